@@ -83,6 +83,61 @@ void zgemm(cudaStream_t st, int batch, int m, int n, int k, double2 alpha, const
   zgemm_batched<<<grid, block, 0, st>>>(m, n, k, alpha, A, lda, sA, opA, B, ldb, sB, beta, C, ldc, sC);
 }
 
+// Where the FP64 products of a call run: the sliced tensor-core GEMM (oz_gemm.cu) with its digit
+// workspace in the handle, or the CUDA-core kernel above (small products, no handle, no memory).
+struct Gemm {
+  Handle* h = nullptr;
+  cudaStream_t st = nullptr;
+  int* err = nullptr;              // device flag of expired waits
+  cudaError_t fail = cudaSuccess;  // first launch error
+};
+
+// the flag lives in the handle's workspace 9; false: products stay on the CUDA cores
+rsfd_status gemm_begin(Handle* h, Gemm& g) {
+  g.h = h;
+  g.st = handle_stream(h);
+  void* p = nullptr;
+  const rsfd_status s = handle_ensure(h, 9, 256, &p);
+  if (s != RSFD_OK) return s;
+  g.err = (int*)p;
+  g.fail = cudaMemsetAsync(g.err, 0, sizeof(int), g.st);
+  return RSFD_OK;
+}
+
+// after the last product: waits for the stream and turns a failed launch or an expired wait into a status
+rsfd_status gemm_end(Gemm& g, const char* who) {
+  int flag = 0;
+  cudaError_t e = g.fail != cudaSuccess ? g.fail : cudaMemcpyAsync(&flag, g.err, sizeof(int), cudaMemcpyDeviceToHost, g.st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(g.st);
+  if (e != cudaSuccess) return handle_fail(g.h, RSFD_ERR_CUDA, std::string(who) + ": " + cudaGetErrorString(e));
+  if (flag) return handle_fail(g.h, RSFD_ERR_TIMEOUT, std::string(who) + ": tensor-core GEMM wait expired");
+  return RSFD_OK;
+}
+
+constexpr size_t kOzWorkMax = (size_t)4 << 30;   // digit workspace of one product, unless one matrix needs more
+
+// C[b] = sign * op(A[b]) B[b] + (add ? C[b] : 0).  Sliced from 8e6 complex multiply-adds on: its three launches
+// cost about 17 us a product, which the FP64 pipe (1.3e11 complex multiply-adds/s) earns back from there.
+// Two products of ns x ns x ns and the rest of rsfd_transmission, CUDA cores / sliced, us: ns = 64, 16 energies
+// (4.2e6) 143 / 154; 192, 1 (7.1e6) 251 / 266; 128, 4 (8.4e6) 242 / 208; 96, 16 (1.4e7) 291 / 190; 256, 16
+// (2.7e8) 3869 / 600.
+void gemm(Gemm& g, int batch, int m, int n, int k, double sign, const double2* A, int lda, long long sA, int opA,
+          const double2* B, int ldb, long long sB, bool add, double2* C, int ldc, long long sC) {
+  if (g.h && k >= 32 && m >= 32 && n >= 16 && (double)m * n * k * batch >= 8e6) {
+    const size_t per = oz_bytes(m, n, k);
+    const size_t want = per * batch < kOzWorkMax ? per * batch : (per > kOzWorkMax ? per : kOzWorkMax);
+    void* w = nullptr;
+    if (handle_ensure(g.h, 8, want, &w) == RSFD_OK) {
+      const cudaError_t e = oz_zgemm(g.st, batch, m, n, k, sign, A, lda, sA, opA, B, ldb, sB, add ? 1 : 0, C, ldc, sC, w,
+                                     want, g.err);
+      if (e != cudaSuccess && g.fail == cudaSuccess) g.fail = e;
+      return;
+    }
+  }
+  zgemm(g.st, batch, m, n, k, make_double2(sign, 0.0), A, lda, sA, opA, B, ldb, sB, make_double2(add ? 1.0 : 0.0, 0.0), C,
+        ldc, sC);
+}
+
 template <typename T>
 __global__ void to_c128(const T* src, double2* dst, long long n) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
@@ -345,8 +400,8 @@ int grid_for(long long n) {
 }
 
 // batched blocked LU of K matrices nb x nb (column-major, contiguous), in place
-void getrf_blocked(cudaStream_t st, double2* M, int nb, int K, int* piv, int* info) {
-  const double2 m1 = make_double2(-1.0, 0.0), one = make_double2(1.0, 0.0);
+void getrf_blocked(Gemm& gc, double2* M, int nb, int K, int* piv, int* info) {
+  cudaStream_t st = gc.st;
   const long long n2 = (long long)nb * nb;
   for (int j0 = 0; j0 < nb; j0 += kPanel) {
     const int jb = nb - j0 < kPanel ? nb - j0 : kPanel;
@@ -356,8 +411,8 @@ void getrf_blocked(cudaStream_t st, double2* M, int nb, int K, int* piv, int* in
     if (rest > 0) {
       panel_trsm<<<grid_for((long long)rest * K), 256, 0, st>>>(M, nb, j0, jb, K);
       // A22 -= L21 U12
-      zgemm(st, K, rest, rest, jb, m1, M + (long long)j0 * nb + j0 + jb, nb, n2, 0, M + (long long)(j0 + jb) * nb + j0,
-            nb, n2, one, M + (long long)(j0 + jb) * nb + j0 + jb, nb, n2);
+      gemm(gc, K, rest, rest, jb, -1.0, M + (long long)j0 * nb + j0 + jb, nb, n2, 0, M + (long long)(j0 + jb) * nb + j0,
+            nb, n2, true, M + (long long)(j0 + jb) * nb + j0 + jb, nb, n2);
     }
   }
 }
@@ -413,12 +468,14 @@ rsfd_status dyson_tc_run(Handle* h, const void* G0, const void* SL, const void* 
   if ((s = handle_ensure(h, 3, sx * Kc * sizeof(double2), &pX)) != RSFD_OK) return s;
   if ((s = handle_ensure(h, 4, sx * Kc * sizeof(double2), &pR)) != RSFD_OK) return s;
   if ((s = handle_ensure(h, 2, (n2 + sx) * Kc * sizeof(float2), &pF)) != RSFD_OK) return s;
-  if ((s = handle_ensure(h, 5, ((long long)Kc * (2 * nb + 1) + 1) * sizeof(int), &pPiv)) != RSFD_OK) return s;
+  if ((s = handle_ensure(h, 5, (long long)Kc * (2 * nb + 1) * sizeof(int), &pPiv)) != RSFD_OK) return s;
   if ((s = handle_ensure(h, 6, (long long)2 * K * sizeof(double), &pRed)) != RSFD_OK) return s;
   if (!fp64in && (s = handle_ensure(h, 0, n2 * Kc * sizeof(double2), &pG0)) != RSFD_OK) return s;
   if (nc < nb && (s = handle_ensure(h, 7, sx * Kc * sizeof(double2), &pB)) != RSFD_OK) return s;
   if ((s = handle_begin(h)) != RSFD_OK) return s;
   cudaStream_t st = handle_stream(h);
+  Gemm gc;
+  if ((s = gemm_begin(h, gc)) != RSFD_OK) return s;
   double2* dM = (double2*)pM;
   double2* dX = (double2*)pX;
   double2* dR = (double2*)pR;
@@ -427,10 +484,8 @@ rsfd_status dyson_tc_run(Handle* h, const void* G0, const void* SL, const void* 
   int* piv = (int*)pPiv;
   int* perm = piv + (long long)Kc * nb;
   int* info = perm + (long long)Kc * nb;
-  int* err = info + Kc;
+  int* err = gc.err;
   double* red = (double*)pRed;
-  const double2 m1 = make_double2(-1.0, 0.0), one = make_double2(1.0, 0.0);
-  DY_CK(h, cudaMemsetAsync(err, 0, sizeof(int), st));
   std::vector<int> hinfo(K, 0);
   for (int k0 = 0; k0 < K; k0 += Kc) {
     const int kb = K - k0 < Kc ? K - k0 : Kc;
@@ -451,8 +506,8 @@ rsfd_status dyson_tc_run(Handle* h, const void* G0, const void* SL, const void* 
     const double2* sl = (const double2*)SL + s2 * k0;
     const double2* sr = (const double2*)SR + s2 * k0;
     set_identity<<<grid_for(tot), 256, 0, st>>>(dM, nb, kb);
-    zgemm(st, kb, nb, ns, ns, m1, g0, nb, n2, 0, sl, ns, s2, one, dM, nb, n2);
-    zgemm(st, kb, nb, ns, ns, m1, g0 + (long long)ns * nb, nb, n2, 0, sr, ns, s2, one, dM + (long long)ns * nb, nb, n2);
+    gemm(gc, kb, nb, ns, ns, -1.0, g0, nb, n2, 0, sl, ns, s2, true, dM, nb, n2);
+    gemm(gc, kb, nb, ns, ns, -1.0, g0 + (long long)ns * nb, nb, n2, 0, sr, ns, s2, true, dM + (long long)ns * nb, nb, n2);
     to_f32_c<<<grid_for(tot), 256, 0, st>>>(dM, dF, tot);
     DY_CK(h, cudaMemsetAsync(info, 0, kb * sizeof(int), st));
     DY_CK(h, getrf_f32_tc(st, dF, nb, kb, piv, info, err));
@@ -460,13 +515,13 @@ rsfd_status dyson_tc_run(Handle* h, const void* G0, const void* SL, const void* 
     set_f32_to_c128<<<grid_for(totx), 256, 0, st>>>(dX, dXf, totx);
     for (int it = 0; it < nref; ++it) {
       copy_c128<<<grid_for(totx), 256, 0, st>>>(b0, dR, totx);
-      zgemm(st, kb, nb, nc, nb, m1, dM, nb, n2, 0, dX, nb, sx, one, dR, nb, sx);
+      gemm(gc, kb, nb, nc, nb, -1.0, dM, nb, n2, 0, dX, nb, sx, true, dR, nb, sx);
       DY_CK(h, getrs_f32_tc(st, dF, piv, nb, kb, (const double2*)dR, nc, dXf, perm, err));
       add_f32_to_c128<<<grid_for(totx), 256, 0, st>>>(dX, dXf, totx);
     }
     if (refres) {
       copy_c128<<<grid_for(totx), 256, 0, st>>>(b0, dR, totx);
-      zgemm(st, kb, nb, nc, nb, m1, dM, nb, n2, 0, dX, nb, sx, one, dR, nb, sx);
+      gemm(gc, kb, nb, nc, nb, -1.0, dM, nb, n2, 0, dX, nb, sx, true, dR, nb, sx);
       frob2_batched<<<kb, 256, 0, st>>>(dR, sx, red + k0);
       frob2_batched<<<kb, 256, 0, st>>>(b0, sx, red + K + k0);
     }
@@ -480,13 +535,10 @@ rsfd_status dyson_tc_run(Handle* h, const void* G0, const void* SL, const void* 
     DY_CK(h, cudaGetLastError());
     DY_CK(h, cudaMemcpyAsync(hinfo.data() + k0, info, kb * sizeof(int), cudaMemcpyDeviceToHost, st));
   }
-  int herr = 0;
-  DY_CK(h, cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, st));
   std::vector<double> hred(2 * K);
   if (refres) DY_CK(h, cudaMemcpyAsync(hred.data(), red, 2 * K * sizeof(double), cudaMemcpyDeviceToHost, st));
-  DY_CK(h, cudaStreamSynchronize(st));
+  if ((s = gemm_end(gc, "rsfd_dyson_boundary")) != RSFD_OK) return s;
   if ((s = handle_end(h)) != RSFD_OK) return s;
-  if (herr) return handle_fail(h, RSFD_ERR_TIMEOUT, "rsfd_dyson_boundary: tensor-core GEMM wait expired");
   if (refres)
     for (int k = 0; k < K; ++k) refres[k] = sqrt(hred[k]) / sqrt(hred[K + k] > 0 ? hred[K + k] : 1.0);
   for (int k = 0; k < K; ++k)
@@ -515,6 +567,8 @@ rsfd_status dyson_run(Handle* h, const void* G0, const void* SL, const void* SR,
   if ((s = handle_ensure(h, 6, (long long)2 * K * sizeof(double), &pRed)) != RSFD_OK) return s;
   if ((s = handle_begin(h)) != RSFD_OK) return s;
   cudaStream_t st = handle_stream(h);
+  Gemm gc;
+  if ((s = gemm_begin(h, gc)) != RSFD_OK) return s;
   double2* dG0 = (double2*)pG0;
   double2* dM = (double2*)pM;
   double2* dLU = (double2*)pLU;
@@ -527,14 +581,13 @@ rsfd_status dyson_run(Handle* h, const void* G0, const void* SL, const void* SR,
   if (fp64) copy_c128<<<grid_for(tot), 256, 0, st>>>((const double2*)G0, dG0, tot);
   else to_c128<float2><<<grid_for(tot), 256, 0, st>>>((const float2*)G0, dG0, tot);
   set_identity<<<grid_for(tot), 256, 0, st>>>(dM, nb, K);
-  const double2 m1 = make_double2(-1.0, 0.0), one = make_double2(1.0, 0.0), zero = make_double2(0.0, 0.0);
   // M[:, :ns] -= G0[:, :ns] SL ;  M[:, ns:] -= G0[:, ns:] SR
-  zgemm(st, K, nb, ns, ns, m1, dG0, nb, n2, 0, (const double2*)SL, ns, (long long)ns * ns, one, dM, nb, n2);
-  zgemm(st, K, nb, ns, ns, m1, dG0 + (long long)ns * nb, nb, n2, 0, (const double2*)SR, ns, (long long)ns * ns, one,
+  gemm(gc, K, nb, ns, ns, -1.0, dG0, nb, n2, 0, (const double2*)SL, ns, (long long)ns * ns, true, dM, nb, n2);
+  gemm(gc, K, nb, ns, ns, -1.0, dG0 + (long long)ns * nb, nb, n2, 0, (const double2*)SR, ns, (long long)ns * ns, true,
         dM + (long long)ns * nb, nb, n2);
   copy_c128<<<grid_for(tot), 256, 0, st>>>(dM, dLU, tot);
   DY_CK(h, cudaMemsetAsync(info, 0, K * sizeof(int), st));
-  getrf_blocked(st, dLU, nb, K, piv, info);
+  getrf_blocked(gc, dLU, nb, K, piv, info);
   // right-hand sides: the first nc columns of every energy, compact (stride sx)
   const double2* b0 = dG0;
   if (nc < nb) {
@@ -551,14 +604,14 @@ rsfd_status dyson_run(Handle* h, const void* G0, const void* SL, const void* SR,
   // iterative refinement in FP64
   for (int it = 0; it < 2; ++it) {
     copy_c128<<<grid_for(totx), 256, 0, st>>>(b0, dR, totx);
-    zgemm(st, K, nb, nc, nb, m1, dM, nb, n2, 0, dX, nb, sx, one, dR, nb, sx);
+    gemm(gc, K, nb, nc, nb, -1.0, dM, nb, n2, 0, dX, nb, sx, true, dR, nb, sx);
     dim3 g((nc + 127) / 128, K);
     zgetrs_batched<<<g, 128, 0, st>>>(dLU, piv, dR, nb, nc);
     axpy_c128<<<grid_for(totx), 256, 0, st>>>(dX, dR, totx);
   }
   if (refres) {
     copy_c128<<<grid_for(totx), 256, 0, st>>>(b0, dR, totx);
-    zgemm(st, K, nb, nc, nb, m1, dM, nb, n2, 0, dX, nb, sx, one, dR, nb, sx);
+    gemm(gc, K, nb, nc, nb, -1.0, dM, nb, n2, 0, dX, nb, sx, true, dR, nb, sx);
     frob2_batched<<<K, 256, 0, st>>>(dR, sx, red);
     frob2_batched<<<K, 256, 0, st>>>(b0, sx, red + K);
   }
@@ -574,14 +627,13 @@ rsfd_status dyson_run(Handle* h, const void* G0, const void* SL, const void* SR,
   DY_CK(h, cudaMemcpyAsync(hinfo.data(), info, K * sizeof(int), cudaMemcpyDeviceToHost, st));
   std::vector<double> hred(2 * K);
   if (refres) DY_CK(h, cudaMemcpyAsync(hred.data(), red, 2 * K * sizeof(double), cudaMemcpyDeviceToHost, st));
-  DY_CK(h, cudaStreamSynchronize(st));
+  if ((s = gemm_end(gc, "rsfd_dyson_boundary")) != RSFD_OK) return s;
   if ((s = handle_end(h)) != RSFD_OK) return s;
   if (refres)
     for (int k = 0; k < K; ++k) refres[k] = sqrt(hred[k]) / sqrt(hred[K + k] > 0 ? hred[K + k] : 1.0);
   for (int k = 0; k < K; ++k)
     if (hinfo[k] != 0)
       return handle_fail(h, RSFD_ERR_BREAKDOWN, "rsfd_dyson_boundary: singular I - G0 Sigma at energy " + std::to_string(k));
-  (void)zero;
   return RSFD_OK;
 }
 
@@ -605,6 +657,8 @@ rsfd_status dyson_tracked_run(Handle* h, int nr, const void* G0, const void* SL,
   if ((s = handle_ensure(h, 7, (2 * bn + r2) * K * sizeof(double2), &pW)) != RSFD_OK) return s;
   if ((s = handle_begin(h)) != RSFD_OK) return s;
   cudaStream_t st = handle_stream(h);
+  Gemm gc;
+  if ((s = gemm_begin(h, gc)) != RSFD_OK) return s;
   double2* dG0 = (double2*)pG0;
   double2* dM = (double2*)pM;
   double2* dLU = (double2*)pLU;
@@ -619,15 +673,14 @@ rsfd_status dyson_tracked_run(Handle* h, int nr, const void* G0, const void* SL,
   const long long rtot = r2 * K, btot = b2 * K, ntot = bn * K;
   if (fp64) copy_c128<<<grid_for(rtot), 256, 0, st>>>((const double2*)G0, dG0, rtot);
   else to_c128<float2><<<grid_for(rtot), 256, 0, st>>>((const float2*)G0, dG0, rtot);
-  const double2 m1 = make_double2(-1.0, 0.0), one = make_double2(1.0, 0.0), zero = make_double2(0.0, 0.0);
   // M = I - G0_bb Sigma (G0_bb: the leading nb x nb block of G0, leading dimension nr)
   set_identity<<<grid_for(btot), 256, 0, st>>>(dM, nb, K);
-  zgemm(st, K, nb, ns, ns, m1, dG0, nr, r2, 0, (const double2*)SL, ns, (long long)ns * ns, one, dM, nb, b2);
-  zgemm(st, K, nb, ns, ns, m1, dG0 + (long long)ns * nr, nr, r2, 0, (const double2*)SR, ns, (long long)ns * ns, one,
+  gemm(gc, K, nb, ns, ns, -1.0, dG0, nr, r2, 0, (const double2*)SL, ns, (long long)ns * ns, true, dM, nb, b2);
+  gemm(gc, K, nb, ns, ns, -1.0, dG0 + (long long)ns * nr, nr, r2, 0, (const double2*)SR, ns, (long long)ns * ns, true,
         dM + (long long)ns * nb, nb, b2);
   copy_c128<<<grid_for(btot), 256, 0, st>>>(dM, dLU, btot);
   DY_CK(h, cudaMemsetAsync(info, 0, K * sizeof(int), st));
-  getrf_blocked(st, dLU, nb, K, piv, info);
+  getrf_blocked(gc, dLU, nb, K, piv, info);
   // Y = M^{-1} G0[b, :] with two FP64 refinement steps
   copy_rows_c128<<<grid_for(ntot), 256, 0, st>>>(dG0, nr, dRHS, nb, nb, nr, K);
   copy_c128<<<grid_for(ntot), 256, 0, st>>>(dRHS, dY, ntot);
@@ -635,21 +688,21 @@ rsfd_status dyson_tracked_run(Handle* h, int nr, const void* G0, const void* SL,
   zgetrs_batched<<<g, 128, 0, st>>>(dLU, piv, dY, nb, nr);
   for (int it = 0; it < 2; ++it) {
     copy_c128<<<grid_for(ntot), 256, 0, st>>>(dRHS, dR, ntot);
-    zgemm(st, K, nb, nr, nb, m1, dM, nb, b2, 0, dY, nb, bn, one, dR, nb, bn);
+    gemm(gc, K, nb, nr, nb, -1.0, dM, nb, b2, 0, dY, nb, bn, true, dR, nb, bn);
     zgetrs_batched<<<g, 128, 0, st>>>(dLU, piv, dR, nb, nr);
     axpy_c128<<<grid_for(ntot), 256, 0, st>>>(dY, dR, ntot);
   }
   if (refres) {
     copy_c128<<<grid_for(ntot), 256, 0, st>>>(dRHS, dR, ntot);
-    zgemm(st, K, nb, nr, nb, m1, dM, nb, b2, 0, dY, nb, bn, one, dR, nb, bn);
+    gemm(gc, K, nb, nr, nb, -1.0, dM, nb, b2, 0, dY, nb, bn, true, dR, nb, bn);
     frob2_batched<<<K, 256, 0, st>>>(dR, bn, red);
     frob2_batched<<<K, 256, 0, st>>>(dRHS, bn, red + K);
   }
   // W = Sigma Y (block-diagonal Sigma), then G = G0 + G0[:, b] W
-  zgemm(st, K, ns, nr, ns, one, (const double2*)SL, ns, (long long)ns * ns, 0, dY, nb, bn, zero, dW, nb, bn);
-  zgemm(st, K, ns, nr, ns, one, (const double2*)SR, ns, (long long)ns * ns, 0, dY + ns, nb, bn, zero, dW + ns, nb, bn);
+  gemm(gc, K, ns, nr, ns, 1.0, (const double2*)SL, ns, (long long)ns * ns, 0, dY, nb, bn, false, dW, nb, bn);
+  gemm(gc, K, ns, nr, ns, 1.0, (const double2*)SR, ns, (long long)ns * ns, 0, dY + ns, nb, bn, false, dW + ns, nb, bn);
   copy_c128<<<grid_for(rtot), 256, 0, st>>>(dG0, dX, rtot);
-  zgemm(st, K, nr, nr, nb, one, dG0, nr, r2, 0, dW, nb, bn, one, dX, nr, r2);
+  gemm(gc, K, nr, nr, nb, 1.0, dG0, nr, r2, 0, dW, nb, bn, true, dX, nr, r2);
   if (fp64) copy_c128<<<grid_for(rtot), 256, 0, st>>>(dX, (double2*)G, rtot);
   else from_c128_f<<<grid_for(rtot), 256, 0, st>>>(dX, (float2*)G, rtot);
   DY_CK(h, cudaGetLastError());
@@ -657,7 +710,7 @@ rsfd_status dyson_tracked_run(Handle* h, int nr, const void* G0, const void* SL,
   DY_CK(h, cudaMemcpyAsync(hinfo.data(), info, K * sizeof(int), cudaMemcpyDeviceToHost, st));
   std::vector<double> hred(2 * K);
   if (refres) DY_CK(h, cudaMemcpyAsync(hred.data(), red, 2 * K * sizeof(double), cudaMemcpyDeviceToHost, st));
-  DY_CK(h, cudaStreamSynchronize(st));
+  if ((s = gemm_end(gc, "rsfd_dyson_tracked")) != RSFD_OK) return s;
   if ((s = handle_end(h)) != RSFD_OK) return s;
   if (refres)
     for (int k = 0; k < K; ++k) refres[k] = sqrt(hred[k]) / sqrt(hred[K + k] > 0 ? hred[K + k] : 1.0);
@@ -778,6 +831,8 @@ rsfd_status lead_decimation_run(Handle* h, const double* VL, const double* VR, c
   if ((s = handle_ensure(h, 6, (size_t)Kc * (sizeof(double2) + sizeof(double)), &pZ)) != RSFD_OK) return s;
   if ((s = handle_begin(h)) != RSFD_OK) return s;
   cudaStream_t st = handle_stream(h);
+  Gemm gc;
+  if ((s = gemm_begin(h, gc)) != RSFD_OK) return s;
   double2* W = (double2*)pW;
   double2 *eps_s = W, *eps = W + n2 * Kc, *al = W + 2 * n2 * Kc, *be = W + 3 * n2 * Kc, *A = W + 4 * n2 * Kc;
   double2 *Y = W + 5 * n2 * Kc, *rhs = W + 7 * n2 * Kc, *P1 = W + 9 * n2 * Kc, *P2 = W + 10 * n2 * Kc;
@@ -786,7 +841,6 @@ rsfd_status lead_decimation_run(Handle* h, const double* VL, const double* VR, c
   int* info = piv + (long long)Kc * n;
   double2* dZ = (double2*)pZ;
   double* dmax = (double*)(dZ + Kc);
-  const double2 one = make_double2(1.0, 0.0), zero = make_double2(0.0, 0.0);
   DY_CK(h, cudaMemcpyAsync(dH01, H01.data(), n2 * sizeof(double2), cudaMemcpyHostToDevice, st));
   DY_CK(h, cudaMemcpyAsync(dH01T, H01T.data(), n2 * sizeof(double2), cudaMemcpyHostToDevice, st));
   int it_max = 0;
@@ -818,7 +872,7 @@ rsfd_status lead_decimation_run(Handle* h, const double* VL, const double* VR, c
         // g [alpha | beta] by LU of Z - eps
         zi_minus<<<grid_for(tot), 256, 0, st>>>(A, eps, dZ, n, kb);
         DY_CK(h, cudaMemsetAsync(info, 0, kb * sizeof(int), st));
-        getrf_blocked(st, A, n, kb, piv, info);
+        getrf_blocked(gc, A, n, kb, piv, info);
         concat_cols<<<grid_for(2 * tot), 256, 0, st>>>(al, be, rhs, n2, kb);
         copy_c128<<<grid_for(2 * tot), 256, 0, st>>>(rhs, Y, 2 * tot);
         {
@@ -828,14 +882,14 @@ rsfd_status lead_decimation_run(Handle* h, const double* VL, const double* VR, c
         const double2* ga = Y;        // g alpha, per energy stride 2 n2
         const double2* gb = Y + n2;   // g beta
         // P1 = alpha g beta, P2 = beta g alpha
-        zgemm(st, kb, n, n, n, one, al, n, n2, 0, gb, n, 2 * n2, zero, P1, n, n2);
-        zgemm(st, kb, n, n, n, one, be, n, n2, 0, ga, n, 2 * n2, zero, P2, n, n2);
+        gemm(gc, kb, n, n, n, 1.0, al, n, n2, 0, gb, n, 2 * n2, false, P1, n, n2);
+        gemm(gc, kb, n, n, n, 1.0, be, n, n2, 0, ga, n, 2 * n2, false, P2, n, n2);
         axpy_c128<<<grid_for(tot), 256, 0, st>>>(eps_s, P1, tot);
         axpy_c128<<<grid_for(tot), 256, 0, st>>>(eps, P1, tot);
         axpy_c128<<<grid_for(tot), 256, 0, st>>>(eps, P2, tot);
         // alpha <- alpha g alpha, beta <- beta g beta (through the product buffers)
-        zgemm(st, kb, n, n, n, one, al, n, n2, 0, ga, n, 2 * n2, zero, P1, n, n2);
-        zgemm(st, kb, n, n, n, one, be, n, n2, 0, gb, n, 2 * n2, zero, P2, n, n2);
+        gemm(gc, kb, n, n, n, 1.0, al, n, n2, 0, ga, n, 2 * n2, false, P1, n, n2);
+        gemm(gc, kb, n, n, n, 1.0, be, n, n2, 0, gb, n, 2 * n2, false, P2, n, n2);
         copy_c128<<<grid_for(tot), 256, 0, st>>>(P1, al, tot);
         copy_c128<<<grid_for(tot), 256, 0, st>>>(P2, be, tot);
       }
@@ -845,16 +899,16 @@ rsfd_status lead_decimation_run(Handle* h, const double* VL, const double* VR, c
       //   Sigma_R = H01 g_s H01^T, Sigma_L = H01^T g_s H01
       zi_minus<<<grid_for(tot), 256, 0, st>>>(A, eps_s, dZ, n, kb);
       DY_CK(h, cudaMemsetAsync(info, 0, kb * sizeof(int), st));
-      getrf_blocked(st, A, n, kb, piv, info);
+      getrf_blocked(gc, A, n, kb, piv, info);
       bcast_c128<<<grid_for(tot), 256, 0, st>>>(lead == 0 ? dH01T : dH01, Y, n2, kb);
       {
         dim3 g((n + 127) / 128, kb);
         zgetrs_batched<<<g, 128, 0, st>>>(A, piv, Y, n, n);
       }
-      zgemm(st, kb, n, n, n, one, lead == 0 ? dH01 : dH01T, n, 0, 0, Y, n, n2, zero, out + n2 * k0, n, n2);
+      gemm(gc, kb, n, n, n, 1.0, lead == 0 ? dH01 : dH01T, n, 0, 0, Y, n, n2, false, out + n2 * k0, n, n2);
       std::vector<int> hinfo(kb);
       DY_CK(h, cudaMemcpyAsync(hinfo.data(), info, kb * sizeof(int), cudaMemcpyDeviceToHost, st));
-      DY_CK(h, cudaStreamSynchronize(st));
+      if ((s = gemm_end(gc, "rsfd_lead_sigma_decimation")) != RSFD_OK) return s;
       for (int k = 0; k < kb; ++k)
         if (hinfo[k] != 0)
           return handle_fail(h, RSFD_ERR_BREAKDOWN, "rsfd_lead_sigma_decimation: singular Z - eps at energy " +
@@ -884,23 +938,24 @@ rsfd_status transmission_run(Handle* h, const void* G, const void* SL, const voi
   if ((s = handle_ensure(h, 6, (long long)2 * K * sizeof(double), &pT)) != RSFD_OK) return s;
   if ((s = handle_begin(h)) != RSFD_OK) return s;
   cudaStream_t st = handle_stream(h);
+  Gemm gc;
+  if ((s = gemm_begin(h, gc)) != RSFD_OK) return s;
   double2* dG = (double2*)pG;
   const long long tot = n2 * K;
   if (fp64) copy_c128<<<grid_for(tot), 256, 0, st>>>((const double2*)G, dG, tot);
   else to_c128<float2><<<grid_for(tot), 256, 0, st>>>((const float2*)G, dG, tot);
   gamma_batched<<<grid_for(s2 * K), 256, 0, st>>>((const double2*)SL, (double2*)pGL, ns, K);
   gamma_batched<<<grid_for(s2 * K), 256, 0, st>>>((const double2*)SR, (double2*)pGR, ns, K);
-  const double2 one = make_double2(1.0, 0.0), zero = make_double2(0.0, 0.0);
   const double2* GRL = dG + ns;   // rows ns.., cols 0..ns-1, leading dimension nb
   // W1 = Gamma_R G_RL ; W2 = G_RL^H W1
-  zgemm(st, K, ns, ns, ns, one, (const double2*)pGR, ns, s2, 0, GRL, nb, n2, zero, (double2*)pW1, ns, s2);
-  zgemm(st, K, ns, ns, ns, one, GRL, nb, n2, 1, (const double2*)pW1, ns, s2, zero, (double2*)pW2, ns, s2);
+  gemm(gc, K, ns, ns, ns, 1.0, (const double2*)pGR, ns, s2, 0, GRL, nb, n2, false, (double2*)pW1, ns, s2);
+  gemm(gc, K, ns, ns, ns, 1.0, GRL, nb, n2, 1, (const double2*)pW1, ns, s2, false, (double2*)pW2, ns, s2);
   double* dT = (double*)pT;
   trace_prod_batched<<<K, 256, 0, st>>>((const double2*)pGL, (const double2*)pW2, ns, dT, dT + K);
   DY_CK(h, cudaGetLastError());
   std::vector<double> hT(2 * K);
   DY_CK(h, cudaMemcpyAsync(hT.data(), dT, 2 * K * sizeof(double), cudaMemcpyDeviceToHost, st));
-  DY_CK(h, cudaStreamSynchronize(st));
+  if ((s = gemm_end(gc, "rsfd_transmission")) != RSFD_OK) return s;
   if ((s = handle_end(h)) != RSFD_OK) return s;
   for (int k = 0; k < K; ++k) T[k] = hT[k];
   return RSFD_OK;
@@ -990,32 +1045,33 @@ rsfd_status dyson_noalloc_run(int32_t nb, int32_t K, const void* G0_bb, const vo
   base += align256((size_t)3 * K * sizeof(double));
   int* bad = (int*)base;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  Gemm gc;   // no handle: the CUDA-core products
+  gc.st = st;
   const double2* G0 = (const double2*)G0_bb;
   double2* dX = (double2*)G_bb;
   const long long tot = n2 * K;
-  const double2 m1 = make_double2(-1.0, 0.0), one = make_double2(1.0, 0.0);
   // the scratch keeps the previous call's contents: clear the flags that must start at zero
   e = cudaMemsetAsync(info, 0, K * sizeof(int), st);
   if (e != cudaSuccess) return handle_fail(nullptr, RSFD_ERR_CUDA, std::string("cudaMemsetAsync: ") + cudaGetErrorString(e));
   fill_int<<<1, 1, 0, st>>>(bad, K);
   set_identity<<<grid_for(tot), 256, 0, st>>>(dM, nb, K);
   const int ns = nb / 2;
-  zgemm(st, K, nb, ns, ns, m1, G0, nb, n2, 0, (const double2*)Sigma_L, ns, (long long)ns * ns, one, dM, nb, n2);
-  zgemm(st, K, nb, ns, ns, m1, G0 + (long long)ns * nb, nb, n2, 0, (const double2*)Sigma_R, ns, (long long)ns * ns, one,
+  gemm(gc, K, nb, ns, ns, -1.0, G0, nb, n2, 0, (const double2*)Sigma_L, ns, (long long)ns * ns, true, dM, nb, n2);
+  gemm(gc, K, nb, ns, ns, -1.0, G0 + (long long)ns * nb, nb, n2, 0, (const double2*)Sigma_R, ns, (long long)ns * ns, true,
         dM + (long long)ns * nb, nb, n2);
   copy_c128<<<grid_for(tot), 256, 0, st>>>(dM, dLU, tot);
-  getrf_blocked(st, dLU, nb, K, piv, info);
+  getrf_blocked(gc, dLU, nb, K, piv, info);
   copy_c128<<<grid_for(tot), 256, 0, st>>>(G0, dX, tot);
   dim3 g((nb + 127) / 128, K);
   zgetrs_batched<<<g, 128, 0, st>>>(dLU, piv, dX, nb, nb);
   for (int it = 0; it < 2; ++it) {
     copy_c128<<<grid_for(tot), 256, 0, st>>>(G0, dR, tot);
-    zgemm(st, K, nb, nb, nb, m1, dM, nb, n2, 0, dX, nb, n2, one, dR, nb, n2);
+    gemm(gc, K, nb, nb, nb, -1.0, dM, nb, n2, 0, dX, nb, n2, true, dR, nb, n2);
     zgetrs_batched<<<g, 128, 0, st>>>(dLU, piv, dR, nb, nb);
     axpy_c128<<<grid_for(tot), 256, 0, st>>>(dX, dR, tot);
   }
   copy_c128<<<grid_for(tot), 256, 0, st>>>(G0, dR, tot);
-  zgemm(st, K, nb, nb, nb, m1, dM, nb, n2, 0, dX, nb, n2, one, dR, nb, n2);
+  gemm(gc, K, nb, nb, nb, -1.0, dM, nb, n2, 0, dX, nb, n2, true, dR, nb, n2);
   frob2_batched<<<K, 256, 0, st>>>(dR, n2, red);
   frob2_batched<<<K, 256, 0, st>>>(G0, n2, red + K);
   noalloc_finish<<<1, 256, 0, st>>>(info, red, K, bad, red + 2 * K);

@@ -1,0 +1,526 @@
+// Complex FP64 GEMM on the tensor cores by error-free slicing (the scheme of Ozaki, Ogita, Oishi and
+// Rump, "Error-free transformations of matrix multiplication by using fast routines of matrix
+// multiplication and its applications", Numer. Algorithms 59, 2012), for the Dyson step, the
+// transmission and the lead decimation, whose matrix products are FP64.
+//
+// Why: the FP64 pipe of this GPU does about 0.5e12 FMA/s, 1/68 of its FP32 rate and 1/2000 of its
+// 16-bit tensor rate, and those products were 85-97 % of the Dyson step.
+//
+// Arithmetic.  Every row of A (column of B) is scaled by a power of two so that its largest component
+// is below 1 and written as a 62-bit fixed-point integer X = rint(x 2^62); X is cut into 8 balanced
+// base-256 digits in [-128, 127] (the leading one within +-65), which are exact in bf16.  A product of
+// digits is at most 2^14, so the tensor core's FP32 sums are exact while a sum has at most 2^10 terms.
+// Digit pairs (i, j) of equal weight 256^-(i+j) share an accumulator; pairs with i + j <= 9 are kept (36
+// of 64; the dropped ones are below 2^-62 of the row and column maxima per term).  The accumulators are
+// emptied every 128 complex k (256 real products): the sums of weights 0..3 then have at most 4 x 256
+// terms and are exact; those of weights 4..7 (2^-32 and less) may round once at 2^-24, below 2^-56.
+// They are added to 64-bit integers, so the k-sum has no further rounding; the result is rounded to
+// FP64 once.  Elements below 2^-9 of their row's (column's) largest lose bits below 2^-63 of it.
+//
+// Kernel.  One CTA makes a 128 x 32 tile of complex C: eight accumulators of 128 x 32 for Re and eight for
+// Im fill the 512 columns of tensor memory.  The digit planes are laid out in global memory exactly as
+// the tensor core wants them in shared memory (K-major core matrices, no swizzle), so a k-step of 16
+// is three contiguous bulk copies: one plane of A (8 digits x 128 rows, 32 KB), the other, and both
+// planes of B (8 digits x 32 columns each, 16 KB).  The 8 digits of B are stacked along N, so digit i of A
+// meets digits 1..9-i of B in ONE MMA of N = 32 (9 - i) whose columns fall onto the accumulators of
+// weights i-1..7.  18 warps: 16 read the accumulators, one thread of the 17th issues the copies,
+// one thread of the 18th the MMAs.
+//
+// Bound: tensor rate (144 real bf16 MACs per complex FP64 MAC; 36 B per clock and SM of operands from L2).
+// Measured: 16 products of 1024^3 in 4.6 ms, 3.8e12 complex multiply-adds/s, 1.08 PFLOP/s of bf16 MMAs = 0.56 of
+// the measured cuBLAS bf16 burst; the CUDA-core kernel takes 132 ms for the same (FP64 pipe, 1.3e11/s).
+
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include "rsfd_internal.cuh"
+
+namespace rsfd {
+namespace {
+
+constexpr int OZ_S = 8;                       // digits
+constexpr int OZ_BM = 128;                    // rows of C per CTA
+constexpr int OZ_BN = 32;                     // columns of C per CTA
+constexpr int OZ_KS = 16;                     // complex k per step (one MMA depth)
+constexpr int OZ_CHUNK = 8;                   // k-steps between two emptyings of the accumulators
+constexpr int OZ_ABLK = OZ_S * OZ_BM * OZ_KS * 2;        // bytes of one plane of A per k-step (32 KB)
+constexpr int OZ_BPLANE = OZ_S * OZ_BN * OZ_KS * 2;      // bytes of one plane of B per k-step (8 KB)
+constexpr int OZ_BBLK = 2 * OZ_BPLANE;
+constexpr int OZ_NA = 5;                      // ring of A planes
+constexpr int OZ_NB = 3;                      // ring of B blocks
+constexpr int OZ_SMEM = OZ_NA * OZ_ABLK + OZ_NB * OZ_BBLK + 1024;
+constexpr int OZ_EPI = 512;                   // epilogue threads (16 warps: 64 accumulator registers each)
+constexpr int OZ_EC = OZ_BN / (OZ_EPI / 128); // columns per epilogue thread
+constexpr int OZ_THREADS = OZ_EPI + 64;
+static_assert(OZ_EC == 8, "the accumulators are read eight columns at a time");
+constexpr uint32_t OZ_SBO = 128;
+constexpr uint32_t OZ_LBO_A = (OZ_BM / 8) * 128;
+constexpr uint32_t OZ_LBO_B = (OZ_S * OZ_BN / 8) * 128;
+constexpr int kOzWaitCap = 1 << 12;           // attempts of a bounded wait, each up to 1 ms
+constexpr uint32_t kOzHintNs = 1000000;
+
+__device__ __forceinline__ uint32_t oz_saddr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+__device__ __forceinline__ bool oz_wait(uint32_t bar, uint32_t parity) {
+  for (int i = 0; i < kOzWaitCap; ++i) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity), "r"(kOzHintNs)
+        : "memory");
+    if (ok) return true;
+  }
+  return false;
+}
+__device__ __forceinline__ void oz_bulk(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(bar)
+               : "memory");
+}
+__device__ __forceinline__ uint64_t oz_desc(uint32_t saddr, uint32_t lbo) {
+  uint64_t d = 0;
+  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
+  d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
+  d |= (uint64_t)((OZ_SBO >> 4) & 0x3FFFu) << 32;
+  d |= (uint64_t)1 << 46;
+  return d;
+}
+// kind::f16 instruction descriptor: FP32 accumulator, bf16 A and B, both K-major, M = 128
+__host__ __device__ constexpr uint32_t oz_idesc(int N, int negA) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)negA << 13) | ((uint32_t)(N >> 3) << 17) |
+         ((uint32_t)(OZ_BM >> 4) << 24);
+}
+__device__ __forceinline__ void oz_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
+      "l"(a), "l"(b), "r"(idesc), "r"(acc)
+      : "memory");
+}
+__device__ __forceinline__ void oz_commit(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void oz_tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+}
+
+// one operand: element (row, k) of matrix b at p[b sb + row rs + k ks] (row: a row of op(A) or a column of B)
+struct OzOperand {
+  const double2* p;
+  long long sb, rs, ks;
+  int rows;         // m or n
+  int conj;
+  int is_b;
+  unsigned int* ex;     // [batch][rows_pad] high words of the largest component
+  unsigned char* dig;   // digit planes
+  int rows_pad;
+};
+struct OzSplit {
+  OzOperand o[2];
+  int k, ksteps, batch;
+};
+
+// Largest component of every row: high words (sign cleared) compared as integers.  Rows contiguous in
+// memory (rs = 1): a thread per row; k contiguous: a warp per row.  Bound: one read of the operand.
+__global__ void __launch_bounds__(256) oz_rowmax(OzSplit q) {
+  const OzOperand& o = q.o[blockIdx.z & 1];
+  const int b = blockIdx.z >> 1;
+  const double2* p = o.p + b * o.sb;
+  if (o.ks != 1) {
+    const int row = blockIdx.x * 32 + (threadIdx.x & 31);
+    unsigned int m = 0;
+    if (row < o.rows)
+      for (int k = blockIdx.y * 64 + (threadIdx.x >> 5); k < min(q.k, (int)blockIdx.y * 64 + 64); k += 8) {
+        const double2 v = p[row * o.rs + k * o.ks];
+        m = max(m, max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu));
+      }
+    __shared__ unsigned int s[8][32];
+    s[threadIdx.x >> 5][threadIdx.x & 31] = m;
+    __syncthreads();
+    if (threadIdx.x < 32 && row < o.rows) {
+#pragma unroll
+      for (int w = 1; w < 8; ++w) m = max(m, s[w][threadIdx.x]);
+      atomicMax(o.ex + (size_t)b * o.rows_pad + row, m);
+    }
+  } else {
+    // 32 rows per block, a warp takes 4 of them
+    for (int r = threadIdx.x >> 5; r < 32; r += 8) {
+      const int row = blockIdx.x * 32 + r;
+      if (row >= o.rows) break;
+      unsigned int m = 0;
+      for (int k = blockIdx.y * 64 + (threadIdx.x & 31); k < min(q.k, (int)blockIdx.y * 64 + 64); k += 32) {
+        const double2 v = p[row * o.rs + k];
+        m = max(m, max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu));
+      }
+      m = __reduce_max_sync(0xffffffffu, m);
+      if ((threadIdx.x & 31) == 0) atomicMax(o.ex + (size_t)b * o.rows_pad + row, m);
+    }
+  }
+}
+
+// binary exponent se with |x| < 2^se for every component of a row whose largest high word is w
+__device__ __forceinline__ int oz_exponent(unsigned int w) {
+  const int e = (int)(w >> 20);
+  return (e < 1 ? 1 : e) - 1022;
+}
+
+// fixed point rint(x 2^(62 - se)), integer arithmetic only
+__device__ __forceinline__ long long oz_fixed(double x, int se) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+  const int e = (int)((u >> 52) & 0x7ff);
+  unsigned long long m = u & 0xfffffffffffffull;
+  if (e > 0) m |= 1ull << 52;
+  const int sh = (e < 1 ? 1 : e) - 1075 - se + 62;   // at most 9
+  if (sh >= 0) m <<= sh;
+  else m = sh > -62 ? (m + (1ull << (-sh - 1))) >> (-sh) : 0ull;
+  return (u >> 63) ? -(long long)m : (long long)m;
+}
+
+// Digit planes.  A thread takes 8 consecutive k of one row: 8 loads, then one 16-byte store per digit and
+// plane (consecutive rows are 16 bytes apart, so a warp stores 512 contiguous bytes).
+// Bound: the stores (32 bytes per element) and one read.
+__global__ void __launch_bounds__(256) oz_digits(OzSplit q) {
+  const OzOperand& o = q.o[blockIdx.z & 1];
+  const int b = blockIdx.z >> 1;
+  const int row = blockIdx.x * 32 + (threadIdx.x & 31);
+  const int kg = blockIdx.y * 8 + (threadIdx.x >> 5);   // group of 8 k
+  if (row >= o.rows_pad || kg >= 2 * q.ksteps) return;
+  const double2* p = o.p + b * o.sb + (long long)row * o.rs;
+  const int se = row < o.rows ? oz_exponent(o.ex[(size_t)b * o.rows_pad + row]) : 0;
+  long long xr[8], xi[8];
+#pragma unroll
+  for (int t = 0; t < 8; ++t) {
+    const int k = kg * 8 + t;
+    double2 v = make_double2(0.0, 0.0);
+    if (row < o.rows && k < q.k) v = p[k * o.ks];
+    if (o.conj) v.y = -v.y;
+    xr[t] = oz_fixed(v.x, se);
+    xi[t] = oz_fixed(v.y, se);
+  }
+  const int ks = kg >> 1, kh = kg & 1;
+  unsigned char *d0, *d1;   // digit 0 (leading) of the two planes
+  uint32_t step;            // bytes from one digit to the next
+  if (o.is_b) {
+    const int nt = row / OZ_BN, r = row % OZ_BN;
+    unsigned char* blk = o.dig + (((size_t)b * (o.rows_pad / OZ_BN) + nt) * q.ksteps + ks) * OZ_BBLK;
+    d0 = blk + kh * OZ_LBO_B + r * 16;      // stacked row = digit * 32 + r
+    d1 = d0 + OZ_BPLANE;
+    step = OZ_BN * 16;
+  } else {
+    const int mt = row / OZ_BM, r = row % OZ_BM;
+    unsigned char* blk = o.dig + (((size_t)b * (o.rows_pad / OZ_BM) + mt) * q.ksteps + ks) * (2 * OZ_ABLK);
+    d0 = blk + kh * OZ_LBO_A + r * 16;
+    d1 = d0 + OZ_ABLK;
+    step = OZ_BM * OZ_KS * 2;
+  }
+#pragma unroll
+  for (int s = OZ_S - 1; s >= 0; --s) {
+    uint32_t wr[4], wi[4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      float f[4];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        long long &a = xr[2 * t + h], &c = xi[2 * t + h];
+        const int da = s > 0 ? (int)(signed char)(a & 0xff) : (int)a;
+        const int dc = s > 0 ? (int)(signed char)(c & 0xff) : (int)c;
+        a = (a - da) >> 8;
+        c = (c - dc) >> 8;
+        f[h] = (float)da;
+        f[2 + h] = (float)dc;
+      }
+      asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(wr[t]) : "f"(f[1]), "f"(f[0]));
+      asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(wi[t]) : "f"(f[3]), "f"(f[2]));
+    }
+    *(uint4*)(d0 + (size_t)s * step) = make_uint4(wr[0], wr[1], wr[2], wr[3]);
+    *(uint4*)(d1 + (size_t)s * step) = make_uint4(wi[0], wi[1], wi[2], wi[3]);
+  }
+}
+
+struct OzGemm {
+  const unsigned char *A, *B;
+  const unsigned int *exA, *exB;
+  int m, n, m_pad, n_pad, ksteps;
+  double sign;        // alpha (+1 or -1)
+  int add;            // 1: add C
+  double2* C;
+  int ldc;
+  long long sC;
+  int* err;
+};
+
+__global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_kernel(OzGemm q) {
+  extern __shared__ __align__(1024) unsigned char oz_smem_raw[];
+  __shared__ __align__(8) uint64_t fullA[OZ_NA], emptyA[OZ_NA], fullB[OZ_NB], emptyB[OZ_NB], accFull, accEmpty, mmaDone;
+  __shared__ uint32_t tmem_s;
+  __shared__ volatile int s_abort;
+  unsigned char* smem = (unsigned char*)(((uintptr_t)oz_smem_raw + 1023) & ~(uintptr_t)1023);
+  unsigned char* sA = smem;
+  unsigned char* sB = smem + OZ_NA * OZ_ABLK;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int mt = blockIdx.x, nt = blockIdx.y, b = blockIdx.z;
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(oz_saddr(&tmem_s)), "r"(512)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  if (tid == 0) {
+    for (int i = 0; i < OZ_NA; ++i) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(oz_saddr(&fullA[i])) : "memory");
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(oz_saddr(&emptyA[i])) : "memory");
+    }
+    for (int i = 0; i < OZ_NB; ++i) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(oz_saddr(&fullB[i])) : "memory");
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(oz_saddr(&emptyB[i])) : "memory");
+    }
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(oz_saddr(&accFull)) : "memory");
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(oz_saddr(&mmaDone)) : "memory");
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(oz_saddr(&accEmpty)), "r"(OZ_EPI) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    s_abort = 0;
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = tmem_s;
+  const int ksteps = q.ksteps;
+  const int nchunks = (ksteps + OZ_CHUNK - 1) / OZ_CHUNK;
+
+  if (warp == OZ_EPI / 32) {
+    // copies: per k-step B (both planes), then the two planes of A
+    if (lane == 0) {
+      const unsigned char* gA = q.A + ((size_t)b * (q.m_pad / OZ_BM) + mt) * ksteps * (2 * OZ_ABLK);
+      const unsigned char* gB = q.B + ((size_t)b * (q.n_pad / OZ_BN) + nt) * ksteps * OZ_BBLK;
+      bool ok = true;
+      int issuedA = 0, issuedB = 0;
+      for (int t = 0; t < ksteps && ok; ++t) {
+        const int sb = t % OZ_NB;
+        if (t >= OZ_NB) ok = oz_wait(oz_saddr(&emptyB[sb]), (uint32_t)((t / OZ_NB - 1) & 1));
+        if (!ok || s_abort) break;
+        oz_bulk(oz_saddr(sB + sb * OZ_BBLK), gB + (size_t)t * OZ_BBLK, OZ_BBLK, oz_saddr(&fullB[sb]));
+        issuedB = t + 1;
+        for (int h = 0; h < 2 && ok; ++h) {
+          const int a = 2 * t + h, sa = a % OZ_NA;
+          if (a >= OZ_NA) ok = oz_wait(oz_saddr(&emptyA[sa]), (uint32_t)((a / OZ_NA - 1) & 1));
+          if (!ok || s_abort) break;
+          oz_bulk(oz_saddr(sA + sa * OZ_ABLK), gA + (size_t)a * OZ_ABLK, OZ_ABLK, oz_saddr(&fullA[sa]));
+          issuedA = a + 1;
+        }
+      }
+      if (!ok || s_abort) {
+        // let the copies in flight land before the CTA's shared memory is released: per ring entry
+        // the last one issued (earlier ones completed before the entry was refilled)
+        s_abort = 1;
+        atomicExch(q.err, 1);
+        for (int a = max(0, issuedA - OZ_NA); a < issuedA; ++a)
+          oz_wait(oz_saddr(&fullA[a % OZ_NA]), (uint32_t)((a / OZ_NA) & 1));
+        for (int c = max(0, issuedB - OZ_NB); c < issuedB; ++c)
+          oz_wait(oz_saddr(&fullB[c % OZ_NB]), (uint32_t)((c / OZ_NB) & 1));
+      }
+    }
+  } else if (warp == OZ_EPI / 32 + 1) {
+    if (lane == 0) {
+      bool ok = true;
+      for (int t = 0; t < ksteps && ok; ++t) {
+        const int c = t / OZ_CHUNK;
+        const bool first = t % OZ_CHUNK == 0;
+        if (first && c > 0) {
+          ok = oz_wait(oz_saddr(&accEmpty), (uint32_t)((c - 1) & 1));
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        }
+        const int sb = t % OZ_NB;
+        ok = ok && oz_wait(oz_saddr(&fullB[sb]), (uint32_t)((t / OZ_NB) & 1));
+        const uint32_t b0 = oz_saddr(sB + sb * OZ_BBLK);
+        const uint64_t bre = oz_desc(b0, OZ_LBO_B), bim = oz_desc(b0 + OZ_BPLANE, OZ_LBO_B);
+        for (int h = 0; h < 2 && ok; ++h) {
+          const int a = 2 * t + h, sa = a % OZ_NA;
+          ok = oz_wait(oz_saddr(&fullA[sa]), (uint32_t)((a / OZ_NA) & 1));
+          if (!ok || s_abort) {
+            ok = false;
+            break;
+          }
+          const uint32_t a0 = oz_saddr(sA + sa * OZ_ABLK);
+          // h = 0: Re += Ar Br, Im += Ar Bi;  h = 1: Re -= Ai Bi, Im += Ai Br
+#pragma unroll
+          for (int i = 0; i < OZ_S; ++i) {
+            const uint64_t ad = oz_desc(a0 + i * (OZ_BM * OZ_KS * 2), OZ_LBO_A);
+            const uint32_t acc = (first && h == 0 && i == 0) ? 0u : 1u;
+            const int N = OZ_BN * (OZ_S - i);
+            oz_mma(tmem + i * OZ_BN, ad, h ? bim : bre, h ? oz_idesc(N, 1) : oz_idesc(N, 0), acc);
+            oz_mma(tmem + 256 + i * OZ_BN, ad, h ? bre : bim, oz_idesc(N, 0), acc);
+          }
+          oz_commit(oz_saddr(&emptyA[sa]));
+        }
+        if (!ok) break;
+        oz_commit(oz_saddr(&emptyB[sb]));
+        if (t % OZ_CHUNK == OZ_CHUNK - 1 || t == ksteps - 1) oz_commit(oz_saddr(&accFull));
+      }
+      if (!ok) {
+        // the MMAs issued so far end before the tensor memory is given back
+        s_abort = 1;
+        atomicExch(q.err, 1);
+        oz_commit(oz_saddr(&mmaDone));
+        oz_wait(oz_saddr(&mmaDone), 0);
+      }
+    }
+  } else {
+    // epilogue threads: row 32 (warp % 4) + lane, columns OZ_EC (warp / 4) ... of Re and of Im
+    const int ch = (warp >> 2) * OZ_EC;
+    const uint32_t tl = tmem + ((uint32_t)((warp & 3) * 32) << 16) + ch;
+    long long hi[2][OZ_EC], lo[2][OZ_EC];
+#pragma unroll
+    for (int p = 0; p < 2; ++p)
+#pragma unroll
+      for (int j = 0; j < OZ_EC; ++j) hi[p][j] = lo[p][j] = 0;
+    bool ok = true;
+    for (int c = 0; c < nchunks; ++c) {
+      ok = oz_wait(oz_saddr(&accFull), (uint32_t)(c & 1));
+      if (!ok || s_abort) {
+        ok = false;
+        break;
+      }
+      __syncwarp();
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+      for (int p = 0; p < 2; ++p) {
+#pragma unroll
+        for (int d = 0; d < OZ_S; d += 2) {
+          uint32_t r0[OZ_EC], r1[OZ_EC];
+          oz_tmem_ld8(tl + p * 256 + d * OZ_BN, r0);
+          oz_tmem_ld8(tl + p * 256 + (d + 1) * OZ_BN, r1);
+          // the registers pass through the wait so that no use moves above it
+          asm volatile("tcgen05.wait::ld.sync.aligned;"
+                       : "+r"(r0[0]), "+r"(r0[1]), "+r"(r0[2]), "+r"(r0[3]), "+r"(r0[4]), "+r"(r0[5]), "+r"(r0[6]),
+                         "+r"(r0[7]), "+r"(r1[0]), "+r"(r1[1]), "+r"(r1[2]), "+r"(r1[3]), "+r"(r1[4]), "+r"(r1[5]),
+                         "+r"(r1[6]), "+r"(r1[7])
+                       :
+                       : "memory");
+#pragma unroll
+          for (int j = 0; j < OZ_EC; ++j) {
+            long long& acc = d < 4 ? hi[p][j] : lo[p][j];
+            acc += (long long)__float2int_rn(__uint_as_float(r0[j])) * (1ll << (8 * (3 - (d & 3))));
+            acc += (long long)__float2int_rn(__uint_as_float(r1[j])) * (1ll << (8 * (2 - (d & 3))));
+          }
+        }
+      }
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(oz_saddr(&accEmpty)) : "memory");
+    }
+    if (!ok) {
+      s_abort = 1;
+      atomicExch(q.err, 1);
+    }
+    const int row = mt * OZ_BM + (warp & 3) * 32 + lane;
+    if (ok && row < q.m) {
+      const unsigned int wa = q.exA[(size_t)b * q.m_pad + row];
+      const int ea = oz_exponent(wa);
+#pragma unroll
+      for (int j = 0; j < OZ_EC; ++j) {
+        const int col = nt * OZ_BN + ch + j;
+        if (col < q.n) {
+          const unsigned int wb = q.exB[(size_t)b * q.n_pad + col];
+          const int e = ea + oz_exponent(wb) - 68;
+          double re = scalbn(fma((double)hi[0][j], 0x1p32, (double)lo[0][j]), e) * q.sign;
+          double im = scalbn(fma((double)hi[1][j], 0x1p32, (double)lo[1][j]), e) * q.sign;
+          if (wa >= 0x7ff00000u || wb >= 0x7ff00000u) re = im = __longlong_as_double(0x7ff8000000000000ll);
+          double2* cp = q.C + b * q.sC + (long long)col * q.ldc + row;
+          if (q.add) {
+            const double2 o = *cp;
+            re += o.x;
+            im += o.y;
+          }
+          *cp = make_double2(re, im);
+        }
+      }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  }
+  __syncthreads();
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+}
+
+size_t up(size_t x, size_t a) { return (x + a - 1) / a * a; }
+
+}  // namespace
+
+// bytes of digits and exponents for one matrix product m x n x k
+size_t oz_bytes(int m, int n, int k) {
+  const size_t mp = up(m, OZ_BM), np = up(n, OZ_BN), ks = (k + OZ_KS - 1) / OZ_KS;
+  return mp / OZ_BM * ks * 2 * OZ_ABLK + np / OZ_BN * ks * OZ_BBLK + up((mp + np) * sizeof(unsigned int), 256);
+}
+
+cudaError_t oz_zgemm(cudaStream_t st, int batch, int m, int n, int k, double sign, const double2* A, int lda,
+                     long long sA, int opA, const double2* B, int ldb, long long sB, int add, double2* C, int ldc,
+                     long long sC, void* work, size_t work_bytes, int* err) {
+  const size_t per = oz_bytes(m, n, k);
+  int nb = (int)(work_bytes / per < (size_t)batch ? work_bytes / per : (size_t)batch);
+  if (nb < 1) return cudaErrorInvalidValue;
+  if (nb > 32767) nb = 32767;   // gridDim.z carries (matrix, operand)
+  const int mp = (int)up(m, OZ_BM), np = (int)up(n, OZ_BN), ks = (k + OZ_KS - 1) / OZ_KS;
+  cudaError_t e = cudaFuncSetAttribute(oz_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM);
+  if (e != cudaSuccess) return e;
+  for (int b0 = 0; b0 < batch; b0 += nb) {
+    const int bn = batch - b0 < nb ? batch - b0 : nb;
+    unsigned char* dA = (unsigned char*)work;
+    unsigned char* dB = dA + (size_t)bn * (mp / OZ_BM) * ks * 2 * OZ_ABLK;
+    unsigned int* xA = (unsigned int*)(dB + (size_t)bn * (np / OZ_BN) * ks * OZ_BBLK);
+    unsigned int* xB = xA + (size_t)bn * mp;
+    OzSplit q;
+    q.k = k;
+    q.ksteps = ks;
+    q.batch = bn;
+    q.o[0].p = A + b0 * sA;
+    q.o[0].sb = sA;
+    q.o[0].rs = opA ? lda : 1;
+    q.o[0].ks = opA ? 1 : lda;
+    q.o[0].rows = m;
+    q.o[0].conj = opA;
+    q.o[0].is_b = 0;
+    q.o[0].ex = xA;
+    q.o[0].dig = dA;
+    q.o[0].rows_pad = mp;
+    q.o[1].p = B + b0 * sB;
+    q.o[1].sb = sB;
+    q.o[1].rs = ldb;
+    q.o[1].ks = 1;
+    q.o[1].rows = n;
+    q.o[1].conj = 0;
+    q.o[1].is_b = 1;
+    q.o[1].ex = xB;
+    q.o[1].dig = dB;
+    q.o[1].rows_pad = np;
+    e = cudaMemsetAsync(xA, 0, (size_t)bn * (mp + np) * sizeof(unsigned int), st);
+    if (e != cudaSuccess) return e;
+    const int rows = m > n ? m : n, rpad = mp > np ? mp : np;
+    oz_rowmax<<<dim3((rows + 31) / 32, (k + 63) / 64, 2 * bn), 256, 0, st>>>(q);
+    oz_digits<<<dim3((rpad + 31) / 32, (2 * ks + 7) / 8, 2 * bn), 256, 0, st>>>(q);
+    OzGemm g;
+    g.A = dA;
+    g.B = dB;
+    g.exA = xA;
+    g.exB = xB;
+    g.m = m;
+    g.n = n;
+    g.m_pad = mp;
+    g.n_pad = np;
+    g.ksteps = ks;
+    g.sign = sign;
+    g.add = add;
+    g.C = C + b0 * sC;
+    g.ldc = ldc;
+    g.sC = sC;
+    g.err = err;
+    oz_gemm_kernel<<<dim3(mp / OZ_BM, np / OZ_BN, bn), OZ_THREADS, OZ_SMEM, st>>>(g);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+}  // namespace rsfd

@@ -229,7 +229,7 @@ cudaError_t kernels_init();
 int pass_threads(int R, int tile_y);
 
 // Handle services used by other translation units (rsfd_api.cu).
-rsfd_status handle_ensure(Handle* h, int idx, size_t bytes, void** out);   // workspace slot idx < 8
+rsfd_status handle_ensure(Handle* h, int idx, size_t bytes, void** out);   // workspace slot idx < 10
 cudaStream_t handle_stream(Handle* h);
 int handle_prec(Handle* h);
 int handle_nb(Handle* h);
@@ -256,6 +256,13 @@ cudaError_t getrs_f32_tc(cudaStream_t st, const float2* LU, const int* piv, int 
 cudaError_t getrs_f32_tc(cudaStream_t st, const float2* LU, const int* piv, int nb, int K, const float2* B, int nrhs,
                          float2* X, int* perm, int* err);
 int tc_panel();
+
+// FP64-accurate complex GEMM on the tensor cores (oz_gemm.cu): C = sign op(A) B + (add ? C : 0), op = N or
+// conjugate transpose, batched; work holds at least oz_bytes(m, n, k); err is set when a bounded wait expires.
+size_t oz_bytes(int m, int n, int k);
+cudaError_t oz_zgemm(cudaStream_t st, int batch, int m, int n, int k, double sign, const double2* A, int lda,
+                     long long sA, int opA, const double2* B, int ldb, long long sB, int add, double2* C, int ldc,
+                     long long sC, void* work, size_t work_bytes, int* err);
 
 // Dyson / transmission launchers (dyson.cu).
 rsfd_status dyson_run(Handle* h, const void* G0, const void* SL, const void* SR, int K, void* G, double* refres);
