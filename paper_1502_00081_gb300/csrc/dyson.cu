@@ -5,9 +5,8 @@
 // (equivalent to the block formulas Eqs. sec3-02 ... sec3-06).  Every energy is an independent
 // dense complex solve of size nb; the batch is processed with:
 //   1. M = I - G0 Sigma           (batched complex GEMM, FP64)
-//   2. M = P L U                  (batched blocked right-looking LU with partial pivoting, FP64;
-//                                  panels of 32 columns, trailing updates by the batched GEMM)
-//   3. G = U^{-1} L^{-1} P G0     (batched triangular solves)
+//   2. M = P L U                  (batched blocked right-looking LU with partial pivoting, lu.cu)
+//   3. G = U^{-1} L^{-1} P G0     (batched blocked triangular solves, lu.cu)
 //   4. FP64 iterative refinement: R = G0 - M G, G += M^{-1} R (twice), reporting ||R||/||G0||.
 // T(E) = Tr[Gamma_L G_RL^H Gamma_R G_RL] (Eq. TF) with Gamma = i (Sigma - Sigma^H) is two
 // GEMMs and a trace per energy.  All matrices are column-major per energy.
@@ -21,7 +20,7 @@
 #include <string>
 #include <vector>
 
-#include "rsfd_internal.cuh"
+#include "dense.cuh"
 
 namespace rsfd {
 namespace {
@@ -83,15 +82,6 @@ void zgemm(cudaStream_t st, int batch, int m, int n, int k, double2 alpha, const
   zgemm_batched<<<grid, block, 0, st>>>(m, n, k, alpha, A, lda, sA, opA, B, ldb, sB, beta, C, ldc, sC);
 }
 
-// Where the FP64 products of a call run: the sliced tensor-core GEMM (oz_gemm.cu) with its digit
-// workspace in the handle, or the CUDA-core kernel above (small products, no handle, no memory).
-struct Gemm {
-  Handle* h = nullptr;
-  cudaStream_t st = nullptr;
-  int* err = nullptr;              // device flag of expired waits
-  cudaError_t fail = cudaSuccess;  // first launch error
-};
-
 // the flag lives in the handle's workspace 9; false: products stay on the CUDA cores
 rsfd_status gemm_begin(Handle* h, Gemm& g) {
   g.h = h;
@@ -114,29 +104,47 @@ rsfd_status gemm_end(Gemm& g, const char* who) {
   return RSFD_OK;
 }
 
-constexpr size_t kOzWorkMax = (size_t)4 << 30;   // digit workspace of one product, unless one matrix needs more
+// digits of one product: up to 4 GB for a batch, or what one matrix needs
+template <typename T> void* oz_work(Gemm& g, int batch, int m, int n, int k, size_t& bytes) {
+  const size_t lim = (size_t)4 << 30, per = oz_bytes(m, n, k, sizeof(T) == 16);
+  bytes = per * batch < lim ? per * batch : (per > lim ? per : lim);
+  void* w = nullptr;
+  return handle_ensure(g.h, 8, bytes, &w) == RSFD_OK ? w : nullptr;
+}
 
-// C[b] = sign * op(A[b]) B[b] + (add ? C[b] : 0).  Sliced from 8e6 complex multiply-adds on: its three launches
-// cost about 17 us a product, which the FP64 pipe (1.3e11 complex multiply-adds/s) earns back from there.
-// Two products of ns x ns x ns and the rest of rsfd_transmission, CUDA cores / sliced, us: ns = 64, 16 energies
-// (4.2e6) 143 / 154; 192, 1 (7.1e6) 251 / 266; 128, 4 (8.4e6) 242 / 208; 96, 16 (1.4e7) 291 / 190; 256, 16
-// (2.7e8) 3869 / 600.
+}  // namespace
+
+// Sliced from 8e6 complex multiply-adds on: its three launches cost about 17 us a product, which the FP64 pipe
+// (1.3e11 complex multiply-adds/s) earns back from there.  Two products of ns x ns x ns and the rest of
+// rsfd_transmission, CUDA cores / sliced, us: ns = 64, 16 energies (4.2e6) 143 / 154; 192, 1 (7.1e6) 251 / 266;
+// 128, 4 (8.4e6) 242 / 208; 96, 16 (1.4e7) 291 / 190; 256, 16 (2.7e8) 3869 / 600.
 void gemm(Gemm& g, int batch, int m, int n, int k, double sign, const double2* A, int lda, long long sA, int opA,
           const double2* B, int ldb, long long sB, bool add, double2* C, int ldc, long long sC) {
-  if (g.h && k >= 32 && m >= 32 && n >= 16 && (double)m * n * k * batch >= 8e6) {
-    const size_t per = oz_bytes(m, n, k);
-    const size_t want = per * batch < kOzWorkMax ? per * batch : (per > kOzWorkMax ? per : kOzWorkMax);
-    void* w = nullptr;
-    if (handle_ensure(g.h, 8, want, &w) == RSFD_OK) {
-      const cudaError_t e = oz_zgemm(g.st, batch, m, n, k, sign, A, lda, sA, opA, B, ldb, sB, add ? 1 : 0, C, ldc, sC, w,
-                                     want, g.err);
-      if (e != cudaSuccess && g.fail == cudaSuccess) g.fail = e;
-      return;
-    }
-  }
-  zgemm(g.st, batch, m, n, k, make_double2(sign, 0.0), A, lda, sA, opA, B, ldb, sB, make_double2(add ? 1.0 : 0.0, 0.0), C,
-        ldc, sC);
+  size_t wb = 0;
+  void* w = g.h && k >= 32 && m >= 32 && n >= 16 && (double)m * n * k * batch >= 8e6
+                ? oz_work<double2>(g, batch, m, n, k, wb)
+                : nullptr;
+  if (w)
+    g.note(oz_gemm(g.st, batch, m, n, k, sign < 0 ? -1 : 1, A, lda, sA, opA, B, ldb, sB, add ? 1 : 0, C, ldc, sC, w, wb, g.err));
+  else
+    zgemm(g.st, batch, m, n, k, make_double2(sign, 0.0), A, lda, sA, opA, B, ldb, sB, make_double2(add ? 1.0 : 0.0, 0.0),
+          C, ldc, sC);
 }
+
+// FP32 operands (the updates of the FP32 LU and solves): always sliced; without memory for the digits the
+// 3xTF32 GEMM.
+void gemm(Gemm& g, int batch, int m, int n, int k, double sign, const float2* A, int lda, long long sA, int opA,
+          const float2* B, int ldb, long long sB, bool add, float2* C, int ldc, long long sC) {
+  size_t wb = 0;
+  void* w = oz_work<float2>(g, batch, m, n, k, wb);
+  if (w)
+    g.note(oz_gemm(g.st, batch, m, n, k, sign < 0 ? -1 : 1, A, lda, sA, opA, B, ldb, sB, add ? 1 : 0, C, ldc, sC, w, wb, g.err));
+  else
+    g.note(cgemm_tf32x3(g.st, batch, m, n, k, make_float2((float)sign, 0.f), A, lda, sA, B, ldb, sB, add ? 1.f : 0.f, C, ldc,
+                        sC, g.err));
+}
+
+namespace {
 
 template <typename T>
 __global__ void to_c128(const T* src, double2* dst, long long n) {
@@ -188,155 +196,51 @@ __global__ void set_identity(double2* M, int nb, int batch) {
   }
 }
 
-// Blocked right-looking LU with partial pivoting (LAPACK getrf order: piv[j] is the row exchanged
-// with row j at step j).  Panels of kPanel columns are factorised by one CTA per matrix; the row
-// exchanges are then applied to the other columns, U12 = L11^{-1} A12 is solved, and the trailing
-// block is updated by the batched GEMM, which spreads the O(nb^3) work over every SM.
-constexpr int kPanel = 32;
-
-__global__ void __launch_bounds__(256) panel_getrf(double2* M, int nb, int j0, int jb, int* piv, int* info) {
-  const int b = blockIdx.x;
-  double2* A = M + (long long)b * nb * nb;
-  int* pv = piv + (long long)b * nb;
-  __shared__ double s_val[256];
-  __shared__ int s_idx[256];
-  __shared__ int s_p;
-  const int tid = threadIdx.x, nt = blockDim.x;
-  for (int j = j0; j < j0 + jb; ++j) {
-    double best = -1.0;
-    int bi = j;
-    for (int i = j + tid; i < nb; i += nt) {
-      const double v = cabs2(A[(long long)j * nb + i]);
-      if (v > best) { best = v; bi = i; }
-    }
-    s_val[tid] = best;
-    s_idx[tid] = bi;
-    __syncthreads();
-    for (int s2 = nt / 2; s2 > 0; s2 >>= 1) {
-      if (tid < s2) {
-        if (s_val[tid + s2] > s_val[tid] || (s_val[tid + s2] == s_val[tid] && s_idx[tid + s2] < s_idx[tid])) {
-          s_val[tid] = s_val[tid + s2];
-          s_idx[tid] = s_idx[tid + s2];
-        }
-      }
-      __syncthreads();
-    }
-    if (tid == 0) {
-      s_p = s_idx[0];
-      pv[j] = s_p;
-      if (!(s_val[0] > 0.0) && info[b] == 0) info[b] = j + 1;
-    }
-    __syncthreads();
-    const int p = s_p;
-    if (p != j) {   // exchange rows j and p inside the panel
-      for (int c = j0 + tid; c < j0 + jb; c += nt) {
-        const double2 t = A[(long long)c * nb + j];
-        A[(long long)c * nb + j] = A[(long long)c * nb + p];
-        A[(long long)c * nb + p] = t;
-      }
-    }
-    __syncthreads();
-    const double2 d = A[(long long)j * nb + j];
-    const double2 inv = (d.x != 0.0 || d.y != 0.0) ? cdiv(make_double2(1.0, 0.0), d) : make_double2(0.0, 0.0);
-    for (int i = j + 1 + tid; i < nb; i += nt) A[(long long)j * nb + i] = cmul(A[(long long)j * nb + i], inv);
-    __syncthreads();
-    const int rem_r = nb - j - 1, rem_c = j0 + jb - j - 1;
-    const long long tot = (long long)rem_r * rem_c;
-    for (long long t = tid; t < tot; t += nt) {
-      const int c = j + 1 + (int)(t / rem_r), i = j + 1 + (int)(t % rem_r);
-      const double2 l = A[(long long)j * nb + i], u = A[(long long)c * nb + j];
-      double2& a = A[(long long)c * nb + i];
-      a = csub(a, cmul(l, u));
-    }
-    __syncthreads();
-  }
-}
-
-// apply the exchanges of rows j0 .. j0 + jb - 1 (in order) to every column outside the panel
-__global__ void panel_laswp(double2* M, int nb, int j0, int jb, const int* piv, int batch) {
-  const int ncol = nb - jb;
-  const long long tot = (long long)ncol * batch;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < tot; t += (long long)gridDim.x * blockDim.x) {
-    const int b = (int)(t / ncol);
-    int c = (int)(t - (long long)b * ncol);
-    if (c >= j0) c += jb;
-    double2* col = M + (long long)b * nb * nb + (long long)c * nb;
-    const int* pv = piv + (long long)b * nb;
-    for (int j = j0; j < j0 + jb; ++j) {
-      const int p = pv[j];
-      if (p != j) {
-        const double2 x = col[j];
-        col[j] = col[p];
-        col[p] = x;
-      }
-    }
-  }
-}
-
-// U12 = L11^{-1} A12 (L11 unit lower jb x jb), one thread per column right of the panel
-__global__ void panel_trsm(double2* M, int nb, int j0, int jb, int batch) {
-  const int ncol = nb - j0 - jb;
-  const long long tot = (long long)ncol * batch;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < tot; t += (long long)gridDim.x * blockDim.x) {
-    const int b = (int)(t / ncol);
-    const int c = j0 + jb + (int)(t - (long long)b * ncol);
-    double2* A = M + (long long)b * nb * nb;
-    double2* col = A + (long long)c * nb;
-    for (int i = j0 + 1; i < j0 + jb; ++i) {
-      double2 s = col[i];
-      for (int k = j0; k < i; ++k) s = csub(s, cmul(A[(long long)k * nb + i], col[k]));
-      col[i] = s;
-    }
-  }
-}
-
-// Solve (P L U) X = B in place for nrhs columns; one thread per right-hand side column.
-__global__ void zgetrs_batched(const double2* LU, const int* piv, double2* B, int nb, int nrhs) {
-  const int b = blockIdx.y;
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= nrhs) return;
-  const double2* A = LU + (long long)b * nb * nb;
-  const int* pv = piv + (long long)b * nb;
-  double2* x = B + ((long long)b * nrhs + c) * nb;
-  for (int j = 0; j < nb; ++j) {
-    const int p = pv[j];
-    if (p != j) {
-      const double2 t = x[j];
-      x[j] = x[p];
-      x[p] = t;
-    }
-  }
-  for (int i = 0; i < nb; ++i) {       // unit lower
-    double2 s = x[i];
-    for (int k = 0; k < i; ++k) s = csub(s, cmul(A[(long long)k * nb + i], x[k]));
-    x[i] = s;
-  }
-  for (int i = nb - 1; i >= 0; --i) {  // upper
-    double2 s = x[i];
-    for (int k = i + 1; k < nb; ++k) s = csub(s, cmul(A[(long long)k * nb + i], x[k]));
-    x[i] = cdiv(s, A[(long long)i * nb + i]);
-  }
-}
-
 __global__ void axpy_c128(double2* y, const double2* x, long long n) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     y[i] = cadd(y[i], x[i]);
 }
 
-// out[b] = sum |A[b]|^2 over n2 entries (FP64, block per batch entry)
-__global__ void frob2_batched(const double2* A, long long n2, double* out) {
-  const int b = blockIdx.x;
-  const double2* a = A + (long long)b * n2;
-  double s = 0.0;
-  for (long long i = threadIdx.x; i < n2; i += blockDim.x) s += cabs2(a[i]);
-  __shared__ double red[256];
-  red[threadIdx.x] = s;
+// Sums over a matrix per batch entry in two launches: kRed blocks an entry leave partial sums in part
+// [batch][kRed] (fixed ranges), one warp an entry adds them in order.
+constexpr int kRed = 64;
+__device__ __forceinline__ double block_sum256(double s) {
+  __shared__ double red[8];
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
   __syncthreads();
-  for (int k = blockDim.x / 2; k > 0; k >>= 1) {
-    if (threadIdx.x < k) red[threadIdx.x] += red[threadIdx.x + k];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) out[b] = red[0];
+  double t = 0.0;
+  if (threadIdx.x == 0)
+    for (int w = 0; w < 8; ++w) t += red[w];
+  return t;   // thread 0
+}
+__global__ void __launch_bounds__(256) frob2_part(const double2* A, long long n2, double* part) {
+  const double2* a = A + blockIdx.y * n2;
+  const long long i1 = n2 * (blockIdx.x + 1) / kRed;
+  double s = 0.0;
+  for (long long i = n2 * blockIdx.x / kRed + threadIdx.x; i < i1; i += 256) s += cabs2(a[i]);
+  s = block_sum256(s);
+  if (threadIdx.x == 0) part[blockIdx.y * kRed + blockIdx.x] = s;
+}
+__global__ void sum_parts(const double* part, double* out, int batch) {
+  const int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (b >= batch) return;
+  double s = 0.0;
+  for (int k = lane; k < kRed; k += 32) s += part[b * kRed + k];
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  if (lane == 0) out[b] = s;
+}
+// the same in one launch without scratch, a block per entry
+__global__ void __launch_bounds__(256) frob2_one(const double2* A, long long n2, double* out) {
+  const double2* a = A + blockIdx.x * n2;
+  double s = 0.0;
+  for (long long i = threadIdx.x; i < n2; i += 256) s += cabs2(a[i]);
+  s = block_sum256(s);
+  if (threadIdx.x == 0) out[blockIdx.x] = s;
+}
+void frob2_batched(cudaStream_t st, const double2* A, long long n2, int batch, double* part, double* out) {
+  frob2_part<<<dim3(kRed, batch), 256, 0, st>>>(A, n2, part);
+  sum_parts<<<(batch + 7) / 8, 256, 0, st>>>(part, out, batch);
 }
 
 // Gamma = i (S - S^H) for a batch of ns x ns matrices
@@ -353,34 +257,28 @@ __global__ void gamma_batched(const double2* S, double2* G, int ns, int batch) {
   }
 }
 
-// T[b] = Re sum_{a,c} GL[a,c] * W[c,a]
-__global__ void trace_prod_batched(const double2* GL, const double2* W, int ns, double* T, double* Ti) {
-  const int b = blockIdx.x;
+// part sums of T[b] = Re sum_{a,c} GL[a,c] W[c,a]: block x of an entry takes a band of 16 x 16 tiles, W through
+// shared memory so that both operands are read along their columns
+__global__ void __launch_bounds__(256) trace_prod_part(const double2* GL, const double2* W, int ns, double* part) {
+  __shared__ double2 tw[16][17];
   const long long n2 = (long long)ns * ns;
-  const double2* g = GL + (long long)b * n2;
-  const double2* w = W + (long long)b * n2;
-  double sr = 0.0, si = 0.0;
-  for (long long t = threadIdx.x; t < n2; t += blockDim.x) {
-    const int c = (int)(t / ns), a = (int)(t - (long long)c * ns);
-    const double2 x = g[t], y = w[(long long)a * ns + c];   // GL[a,c], W[c,a]
-    sr += x.x * y.x - x.y * y.y;
-    si += x.x * y.y + x.y * y.x;
-  }
-  __shared__ double r1[256], r2[256];
-  r1[threadIdx.x] = sr;
-  r2[threadIdx.x] = si;
-  __syncthreads();
-  for (int k = blockDim.x / 2; k > 0; k >>= 1) {
-    if (threadIdx.x < k) {
-      r1[threadIdx.x] += r1[threadIdx.x + k];
-      r2[threadIdx.x] += r2[threadIdx.x + k];
-    }
+  const double2* g = GL + blockIdx.y * n2;
+  const double2* w = W + blockIdx.y * n2;
+  const int nt = (ns + 15) / 16, tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  double s = 0.0;
+  for (int t = blockIdx.x; t < nt * nt; t += kRed) {
+    const int a0 = (t % nt) * 16, c0 = (t / nt) * 16;
     __syncthreads();
+    // W[c, a] sits at a ns + c: read along c
+    tw[ty][tx] = (a0 + ty < ns && c0 + tx < ns) ? w[(long long)(a0 + ty) * ns + c0 + tx] : make_double2(0.0, 0.0);
+    __syncthreads();
+    if (a0 + tx < ns && c0 + ty < ns) {
+      const double2 x = g[(long long)(c0 + ty) * ns + a0 + tx], y = tw[tx][ty];
+      s += x.x * y.x - x.y * y.y;
+    }
   }
-  if (threadIdx.x == 0) {
-    T[b] = r1[0];
-    Ti[b] = r2[0];
-  }
+  s = block_sum256(s);
+  if (threadIdx.x == 0) part[blockIdx.y * kRed + blockIdx.x] = s;
 }
 
 // dst[b][c][0:nrow] = src[b][c][0:nrow] for ncol columns: the leading rows of a column-major block
@@ -397,24 +295,6 @@ __global__ void copy_rows_c128(const double2* src, int lds, double2* dst, int ld
 int grid_for(long long n) {
   long long g = (n + 255) / 256;
   return (int)(g < 4096 ? (g < 1 ? 1 : g) : 4096);
-}
-
-// batched blocked LU of K matrices nb x nb (column-major, contiguous), in place
-void getrf_blocked(Gemm& gc, double2* M, int nb, int K, int* piv, int* info) {
-  cudaStream_t st = gc.st;
-  const long long n2 = (long long)nb * nb;
-  for (int j0 = 0; j0 < nb; j0 += kPanel) {
-    const int jb = nb - j0 < kPanel ? nb - j0 : kPanel;
-    panel_getrf<<<K, 256, 0, st>>>(M, nb, j0, jb, piv, info);
-    if (nb > jb) panel_laswp<<<grid_for((long long)(nb - jb) * K), 256, 0, st>>>(M, nb, j0, jb, piv, K);
-    const int rest = nb - j0 - jb;
-    if (rest > 0) {
-      panel_trsm<<<grid_for((long long)rest * K), 256, 0, st>>>(M, nb, j0, jb, K);
-      // A22 -= L21 U12
-      gemm(gc, K, rest, rest, jb, -1.0, M + (long long)j0 * nb + j0 + jb, nb, n2, 0, M + (long long)(j0 + jb) * nb + j0,
-            nb, n2, true, M + (long long)(j0 + jb) * nb + j0 + jb, nb, n2);
-    }
-  }
 }
 
 }  // namespace
@@ -468,8 +348,8 @@ rsfd_status dyson_tc_run(Handle* h, const void* G0, const void* SL, const void* 
   if ((s = handle_ensure(h, 3, sx * Kc * sizeof(double2), &pX)) != RSFD_OK) return s;
   if ((s = handle_ensure(h, 4, sx * Kc * sizeof(double2), &pR)) != RSFD_OK) return s;
   if ((s = handle_ensure(h, 2, (n2 + sx) * Kc * sizeof(float2), &pF)) != RSFD_OK) return s;
-  if ((s = handle_ensure(h, 5, (long long)Kc * (2 * nb + 1) * sizeof(int), &pPiv)) != RSFD_OK) return s;
-  if ((s = handle_ensure(h, 6, (long long)2 * K * sizeof(double), &pRed)) != RSFD_OK) return s;
+  if ((s = handle_ensure(h, 5, (long long)Kc * (nb + 1 + lu_swap_ints(nb)) * sizeof(int), &pPiv)) != RSFD_OK) return s;
+  if ((s = handle_ensure(h, 6, (long long)(2 + kRed) * K * sizeof(double), &pRed)) != RSFD_OK) return s;
   if (!fp64in && (s = handle_ensure(h, 0, n2 * Kc * sizeof(double2), &pG0)) != RSFD_OK) return s;
   if (nc < nb && (s = handle_ensure(h, 7, sx * Kc * sizeof(double2), &pB)) != RSFD_OK) return s;
   if ((s = handle_begin(h)) != RSFD_OK) return s;
@@ -481,10 +361,9 @@ rsfd_status dyson_tc_run(Handle* h, const void* G0, const void* SL, const void* 
   double2* dR = (double2*)pR;
   float2* dF = (float2*)pF;
   float2* dXf = dF + n2 * Kc;
-  int* piv = (int*)pPiv;
-  int* perm = piv + (long long)Kc * nb;
+  int* perm = (int*)pPiv;
   int* info = perm + (long long)Kc * nb;
-  int* err = gc.err;
+  int* swp = info + Kc;
   double* red = (double*)pRed;
   std::vector<int> hinfo(K, 0);
   for (int k0 = 0; k0 < K; k0 += Kc) {
@@ -510,20 +389,22 @@ rsfd_status dyson_tc_run(Handle* h, const void* G0, const void* SL, const void* 
     gemm(gc, kb, nb, ns, ns, -1.0, g0 + (long long)ns * nb, nb, n2, 0, sr, ns, s2, true, dM + (long long)ns * nb, nb, n2);
     to_f32_c<<<grid_for(tot), 256, 0, st>>>(dM, dF, tot);
     DY_CK(h, cudaMemsetAsync(info, 0, kb * sizeof(int), st));
-    DY_CK(h, getrf_f32_tc(st, dF, nb, kb, piv, info, err));
-    DY_CK(h, getrs_f32_tc(st, dF, piv, nb, kb, b0, nc, dXf, perm, err));
+    lu_factor(gc, dF, nb, kb, perm, info, swp);
+    lu_permute(gc, b0, nb, kb, perm, dXf, nc);
+    lu_solve(gc, dF, nb, kb, dXf, nc);
     set_f32_to_c128<<<grid_for(totx), 256, 0, st>>>(dX, dXf, totx);
     for (int it = 0; it < nref; ++it) {
       copy_c128<<<grid_for(totx), 256, 0, st>>>(b0, dR, totx);
       gemm(gc, kb, nb, nc, nb, -1.0, dM, nb, n2, 0, dX, nb, sx, true, dR, nb, sx);
-      DY_CK(h, getrs_f32_tc(st, dF, piv, nb, kb, (const double2*)dR, nc, dXf, perm, err));
+      lu_permute(gc, dR, nb, kb, perm, dXf, nc);
+      lu_solve(gc, dF, nb, kb, dXf, nc);
       add_f32_to_c128<<<grid_for(totx), 256, 0, st>>>(dX, dXf, totx);
     }
     if (refres) {
       copy_c128<<<grid_for(totx), 256, 0, st>>>(b0, dR, totx);
       gemm(gc, kb, nb, nc, nb, -1.0, dM, nb, n2, 0, dX, nb, sx, true, dR, nb, sx);
-      frob2_batched<<<kb, 256, 0, st>>>(dR, sx, red + k0);
-      frob2_batched<<<kb, 256, 0, st>>>(b0, sx, red + K + k0);
+      frob2_batched(st, dR, sx, kb, red + 2 * K, red + k0);
+      frob2_batched(st, b0, sx, kb, red + 2 * K, red + K + k0);
     }
     if (fp64in) {
       copy_batched<double2, double2><<<grid_for(totx), 256, 0, st>>>(dX, sx, (double2*)G + n2 * k0, n2, sx, kb);
@@ -563,8 +444,8 @@ rsfd_status dyson_run(Handle* h, const void* G0, const void* SL, const void* SR,
   const long long sx = (long long)nb * nc, totx = sx * K;
   if ((s = handle_ensure(h, 3, sx * K * sizeof(double2), &pX)) != RSFD_OK) return s;
   if ((s = handle_ensure(h, 4, sx * K * sizeof(double2), &pR)) != RSFD_OK) return s;
-  if ((s = handle_ensure(h, 5, (long long)K * (nb + 1) * sizeof(int), &pPiv)) != RSFD_OK) return s;
-  if ((s = handle_ensure(h, 6, (long long)2 * K * sizeof(double), &pRed)) != RSFD_OK) return s;
+  if ((s = handle_ensure(h, 5, (long long)K * (nb + 1 + lu_swap_ints(nb)) * sizeof(int), &pPiv)) != RSFD_OK) return s;
+  if ((s = handle_ensure(h, 6, (long long)(2 + kRed) * K * sizeof(double), &pRed)) != RSFD_OK) return s;
   if ((s = handle_begin(h)) != RSFD_OK) return s;
   cudaStream_t st = handle_stream(h);
   Gemm gc;
@@ -574,8 +455,9 @@ rsfd_status dyson_run(Handle* h, const void* G0, const void* SL, const void* SR,
   double2* dLU = (double2*)pLU;
   double2* dX = (double2*)pX;
   double2* dR = (double2*)pR;
-  int* piv = (int*)pPiv;
-  int* info = piv + (long long)K * nb;
+  int* perm = (int*)pPiv;
+  int* info = perm + (long long)K * nb;
+  int* swp = info + K;
   double* red = (double*)pRed;
   const long long tot = n2 * K;
   if (fp64) copy_c128<<<grid_for(tot), 256, 0, st>>>((const double2*)G0, dG0, tot);
@@ -587,7 +469,7 @@ rsfd_status dyson_run(Handle* h, const void* G0, const void* SL, const void* SR,
         dM + (long long)ns * nb, nb, n2);
   copy_c128<<<grid_for(tot), 256, 0, st>>>(dM, dLU, tot);
   DY_CK(h, cudaMemsetAsync(info, 0, K * sizeof(int), st));
-  getrf_blocked(gc, dLU, nb, K, piv, info);
+  lu_factor(gc, dLU, nb, K, perm, info, swp);
   // right-hand sides: the first nc columns of every energy, compact (stride sx)
   const double2* b0 = dG0;
   if (nc < nb) {
@@ -596,24 +478,21 @@ rsfd_status dyson_run(Handle* h, const void* G0, const void* SL, const void* SR,
     copy_batched<double2, double2><<<grid_for(totx), 256, 0, st>>>(dG0, n2, (double2*)pB, sx, sx, K);
     b0 = (const double2*)pB;
   }
-  copy_c128<<<grid_for(totx), 256, 0, st>>>(b0, dX, totx);
-  {
-    dim3 g((nc + 127) / 128, K);
-    zgetrs_batched<<<g, 128, 0, st>>>(dLU, piv, dX, nb, nc);
-  }
+  lu_permute(gc, b0, nb, K, perm, dX, nc);
+  lu_solve(gc, dLU, nb, K, dX, nc);
   // iterative refinement in FP64
   for (int it = 0; it < 2; ++it) {
     copy_c128<<<grid_for(totx), 256, 0, st>>>(b0, dR, totx);
     gemm(gc, K, nb, nc, nb, -1.0, dM, nb, n2, 0, dX, nb, sx, true, dR, nb, sx);
-    dim3 g((nc + 127) / 128, K);
-    zgetrs_batched<<<g, 128, 0, st>>>(dLU, piv, dR, nb, nc);
+    lu_permute(gc, dR, nb, K, perm, dR, nc);
+    lu_solve(gc, dLU, nb, K, dR, nc);
     axpy_c128<<<grid_for(totx), 256, 0, st>>>(dX, dR, totx);
   }
   if (refres) {
     copy_c128<<<grid_for(totx), 256, 0, st>>>(b0, dR, totx);
     gemm(gc, K, nb, nc, nb, -1.0, dM, nb, n2, 0, dX, nb, sx, true, dR, nb, sx);
-    frob2_batched<<<K, 256, 0, st>>>(dR, sx, red);
-    frob2_batched<<<K, 256, 0, st>>>(b0, sx, red + K);
+    frob2_batched(st, dR, sx, K, red + 2 * K, red);
+    frob2_batched(st, b0, sx, K, red + 2 * K, red + K);
   }
   if (fp64) {
     copy_batched<double2, double2><<<grid_for(totx), 256, 0, st>>>(dX, sx, (double2*)G, n2, sx, K);
@@ -652,8 +531,8 @@ rsfd_status dyson_tracked_run(Handle* h, int nr, const void* G0, const void* SL,
   if ((s = handle_ensure(h, 2, b2 * K * sizeof(double2), &pLU)) != RSFD_OK) return s;
   if ((s = handle_ensure(h, 3, bn * K * sizeof(double2), &pY)) != RSFD_OK) return s;
   if ((s = handle_ensure(h, 4, bn * K * sizeof(double2), &pR)) != RSFD_OK) return s;
-  if ((s = handle_ensure(h, 5, (long long)K * (nb + 1) * sizeof(int), &pPiv)) != RSFD_OK) return s;
-  if ((s = handle_ensure(h, 6, (long long)2 * K * sizeof(double), &pRed)) != RSFD_OK) return s;
+  if ((s = handle_ensure(h, 5, (long long)K * (nb + 1 + lu_swap_ints(nb)) * sizeof(int), &pPiv)) != RSFD_OK) return s;
+  if ((s = handle_ensure(h, 6, (long long)(2 + kRed) * K * sizeof(double), &pRed)) != RSFD_OK) return s;
   if ((s = handle_ensure(h, 7, (2 * bn + r2) * K * sizeof(double2), &pW)) != RSFD_OK) return s;
   if ((s = handle_begin(h)) != RSFD_OK) return s;
   cudaStream_t st = handle_stream(h);
@@ -667,8 +546,9 @@ rsfd_status dyson_tracked_run(Handle* h, int nr, const void* G0, const void* SL,
   double2* dRHS = (double2*)pW;
   double2* dW = dRHS + bn * K;
   double2* dX = dW + bn * K;
-  int* piv = (int*)pPiv;
-  int* info = piv + (long long)K * nb;
+  int* perm = (int*)pPiv;
+  int* info = perm + (long long)K * nb;
+  int* swp = info + K;
   double* red = (double*)pRed;
   const long long rtot = r2 * K, btot = b2 * K, ntot = bn * K;
   if (fp64) copy_c128<<<grid_for(rtot), 256, 0, st>>>((const double2*)G0, dG0, rtot);
@@ -680,23 +560,23 @@ rsfd_status dyson_tracked_run(Handle* h, int nr, const void* G0, const void* SL,
         dM + (long long)ns * nb, nb, b2);
   copy_c128<<<grid_for(btot), 256, 0, st>>>(dM, dLU, btot);
   DY_CK(h, cudaMemsetAsync(info, 0, K * sizeof(int), st));
-  getrf_blocked(gc, dLU, nb, K, piv, info);
+  lu_factor(gc, dLU, nb, K, perm, info, swp);
   // Y = M^{-1} G0[b, :] with two FP64 refinement steps
   copy_rows_c128<<<grid_for(ntot), 256, 0, st>>>(dG0, nr, dRHS, nb, nb, nr, K);
-  copy_c128<<<grid_for(ntot), 256, 0, st>>>(dRHS, dY, ntot);
-  dim3 g((nr + 127) / 128, K);
-  zgetrs_batched<<<g, 128, 0, st>>>(dLU, piv, dY, nb, nr);
+  lu_permute(gc, dRHS, nb, K, perm, dY, nr);
+  lu_solve(gc, dLU, nb, K, dY, nr);
   for (int it = 0; it < 2; ++it) {
     copy_c128<<<grid_for(ntot), 256, 0, st>>>(dRHS, dR, ntot);
     gemm(gc, K, nb, nr, nb, -1.0, dM, nb, b2, 0, dY, nb, bn, true, dR, nb, bn);
-    zgetrs_batched<<<g, 128, 0, st>>>(dLU, piv, dR, nb, nr);
+    lu_permute(gc, dR, nb, K, perm, dR, nr);
+    lu_solve(gc, dLU, nb, K, dR, nr);
     axpy_c128<<<grid_for(ntot), 256, 0, st>>>(dY, dR, ntot);
   }
   if (refres) {
     copy_c128<<<grid_for(ntot), 256, 0, st>>>(dRHS, dR, ntot);
     gemm(gc, K, nb, nr, nb, -1.0, dM, nb, b2, 0, dY, nb, bn, true, dR, nb, bn);
-    frob2_batched<<<K, 256, 0, st>>>(dR, bn, red);
-    frob2_batched<<<K, 256, 0, st>>>(dRHS, bn, red + K);
+    frob2_batched(st, dR, bn, K, red + 2 * K, red);
+    frob2_batched(st, dRHS, bn, K, red + 2 * K, red + K);
   }
   // W = Sigma Y (block-diagonal Sigma), then G = G0 + G0[:, b] W
   gemm(gc, K, ns, nr, ns, 1.0, (const double2*)SL, ns, (long long)ns * ns, 0, dY, nb, bn, false, dW, nb, bn);
@@ -816,7 +696,7 @@ rsfd_status lead_decimation_run(Handle* h, const double* VL, const double* VR, c
   for (int r = 0; r < n; ++r)
     for (int c = 0; c < n; ++c) H01T[(size_t)c * n + r] = H01[(size_t)r * n + c];
   // per energy: eps_s, eps, alpha, beta, A (LU), Y (n x 2n), rhs (n x 2n), 2 products
-  const long long per = n2 * 11 * (long long)sizeof(double2) + (n + 64) * (long long)sizeof(int) + 64;
+  const long long per = n2 * 11 * (long long)sizeof(double2) + (n + 1 + lu_swap_ints(n)) * (long long)sizeof(int) + 64;
   size_t free_b = 0, tot_b = 0;
   DY_CK(h, cudaMemGetInfo(&free_b, &tot_b));
   long long kc = (long long)(0.5 * (double)free_b) / per;
@@ -827,7 +707,7 @@ rsfd_status lead_decimation_run(Handle* h, const double* VL, const double* VR, c
   void *pW, *pC, *pPiv, *pZ;
   if ((s = handle_ensure(h, 1, (size_t)n2 * 11 * Kc * sizeof(double2), &pW)) != RSFD_OK) return s;
   if ((s = handle_ensure(h, 2, (size_t)n2 * 3 * sizeof(double2), &pC)) != RSFD_OK) return s;
-  if ((s = handle_ensure(h, 5, ((size_t)Kc * (n + 1) + 64) * sizeof(int), &pPiv)) != RSFD_OK) return s;
+  if ((s = handle_ensure(h, 5, (size_t)Kc * (n + 1 + lu_swap_ints(n)) * sizeof(int), &pPiv)) != RSFD_OK) return s;
   if ((s = handle_ensure(h, 6, (size_t)Kc * (sizeof(double2) + sizeof(double)), &pZ)) != RSFD_OK) return s;
   if ((s = handle_begin(h)) != RSFD_OK) return s;
   cudaStream_t st = handle_stream(h);
@@ -837,8 +717,9 @@ rsfd_status lead_decimation_run(Handle* h, const double* VL, const double* VR, c
   double2 *eps_s = W, *eps = W + n2 * Kc, *al = W + 2 * n2 * Kc, *be = W + 3 * n2 * Kc, *A = W + 4 * n2 * Kc;
   double2 *Y = W + 5 * n2 * Kc, *rhs = W + 7 * n2 * Kc, *P1 = W + 9 * n2 * Kc, *P2 = W + 10 * n2 * Kc;
   double2 *dH00 = (double2*)pC, *dH01 = dH00 + n2, *dH01T = dH00 + 2 * n2;
-  int* piv = (int*)pPiv;
-  int* info = piv + (long long)Kc * n;
+  int* perm = (int*)pPiv;
+  int* info = perm + (long long)Kc * n;
+  int* swp = info + Kc;
   double2* dZ = (double2*)pZ;
   double* dmax = (double*)(dZ + Kc);
   DY_CK(h, cudaMemcpyAsync(dH01, H01.data(), n2 * sizeof(double2), cudaMemcpyHostToDevice, st));
@@ -872,13 +753,10 @@ rsfd_status lead_decimation_run(Handle* h, const double* VL, const double* VR, c
         // g [alpha | beta] by LU of Z - eps
         zi_minus<<<grid_for(tot), 256, 0, st>>>(A, eps, dZ, n, kb);
         DY_CK(h, cudaMemsetAsync(info, 0, kb * sizeof(int), st));
-        getrf_blocked(gc, A, n, kb, piv, info);
+        lu_factor(gc, A, n, kb, perm, info, swp);
         concat_cols<<<grid_for(2 * tot), 256, 0, st>>>(al, be, rhs, n2, kb);
-        copy_c128<<<grid_for(2 * tot), 256, 0, st>>>(rhs, Y, 2 * tot);
-        {
-          dim3 g((2 * n + 127) / 128, kb);
-          zgetrs_batched<<<g, 128, 0, st>>>(A, piv, Y, n, 2 * n);
-        }
+        lu_permute(gc, rhs, n, kb, perm, Y, 2 * n);
+        lu_solve(gc, A, n, kb, Y, 2 * n);
         const double2* ga = Y;        // g alpha, per energy stride 2 n2
         const double2* gb = Y + n2;   // g beta
         // P1 = alpha g beta, P2 = beta g alpha
@@ -899,12 +777,10 @@ rsfd_status lead_decimation_run(Handle* h, const double* VL, const double* VR, c
       //   Sigma_R = H01 g_s H01^T, Sigma_L = H01^T g_s H01
       zi_minus<<<grid_for(tot), 256, 0, st>>>(A, eps_s, dZ, n, kb);
       DY_CK(h, cudaMemsetAsync(info, 0, kb * sizeof(int), st));
-      getrf_blocked(gc, A, n, kb, piv, info);
-      bcast_c128<<<grid_for(tot), 256, 0, st>>>(lead == 0 ? dH01T : dH01, Y, n2, kb);
-      {
-        dim3 g((n + 127) / 128, kb);
-        zgetrs_batched<<<g, 128, 0, st>>>(A, piv, Y, n, n);
-      }
+      lu_factor(gc, A, n, kb, perm, info, swp);
+      bcast_c128<<<grid_for(tot), 256, 0, st>>>(lead == 0 ? dH01T : dH01, rhs, n2, kb);
+      lu_permute(gc, rhs, n, kb, perm, Y, n);
+      lu_solve(gc, A, n, kb, Y, n);
       gemm(gc, kb, n, n, n, 1.0, lead == 0 ? dH01 : dH01T, n, 0, 0, Y, n, n2, false, out + n2 * k0, n, n2);
       std::vector<int> hinfo(kb);
       DY_CK(h, cudaMemcpyAsync(hinfo.data(), info, kb * sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -935,7 +811,7 @@ rsfd_status transmission_run(Handle* h, const void* G, const void* SL, const voi
   if ((s = handle_ensure(h, 2, s2 * K * sizeof(double2), &pGR)) != RSFD_OK) return s;
   if ((s = handle_ensure(h, 3, s2 * K * sizeof(double2), &pW1)) != RSFD_OK) return s;
   if ((s = handle_ensure(h, 4, s2 * K * sizeof(double2), &pW2)) != RSFD_OK) return s;
-  if ((s = handle_ensure(h, 6, (long long)2 * K * sizeof(double), &pT)) != RSFD_OK) return s;
+  if ((s = handle_ensure(h, 6, (long long)(1 + kRed) * K * sizeof(double), &pT)) != RSFD_OK) return s;
   if ((s = handle_begin(h)) != RSFD_OK) return s;
   cudaStream_t st = handle_stream(h);
   Gemm gc;
@@ -951,10 +827,11 @@ rsfd_status transmission_run(Handle* h, const void* G, const void* SL, const voi
   gemm(gc, K, ns, ns, ns, 1.0, (const double2*)pGR, ns, s2, 0, GRL, nb, n2, false, (double2*)pW1, ns, s2);
   gemm(gc, K, ns, ns, ns, 1.0, GRL, nb, n2, 1, (const double2*)pW1, ns, s2, false, (double2*)pW2, ns, s2);
   double* dT = (double*)pT;
-  trace_prod_batched<<<K, 256, 0, st>>>((const double2*)pGL, (const double2*)pW2, ns, dT, dT + K);
+  trace_prod_part<<<dim3(kRed, K), 256, 0, st>>>((const double2*)pGL, (const double2*)pW2, ns, dT + K);
+  sum_parts<<<(K + 7) / 8, 256, 0, st>>>(dT + K, dT, K);
   DY_CK(h, cudaGetLastError());
-  std::vector<double> hT(2 * K);
-  DY_CK(h, cudaMemcpyAsync(hT.data(), dT, 2 * K * sizeof(double), cudaMemcpyDeviceToHost, st));
+  std::vector<double> hT(K);
+  DY_CK(h, cudaMemcpyAsync(hT.data(), dT, K * sizeof(double), cudaMemcpyDeviceToHost, st));
   if ((s = gemm_end(gc, "rsfd_transmission")) != RSFD_OK) return s;
   if ((s = handle_end(h)) != RSFD_OK) return s;
   for (int k = 0; k < K; ++k) T[k] = hT[k];
@@ -1038,12 +915,17 @@ rsfd_status dyson_noalloc_run(int32_t nb, int32_t K, const void* G0_bb, const vo
   base += align256((size_t)n2 * K * sizeof(double2));
   double2* dR = (double2*)base;
   base += align256((size_t)n2 * K * sizeof(double2));
-  int* piv = (int*)base;
-  int* info = piv + (size_t)K * nb;
+  int* perm = (int*)base;
+  int* info = perm + (size_t)K * nb;
   base += align256((size_t)K * (nb + 1) * sizeof(int));
   double* red = (double*)base;   // [2K] squared norms, [K] ratios
   base += align256((size_t)3 * K * sizeof(double));
   int* bad = (int*)base;
+  base += align256(sizeof(int));
+  // the LU's exchange lists: behind the rest, or, when that is full, in the residual's place (not yet in use,
+  // and at least as large from nb = 4 on)
+  const size_t swp_bytes = (size_t)K * lu_swap_ints(nb) * sizeof(int);
+  int* swp = need + swp_bytes <= kNoAllocScratchBytes ? (int*)base : (int*)dR;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   Gemm gc;   // no handle: the CUDA-core products
   gc.st = st;
@@ -1060,22 +942,22 @@ rsfd_status dyson_noalloc_run(int32_t nb, int32_t K, const void* G0_bb, const vo
   gemm(gc, K, nb, ns, ns, -1.0, G0 + (long long)ns * nb, nb, n2, 0, (const double2*)Sigma_R, ns, (long long)ns * ns, true,
         dM + (long long)ns * nb, nb, n2);
   copy_c128<<<grid_for(tot), 256, 0, st>>>(dM, dLU, tot);
-  getrf_blocked(gc, dLU, nb, K, piv, info);
-  copy_c128<<<grid_for(tot), 256, 0, st>>>(G0, dX, tot);
-  dim3 g((nb + 127) / 128, K);
-  zgetrs_batched<<<g, 128, 0, st>>>(dLU, piv, dX, nb, nb);
+  lu_factor(gc, dLU, nb, K, perm, info, swp);
+  lu_permute(gc, G0, nb, K, perm, dX, nb);
+  lu_solve(gc, dLU, nb, K, dX, nb);
   for (int it = 0; it < 2; ++it) {
     copy_c128<<<grid_for(tot), 256, 0, st>>>(G0, dR, tot);
     gemm(gc, K, nb, nb, nb, -1.0, dM, nb, n2, 0, dX, nb, n2, true, dR, nb, n2);
-    zgetrs_batched<<<g, 128, 0, st>>>(dLU, piv, dR, nb, nb);
+    lu_permute(gc, dR, nb, K, perm, dR, nb);
+    lu_solve(gc, dLU, nb, K, dR, nb);
     axpy_c128<<<grid_for(tot), 256, 0, st>>>(dX, dR, tot);
   }
   copy_c128<<<grid_for(tot), 256, 0, st>>>(G0, dR, tot);
   gemm(gc, K, nb, nb, nb, -1.0, dM, nb, n2, 0, dX, nb, n2, true, dR, nb, n2);
-  frob2_batched<<<K, 256, 0, st>>>(dR, n2, red);
-  frob2_batched<<<K, 256, 0, st>>>(G0, n2, red + K);
+  frob2_one<<<K, 256, 0, st>>>(dR, n2, red);
+  frob2_one<<<K, 256, 0, st>>>(G0, n2, red + K);
   noalloc_finish<<<1, 256, 0, st>>>(info, red, K, bad, red + 2 * K);
-  e = cudaGetLastError();
+  e = gc.fail != cudaSuccess ? gc.fail : cudaGetLastError();
   int hbad = K;
   if (e == cudaSuccess) e = cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess && refine_residual)

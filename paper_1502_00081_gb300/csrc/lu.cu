@@ -1,0 +1,665 @@
+// Batched LU with partial pivoting and triangular solves in FP32 and FP64 complex arithmetic, for the
+// boundary solve (I - G0 Sigma) G = G0 (Eq. sec3-01a) and the lead decimation.
+//
+// Right-looking, two levels.  Outer blocks of 128 columns end in one tensor-core product
+// A22 -= L21 U12 (k = 128).  Inside an outer block, panels of W columns take three launches:
+//   lu_panel   factorises rows x W: every row of the panel lives in one thread's registers, the rows are
+//              spread over up to 8 CTAs of a cluster, and a column costs one block and one cluster barrier
+//              (the pivot candidates, the pivot row and the row it replaces travel through
+//              distributed shared memory);
+//   lu_swap    applies the panel's exchanges to the outer block's other columns as one permutation of at
+//              most 2 W rows, and solves with the panel's unit lower triangle for those to its right;
+//   lu_update  the rank-W update of the rest of the outer block.
+// The exchanges then reach the other columns (lu_swap_rest), and U12 = L11^{-1} A12 is a triangular solve.
+// Triangular solves: blocks of 64 (FP64) or 128 (FP32) rows by substitution (lu_trsm), the rest by products.
+//
+// Measured (16 matrices of 1024 rows, FP32): panel_getrf + laswp + trsm + 3xTF32 updates 48 ms before, 14 ms now; 4 of
+// 2048: 123 -> 21 ms; 8 of 512 in FP64 with three solves of 512 columns: 213 -> 12 ms (one thread a column before).
+// What bounds it: the panels are a chain of nb column steps (barriers and reductions, ~1-2 us each); the
+// FP64 pipe for lu_update and lu_trsm in FP64; the products run at tensor rate.
+
+#include <cooperative_groups.h>
+#include <cuda_runtime.h>
+
+#include "dense.cuh"
+
+namespace cg = cooperative_groups;
+
+namespace rsfd {
+namespace {
+
+constexpr int kOuter = 128;      // columns per outer block = k of the trailing products
+constexpr int kPanelThreads = 512;
+constexpr int kMaxCluster = 8;   // portable cluster size
+constexpr int kMaxPanels = 16;   // panels of an outer block (at least 8 columns each)
+
+template <typename T> struct Num;
+template <> struct Num<float2> {
+  typedef float R;
+  static constexpr int NBLK = 128;   // rows per substitution block
+  // pivot measure, as in the FP32 form's reference: |re| + |im|
+  static __device__ __forceinline__ float mag(float2 a) { return fabsf(a.x) + fabsf(a.y); }
+  static __device__ __forceinline__ float2 mul(float2 a, float2 b) {
+    return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
+  }
+  // c - a b
+  static __device__ __forceinline__ float2 nma(float2 a, float2 b, float2 c) {
+    return make_float2(fmaf(-a.x, b.x, fmaf(a.y, b.y, c.x)), fmaf(-a.x, b.y, fmaf(-a.y, b.x, c.y)));
+  }
+  static __device__ __forceinline__ float2 recip(float2 d) {   // Smith
+    if (d.x == 0.f && d.y == 0.f) return make_float2(0.f, 0.f);
+    if (fabsf(d.x) >= fabsf(d.y)) {
+      const float r = d.y / d.x, den = d.x + d.y * r;
+      return make_float2(1.f / den, -r / den);
+    }
+    const float r = d.x / d.y, den = d.y + d.x * r;
+    return make_float2(r / den, -1.f / den);
+  }
+};
+template <> struct Num<double2> {
+  typedef double R;
+  static constexpr int NBLK = 64;
+  static __device__ __forceinline__ double mag(double2 a) { return cabs2(a); }
+  static __device__ __forceinline__ double2 mul(double2 a, double2 b) { return cmul(a, b); }
+  static __device__ __forceinline__ double2 nma(double2 a, double2 b, double2 c) {
+    return make_double2(fma(-a.x, b.x, fma(a.y, b.y, c.x)), fma(-a.x, b.y, fma(-a.y, b.x, c.y)));
+  }
+  static __device__ __forceinline__ double2 recip(double2 d) {
+    if (d.x == 0.0 && d.y == 0.0) return make_double2(0.0, 0.0);
+    return cdiv(make_double2(1.0, 0.0), d);
+  }
+};
+
+__device__ __forceinline__ float2 shfl(float2 v, int l) {
+  return make_float2(__shfl_sync(0xffffffffu, v.x, l), __shfl_sync(0xffffffffu, v.y, l));
+}
+__device__ __forceinline__ double2 shfl(double2 v, int l) {
+  return make_double2(__shfl_sync(0xffffffffu, v.x, l), __shfl_sync(0xffffffffu, v.y, l));
+}
+
+// The panel's exchanges (row j0 + t with row piv[t], t = 0 .. jw - 1 in order) as one permutation of at
+// most 2 W rows: entry e moves row src[e] to row dst[e] (dst < 0: unused).  One warp.
+template <int W> __device__ void swap_list(const int* piv, int j0, int jw, int* out) {
+  const int lane = threadIdx.x & 31;
+  int row = -1 - lane;
+  if (lane < W) {
+    if (lane < jw) row = j0 + lane;
+  } else if (lane < 2 * W && lane - W < jw) {
+    row = piv[lane - W];
+  }
+  const int first = __ffs(__match_any_sync(0xffffffffu, row)) - 1;   // the entry that stands for this row
+  int label = row;
+  for (int t = 0; t < jw; ++t) {
+    const int q = __shfl_sync(0xffffffffu, first, W + t);
+    const int a = __shfl_sync(0xffffffffu, label, t), c = __shfl_sync(0xffffffffu, label, q);
+    if (lane == t) label = c;
+    if (lane == q) label = a;
+  }
+  const bool valid = row >= 0 && lane == first;
+  out[lane] = valid ? row : -1;
+  out[32 + lane] = label;
+}
+
+// Factorise columns j0 .. j0 + jw - 1 (jw <= W <= 16) of matrix blockIdx.y, rows j0 .. nb - 1; grid (cluster size, K).
+// Ties in the pivot search go to the lowest row.
+template <typename T, int W, int RPT>
+__global__ void __launch_bounds__(kPanelThreads) lu_panel(T* M, int nb, int j0, int jw, int* swp, int ss, int* info) {
+  typedef Num<T> N;
+  typedef typename N::R R;
+  cg::cluster_group cl = cg::this_cluster();
+  const int C = gridDim.x, rank = blockIdx.x, b = blockIdx.y;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockDim.x, nw = nt >> 5;
+  // what a CTA shows to its cluster, double-buffered by column parity: a CTA that writes entry (jj + 2) has
+  // passed the barrier of column jj + 1, at which every CTA has finished reading column jj
+  __shared__ T s_cand[2][W], s_rowj[2][W], s_inv[2];
+  __shared__ R s_bv[2];
+  __shared__ int s_bi[2];
+  __shared__ R s_wv[kPanelThreads / 32];
+  __shared__ int s_wi[kPanelThreads / 32];
+  __shared__ T s_w[kPanelThreads / 32][2 * W + 1];   // per warp: pivot row, replaced row, 1 / pivot
+  __shared__ int s_piv[W];
+  T* A = M + (long long)b * nb * nb + (long long)j0 * nb;
+  const int row0 = j0 + rank * nt * RPT + tid;
+  T a[RPT][W];
+#pragma unroll
+  for (int r = 0; r < RPT; ++r)
+#pragma unroll
+    for (int c = 0; c < W; ++c) {
+      const int i = row0 + r * nt;
+      a[r][c] = (i < nb && c < jw) ? A[(long long)c * nb + i] : T();
+    }
+#pragma unroll
+  for (int jj = 0; jj < W; ++jj) {
+    if (jj < jw) {
+      const int gj = j0 + jj, par = jj & 1;
+      R best = (R)-1;
+      int bi = 0x7fffffff;
+#pragma unroll
+      for (int r = 0; r < RPT; ++r) {
+        const int i = row0 + r * nt;
+        const R v = N::mag(a[r][jj]);
+        if (i >= gj && i < nb && v > best) {
+          best = v;
+          bi = i;
+        }
+      }
+      for (int o = 16; o > 0; o >>= 1) {
+        const R ov = __shfl_xor_sync(0xffffffffu, best, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+        if (ov > best || (ov == best && oi < bi)) {
+          best = ov;
+          bi = oi;
+        }
+      }
+      if (lane == 0) {
+        s_wv[warp] = best;
+        s_wi[warp] = bi;
+      }
+      if (rank == 0 && tid == jj) {
+#pragma unroll
+        for (int c = 0; c < W; ++c) s_rowj[par][c] = a[0][c];
+      }
+      __syncthreads();
+      best = s_wv[0];
+      bi = s_wi[0];
+      for (int w = 1; w < nw; ++w) {
+        const R ov = s_wv[w];
+        const int oi = s_wi[w];
+        if (ov > best || (ov == best && oi < bi)) {
+          best = ov;
+          bi = oi;
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < RPT; ++r)
+        if (row0 + r * nt == bi) {
+#pragma unroll
+          for (int c = 0; c < W; ++c) s_cand[par][c] = a[r][c];
+          s_inv[par] = N::recip(a[r][jj]);
+        }
+      if (tid == 0) {
+        s_bv[par] = best;
+        s_bi[par] = bi;
+      }
+      if (C > 1) cl.sync();
+      else __syncthreads();
+      int pr = 0;
+      if (C > 1) {
+        best = (R)-1;
+        bi = 0x7fffffff;
+        if (lane < C) {
+          best = *cl.map_shared_rank(&s_bv[par], lane);
+          bi = *cl.map_shared_rank(&s_bi[par], lane);
+        }
+        for (int o = kMaxCluster / 2; o > 0; o >>= 1) {
+          const R ov = __shfl_xor_sync(0xffffffffu, best, o);
+          const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+          if (ov > best || (ov == best && oi < bi)) {
+            best = ov;
+            bi = oi;
+          }
+        }
+        best = __shfl_sync(0xffffffffu, best, 0);
+        bi = __shfl_sync(0xffffffffu, bi, 0);
+      }
+      const bool none = bi == 0x7fffffff;   // no comparable entry in the column (all NaN)
+      const int gp = none ? gj : bi;
+      pr = (gp - j0) / (nt * RPT);
+      if (lane < W) {
+        const T* rj = C > 1 ? cl.map_shared_rank(&s_rowj[par][0], 0) : &s_rowj[par][0];
+        const T* pv = C > 1 ? cl.map_shared_rank(&s_cand[par][0], pr) : &s_cand[par][0];
+        const T vj = rj[lane];
+        s_w[warp][lane] = none ? vj : pv[lane];
+        s_w[warp][W + lane] = vj;
+      } else if (lane == W) {
+        const T* pi = C > 1 ? cl.map_shared_rank(&s_inv[par], pr) : &s_inv[par];
+        s_w[warp][2 * W] = none ? T() : *pi;
+      }
+      __syncwarp();
+      if (rank == 0 && tid == 0) {
+        s_piv[jj] = gp;
+        if (!(best > (R)0) && info[b] == 0) info[b] = gj + 1;
+      }
+      const T inv = s_w[warp][2 * W];
+#pragma unroll
+      for (int r = 0; r < RPT; ++r) {
+        const int i = row0 + r * nt;
+        if (gp != gj && (i == gp || i == gj)) {
+          const int o = i == gp ? W : 0;
+#pragma unroll
+          for (int c = 0; c < W; ++c) a[r][c] = s_w[warp][o + c];
+        }
+        if (i > gj && i < nb) {
+          const T l = N::mul(a[r][jj], inv);
+          a[r][jj] = l;
+#pragma unroll
+          for (int c = jj + 1; c < W; ++c) a[r][c] = N::nma(l, s_w[warp][c], a[r][c]);
+        }
+      }
+      __syncwarp();
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < RPT; ++r)
+#pragma unroll
+    for (int c = 0; c < W; ++c) {
+      const int i = row0 + r * nt;
+      if (i < nb && c < jw) A[(long long)c * nb + i] = a[r][c];
+    }
+  __syncthreads();
+  if (rank == 0 && warp == 0) swap_list<W>(s_piv, j0, jw, swp + (long long)b * ss);
+  if (C > 1) cl.sync();   // a CTA's shared memory outlives the other CTAs' reads
+}
+
+// The same for panels taller than the clusters hold: one CTA per matrix, the panel stays in global memory.
+template <typename T>
+__global__ void __launch_bounds__(kPanelThreads) lu_panel_global(T* M, int nb, int j0, int jw, int* swp, int ss,
+                                                               int* info) {
+  typedef Num<T> N;
+  typedef typename N::R R;
+  const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, nt = blockDim.x;
+  T* A = M + (long long)b * nb * nb;
+  __shared__ R s_wv[kPanelThreads / 32];
+  __shared__ int s_wi[kPanelThreads / 32];
+  __shared__ T s_inv;
+  __shared__ int s_piv[16];
+  for (int j = j0; j < j0 + jw; ++j) {
+    R best = (R)-1;
+    int bi = 0x7fffffff;
+    for (int i = j + tid; i < nb; i += nt) {
+      const R v = N::mag(A[(long long)j * nb + i]);
+      if (v > best) {
+        best = v;
+        bi = i;
+      }
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      const R ov = __shfl_xor_sync(0xffffffffu, best, o);
+      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+      if (ov > best || (ov == best && oi < bi)) {
+        best = ov;
+        bi = oi;
+      }
+    }
+    if (lane == 0) {
+      s_wv[tid >> 5] = best;
+      s_wi[tid >> 5] = bi;
+    }
+    __syncthreads();
+    best = s_wv[0];
+    bi = s_wi[0];
+    for (int w = 1; w < nt >> 5; ++w)
+      if (s_wv[w] > best || (s_wv[w] == best && s_wi[w] < bi)) {
+        best = s_wv[w];
+        bi = s_wi[w];
+      }
+    const int p = bi == 0x7fffffff ? j : bi;
+    if (tid == 0) {
+      s_piv[j - j0] = p;
+      if (!(best > (R)0) && info[b] == 0) info[b] = j + 1;
+    }
+    if (p != j && tid < jw) {
+      T* c = A + (long long)(j0 + tid) * nb;
+      const T t = c[j];
+      c[j] = c[p];
+      c[p] = t;
+    }
+    __syncthreads();
+    if (tid == 0) s_inv = N::recip(A[(long long)j * nb + j]);
+    __syncthreads();
+    const T inv = s_inv;
+    for (int i = j + 1 + tid; i < nb; i += nt) {
+      const T l = N::mul(A[(long long)j * nb + i], inv);
+      A[(long long)j * nb + i] = l;
+      for (int c = j + 1; c < j0 + jw; ++c) A[(long long)c * nb + i] = N::nma(l, A[(long long)c * nb + j], A[(long long)c * nb + i]);
+    }
+    __syncthreads();
+  }
+  if (tid < 32) swap_list<16>(s_piv, j0, jw, swp + (long long)b * ss);
+}
+
+// Row exchanges of the panel (W, j0, jw) in the outer block's other columns o0 .. oend - 1, one thread per column;
+// those right of the panel are also solved with its unit lower triangle.  Bound: latency of 2 W scattered
+// loads per thread, all in flight together.
+template <typename T, int W>
+__global__ void __launch_bounds__(kOuter) lu_swap(T* M, int nb, int o0, int oend, int j0, int jw, const int* swp, int ss) {
+  typedef Num<T> N;
+  const int b = blockIdx.x;
+  __shared__ int s_dst[2 * W], s_src[2 * W];
+  __shared__ T s_L[W][W];
+  T* A = M + (long long)b * nb * nb;
+  const int* sw = swp + (long long)b * ss;
+  for (int t = threadIdx.x; t < 2 * W; t += blockDim.x) {
+    s_dst[t] = sw[t];
+    s_src[t] = sw[32 + t];
+  }
+  for (int t = threadIdx.x; t < W * W; t += blockDim.x) {
+    const int c = t / W, r = t % W;
+    s_L[r][c] = (r > c && r < jw) ? A[(long long)(j0 + c) * nb + j0 + r] : T();
+  }
+  __syncthreads();
+  const int c = o0 + threadIdx.x;
+  if (c >= oend || (c >= j0 && c < j0 + jw)) return;
+  T* col = A + (long long)c * nb;
+  const bool right = c >= j0 + jw;
+  T v[2 * W];
+#pragma unroll
+  for (int t = 0; t < 2 * W; ++t) {
+    v[t] = T();
+    if (s_dst[t] >= 0 && (s_dst[t] != s_src[t] || (right && t < W))) v[t] = col[s_src[t]];
+  }
+  if (right) {
+#pragma unroll
+    for (int r = 1; r < W; ++r)
+#pragma unroll
+      for (int q = 0; q < r; ++q) v[r] = N::nma(s_L[r][q], v[q], v[r]);
+  }
+#pragma unroll
+  for (int t = 0; t < 2 * W; ++t)
+    if (s_dst[t] >= 0 && (s_dst[t] != s_src[t] || (right && t < W))) col[s_dst[t]] = v[t];
+}
+
+// The exchanges of an outer block's np panels, in order, in the columns outside it and in perm (the last
+// "column"), one thread per column.
+template <typename V> __device__ __forceinline__ void apply_lists(V* col, const int (*lists)[kSwapInts], int np) {
+  for (int p = 0; p < np; ++p) {
+    V v[32];
+#pragma unroll
+    for (int t = 0; t < 32; ++t)
+      if (lists[p][t] >= 0 && lists[p][t] != lists[p][32 + t]) v[t] = col[lists[p][32 + t]];
+#pragma unroll
+    for (int t = 0; t < 32; ++t)
+      if (lists[p][t] >= 0 && lists[p][t] != lists[p][32 + t]) col[lists[p][t]] = v[t];
+  }
+}
+template <typename T>
+__global__ void __launch_bounds__(64) lu_swap_rest(T* M, int nb, int o0, int oend, int np, const int* swp, int ss, int* perm) {
+  __shared__ int s_l[kMaxPanels][kSwapInts];
+  const int b = blockIdx.y;
+  for (int t = threadIdx.x; t < np * kSwapInts; t += blockDim.x) s_l[t / kSwapInts][t % kSwapInts] = swp[(long long)b * ss + t];
+  __syncthreads();
+  int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= o0) c += oend - o0;
+  if (c > nb) return;
+  if (c == nb) apply_lists(perm + (long long)b * nb, s_l, np);
+  else apply_lists(M + (long long)b * nb * nb + (long long)c * nb, s_l, np);
+}
+
+// A[i, c] -= sum_t A[i, j0 + t] A[j0 + t, c] for rows r0 .. nb - 1 of columns r0 .. oend - 1 (r0 = j0 + jw).  Tiles of 64
+// rows x 16 columns, 128 threads.
+template <typename T, int W>
+__global__ void __launch_bounds__(128) lu_update(T* M, int nb, int j0, int jw, int oend) {
+  typedef Num<T> N;
+  __shared__ T s_u[16][W];
+  const int r0 = j0 + jw;
+  T* A = M + (long long)blockIdx.z * nb * nb;
+  const int rb = r0 + blockIdx.x * 64, cb = r0 + blockIdx.y * 16;
+  for (int e = threadIdx.x; e < 16 * W; e += 128) {
+    const int c = cb + e / W, q = e % W;
+    s_u[e / W][q] = (c < oend && q < jw) ? A[(long long)c * nb + j0 + q] : T();
+  }
+  __syncthreads();
+  const int i = rb + (threadIdx.x & 63), cg0 = (threadIdx.x >> 6) * 8;
+  if (i >= nb) return;
+  T l[W];
+#pragma unroll
+  for (int q = 0; q < W; ++q) l[q] = q < jw ? A[(long long)(j0 + q) * nb + i] : T();
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    const int c = cb + cg0 + e;
+    if (c < oend) {
+      T v = A[(long long)c * nb + i];
+#pragma unroll
+      for (int q = 0; q < W; ++q) v = N::nma(l[q], s_u[cg0 + e][q], v);
+      A[(long long)c * nb + i] = v;
+    }
+  }
+}
+
+// X[r0 .. r0 + ib, :] = T^{-1} X[r0 .. r0 + ib, :] for the diagonal block T of LU at (r0, r0): unit lower (LOWER) or
+// upper triangle.  Eight threads share a column (rows q, q + 8, ...), 32 columns per CTA; T passes through
+// shared memory in strips of 16 columns; the solved element travels by shuffle.  X has nb rows and batch stride sX.  Bound: FP64 (FP32) pipe.
+template <typename T, bool LOWER>
+__global__ void __launch_bounds__(256) lu_trsm(const T* LU, int nb, int r0, int ib, T* X, long long sX, int nrhs) {
+  typedef Num<T> N;
+  constexpr int NB = Num<T>::NBLK, RP = NB / 8, NS = NB / 16;
+  __shared__ T s_t[16][NB];
+  __shared__ T s_d[NB];
+  const int b = blockIdx.y, tid = threadIdx.x, lane = tid & 31, q = tid & 7;
+  const int col = blockIdx.x * 32 + (tid >> 3);
+  const T* F = LU + (long long)b * nb * nb + (long long)r0 * nb + r0;
+  T* x = X + b * sX + (long long)col * nb + r0;
+  if (!LOWER)
+    for (int i = tid; i < ib; i += 256) s_d[i] = N::recip(F[(long long)i * nb + i]);
+  T v[RP];
+#pragma unroll
+  for (int k = 0; k < RP; ++k) {
+    const int r = k * 8 + q;
+    v[k] = (col < nrhs && r < ib) ? x[r] : T();
+  }
+#pragma unroll
+  for (int s = 0; s < NS; ++s) {
+    const int i0 = (LOWER ? s : NS - 1 - s) * 16;
+    __syncthreads();
+    for (int e = tid; e < 16 * NB; e += 256) {
+      const int c = e / NB, r = e % NB;
+      s_t[c][r] = (i0 + c < ib && r < ib) ? F[(long long)(i0 + c) * nb + r] : T();
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < 16; ++u) {
+      const int t = LOWER ? u : 15 - u;
+      const int ki = (LOWER ? s : NS - 1 - s) * 2 + t / 8;   // register of row i = i0 + t in its owner (q = t % 8)
+      T xi = shfl(v[ki], (lane & 24) | (t & 7));
+      if (!LOWER) {
+        if (i0 + t < ib) {   // uniform
+          xi = N::mul(xi, s_d[i0 + t]);
+          if (q == (t & 7)) v[ki] = xi;
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < RP; ++k) {
+        if (LOWER ? k > ki : k < ki) v[k] = N::nma(s_t[t][k * 8 + q], xi, v[k]);
+        if (k == ki && (LOWER ? q > (t & 7) : q < (t & 7))) v[k] = N::nma(s_t[t][k * 8 + q], xi, v[k]);
+      }
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < RP; ++k) {
+    const int r = k * 8 + q;
+    if (col < nrhs && r < ib) x[r] = v[k];
+  }
+}
+
+__global__ void iota_rows(int* perm, int nb, int K) {
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < (long long)nb * K;
+       t += (long long)gridDim.x * blockDim.x)
+    perm[t] = (int)(t % nb);
+}
+
+__device__ __forceinline__ void conv(double2 a, double2& r) { r = a; }
+__device__ __forceinline__ void conv(double2 a, float2& r) { r = make_float2((float)a.x, (float)a.y); }
+
+// X[:, c][i] = B[:, c][perm[i]] between different buffers
+template <typename S, typename T>
+__global__ void permute_rows(const S* B, int nb, int nrhs, const int* perm, T* X, int K) {
+  const long long per = (long long)nb * nrhs;
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < per * K; t += (long long)gridDim.x * blockDim.x) {
+    const long long b = t / per, e = t - b * per;
+    const long long c = e / nb, i = e - c * nb;
+    conv(B[b * per + c * nb + perm[b * nb + i]], X[t]);
+  }
+}
+// in place, one column per CTA through shared memory
+__global__ void permute_rows_inplace(double2* X, int nb, int nrhs, const int* perm) {
+  extern __shared__ double2 s_col[];
+  double2* x = X + ((long long)blockIdx.y * nrhs + blockIdx.x) * nb;
+  for (int i = threadIdx.x; i < nb; i += blockDim.x) s_col[i] = x[i];
+  __syncthreads();
+  const int* pm = perm + (long long)blockIdx.y * nb;
+  for (int i = threadIdx.x; i < nb; i += blockDim.x) x[i] = s_col[pm[i]];
+}
+
+int grid1(long long n) {
+  const long long g = (n + 255) / 256;
+  return (int)(g < 8192 ? (g < 1 ? 1 : g) : 8192);
+}
+
+template <typename T, int W, int RPT>
+void launch_panel(Gemm& g, T* M, int nb, int K, int j0, int jw, int C, int* swp, int ss, int* info) {
+  const int rows = nb - j0;
+  const int per = (rows + C * RPT - 1) / (C * RPT);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(C, K);
+  cfg.blockDim = dim3((per + 31) / 32 * 32);
+  cfg.stream = g.st;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = C;
+  at.val.clusterDim.y = 1;
+  at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  g.note(cudaLaunchKernelEx(&cfg, lu_panel<T, W, RPT>, M, nb, j0, jw, swp, ss, info));
+}
+
+template <typename T, int W>
+void launch_swap_update(Gemm& g, T* M, int nb, int K, int o0, int j0, int jw, int oend, const int* swp, int ss) {
+  if (oend - o0 > jw) lu_swap<T, W><<<K, kOuter, 0, g.st>>>(M, nb, o0, oend, j0, jw, swp, ss);
+  const int r0 = j0 + jw;
+  if (r0 < oend) lu_update<T, W><<<dim3((nb - r0 + 63) / 64, (oend - r0 + 15) / 16, K), 128, 0, g.st>>>(M, nb, j0, jw, oend);
+}
+
+// Panel width and rows per thread by the panel's height: a row takes W registers pairs (quads in FP64), a
+// thread holds 64 of them, and a cluster has at most 8 x 512 threads.  FP64 panels are spread over the cluster
+// from 64 rows per CTA on (an SM does two FP64 FMAs a clock), FP32 panels from 512.
+template <typename T>
+int panel(Gemm& g, T* M, int nb, int K, int o0, int j0, int oend, int* info, int* swp, int ss) {
+  constexpr bool dbl = sizeof(T) == 16;
+  const int rows = nb - j0, left = oend - j0;
+  const int top = kMaxCluster * kPanelThreads;
+  auto cluster = [&](int per) {
+    const int c = (rows + per - 1) / per;
+    return c < 1 ? 1 : (c > kMaxCluster ? kMaxCluster : c);
+  };
+  int jw;
+  if (rows <= top) {
+    jw = left < 16 ? left : 16;
+    launch_panel<T, 16, 1>(g, M, nb, K, j0, jw, cluster(dbl ? 64 : kPanelThreads), swp, ss, info);
+    launch_swap_update<T, 16>(g, M, nb, K, o0, j0, jw, oend, swp, ss);
+  } else if (rows <= 2 * top) {
+    constexpr int W = dbl ? 8 : 16;
+    jw = left < W ? left : W;
+    launch_panel<T, W, 2>(g, M, nb, K, j0, jw, kMaxCluster, swp, ss, info);
+    launch_swap_update<T, W>(g, M, nb, K, o0, j0, jw, oend, swp, ss);
+  } else if (!dbl && rows <= 4 * top) {
+    jw = left < 8 ? left : 8;
+    launch_panel<T, 8, dbl ? 2 : 4>(g, M, nb, K, j0, jw, kMaxCluster, swp, ss, info);
+    launch_swap_update<T, 8>(g, M, nb, K, o0, j0, jw, oend, swp, ss);
+  } else {
+    jw = left < 16 ? left : 16;
+    lu_panel_global<T><<<K, kPanelThreads, 0, g.st>>>(M, nb, j0, jw, swp, ss, info);
+    launch_swap_update<T, 16>(g, M, nb, K, o0, j0, jw, oend, swp, ss);
+  }
+  return jw;
+}
+
+// X = T^{-1} X for the unit lower triangle (LOWER) or the upper triangle of rows and columns r0 .. r1 - 1 of LU
+template <typename T, bool LOWER>
+void solve_range(Gemm& g, const T* LU, int nb, int K, int r0, int r1, T* X, long long sX, int nrhs) {
+  constexpr int NB = Num<T>::NBLK;
+  const long long n2 = (long long)nb * nb;
+  const dim3 grid((nrhs + 31) / 32, K);
+  const int nblk = (r1 - r0 + NB - 1) / NB;
+  for (int bi = 0; bi < nblk; ++bi) {
+    const int s0 = r0 + (LOWER ? bi : nblk - 1 - bi) * NB, ib = r1 - s0 < NB ? r1 - s0 : NB;
+    lu_trsm<T, LOWER><<<grid, 256, 0, g.st>>>(LU, nb, s0, ib, X, sX, nrhs);
+    const int d0 = LOWER ? s0 + ib : r0, d1 = LOWER ? r1 : s0;   // rows still to be updated
+    if (d1 > d0)
+      gemm(g, K, d1 - d0, nrhs, ib, -1.0, LU + (long long)s0 * nb + d0, nb, n2, 0, X + s0, nb, sX, true, X + d0, nb, sX);
+  }
+}
+
+template <typename T> void lu_factor_t(Gemm& g, T* M, int nb, int K, int* perm, int* info, int* swp) {
+  const long long n2 = (long long)nb * nb;
+  const int ss = lu_swap_ints(nb);
+  iota_rows<<<grid1((long long)nb * K), 256, 0, g.st>>>(perm, nb, K);
+  for (int o0 = 0; o0 < nb; o0 += kOuter) {
+    const int oend = nb - o0 < kOuter ? nb : o0 + kOuter, out = nb - (oend - o0) + 1, rest = nb - oend;
+    int np = 0;
+    for (int j0 = o0; j0 < oend; ++np) {
+      int* lists = swp + np * kSwapInts;
+      // nb <= kOuter: one list per matrix, applied to perm after every panel
+      if (ss == kSwapInts) lists = swp;
+      j0 += panel<T>(g, M, nb, K, o0, j0, oend, info, lists, ss);
+      if (ss == kSwapInts) lu_swap_rest<T><<<dim3(1, K), 64, 0, g.st>>>(M, nb, o0, oend, 1, swp, ss, perm);
+    }
+    if (ss == kSwapInts) continue;
+    lu_swap_rest<T><<<dim3((out + 63) / 64, K), 64, 0, g.st>>>(M, nb, o0, oend, np, swp, ss, perm);
+    if (rest > 0) {
+      // U12 = L11^{-1} A12, then A22 -= L21 U12
+      solve_range<T, true>(g, M, nb, K, o0, oend, M + (long long)oend * nb, n2, rest);
+      gemm(g, K, rest, rest, oend - o0, -1.0, M + (long long)o0 * nb + oend, nb, n2, 0, M + (long long)oend * nb + o0, nb, n2,
+           true, M + (long long)oend * nb + oend, nb, n2);
+    }
+  }
+  g.note(cudaGetLastError());
+}
+
+template <typename T> void lu_solve_t(Gemm& g, const T* LU, int nb, int K, T* X, int nrhs) {
+  const long long sx = (long long)nb * nrhs;
+  solve_range<T, true>(g, LU, nb, K, 0, nb, X, sx, nrhs);
+  solve_range<T, false>(g, LU, nb, K, 0, nb, X, sx, nrhs);
+  g.note(cudaGetLastError());
+}
+
+}  // namespace
+
+int lu_swap_ints(int nb) { return nb <= kOuter ? kSwapInts : kMaxPanels * kSwapInts; }
+
+void lu_factor(Gemm& g, double2* M, int nb, int K, int* perm, int* info, int* swp) {
+  lu_factor_t<double2>(g, M, nb, K, perm, info, swp);
+}
+void lu_factor(Gemm& g, float2* M, int nb, int K, int* perm, int* info, int* swp) {
+  lu_factor_t<float2>(g, M, nb, K, perm, info, swp);
+}
+void lu_solve(Gemm& g, const double2* LU, int nb, int K, double2* X, int nrhs) { lu_solve_t<double2>(g, LU, nb, K, X, nrhs); }
+void lu_solve(Gemm& g, const float2* LU, int nb, int K, float2* X, int nrhs) { lu_solve_t<float2>(g, LU, nb, K, X, nrhs); }
+
+void lu_permute(Gemm& g, const double2* B, int nb, int K, const int* perm, float2* X, int nrhs) {
+  permute_rows<double2, float2><<<grid1((long long)nb * nrhs * K), 256, 0, g.st>>>(B, nb, nrhs, perm, X, K);
+  g.note(cudaGetLastError());
+}
+
+void lu_permute(Gemm& g, const double2* B, int nb, int K, const int* perm, double2* X, int nrhs) {
+  if (B != X) {
+    permute_rows<double2, double2><<<grid1((long long)nb * nrhs * K), 256, 0, g.st>>>(B, nb, nrhs, perm, X, K);
+    g.note(cudaGetLastError());
+    return;
+  }
+  const size_t smem = (size_t)nb * sizeof(double2);
+  if (smem <= 216 * 1024) {
+    g.note(cudaFuncSetAttribute(permute_rows_inplace, cudaFuncAttributeMaxDynamicSharedMemorySize, 216 * 1024));
+    permute_rows_inplace<<<dim3(nrhs, K), nb < 256 ? 64 : 256, smem, g.st>>>(X, nb, nrhs, perm);
+    g.note(cudaGetLastError());
+    return;
+  }
+  // taller columns: through a copy of a few columns at a time
+  const int cols = 64;
+  void* w = nullptr;
+  if (!g.h || handle_ensure(g.h, 8, (size_t)nb * cols * sizeof(double2), &w) != RSFD_OK) {
+    g.note(cudaErrorMemoryAllocation);
+    return;
+  }
+  for (int b = 0; b < K; ++b)
+    for (int c0 = 0; c0 < nrhs; c0 += cols) {
+      const int nc = nrhs - c0 < cols ? nrhs - c0 : cols;
+      double2* x = X + ((long long)b * nrhs + c0) * nb;
+      g.note(cudaMemcpyAsync(w, x, (size_t)nb * nc * sizeof(double2), cudaMemcpyDeviceToDevice, g.st));
+      permute_rows<double2, double2><<<grid1((long long)nb * nc), 256, 0, g.st>>>((const double2*)w, nb, nc,
+                                                                                perm + (long long)b * nb, x, 1);
+    }
+  g.note(cudaGetLastError());
+}
+
+}  // namespace rsfd

@@ -31,6 +31,7 @@
 // the measured cuBLAS bf16 burst; the CUDA-core kernel takes 132 ms for the same (FP64 pipe, 1.3e11/s).
 
 #include <cuda_runtime.h>
+#include <math_constants.h>
 #include <stdint.h>
 
 #include "rsfd_internal.cuh"
@@ -38,24 +39,30 @@
 namespace rsfd {
 namespace {
 
-constexpr int OZ_S = 8;                       // digits
+// digits per element: 8 for FP64 operands, 4 for FP32 operands
+template <typename T> struct OzOf;
+template <> struct OzOf<double2> { static constexpr int S = 8, NA = 5; };
+template <> struct OzOf<float2> { static constexpr int S = 4, NA = 10; };
+
 constexpr int OZ_BM = 128;                    // rows of C per CTA
-constexpr int OZ_BN = 32;                     // columns of C per CTA
 constexpr int OZ_KS = 16;                     // complex k per step (one MMA depth)
 constexpr int OZ_CHUNK = 8;                   // k-steps between two emptyings of the accumulators
-constexpr int OZ_ABLK = OZ_S * OZ_BM * OZ_KS * 2;        // bytes of one plane of A per k-step (32 KB)
-constexpr int OZ_BPLANE = OZ_S * OZ_BN * OZ_KS * 2;      // bytes of one plane of B per k-step (8 KB)
-constexpr int OZ_BBLK = 2 * OZ_BPLANE;
-constexpr int OZ_NA = 5;                      // ring of A planes
 constexpr int OZ_NB = 3;                      // ring of B blocks
-constexpr int OZ_SMEM = OZ_NA * OZ_ABLK + OZ_NB * OZ_BBLK + 1024;
+constexpr int OZ_BPLANE = 256 * OZ_KS * 2;    // bytes of one plane of B per k-step: digits x columns = 256 rows
+constexpr int OZ_BBLK = 2 * OZ_BPLANE;
 constexpr int OZ_EPI = 512;                   // epilogue threads (16 warps: 64 accumulator registers each)
-constexpr int OZ_EC = OZ_BN / (OZ_EPI / 128); // columns per epilogue thread
 constexpr int OZ_THREADS = OZ_EPI + 64;
-static_assert(OZ_EC == 8, "the accumulators are read eight columns at a time");
+template <int S> struct OzDim {
+  static constexpr int BN = 256 / S;                 // columns of C per CTA
+  static constexpr int EC = BN / (OZ_EPI / 128);     // columns per epilogue thread
+  static constexpr int ABLK = S * OZ_BM * OZ_KS * 2; // bytes of one plane of A per k-step
+};
+template <typename T> constexpr int oz_smem() {
+  return OzOf<T>::NA * OzDim<OzOf<T>::S>::ABLK + OZ_NB * OZ_BBLK + 1024;
+}
 constexpr uint32_t OZ_SBO = 128;
 constexpr uint32_t OZ_LBO_A = (OZ_BM / 8) * 128;
-constexpr uint32_t OZ_LBO_B = (OZ_S * OZ_BN / 8) * 128;
+constexpr uint32_t OZ_LBO_B = (256 / 8) * 128;
 constexpr int kOzWaitCap = 1 << 12;           // attempts of a bounded wait, each up to 1 ms
 constexpr uint32_t kOzHintNs = 1000000;
 
@@ -111,8 +118,8 @@ __device__ __forceinline__ void oz_tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
 }
 
 // one operand: element (row, k) of matrix b at p[b sb + row rs + k ks] (row: a row of op(A) or a column of B)
-struct OzOperand {
-  const double2* p;
+template <typename T> struct OzOperand {
+  const T* p;
   long long sb, rs, ks;
   int rows;         // m or n
   int conj;
@@ -121,25 +128,30 @@ struct OzOperand {
   unsigned char* dig;   // digit planes
   int rows_pad;
 };
-struct OzSplit {
-  OzOperand o[2];
+template <typename T> struct OzSplit {
+  OzOperand<T> o[2];
   int k, ksteps, batch;
 };
 
-// Largest component of every row: high words (sign cleared) compared as integers.  Rows contiguous in
-// memory (rs = 1): a thread per row; k contiguous: a warp per row.  Bound: one read of the operand.
-__global__ void __launch_bounds__(256) oz_rowmax(OzSplit q) {
-  const OzOperand& o = q.o[blockIdx.z & 1];
+// sign-cleared leading word of a component: ordered like its magnitude
+__device__ __forceinline__ unsigned oz_word(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
+__device__ __forceinline__ unsigned oz_word(float x) { return __float_as_uint(x) & 0x7fffffffu; }
+template <typename T> __device__ __forceinline__ unsigned oz_word2(T v) { return max(oz_word(v.x), oz_word(v.y)); }
+// words of infinities and NaN start here
+template <typename T> __host__ __device__ constexpr unsigned oz_nonfinite() { return sizeof(T) == 16 ? 0x7ff00000u : 0x7f800000u; }
+
+// Largest component of every row: leading words compared as integers.  Rows contiguous in memory
+// (rs = 1): a thread per row; k contiguous: a warp per row.  Bound: one read of the operand.
+template <typename T> __global__ void __launch_bounds__(256) oz_rowmax(OzSplit<T> q) {
+  const OzOperand<T>& o = q.o[blockIdx.z & 1];
   const int b = blockIdx.z >> 1;
-  const double2* p = o.p + b * o.sb;
+  const T* p = o.p + b * o.sb;
   if (o.ks != 1) {
     const int row = blockIdx.x * 32 + (threadIdx.x & 31);
     unsigned int m = 0;
     if (row < o.rows)
-      for (int k = blockIdx.y * 64 + (threadIdx.x >> 5); k < min(q.k, (int)blockIdx.y * 64 + 64); k += 8) {
-        const double2 v = p[row * o.rs + k * o.ks];
-        m = max(m, max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu));
-      }
+      for (int k = blockIdx.y * 64 + (threadIdx.x >> 5); k < min(q.k, (int)blockIdx.y * 64 + 64); k += 8)
+        m = max(m, oz_word2(p[row * o.rs + k * o.ks]));
     __shared__ unsigned int s[8][32];
     s[threadIdx.x >> 5][threadIdx.x & 31] = m;
     __syncthreads();
@@ -154,23 +166,21 @@ __global__ void __launch_bounds__(256) oz_rowmax(OzSplit q) {
       const int row = blockIdx.x * 32 + r;
       if (row >= o.rows) break;
       unsigned int m = 0;
-      for (int k = blockIdx.y * 64 + (threadIdx.x & 31); k < min(q.k, (int)blockIdx.y * 64 + 64); k += 32) {
-        const double2 v = p[row * o.rs + k];
-        m = max(m, max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu));
-      }
+      for (int k = blockIdx.y * 64 + (threadIdx.x & 31); k < min(q.k, (int)blockIdx.y * 64 + 64); k += 32)
+        m = max(m, oz_word2(p[row * o.rs + k]));
       m = __reduce_max_sync(0xffffffffu, m);
       if ((threadIdx.x & 31) == 0) atomicMax(o.ex + (size_t)b * o.rows_pad + row, m);
     }
   }
 }
 
-// binary exponent se with |x| < 2^se for every component of a row whose largest high word is w
-__device__ __forceinline__ int oz_exponent(unsigned int w) {
-  const int e = (int)(w >> 20);
-  return (e < 1 ? 1 : e) - 1022;
+// binary exponent se with |x| < 2^se for every component of a row whose largest leading word is w
+template <typename T> __device__ __forceinline__ int oz_exponent(unsigned int w) {
+  const int e = (int)(w >> (sizeof(T) == 16 ? 20 : 23));
+  return (e < 1 ? 1 : e) - (sizeof(T) == 16 ? 1022 : 126);
 }
 
-// fixed point rint(x 2^(62 - se)), integer arithmetic only
+// fixed point rint(x 2^(62 - se)) (FP64) or rint(x 2^(30 - se)) (FP32), integer arithmetic only
 __device__ __forceinline__ long long oz_fixed(double x, int se) {
   const unsigned long long u = (unsigned long long)__double_as_longlong(x);
   const int e = (int)((u >> 52) & 0x7ff);
@@ -181,23 +191,35 @@ __device__ __forceinline__ long long oz_fixed(double x, int se) {
   else m = sh > -62 ? (m + (1ull << (-sh - 1))) >> (-sh) : 0ull;
   return (u >> 63) ? -(long long)m : (long long)m;
 }
+__device__ __forceinline__ int oz_fixed(float x, int se) {
+  const unsigned u = __float_as_uint(x);
+  const int e = (int)((u >> 23) & 0xff);
+  unsigned m = u & 0x7fffffu;
+  if (e > 0) m |= 1u << 23;
+  const int sh = (e < 1 ? 1 : e) - 150 - se + 30;    // at most 6
+  if (sh >= 0) m <<= sh;
+  else m = sh > -30 ? (m + (1u << (-sh - 1))) >> (-sh) : 0u;
+  return (u >> 31) ? -(int)m : (int)m;
+}
 
 // Digit planes.  A thread takes 8 consecutive k of one row: 8 loads, then one 16-byte store per digit and
 // plane (consecutive rows are 16 bytes apart, so a warp stores 512 contiguous bytes).
-// Bound: the stores (32 bytes per element) and one read.
-__global__ void __launch_bounds__(256) oz_digits(OzSplit q) {
-  const OzOperand& o = q.o[blockIdx.z & 1];
+// Bound: the stores (4 bytes per digit and element) and one read.
+template <typename T> __global__ void __launch_bounds__(256) oz_digits(OzSplit<T> q) {
+  constexpr int S = OzOf<T>::S, BN = OzDim<S>::BN, ABLK = OzDim<S>::ABLK;
+  typedef decltype(oz_fixed(T().x, 0)) I;
+  const OzOperand<T>& o = q.o[blockIdx.z & 1];
   const int b = blockIdx.z >> 1;
   const int row = blockIdx.x * 32 + (threadIdx.x & 31);
   const int kg = blockIdx.y * 8 + (threadIdx.x >> 5);   // group of 8 k
   if (row >= o.rows_pad || kg >= 2 * q.ksteps) return;
-  const double2* p = o.p + b * o.sb + (long long)row * o.rs;
-  const int se = row < o.rows ? oz_exponent(o.ex[(size_t)b * o.rows_pad + row]) : 0;
-  long long xr[8], xi[8];
+  const T* p = o.p + b * o.sb + (long long)row * o.rs;
+  const int se = row < o.rows ? oz_exponent<T>(o.ex[(size_t)b * o.rows_pad + row]) : 0;
+  I xr[8], xi[8];
 #pragma unroll
   for (int t = 0; t < 8; ++t) {
     const int k = kg * 8 + t;
-    double2 v = make_double2(0.0, 0.0);
+    T v = T();
     if (row < o.rows && k < q.k) v = p[k * o.ks];
     if (o.conj) v.y = -v.y;
     xr[t] = oz_fixed(v.x, se);
@@ -207,27 +229,27 @@ __global__ void __launch_bounds__(256) oz_digits(OzSplit q) {
   unsigned char *d0, *d1;   // digit 0 (leading) of the two planes
   uint32_t step;            // bytes from one digit to the next
   if (o.is_b) {
-    const int nt = row / OZ_BN, r = row % OZ_BN;
-    unsigned char* blk = o.dig + (((size_t)b * (o.rows_pad / OZ_BN) + nt) * q.ksteps + ks) * OZ_BBLK;
-    d0 = blk + kh * OZ_LBO_B + r * 16;      // stacked row = digit * 32 + r
+    const int nt = row / BN, r = row % BN;
+    unsigned char* blk = o.dig + (((size_t)b * (o.rows_pad / BN) + nt) * q.ksteps + ks) * OZ_BBLK;
+    d0 = blk + kh * OZ_LBO_B + r * 16;      // stacked row = digit * BN + r
     d1 = d0 + OZ_BPLANE;
-    step = OZ_BN * 16;
+    step = BN * 16;
   } else {
     const int mt = row / OZ_BM, r = row % OZ_BM;
-    unsigned char* blk = o.dig + (((size_t)b * (o.rows_pad / OZ_BM) + mt) * q.ksteps + ks) * (2 * OZ_ABLK);
+    unsigned char* blk = o.dig + (((size_t)b * (o.rows_pad / OZ_BM) + mt) * q.ksteps + ks) * (2 * ABLK);
     d0 = blk + kh * OZ_LBO_A + r * 16;
-    d1 = d0 + OZ_ABLK;
+    d1 = d0 + ABLK;
     step = OZ_BM * OZ_KS * 2;
   }
 #pragma unroll
-  for (int s = OZ_S - 1; s >= 0; --s) {
+  for (int s = S - 1; s >= 0; --s) {
     uint32_t wr[4], wi[4];
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
       float f[4];
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        long long &a = xr[2 * t + h], &c = xi[2 * t + h];
+        I &a = xr[2 * t + h], &c = xi[2 * t + h];
         const int da = s > 0 ? (int)(signed char)(a & 0xff) : (int)a;
         const int dc = s > 0 ? (int)(signed char)(c & 0xff) : (int)c;
         a = (a - da) >> 8;
@@ -243,26 +265,70 @@ __global__ void __launch_bounds__(256) oz_digits(OzSplit q) {
   }
 }
 
-struct OzGemm {
+template <typename T> struct OzGemm {
   const unsigned char *A, *B;
   const unsigned int *exA, *exB;
   int m, n, m_pad, n_pad, ksteps;
-  double sign;        // alpha (+1 or -1)
+  int sign;           // alpha (+1 or -1)
   int add;            // 1: add C
-  double2* C;
+  T* C;
   int ldc;
   long long sC;
   int* err;
 };
 
-__global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_kernel(OzGemm q) {
+// (hi 2^32 + lo) 2^e rounded to nearest, by integer arithmetic (conversions and FP64 arithmetic run at 2 a
+// clock and SM): FP64 result of the 8-digit form
+__device__ __forceinline__ double oz_round(long long hi, long long lo, int e) {
+  long long h = hi + (lo >> 32);
+  unsigned l = (unsigned)lo;
+  const bool neg = h < 0;
+  if (neg) {
+    h = -h - (l != 0u);
+    l = 0u - l;
+  }
+  unsigned long long m;     // leading 64 bits of the magnitude, top bit at 63
+  int x;                    // value = m 2^x (bits below m only matter as a rounding tie and are dropped)
+  if (h != 0) {
+    const int z = __clzll(h);
+    m = (unsigned long long)h << z;
+    if (z <= 32) m |= (unsigned long long)l >> (32 - z);
+    else m |= (unsigned long long)l << (z - 32);
+    x = 32 - z;
+  } else {
+    if (l == 0u) return 0.0;
+    const int z = __clz(l);
+    m = (unsigned long long)l << (32 + z);
+    x = -32 - z;
+  }
+  const int ex = x + e + 63 + 1023;   // biased exponent of the leading bit
+  if (ex <= 0 || ex >= 2046) {        // near the ends of the range: the library's scaling
+    const double v = scalbn((double)m, x + e);
+    return neg ? -v : v;
+  }
+  // 53 bits, round half up; a carry out of the mantissa raises the exponent field by itself
+  const unsigned long long r = (m + 0x400ull) >> 11;
+  const unsigned long long bits = r < (1ull << 52) ? ((unsigned long long)(ex + 1) << 52)   // m + 0x400 wrapped
+                                                   : ((unsigned long long)(ex - 1) << 52) + r;
+  return __longlong_as_double((long long)(bits | (neg ? 1ull << 63 : 0ull)));
+}
+// FP32 result of the 4-digit form: hi 2^e
+__device__ __forceinline__ float oz_round(long long hi, int e) {
+  const int h = (int)(hi >> 32);
+  const unsigned l = (unsigned)hi;
+  return scalbnf(fmaf((float)h, 0x1p32f, (float)l), e);
+}
+
+template <typename T> __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_kernel(OzGemm<T> q) {
+  constexpr int S = OzOf<T>::S, NA = OzOf<T>::NA, BN = OzDim<S>::BN, EC = OzDim<S>::EC, ABLK = OzDim<S>::ABLK;
+  constexpr int SW = S / 4;   // 64-bit sums per component
   extern __shared__ __align__(1024) unsigned char oz_smem_raw[];
-  __shared__ __align__(8) uint64_t fullA[OZ_NA], emptyA[OZ_NA], fullB[OZ_NB], emptyB[OZ_NB], accFull, accEmpty, mmaDone;
+  __shared__ __align__(8) uint64_t fullA[NA], emptyA[NA], fullB[OZ_NB], emptyB[OZ_NB], accFull, accEmpty, mmaDone;
   __shared__ uint32_t tmem_s;
   __shared__ volatile int s_abort;
   unsigned char* smem = (unsigned char*)(((uintptr_t)oz_smem_raw + 1023) & ~(uintptr_t)1023);
   unsigned char* sA = smem;
-  unsigned char* sB = smem + OZ_NA * OZ_ABLK;
+  unsigned char* sB = smem + NA * ABLK;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int mt = blockIdx.x, nt = blockIdx.y, b = blockIdx.z;
   if (warp == 0) {
@@ -271,17 +337,20 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_kernel(OzGemm q) {
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   if (tid == 0) {
-    for (int i = 0; i < OZ_NA; ++i) {
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(oz_saddr(&fullA[i])) : "memory");
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(oz_saddr(&emptyA[i])) : "memory");
+    auto init = [](uint64_t* bar, int count) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(oz_saddr(bar)), "r"(count) : "memory");
+    };
+    for (int i = 0; i < NA; ++i) {
+      init(&fullA[i], 1);
+      init(&emptyA[i], 1);
     }
     for (int i = 0; i < OZ_NB; ++i) {
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(oz_saddr(&fullB[i])) : "memory");
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(oz_saddr(&emptyB[i])) : "memory");
+      init(&fullB[i], 1);
+      init(&emptyB[i], 1);
     }
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(oz_saddr(&accFull)) : "memory");
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(oz_saddr(&mmaDone)) : "memory");
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(oz_saddr(&accEmpty)), "r"(OZ_EPI) : "memory");
+    init(&accFull, 1);
+    init(&mmaDone, 1);
+    init(&accEmpty, OZ_EPI);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     s_abort = 0;
   }
@@ -295,8 +364,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_kernel(OzGemm q) {
   if (warp == OZ_EPI / 32) {
     // copies: per k-step B (both planes), then the two planes of A
     if (lane == 0) {
-      const unsigned char* gA = q.A + ((size_t)b * (q.m_pad / OZ_BM) + mt) * ksteps * (2 * OZ_ABLK);
-      const unsigned char* gB = q.B + ((size_t)b * (q.n_pad / OZ_BN) + nt) * ksteps * OZ_BBLK;
+      const unsigned char* gA = q.A + ((size_t)b * (q.m_pad / OZ_BM) + mt) * ksteps * (2 * ABLK);
+      const unsigned char* gB = q.B + ((size_t)b * (q.n_pad / BN) + nt) * ksteps * OZ_BBLK;
       bool ok = true;
       int issuedA = 0, issuedB = 0;
       for (int t = 0; t < ksteps && ok; ++t) {
@@ -306,10 +375,10 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_kernel(OzGemm q) {
         oz_bulk(oz_saddr(sB + sb * OZ_BBLK), gB + (size_t)t * OZ_BBLK, OZ_BBLK, oz_saddr(&fullB[sb]));
         issuedB = t + 1;
         for (int h = 0; h < 2 && ok; ++h) {
-          const int a = 2 * t + h, sa = a % OZ_NA;
-          if (a >= OZ_NA) ok = oz_wait(oz_saddr(&emptyA[sa]), (uint32_t)((a / OZ_NA - 1) & 1));
+          const int a = 2 * t + h, sa = a % NA;
+          if (a >= NA) ok = oz_wait(oz_saddr(&emptyA[sa]), (uint32_t)((a / NA - 1) & 1));
           if (!ok || s_abort) break;
-          oz_bulk(oz_saddr(sA + sa * OZ_ABLK), gA + (size_t)a * OZ_ABLK, OZ_ABLK, oz_saddr(&fullA[sa]));
+          oz_bulk(oz_saddr(sA + sa * ABLK), gA + (size_t)a * ABLK, ABLK, oz_saddr(&fullA[sa]));
           issuedA = a + 1;
         }
       }
@@ -318,8 +387,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_kernel(OzGemm q) {
         // the last one issued (earlier ones completed before the entry was refilled)
         s_abort = 1;
         atomicExch(q.err, 1);
-        for (int a = max(0, issuedA - OZ_NA); a < issuedA; ++a)
-          oz_wait(oz_saddr(&fullA[a % OZ_NA]), (uint32_t)((a / OZ_NA) & 1));
+        for (int a = max(0, issuedA - NA); a < issuedA; ++a)
+          oz_wait(oz_saddr(&fullA[a % NA]), (uint32_t)((a / NA) & 1));
         for (int c = max(0, issuedB - OZ_NB); c < issuedB; ++c)
           oz_wait(oz_saddr(&fullB[c % OZ_NB]), (uint32_t)((c / OZ_NB) & 1));
       }
@@ -339,21 +408,21 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_kernel(OzGemm q) {
         const uint32_t b0 = oz_saddr(sB + sb * OZ_BBLK);
         const uint64_t bre = oz_desc(b0, OZ_LBO_B), bim = oz_desc(b0 + OZ_BPLANE, OZ_LBO_B);
         for (int h = 0; h < 2 && ok; ++h) {
-          const int a = 2 * t + h, sa = a % OZ_NA;
-          ok = oz_wait(oz_saddr(&fullA[sa]), (uint32_t)((a / OZ_NA) & 1));
+          const int a = 2 * t + h, sa = a % NA;
+          ok = oz_wait(oz_saddr(&fullA[sa]), (uint32_t)((a / NA) & 1));
           if (!ok || s_abort) {
             ok = false;
             break;
           }
-          const uint32_t a0 = oz_saddr(sA + sa * OZ_ABLK);
+          const uint32_t a0 = oz_saddr(sA + sa * ABLK);
           // h = 0: Re += Ar Br, Im += Ar Bi;  h = 1: Re -= Ai Bi, Im += Ai Br
 #pragma unroll
-          for (int i = 0; i < OZ_S; ++i) {
+          for (int i = 0; i < S; ++i) {
             const uint64_t ad = oz_desc(a0 + i * (OZ_BM * OZ_KS * 2), OZ_LBO_A);
             const uint32_t acc = (first && h == 0 && i == 0) ? 0u : 1u;
-            const int N = OZ_BN * (OZ_S - i);
-            oz_mma(tmem + i * OZ_BN, ad, h ? bim : bre, h ? oz_idesc(N, 1) : oz_idesc(N, 0), acc);
-            oz_mma(tmem + 256 + i * OZ_BN, ad, h ? bre : bim, oz_idesc(N, 0), acc);
+            const int N = BN * (S - i);
+            oz_mma(tmem + i * BN, ad, h ? bim : bre, h ? oz_idesc(N, 1) : oz_idesc(N, 0), acc);
+            oz_mma(tmem + 256 + i * BN, ad, h ? bre : bim, oz_idesc(N, 0), acc);
           }
           oz_commit(oz_saddr(&emptyA[sa]));
         }
@@ -370,14 +439,16 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_kernel(OzGemm q) {
       }
     }
   } else {
-    // epilogue threads: row 32 (warp % 4) + lane, columns OZ_EC (warp / 4) ... of Re and of Im
-    const int ch = (warp >> 2) * OZ_EC;
+    // epilogue threads: row 32 (warp % 4) + lane, columns EC (warp / 4) ... of Re and of Im
+    const int ch = (warp >> 2) * EC;
     const uint32_t tl = tmem + ((uint32_t)((warp & 3) * 32) << 16) + ch;
-    long long hi[2][OZ_EC], lo[2][OZ_EC];
+    long long sum[2][SW][EC];
 #pragma unroll
     for (int p = 0; p < 2; ++p)
 #pragma unroll
-      for (int j = 0; j < OZ_EC; ++j) hi[p][j] = lo[p][j] = 0;
+      for (int w = 0; w < SW; ++w)
+#pragma unroll
+        for (int j = 0; j < EC; ++j) sum[p][w][j] = 0;
     bool ok = true;
     for (int c = 0; c < nchunks; ++c) {
       ok = oz_wait(oz_saddr(&accFull), (uint32_t)(c & 1));
@@ -390,22 +461,25 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_kernel(OzGemm q) {
 #pragma unroll
       for (int p = 0; p < 2; ++p) {
 #pragma unroll
-        for (int d = 0; d < OZ_S; d += 2) {
-          uint32_t r0[OZ_EC], r1[OZ_EC];
-          oz_tmem_ld8(tl + p * 256 + d * OZ_BN, r0);
-          oz_tmem_ld8(tl + p * 256 + (d + 1) * OZ_BN, r1);
-          // the registers pass through the wait so that no use moves above it
-          asm volatile("tcgen05.wait::ld.sync.aligned;"
-                       : "+r"(r0[0]), "+r"(r0[1]), "+r"(r0[2]), "+r"(r0[3]), "+r"(r0[4]), "+r"(r0[5]), "+r"(r0[6]),
-                         "+r"(r0[7]), "+r"(r1[0]), "+r"(r1[1]), "+r"(r1[2]), "+r"(r1[3]), "+r"(r1[4]), "+r"(r1[5]),
-                         "+r"(r1[6]), "+r"(r1[7])
-                       :
-                       : "memory");
+        for (int d = 0; d < S; d += 2) {
 #pragma unroll
-          for (int j = 0; j < OZ_EC; ++j) {
-            long long& acc = d < 4 ? hi[p][j] : lo[p][j];
-            acc += (long long)__float2int_rn(__uint_as_float(r0[j])) * (1ll << (8 * (3 - (d & 3))));
-            acc += (long long)__float2int_rn(__uint_as_float(r1[j])) * (1ll << (8 * (2 - (d & 3))));
+          for (int j0 = 0; j0 < EC; j0 += 8) {
+            uint32_t r0[8], r1[8];
+            oz_tmem_ld8(tl + p * 256 + d * BN + j0, r0);
+            oz_tmem_ld8(tl + p * 256 + (d + 1) * BN + j0, r1);
+            // the registers pass through the wait so that no use moves above it
+            asm volatile("tcgen05.wait::ld.sync.aligned;"
+                         : "+r"(r0[0]), "+r"(r0[1]), "+r"(r0[2]), "+r"(r0[3]), "+r"(r0[4]), "+r"(r0[5]), "+r"(r0[6]),
+                           "+r"(r0[7]), "+r"(r1[0]), "+r"(r1[1]), "+r"(r1[2]), "+r"(r1[3]), "+r"(r1[4]), "+r"(r1[5]),
+                           "+r"(r1[6]), "+r"(r1[7])
+                         :
+                         : "memory");
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              long long& acc = sum[p][d / 4][j0 + j];
+              acc += (long long)__float2int_rn(__uint_as_float(r0[j])) * (1ll << (8 * (3 - (d & 3))));
+              acc += (long long)__float2int_rn(__uint_as_float(r1[j])) * (1ll << (8 * (2 - (d & 3))));
+            }
           }
         }
       }
@@ -419,23 +493,33 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_kernel(OzGemm q) {
     const int row = mt * OZ_BM + (warp & 3) * 32 + lane;
     if (ok && row < q.m) {
       const unsigned int wa = q.exA[(size_t)b * q.m_pad + row];
-      const int ea = oz_exponent(wa);
+      const int ea = oz_exponent<T>(wa);
 #pragma unroll
-      for (int j = 0; j < OZ_EC; ++j) {
-        const int col = nt * OZ_BN + ch + j;
+      for (int j = 0; j < EC; ++j) {
+        const int col = nt * BN + ch + j;
         if (col < q.n) {
           const unsigned int wb = q.exB[(size_t)b * q.n_pad + col];
-          const int e = ea + oz_exponent(wb) - 68;
-          double re = scalbn(fma((double)hi[0][j], 0x1p32, (double)lo[0][j]), e) * q.sign;
-          double im = scalbn(fma((double)hi[1][j], 0x1p32, (double)lo[1][j]), e) * q.sign;
-          if (wa >= 0x7ff00000u || wb >= 0x7ff00000u) re = im = __longlong_as_double(0x7ff8000000000000ll);
-          double2* cp = q.C + b * q.sC + (long long)col * q.ldc + row;
-          if (q.add) {
-            const double2 o = *cp;
-            re += o.x;
-            im += o.y;
+          const int e = ea + oz_exponent<T>(wb);
+          T v;
+          if constexpr (S == 8) {
+            v.x = oz_round(sum[0][0][j], sum[0][SW - 1][j], e - 68);
+            v.y = oz_round(sum[1][0][j], sum[1][SW - 1][j], e - 68);
+          } else {
+            v.x = oz_round(sum[0][0][j], e - 36);
+            v.y = oz_round(sum[1][0][j], e - 36);
           }
-          *cp = make_double2(re, im);
+          if (wa >= oz_nonfinite<T>() || wb >= oz_nonfinite<T>()) v.x = v.y = CUDART_NAN_F;
+          T* cp = q.C + b * q.sC + (long long)col * q.ldc + row;
+          T o = T();
+          if (q.add) o = *cp;
+          if (q.sign < 0) {
+            o.x -= v.x;
+            o.y -= v.y;
+          } else {
+            o.x += v.x;
+            o.y += v.y;
+          }
+          *cp = o;
         }
       }
     }
@@ -447,80 +531,64 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_kernel(OzGemm q) {
 
 size_t up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-}  // namespace
-
-// bytes of digits and exponents for one matrix product m x n x k
-size_t oz_bytes(int m, int n, int k) {
-  const size_t mp = up(m, OZ_BM), np = up(n, OZ_BN), ks = (k + OZ_KS - 1) / OZ_KS;
-  return mp / OZ_BM * ks * 2 * OZ_ABLK + np / OZ_BN * ks * OZ_BBLK + up((mp + np) * sizeof(unsigned int), 256);
+template <typename T> size_t oz_bytes_t(int m, int n, int k) {
+  constexpr int S = OzOf<T>::S;
+  const size_t mp = up(m, OZ_BM), np = up(n, OzDim<S>::BN), ks = (k + OZ_KS - 1) / OZ_KS;
+  return mp / OZ_BM * ks * 2 * OzDim<S>::ABLK + np / OzDim<S>::BN * ks * OZ_BBLK + up((mp + np) * sizeof(unsigned int), 256);
 }
 
-cudaError_t oz_zgemm(cudaStream_t st, int batch, int m, int n, int k, double sign, const double2* A, int lda,
-                     long long sA, int opA, const double2* B, int ldb, long long sB, int add, double2* C, int ldc,
-                     long long sC, void* work, size_t work_bytes, int* err) {
-  const size_t per = oz_bytes(m, n, k);
+template <typename T>
+cudaError_t oz_gemm_t(cudaStream_t st, int batch, int m, int n, int k, int sign, const T* A, int lda, long long sA,
+                      int opA, const T* B, int ldb, long long sB, int add, T* C, int ldc, long long sC, void* work,
+                      size_t work_bytes, int* err) {
+  constexpr int S = OzOf<T>::S, BN = OzDim<S>::BN, ABLK = OzDim<S>::ABLK;
+  const size_t per = oz_bytes_t<T>(m, n, k);
   int nb = (int)(work_bytes / per < (size_t)batch ? work_bytes / per : (size_t)batch);
   if (nb < 1) return cudaErrorInvalidValue;
   if (nb > 32767) nb = 32767;   // gridDim.z carries (matrix, operand)
-  const int mp = (int)up(m, OZ_BM), np = (int)up(n, OZ_BN), ks = (k + OZ_KS - 1) / OZ_KS;
-  cudaError_t e = cudaFuncSetAttribute(oz_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM);
+  const int mp = (int)up(m, OZ_BM), np = (int)up(n, BN), ks = (k + OZ_KS - 1) / OZ_KS;
+  cudaError_t e = cudaFuncSetAttribute(oz_gemm_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, oz_smem<T>());
   if (e != cudaSuccess) return e;
   for (int b0 = 0; b0 < batch; b0 += nb) {
     const int bn = batch - b0 < nb ? batch - b0 : nb;
     unsigned char* dA = (unsigned char*)work;
-    unsigned char* dB = dA + (size_t)bn * (mp / OZ_BM) * ks * 2 * OZ_ABLK;
-    unsigned int* xA = (unsigned int*)(dB + (size_t)bn * (np / OZ_BN) * ks * OZ_BBLK);
+    unsigned char* dB = dA + (size_t)bn * (mp / OZ_BM) * ks * 2 * ABLK;
+    unsigned int* xA = (unsigned int*)(dB + (size_t)bn * (np / BN) * ks * OZ_BBLK);
     unsigned int* xB = xA + (size_t)bn * mp;
-    OzSplit q;
+    OzSplit<T> q;
     q.k = k;
     q.ksteps = ks;
     q.batch = bn;
-    q.o[0].p = A + b0 * sA;
-    q.o[0].sb = sA;
-    q.o[0].rs = opA ? lda : 1;
-    q.o[0].ks = opA ? 1 : lda;
-    q.o[0].rows = m;
-    q.o[0].conj = opA;
-    q.o[0].is_b = 0;
-    q.o[0].ex = xA;
-    q.o[0].dig = dA;
-    q.o[0].rows_pad = mp;
-    q.o[1].p = B + b0 * sB;
-    q.o[1].sb = sB;
-    q.o[1].rs = ldb;
-    q.o[1].ks = 1;
-    q.o[1].rows = n;
-    q.o[1].conj = 0;
-    q.o[1].is_b = 1;
-    q.o[1].ex = xB;
-    q.o[1].dig = dB;
-    q.o[1].rows_pad = np;
+    q.o[0] = OzOperand<T>{A + b0 * sA, sA, opA ? lda : 1, opA ? 1 : lda, m, opA, 0, xA, dA, mp};
+    q.o[1] = OzOperand<T>{B + b0 * sB, sB, ldb, 1, n, 0, 1, xB, dB, np};
     e = cudaMemsetAsync(xA, 0, (size_t)bn * (mp + np) * sizeof(unsigned int), st);
     if (e != cudaSuccess) return e;
     const int rows = m > n ? m : n, rpad = mp > np ? mp : np;
-    oz_rowmax<<<dim3((rows + 31) / 32, (k + 63) / 64, 2 * bn), 256, 0, st>>>(q);
-    oz_digits<<<dim3((rpad + 31) / 32, (2 * ks + 7) / 8, 2 * bn), 256, 0, st>>>(q);
-    OzGemm g;
-    g.A = dA;
-    g.B = dB;
-    g.exA = xA;
-    g.exB = xB;
-    g.m = m;
-    g.n = n;
-    g.m_pad = mp;
-    g.n_pad = np;
-    g.ksteps = ks;
-    g.sign = sign;
-    g.add = add;
-    g.C = C + b0 * sC;
-    g.ldc = ldc;
-    g.sC = sC;
-    g.err = err;
-    oz_gemm_kernel<<<dim3(mp / OZ_BM, np / OZ_BN, bn), OZ_THREADS, OZ_SMEM, st>>>(g);
+    oz_rowmax<T><<<dim3((rows + 31) / 32, (k + 63) / 64, 2 * bn), 256, 0, st>>>(q);
+    oz_digits<T><<<dim3((rpad + 31) / 32, (2 * ks + 7) / 8, 2 * bn), 256, 0, st>>>(q);
+    OzGemm<T> g{dA, dB, xA, xB, m, n, mp, np, ks, sign, add, C + b0 * sC, ldc, sC, err};
+    oz_gemm_kernel<T><<<dim3(mp / OZ_BM, np / BN, bn), OZ_THREADS, oz_smem<T>(), st>>>(g);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
+}
+
+}  // namespace
+
+size_t oz_bytes(int m, int n, int k, bool fp64) {
+  return fp64 ? oz_bytes_t<double2>(m, n, k) : oz_bytes_t<float2>(m, n, k);
+}
+
+cudaError_t oz_gemm(cudaStream_t st, int batch, int m, int n, int k, int sign, const double2* A, int lda, long long sA,
+                    int opA, const double2* B, int ldb, long long sB, int add, double2* C, int ldc, long long sC,
+                    void* work, size_t work_bytes, int* err) {
+  return oz_gemm_t<double2>(st, batch, m, n, k, sign, A, lda, sA, opA, B, ldb, sB, add, C, ldc, sC, work, work_bytes, err);
+}
+cudaError_t oz_gemm(cudaStream_t st, int batch, int m, int n, int k, int sign, const float2* A, int lda, long long sA,
+                    int opA, const float2* B, int ldb, long long sB, int add, float2* C, int ldc, long long sC, void* work,
+                    size_t work_bytes, int* err) {
+  return oz_gemm_t<float2>(st, batch, m, n, k, sign, A, lda, sA, opA, B, ldb, sB, add, C, ldc, sC, work, work_bytes, err);
 }
 
 }  // namespace rsfd

@@ -250,19 +250,17 @@ int handle_dyson_cols(Handle* h);     // 0: every column of G_bb; 1: the left sl
 cudaError_t cgemm_tf32x3(cudaStream_t st, int batch, int m, int n, int k, float2 alpha, const float2* A, int lda,
                          long long sA, const float2* B, int ldb, long long sB, float beta, float2* C, int ldc,
                          long long sC, int* err);
-cudaError_t getrf_f32_tc(cudaStream_t st, float2* M, int nb, int K, int* piv, int* info, int* err);
-cudaError_t getrs_f32_tc(cudaStream_t st, const float2* LU, const int* piv, int nb, int K, const double2* B, int nrhs,
-                         float2* X, int* perm, int* err);
-cudaError_t getrs_f32_tc(cudaStream_t st, const float2* LU, const int* piv, int nb, int K, const float2* B, int nrhs,
-                         float2* X, int* perm, int* err);
-int tc_panel();
 
-// FP64-accurate complex GEMM on the tensor cores (oz_gemm.cu): C = sign op(A) B + (add ? C : 0), op = N or
-// conjugate transpose, batched; work holds at least oz_bytes(m, n, k); err is set when a bounded wait expires.
-size_t oz_bytes(int m, int n, int k);
-cudaError_t oz_zgemm(cudaStream_t st, int batch, int m, int n, int k, double sign, const double2* A, int lda,
-                     long long sA, int opA, const double2* B, int ldb, long long sB, int add, double2* C, int ldc,
-                     long long sC, void* work, size_t work_bytes, int* err);
+// Complex GEMM on the tensor cores by digit slices (oz_gemm.cu): C = sign op(A) B + (add ? C : 0), op = N or
+// conjugate transpose, batched, FP64-accurate (double2) or FP32-accurate (float2); work holds at least
+// oz_bytes(m, n, k, fp64); err is set when a bounded wait expires.
+size_t oz_bytes(int m, int n, int k, bool fp64);
+cudaError_t oz_gemm(cudaStream_t st, int batch, int m, int n, int k, int sign, const double2* A, int lda, long long sA,
+                    int opA, const double2* B, int ldb, long long sB, int add, double2* C, int ldc, long long sC,
+                    void* work, size_t work_bytes, int* err);
+cudaError_t oz_gemm(cudaStream_t st, int batch, int m, int n, int k, int sign, const float2* A, int lda, long long sA,
+                    int opA, const float2* B, int ldb, long long sB, int add, float2* C, int ldc, long long sC, void* work,
+                    size_t work_bytes, int* err);
 
 // Dyson / transmission launchers (dyson.cu).
 rsfd_status dyson_run(Handle* h, const void* G0, const void* SL, const void* SR, int K, void* G, double* refres);

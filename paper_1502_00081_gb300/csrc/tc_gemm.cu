@@ -1,6 +1,5 @@
-// Tensor-core pieces of the Dyson step (Eq. sec3-01a on the boundary rows): a batched complex
-// FP32 GEMM on the 5th-generation tensor cores (tcgen05, kind::tf32) with the 3xTF32 split, and the
-// FP32 blocked LU / triangular solves whose O(nb^3) updates it carries.
+// A batched complex FP32 GEMM on the 5th-generation tensor cores (tcgen05, kind::tf32) with the 3xTF32 split:
+// the entry rsfd_cgemm_tf32x3, and the FP32 products of the Dyson step when there is no memory for digit planes.
 //
 // 3xTF32: every FP32 operand x is split into hi = x with the 13 low mantissa bits cleared (exactly a
 // TF32 number) and lo = x - hi (exact in FP32).  A product a*b is taken as
@@ -41,7 +40,6 @@ constexpr uint32_t TC_SBO = 128;
 constexpr uint32_t TC_LBO_A = (TC_BM / 8) * 128;
 constexpr uint32_t TC_LBO_B = (TC_BN / 8) * 128;
 constexpr long long kTcWaitCap = 1ll << 22;
-constexpr int kTcPanel = 64;     // LU panel width = K of the trailing-update GEMMs
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -287,189 +285,6 @@ cgemm_tf32x3_kernel(int m, int n, int k, float2 alpha, const float2* __restrict_
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TC_TMEM_COLS) : "memory");
 }
 
-// ------------------------------------------------------------------------------------------------
-// FP32 blocked LU with partial pivoting and the blocked triangular solves
-// ------------------------------------------------------------------------------------------------
-__device__ __forceinline__ float2 fmulc(float2 a, float2 b) {
-  return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
-}
-__device__ __forceinline__ float2 fsubc(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
-__device__ __forceinline__ float2 frecip(float2 d) {
-  // 1 / d by Smith's algorithm
-  if (fabsf(d.x) >= fabsf(d.y)) {
-    const float r = d.y / d.x, den = d.x + d.y * r;
-    return make_float2(1.f / den, -r / den);
-  }
-  const float r = d.x / d.y, den = d.y + d.x * r;
-  return make_float2(r / den, -1.f / den);
-}
-
-// Factorise columns j0 .. j0+jb-1 of every matrix (one CTA per matrix), LAPACK getrf order:
-// piv[j] is the row exchanged with row j at step j; info[b] = first zero pivot (1-based).
-__global__ void __launch_bounds__(256) panel_getrf_f32(float2* M, int nb, int j0, int jb, int* piv, int* info) {
-  const int b = blockIdx.x;
-  float2* A = M + (long long)b * nb * nb;
-  int* pv = piv + (long long)b * nb;
-  __shared__ float s_val[256];
-  __shared__ int s_idx[256];
-  __shared__ int s_p;
-  const int tid = threadIdx.x, nt = blockDim.x;
-  for (int j = j0; j < j0 + jb; ++j) {
-    float best = -1.f;
-    int bi = j;
-    for (int i = j + tid; i < nb; i += nt) {
-      const float2 a = A[(long long)j * nb + i];
-      const float v = fabsf(a.x) + fabsf(a.y);
-      if (v > best) { best = v; bi = i; }
-    }
-    s_val[tid] = best;
-    s_idx[tid] = bi;
-    __syncthreads();
-    for (int s2 = nt / 2; s2 > 0; s2 >>= 1) {
-      if (tid < s2) {
-        if (s_val[tid + s2] > s_val[tid] || (s_val[tid + s2] == s_val[tid] && s_idx[tid + s2] < s_idx[tid])) {
-          s_val[tid] = s_val[tid + s2];
-          s_idx[tid] = s_idx[tid + s2];
-        }
-      }
-      __syncthreads();
-    }
-    if (tid == 0) {
-      s_p = s_idx[0];
-      pv[j] = s_p;
-      if (!(s_val[0] > 0.f) && info[b] == 0) info[b] = j + 1;
-    }
-    __syncthreads();
-    const int p = s_p;
-    if (p != j) {
-      for (int c = j0 + tid; c < j0 + jb; c += nt) {
-        const float2 t = A[(long long)c * nb + j];
-        A[(long long)c * nb + j] = A[(long long)c * nb + p];
-        A[(long long)c * nb + p] = t;
-      }
-    }
-    __syncthreads();
-    const float2 d = A[(long long)j * nb + j];
-    const float2 inv = (d.x != 0.f || d.y != 0.f) ? frecip(d) : make_float2(0.f, 0.f);
-    for (int i = j + 1 + tid; i < nb; i += nt) A[(long long)j * nb + i] = fmulc(A[(long long)j * nb + i], inv);
-    __syncthreads();
-    const int rem_r = nb - j - 1, rem_c = j0 + jb - j - 1;
-    if (rem_c > 0) {
-      for (int i = j + 1 + tid; i < nb; i += nt) {
-        const float2 l = A[(long long)j * nb + i];
-        for (int c = j + 1; c < j0 + jb; ++c) {
-          float2& a = A[(long long)c * nb + i];
-          a = fsubc(a, fmulc(l, A[(long long)c * nb + j]));
-        }
-      }
-    }
-    (void)rem_r;
-    __syncthreads();
-  }
-}
-
-// apply the exchanges of rows j0 .. j0+jb-1 (in order) to every column outside the panel
-__global__ void laswp_f32(float2* M, int nb, int j0, int jb, const int* piv, int batch) {
-  const int ncol = nb - jb;
-  const long long tot = (long long)ncol * batch;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < tot; t += (long long)gridDim.x * blockDim.x) {
-    const int b = (int)(t / ncol);
-    int c = (int)(t - (long long)b * ncol);
-    if (c >= j0) c += jb;
-    float2* col = M + (long long)b * nb * nb + (long long)c * nb;
-    const int* pv = piv + (long long)b * nb;
-    for (int j = j0; j < j0 + jb; ++j) {
-      const int p = pv[j];
-      if (p != j) {
-        const float2 x = col[j];
-        col[j] = col[p];
-        col[p] = x;
-      }
-    }
-  }
-}
-
-// X[0:ib, c] = T^{-1} X[0:ib, c] for the ib x ib diagonal block T at (r0, r0) of each matrix;
-// lower = 1: unit lower triangle, lower = 0: upper triangle with its diagonal.  T is staged in
-// shared memory; one thread per right-hand-side column.  X has leading dimension ldx and batch
-// stride sX; the factor has leading dimension nb and batch stride nb*nb.
-template <int IB>
-__global__ void __launch_bounds__(128) trsm_diag_f32(const float2* LU, int nb, int r0, int ib, float2* X, int ldx,
-                                                    long long sX, int nrhs, int lower) {
-  __shared__ float2 T[IB][IB + 1];
-  const int b = blockIdx.y;
-  const float2* F = LU + (long long)b * nb * nb;
-  for (int t = threadIdx.x; t < ib * ib; t += blockDim.x) {
-    const int c = t / ib, r = t - c * ib;
-    T[r][c] = F[(long long)(r0 + c) * nb + r0 + r];
-  }
-  __syncthreads();
-  const int col = blockIdx.x * blockDim.x + threadIdx.x;
-  if (col >= nrhs) return;
-  float2* x = X + b * sX + (long long)col * ldx + r0;
-  float2 v[IB];
-#pragma unroll
-  for (int i = 0; i < IB; ++i) v[i] = i < ib ? x[i] : make_float2(0.f, 0.f);
-  if (lower) {
-#pragma unroll
-    for (int i = 1; i < IB; ++i) {
-      float2 s = v[i];
-#pragma unroll
-      for (int q = 0; q < i; ++q) s = fsubc(s, fmulc(T[i][q], v[q]));
-      v[i] = s;
-    }
-  } else {
-#pragma unroll
-    for (int i = IB - 1; i >= 0; --i) {
-      if (i < ib) {
-        float2 s = v[i];
-#pragma unroll
-        for (int q = i + 1; q < IB; ++q)
-          if (q < ib) s = fsubc(s, fmulc(T[i][q], v[q]));
-        v[i] = fmulc(s, frecip(T[i][i]));
-      }
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < IB; ++i)
-    if (i < ib) x[i] = v[i];
-}
-
-// the row permutation of P^T: perm[i] = source row of row i after the exchanges piv[0 .. nb-1]
-__global__ void perm_from_piv(const int* piv, int nb, int batch, int* perm) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= batch) return;
-  const int* pv = piv + (long long)b * nb;
-  int* pm = perm + (long long)b * nb;
-  for (int i = 0; i < nb; ++i) pm[i] = i;
-  for (int j = 0; j < nb; ++j) {
-    const int p = pv[j];
-    if (p != j) {
-      const int t = pm[j];
-      pm[j] = pm[p];
-      pm[p] = t;
-    }
-  }
-}
-
-// dst[b][:, c][i] = src[b][:, c][perm[b][i]]  for nrhs columns of nb rows (FP64 -> FP32 or FP32 -> FP32)
-template <typename S>
-__global__ void gather_rows_f32(const S* src, int nb, int nrhs, const int* perm, float2* dst, int batch) {
-  const long long per = (long long)nb * nrhs;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < per * batch;
-       t += (long long)gridDim.x * blockDim.x) {
-    const long long b = t / per, e = t - b * per;
-    const long long c = e / nb, i = e - c * nb;
-    const S v = src[b * per + c * nb + perm[b * nb + i]];
-    dst[t] = make_float2((float)v.x, (float)v.y);
-  }
-}
-
-int grid_1d(long long n) {
-  long long g = (n + 255) / 256;
-  return (int)(g < 8192 ? (g < 1 ? 1 : g) : 8192);
-}
-
 bool g_tc_attr_set[16] = {false};
 
 }  // namespace
@@ -493,73 +308,6 @@ cudaError_t cgemm_tf32x3(cudaStream_t st, int batch, int m, int n, int k, float2
   cgemm_tf32x3_kernel<<<grid, TC_THREADS, TC_SMEM, st>>>(m, n, k, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC,
                                                          err, vecB);
   return cudaGetLastError();
-}
-
-int tc_panel() { return kTcPanel; }
-
-// Batched blocked LU of K matrices nb x nb (FP32 complex, column-major, contiguous), in place.
-cudaError_t getrf_f32_tc(cudaStream_t st, float2* M, int nb, int K, int* piv, int* info, int* err) {
-  const long long n2 = (long long)nb * nb;
-  const float2 m1 = make_float2(-1.f, 0.f);
-  for (int j0 = 0; j0 < nb; j0 += kTcPanel) {
-    const int jb = nb - j0 < kTcPanel ? nb - j0 : kTcPanel;
-    panel_getrf_f32<<<K, 256, 0, st>>>(M, nb, j0, jb, piv, info);
-    if (nb > jb) laswp_f32<<<grid_1d((long long)(nb - jb) * K), 256, 0, st>>>(M, nb, j0, jb, piv, K);
-    const int rest = nb - j0 - jb;
-    if (rest > 0) {
-      // U12 = L11^{-1} A12: the panel's unit lower diagonal block applied to the columns right of it
-      dim3 g((rest + 127) / 128, K);
-      trsm_diag_f32<kTcPanel><<<g, 128, 0, st>>>(M, nb, j0, jb, M + (long long)(j0 + jb) * nb, nb, n2, rest, 1);
-      // A22 -= L21 U12
-      cudaError_t e = cgemm_tf32x3(st, K, rest, rest, jb, m1, M + (long long)j0 * nb + j0 + jb, nb, n2,
-                                   M + (long long)(j0 + jb) * nb + j0, nb, n2, 1.f,
-                                   M + (long long)(j0 + jb) * nb + j0 + jb, nb, n2, err);
-      if (e != cudaSuccess) return e;
-    }
-  }
-  return cudaGetLastError();
-}
-
-// X = U^{-1} L^{-1} P B for nrhs columns per matrix.  B (FP64 or FP32 complex, [K][nrhs][nb]) is
-// permuted into X (FP32) first; perm is [K][nb] scratch.
-template <typename S>
-cudaError_t getrs_f32_tc_impl(cudaStream_t st, const float2* LU, const int* piv, int nb, int K, const S* B, int nrhs,
-                              float2* X, int* perm, int* err) {
-  const long long n2 = (long long)nb * nb, sx = (long long)nb * nrhs;
-  const float2 m1 = make_float2(-1.f, 0.f);
-  perm_from_piv<<<(K + 127) / 128, 128, 0, st>>>(piv, nb, K, perm);
-  gather_rows_f32<S><<<grid_1d(sx * K), 256, 0, st>>>(B, nb, nrhs, perm, X, K);
-  const int nblk = (nb + kTcPanel - 1) / kTcPanel;
-  dim3 g((nrhs + 127) / 128, K);
-  for (int bi = 0; bi < nblk; ++bi) {   // forward: unit lower L
-    const int r0 = bi * kTcPanel, ib = nb - r0 < kTcPanel ? nb - r0 : kTcPanel;
-    trsm_diag_f32<kTcPanel><<<g, 128, 0, st>>>(LU, nb, r0, ib, X, nb, sx, nrhs, 1);
-    const int rest = nb - r0 - ib;
-    if (rest > 0) {
-      cudaError_t e = cgemm_tf32x3(st, K, rest, nrhs, ib, m1, LU + (long long)r0 * nb + r0 + ib, nb, n2, X + r0, nb,
-                                   sx, 1.f, X + r0 + ib, nb, sx, err);
-      if (e != cudaSuccess) return e;
-    }
-  }
-  for (int bi = nblk - 1; bi >= 0; --bi) {   // backward: upper U
-    const int r0 = bi * kTcPanel, ib = nb - r0 < kTcPanel ? nb - r0 : kTcPanel;
-    trsm_diag_f32<kTcPanel><<<g, 128, 0, st>>>(LU, nb, r0, ib, X, nb, sx, nrhs, 0);
-    if (r0 > 0) {
-      cudaError_t e = cgemm_tf32x3(st, K, r0, nrhs, ib, m1, LU + (long long)r0 * nb, nb, n2, X + r0, nb, sx, 1.f, X,
-                                   nb, sx, err);
-      if (e != cudaSuccess) return e;
-    }
-  }
-  return cudaGetLastError();
-}
-
-cudaError_t getrs_f32_tc(cudaStream_t st, const float2* LU, const int* piv, int nb, int K, const double2* B, int nrhs,
-                         float2* X, int* perm, int* err) {
-  return getrs_f32_tc_impl<double2>(st, LU, piv, nb, K, B, nrhs, X, perm, err);
-}
-cudaError_t getrs_f32_tc(cudaStream_t st, const float2* LU, const int* piv, int nb, int K, const float2* B, int nrhs,
-                         float2* X, int* perm, int* err) {
-  return getrs_f32_tc_impl<float2>(st, LU, piv, nb, K, B, nrhs, X, perm, err);
 }
 
 }  // namespace rsfd
