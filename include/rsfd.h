@@ -109,15 +109,18 @@ typedef struct {
 
 /* Form of the seed iteration's pass (rsfd_solve_opts.pass_kind). */
 typedef enum {
-  RSFD_PASS_AUTO = 0,      /* RSFD_PASS_STORED when the options are not tuned; rsfd_autotune times every form
-                              (on the 64^2 x 128 workload it picks RSFD_PASS_SPLIT_BFP for double-float) */
+  RSFD_PASS_AUTO = 0,      /* RSFD_PASS_SPLIT on tiles cut to the grid when the options are not tuned (double-float: with
+                              the sums in RSFD_PASS_STORED's blocks, so the two agree bit for bit), RSFD_PASS_STORED
+                              when tile_y, tile_x = 16, rows_per_thread > 1, reg_budget or prefetch is given;
+                              rsfd_autotune times every form (on the 64^2 x 128 workload it picks
+                              RSFD_PASS_SPLIT_BFP for double-float) */
   RSFD_PASS_RECOMPUTE = 1, /* three vectors per iteration (r_{n-1}, r_{n-2} in, r_n out); A r_{n-1} is
                               recomputed on the tile plus halo and A r_n again for the dot products */
   RSFD_PASS_STORED = 2,    /* five vectors per iteration (r_{n-1}, r_{n-2}, A r_{n-1} in; r_n, A r_n out);
                               one stencil application per grid point */
   RSFD_PASS_SPLIT = 3,     /* the stored-product iteration as two launches: a pointwise combine (r_n from
                               r_{n-1}, r_{n-2}, A r_{n-1}; four vectors) and a stencil (A r_n from r_n; two
-                              vectors plus its halo); one row per thread, tile width 32, tile_y <= 16 */
+                              vectors plus its halo); two rows per thread, tile width by the grid's, tile_y <= 16 */
   RSFD_PASS_SPLIT_BFP = 4  /* double-float handles: RSFD_PASS_SPLIT with the leading
                               parts of r_n rounded to a per-column, per-iteration quantum q (block floating
                               point, q chosen from a bound on |r_n| so that every leading part is at most
@@ -159,10 +162,7 @@ typedef struct {
   int32_t reg_budget;     /* RSFD_PASS_STORED, double-float, one row per thread: registers per thread of
                              the pass, 0 = at most 96 (CTAs of <= 640 threads; two CTAs of <= 320 threads
                              per SM), 1 = at most 128 (CTAs of <= 512 threads, tile_y <= 14, one CTA per
-                             SM, no register spills); RSFD_PASS_SPLIT_BFP: the stencil launch keeps 0 = at
-                             most 128 / 85 registers (one 512-thread or three 256-thread CTAs per SM) or
-                             1 = at most 64 (two 512-thread or four 256-thread CTAs per SM); other passes
-                             ignore it */
+                             SM, no register spills); other passes ignore it */
   int32_t tile_x;         /* RSFD_PASS_STORED, double-float, one row per thread: tile width in x, 0 or 32
                              (one tile row per warp) or 16 (two tile rows per warp; less idle work when Nx
                              is an odd multiple of 16, e.g. 48 or 80); tile_y must be even */

@@ -567,13 +567,6 @@ struct AccK {
     kahan(ra, ra_c, tra);
     nn = __fmaf_rn(r.x, r.x, __fmaf_rn(r.y, r.y, nn));
   }
-  __device__ __forceinline__ void add_r(float2 r) {
-    kahan(rr, rr_c, make_float2(__fmaf_rn(r.x, r.x, -r.y * r.y), 2.f * r.x * r.y));
-    nn = __fmaf_rn(r.x, r.x, __fmaf_rn(r.y, r.y, nn));
-  }
-  __device__ __forceinline__ void add_ra(float2 r, float2 v) {
-    kahan(ra, ra_c, make_float2(__fmaf_rn(r.x, v.x, -r.y * v.y), __fmaf_rn(r.x, v.y, r.y * v.x)));
-  }
   // The Kahan pairs (s, -c) are double-float values: reduce them over the warp with TwoSum merges
   // (whole warps only) and convert once; lane 0 returns the warp's sums, the other lanes zeros.
   __device__ __forceinline__ void get(double* o) {
@@ -594,9 +587,36 @@ struct AccK {
   }
 };
 
+// complex64 vectors in the split pass: the products are formed exactly (FMA) and summed in double-float, as for
+// double-float vectors without their low parts.  The split kernels are not bound by this arithmetic, and rounded
+// products can keep a solve at small eta from ever reaching its tolerance.
+struct AccX {
+  AccDF a;
+  static __device__ __forceinline__ void addprod(float2& s, float2& l, float2 x, float2 y) {
+    const float2 p = f2mul(x, y);
+    const float2 ne = f2fma(f2neg(x), y, p);   // p - x y, exact
+    float2 t, te;
+    two_sum2(s, p, t, te);
+    s = t;
+    l = f2add(l, f2sub(te, ne));
+  }
+  __device__ __forceinline__ void add_r(float2 r) {
+    addprod(a.rr_s, a.rr_l, bc(r.x), r);
+    addprod(a.rr_s, a.rr_l, make_float2(-r.y, r.y), make_float2(r.y, r.x));
+    a.nn = __fmaf_rn(r.x, r.x, __fmaf_rn(r.y, r.y, a.nn));
+  }
+  __device__ __forceinline__ void add_ra(float2 r, float2 v) {
+    addprod(a.ra_s, a.ra_l, bc(r.x), v);
+    addprod(a.ra_s, a.ra_l, make_float2(-r.y, r.y), make_float2(v.y, v.x));
+  }
+  __device__ __forceinline__ void get(double* o) { a.get(o); }
+};
+
 template <int MODE> struct AccOf { typedef AccDF type; };
 template <> struct AccOf<RSFD_MIXED> { typedef AccK type; };
 template <> struct AccOf<RSFD_FP64> { typedef Acc<double> type; };
+template <int MODE> struct AccSplit { typedef typename AccOf<MODE>::type type; };   // the split pass's
+template <> struct AccSplit<RSFD_MIXED> { typedef AccX type; };
 
 // index of plane z among the recorded planes (boundary planes, then the tracked interior planes),
 // -1 when its rows are not recorded
@@ -677,12 +697,14 @@ __device__ __forceinline__ void block_sum_lane0(double (&v)[NV], double* s_red) 
     for (int k = 0; k < NV; ++k) s_red[wid * NV + k] = v[k];
   }
   __syncthreads();
-  if (tid == 0) {
+  if (wid == 0) {   // lane k adds value k over the warps
+    double t = 0.0;
+    if (lane < NV)
+      for (int w = 0; w < nw; ++w) t += s_red[w * NV + lane];
 #pragma unroll
     for (int k = 0; k < NV; ++k) {
-      double t = 0.0;
-      for (int w = 0; w < nw; ++w) t += s_red[w * NV + k];
-      v[k] = t;
+      const double r = __shfl_sync(0xffffffffu, t, k);
+      if (lane == 0) v[k] = r;
     }
   }
   __syncthreads();
@@ -955,19 +977,20 @@ __device__ void scalar_step(const PassParams& p, int slot, ScalarShared& S) {
 // atomic ticket; the last of the slot's ctas_per_slot CTAs sums all npart partials of the slot in
 // order (warp 0, fixed tree; the split pass's combine kernel has left its partials in entries
 // ctas_per_slot ...) and returns true with (r,r), (r,Ar), ||r||^2 in S.  No CTA waits on another.
-__device__ bool pass_finish(const PassParams& p, int slot, int cta, double (&v5)[5], ScalarShared& S, int& s_last,
-                            float mxu = 0.f) {
-  const int tid = threadIdx.x;
+__device__ bool pass_tail(const PassParams& p, int slot, ScalarShared& S, int& s_last);
+__device__ bool pass_finish(const PassParams& p, int slot, int cta, double (&v5)[5], ScalarShared& S, int& s_last) {
   block_sum_lane0<5>(v5, S.red);
-  if (p.bfp) mxu = block_max0(mxu, reinterpret_cast<float*>(S.red));
-  if (tid == 0) {
+  if (threadIdx.x == 0) {
     double* dst = p.partials + ((size_t)slot * p.d.npart + cta) * 8;
 #pragma unroll
     for (int k = 0; k < 5; ++k) dst[k] = v5[k];
-    if (p.bfp) {
-      dst[5] = 0.0;
-      dst[6] = (double)mxu;
-    }
+  }
+  return pass_tail(p, slot, S, s_last);
+}
+// The ticket and the slot's sums, after thread 0 has written the CTA's partials.
+__device__ bool pass_tail(const PassParams& p, int slot, ScalarShared& S, int& s_last) {
+  const int tid = threadIdx.x;
+  if (tid == 0) {
     __threadfence();
     const unsigned int t = atomicAdd(p.tickets + slot, 1u);
     s_last = (t == (unsigned int)(p.d.ctas_per_slot - 1));
@@ -1624,9 +1647,6 @@ __global__ void __launch_bounds__(NT) passu_kernel(PassParams p, const __grid_co
 // pass's five, in exchange for every grid point's stencil and combine being computed once (no frame
 // recomputation).
 
-// Combine: CTA = 256 threads over a range of z-planes of one slot; each thread walks the plane's
-// padded elements with stride 256 (x, y tracked by a running counter) and handles two elements per
-// step so that six 16-byte loads are in flight.
 constexpr int kCombThreads = 256;
 
 // Block-floating-point rounding of the leading parts (BFP): with Cq = 1.5 2^23 q, fl(h + Cq) - Cq is h
@@ -1646,16 +1666,110 @@ template <> struct Requant<true, dfc> {
   static __device__ __forceinline__ float amax(const dfc& x) { return fmaxf(fabsf(x.h.x), fabsf(x.h.y)); }
 };
 
-// one combine CTA: block cblk (of d.ctas_c, a range of z-planes) of slot `slot`; any block size
-template <int MODE, bool BFP>
-__device__ __forceinline__ void combine_body(const PassParams& p, const int slot, const int cblk) {
+// Combine over a contiguous range (block blockIdx.x of d.ctas_c) of one slot's padded elements (planes are not a unit,
+// so small planes fill the threads too), in 16-byte units (one element, or two of complex64); each thread handles
+// two units per step, so that six 16-byte loads are in flight.  Coordinates are only formed where they are
+// needed: x in padded rows, all of them in the planes whose rows are recorded.
+template <int MODE> __global__ void __launch_bounds__(kCombThreads, 4) combine_kernel(PassParams p) {
+  const int slot = blockIdx.y, cblk = blockIdx.x;
   typedef Ops<MODE> O;
   typedef Stencil<MODE, 1> ST;   // combine() does not depend on the stencil reach
   typedef typename O::C C;
   typedef typename O::H H;
-  typedef Requant<BFP, C> RQ;
   __shared__ double s_red[32 * 5];
   __shared__ typename O::Cplx s_a[3];
+  __shared__ int s_n, s_hc;
+  const SlotState* st = p.slots + slot;
+  if (st->status != SLOT_RUNNING) return;
+  const SolveDims& d = p.d;
+  if (threadIdx.x < 3) s_a[threadIdx.x] = O::cplx(threadIdx.x == 0 ? st->a1 : (threadIdx.x == 1 ? st->a2 : st->aA));
+  if (threadIdx.x == 0) {
+    s_n = st->n;
+    s_hc = st->hcnt;
+  }
+  __syncthreads();
+  const typename O::Cplx a1 = s_a[0], a2 = s_a[1], aA = s_a[2];
+  const int n = s_n;
+  const int i1 = (n + 2) % 3, i2 = (n + 1) % 3, io = n % 3, iu1 = 3 + (n + 1) % 2;
+  const int pe = d.nxp * d.ny;   // padded elements per plane
+  const long long vec = (long long)d.nz * pe;
+  const C* R1 = reinterpret_cast<const C*>(p.rbuf) + ((size_t)slot * 5 + i1) * vec;
+  const C* R2 = reinterpret_cast<const C*>(p.rbuf) + ((size_t)slot * 5 + i2) * vec;
+  const C* U1 = reinterpret_cast<const C*>(p.rbuf) + ((size_t)slot * 5 + iu1) * vec;
+  C* RO = reinterpret_cast<C*>(p.rbuf) + ((size_t)slot * 5 + io) * vec;
+  H* hist = reinterpret_cast<H*>(p.rhist) + ((size_t)slot * p.hist_len + s_hc) * d.nb;
+  constexpr int U = 16 / sizeof(C);   // elements per unit (vec is a multiple of 4)
+  const long long nu = vec / U;         // below 2^32: five such vectors fit the device's memory
+  const unsigned lo = (unsigned)(nu * cblk / d.ctas_c), hi = (unsigned)(nu * (cblk + 1) / d.ctas_c);
+  // elements from which planes are not recorded, and from which they are again
+  const long long in0 = (long long)d.nface * pe, in1 = (long long)(d.nz - d.nface) * pe;
+  const bool padded = d.nxp != d.nx, small = vec < (1ll << 32);
+  typename AccSplit<MODE>::type acc;
+  struct alignas(16) Unit {
+    C c[U];
+  };
+  auto finish = [&](long long e, const C& r) {
+    const bool rec = e < in0 || e >= in1 || d.ntrack > 0;
+    if (padded || rec) {
+      const unsigned row = small ? (unsigned)e / (unsigned)d.nxp : (unsigned)(e / d.nxp);
+      const int x = (int)(e - (long long)row * d.nxp);
+      if (x >= d.nx) return;   // row padding
+      if (rec) {
+        const int z = (int)(row / (unsigned)d.ny), y = (int)(row - (unsigned)z * (unsigned)d.ny);
+        const int pl = recorded_plane(d, z);
+        if (pl >= 0) hist[((size_t)pl * d.ny + y) * d.nx + x] = O::hi(r);
+      }
+    }
+    acc.add_r(r);
+  };
+  auto unit = [&](unsigned u, const Unit& r1, const Unit& r2, const Unit& u1) {
+    if constexpr (U == 1) {
+      const C r = ST::combine(a1, r1.c[0], a2, r2.c[0], aA, u1.c[0]);   // Eq. rvec
+      RO[u] = r;
+      finish(u, r);
+    } else {
+      Unit r;
+#pragma unroll
+      for (int k = 0; k < U; ++k) r.c[k] = ST::combine(a1, r1.c[k], a2, r2.c[k], aA, u1.c[k]);
+      reinterpret_cast<Unit*>(RO)[u] = r;
+#pragma unroll
+      for (int k = 0; k < U; ++k) finish((long long)u * U + k, r.c[k]);
+    }
+  };
+  const Unit *P1 = reinterpret_cast<const Unit*>(R1), *P2 = reinterpret_cast<const Unit*>(R2),
+             *PU = reinterpret_cast<const Unit*>(U1);
+  for (unsigned u = lo + threadIdx.x; u < hi; u += 2 * kCombThreads) {
+    const unsigned u2 = u + kCombThreads;   // may lie past the range
+    const bool has2 = u2 < hi;
+    const Unit r1a = P1[u], r2a = P2[u], ua = PU[u];
+    Unit r1b = r1a, r2b = r2a, ub = ua;
+    if (has2) { r1b = P1[u2]; r2b = P2[u2]; ub = PU[u2]; }
+    unit(u, r1a, r2a, ua);
+    if (has2) unit(u2, r1b, r2b, ub);
+  }
+  double v5[5];
+  acc.get(v5);
+  block_sum_lane0<5>(v5, s_red);
+  if (threadIdx.x == 0) {
+    double* dst = p.partials + ((size_t)slot * d.npart + d.nlog + cblk) * 8;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) dst[k] = v5[k];
+  }
+}
+
+// Combine with its sums, double-float: CTA = 256 threads over a range of z-planes (block blockIdx.x of d.ctas_c); each
+// thread walks the plane's padded elements with stride 256 (x, y tracked by a running counter), two elements per
+// step so that six 16-byte loads are in flight.  The ranges and this order fix the rounding of (r_n, r_n).
+// At most 64 registers: four CTAs (32 warps) per SM keep enough loads in flight for HBM.
+template <bool BFP> __global__ void __launch_bounds__(kCombThreads, 4) combine_planes_kernel(PassParams p) {
+  typedef Ops<RSFD_DF64> O;
+  typedef Stencil<RSFD_DF64, 1> ST;   // combine() does not depend on the stencil reach
+  const int slot = blockIdx.y, cblk = blockIdx.x;
+  typedef O::C C;
+  typedef O::H H;
+  typedef Requant<BFP, C> RQ;
+  __shared__ double s_red[32 * 5];
+  __shared__ O::Cplx s_a[3];
   __shared__ int s_n, s_hc;
   __shared__ float s_cq;
   const SlotState* st = p.slots + slot;
@@ -1670,7 +1784,7 @@ __device__ __forceinline__ void combine_body(const PassParams& p, const int slot
     s_cq = BFP ? (float)(1.5 * 8388608.0 * st->q) : 0.f;
   }
   __syncthreads();
-  const typename O::Cplx a1 = s_a[0], a2 = s_a[1], aA = s_a[2];
+  const O::Cplx a1 = s_a[0], a2 = s_a[1], aA = s_a[2];
   const float2 cq = make_float2(s_cq, s_cq);
   float mxr = 0.f;
   const int n = s_n;
@@ -1688,7 +1802,7 @@ __device__ __forceinline__ void combine_body(const PassParams& p, const int slot
   const int tid = threadIdx.x;
   const int nthr = blockDim.x;
   const int dx = nthr % d.nxp, dy = nthr / d.nxp;
-  typename AccOf<MODE>::type acc;
+  AccDF acc;
   for (int z = za; z < zb; ++z) {
     const long long zo = (long long)z * pe;
     const int pl = recorded_plane(d, z);
@@ -1730,7 +1844,7 @@ __device__ __forceinline__ void combine_body(const PassParams& p, const int slot
   block_sum_lane0<5>(v5, s_red);
   if (BFP) mxr = block_max0(mxr, reinterpret_cast<float*>(s_red));
   if (tid == 0) {
-    double* dst = p.partials + ((size_t)slot * d.npart + d.ctas_per_slot + cblk) * 8;
+    double* dst = p.partials + ((size_t)slot * d.npart + d.nlog + cblk) * 8;
 #pragma unroll
     for (int k = 0; k < 5; ++k) dst[k] = v5[k];
     if (BFP) {
@@ -1740,244 +1854,382 @@ __device__ __forceinline__ void combine_body(const PassParams& p, const int slot
   }
 }
 
-// At most 64 registers: four CTAs (32 warps) per SM keep enough loads in flight for HBM.
-template <int MODE, bool BFP>
-__global__ void __launch_bounds__(kCombThreads, 4) combine_kernel(PassParams p) {
-  combine_body<MODE, BFP>(p, blockIdx.y, blockIdx.x);
+// Combine with its sums in the stored pass's blocks, double-float: CTA = one block of 32 x lty columns and a z-chunk, a
+// thread a column, two planes per step (six 16-byte loads in flight; a warp reads rows of 512 bytes).  Grids of at most
+// 16 (8) columns put two (four) rows into a warp: the missing columns of a row add zeros, which change no sum.
+__global__ void __launch_bounds__(kCombThreads, 4) combine_blocks_kernel(PassParams p) {
+  typedef Ops<RSFD_DF64> O;
+  typedef Stencil<RSFD_DF64, 1> ST;
+  const int slot = blockIdx.y, cta = blockIdx.x;
+  const SlotState* st = p.slots + slot;
+  if (st->status != SLOT_RUNNING) return;
+  __shared__ O::Cplx s_a[3];
+  __shared__ double s_rows[8 * 3];
+  const SolveDims& d = p.d;
+  const int tid = threadIdx.x, lane = tid & 31;
+  if (tid < 3) s_a[tid] = O::cplx(tid == 0 ? st->a1 : (tid == 1 ? st->a2 : st->aA));
+  const int n = st->n, hc = st->hcnt;
+  __syncthreads();
+  const O::Cplx a1 = s_a[0], a2 = s_a[1], aA = s_a[2];
+  const int hw = d.nx <= 8 ? 4 : (d.nx <= 16 ? 2 : 1), wd = 32 / hw;   // rows and columns per warp
+  const int ltx = (d.nx + 31) / 32;
+  const int tz = cta % d.nzchunks, txy = cta / d.nzchunks;
+  const int row = (tid >> 5) * hw + lane / wd;
+  const int x = (txy % ltx) * 32 + lane % wd, y = (txy / ltx) * d.lty + row;
+  const int z0 = tz * d.zchunk, z1 = min(z0 + d.zchunk, d.nz);
+  const bool own = x < d.nx && y < d.ny && row < d.lty;
+  const long long pe = (long long)d.nxp * d.ny, vec = d.nz * pe, o = z0 * pe + (long long)y * d.nxp + x;
+  dfc* base = reinterpret_cast<dfc*>(p.rbuf) + (size_t)slot * 5 * vec + o;
+  const dfc *R1 = base + ((n + 2) % 3) * vec, *R2 = base + ((n + 1) % 3) * vec, *U1 = base + (3 + (n + 1) % 2) * vec;
+  dfc* RO = base + (n % 3) * vec;
+  float2* hist = reinterpret_cast<float2*>(p.rhist) + ((size_t)slot * p.hist_len + hc) * d.nb + (size_t)y * d.nx + x;
+  const size_t nxy = (size_t)d.nx * d.ny;
+  AccDF acc;
+  if (own) {
+    for (int z = z0; z < z1; z += 2) {
+      const bool has2 = z + 1 < z1;
+      const dfc r1a = R1[0], r2a = R2[0], ua = U1[0];
+      dfc r1b = r1a, r2b = r2a, ub = ua;
+      if (has2) { r1b = R1[pe]; r2b = R2[pe]; ub = U1[pe]; }
+      const dfc ra = ST::combine(a1, r1a, a2, r2a, aA, ua);   // Eq. rvec
+      RO[0] = ra;
+      acc.add_r(ra);
+      int pl = recorded_plane(d, z);
+      if (pl >= 0) hist[pl * nxy] = ra.h;
+      if (has2) {
+        const dfc rb = ST::combine(a1, r1b, a2, r2b, aA, ub);
+        RO[pe] = rb;
+        acc.add_r(rb);
+        pl = recorded_plane(d, z + 1);
+        if (pl >= 0) hist[pl * nxy] = rb.h;
+      }
+      R1 += 2 * pe;
+      R2 += 2 * pe;
+      U1 += 2 * pe;
+      RO += 2 * pe;
+    }
+  }
+  // a row's columns in the fixed tree of a whole warp (narrower groups skip its steps over zeros), then the rows
+  for (int off = wd / 2; off > 0; off >>= 1) {
+    const float2 a = AccDF::shfl2(acc.rr_s, off), b = AccDF::shfl2(acc.rr_l, off);
+    AccDF::merge(acc.rr_s, acc.rr_l, a, b);
+    acc.nn += __shfl_down_sync(0xffffffffu, acc.nn, off);
+  }
+  if (lane % wd == 0 && row < d.lty) {
+    s_rows[row * 3] = (double)acc.rr_s.x + (double)acc.rr_l.x;
+    s_rows[row * 3 + 1] = (double)acc.rr_s.y + (double)acc.rr_l.y;
+    s_rows[row * 3 + 2] = (double)acc.nn;
+  }
+  __syncthreads();
+  if (tid < 3) {
+    double t = 0.0;
+    for (int r = 0; r < d.lty; ++r) t += s_rows[r * 3 + tid];
+    p.partials[((size_t)slot * d.npart + cta) * 8 + (tid == 2 ? 4 : tid)] = t;
+  }
 }
 
-// Stencil: CTA = a 32 x TY tile of one slot and a z-range, one thread per tile point (one warp per
-// tile row).  Per z-plane one TMA transfer brings the (32 + 4) x (TY + 2R) box of r_n into a ring of
-// depth + R + 1 shared-memory stages; each thread keeps its own column's r_n on the last 2R + 1
-// planes in registers (ring rotated by unrolling, no moves) and takes its x and y neighbours from
-// the stage of the plane it evaluates.  One barrier per plane.
+// Stencil: CTA = a TX x TY tile of one slot and a z-range.  A thread owns two y-adjacent points of the tile;
+// threads are numbered through the tile, so TX need not divide a warp and follows the grid's width (48, or
+// 32 + 40 for 72 ...).  Per z-plane one TMA transfer brings the (TX + 4) x (TY + 2R)
+// box of r_n and one the tile of V into a ring of depth + R + 1 shared-memory stages; a thread keeps its points'
+// r_n of the last 2R + 1 planes in registers (ring rotated by unrolling, no moves) and takes the other x and y
+// neighbours from the stage of the plane it evaluates: 12 instead of 16 shared loads for two points.
+// There is no CTA-wide barrier per plane: a stage has a "full" mbarrier (the TMA bytes) and an "empty" one
+// on which each warp arrives when it is done with it; thread 0 refills (an extra warp for that would cost a
+// quarter of the register file's third warp slot per scheduler: 96 registers a thread instead of 128).
+// Double-float vectors (LOG): the rounding of the sums is that of blocks of 32 x d.lty columns and a z-chunk (a warp a
+// row, the rows in order), whatever tile the CTA has: a tile is made of such blocks, every column keeps its own
+// accumulators over the z-range, and they are added in that order at the end.
+// BFP (double-float handles): the r_n it reads has block-floating-point leading parts, tmV maps s V, and it
+// stores u_n = s A r_n (StencilBFP) with the largest leading-part component of u_n.
 constexpr int kMaxStagesS = kMaxDepth + 3;
+constexpr int kStencilThreads = 256;
+constexpr int kMaxRowSums = 128;   // rows of 32 columns in a double-float tile (at most 60 wide, 512 points)
 
-// The potential of the plane being evaluated arrives by TMA with the plane of r_n.  There is no
-// CTA-wide barrier per plane: every stage has a "full" mbarrier (the TMA transaction count) and an
-// "empty" one on which each warp arrives once it is done with the stage; thread 0 waits for a stage
-// to be empty before it refills it, so warps run up to the prefetch depth apart.
-// BFP (double-float handles): the r_n it reads has block-floating-point leading parts, tmV maps s V,
-// and it stores u_n = s A r_n (StencilBFP) with the largest leading-part component of u_n.
-// one stencil CTA: tile cta (of d.ctas_per_slot) of slot `slot`; blockDim = 32 x tile_y
+// Two 256-thread CTAs per SM (128 registers): three (80 registers) spill 90 bytes a point and were 1.6 times slower.
 template <int MODE, int R, bool BFP>
-__device__ __forceinline__ void stencil_body(const PassParams& p, const CUtensorMap& tmR, const CUtensorMap& tmV,
-                                             const int slot, const int cta) {
+__global__ void __launch_bounds__(kStencilThreads, MODE == RSFD_MIXED ? 3 : 2)
+stencil_kernel(PassParams p, const __grid_constant__ CUtensorMap tmR, const __grid_constant__ CUtensorMap tmV) {
   static_assert(!BFP || MODE == RSFD_DF64, "the block-floating-point pass is double-float only");
+  constexpr bool LOG = MODE == RSFD_DF64;
   typedef Ops<MODE> O;
   typedef typename O::C C;
   typedef typename O::VT VT;
   constexpr int Q = 2 * R + 1;
-  constexpr int BW = kTileX + 2 * kUBoxOff;
   extern __shared__ unsigned char smem_raw[];
   __shared__ ScalarShared S;
   __shared__ int s_last;
   __shared__ volatile int s_abort;
   __shared__ __align__(8) unsigned long long bars[kMaxStagesS];     // full: TMA bytes landed
-  __shared__ __align__(8) unsigned long long ebars[kMaxStagesS];    // empty: every warp done with it
+  __shared__ __align__(8) unsigned long long ebars[kMaxStagesS];    // empty: every consumer warp done with it
 
+  const int slot = blockIdx.y, cta = blockIdx.x;
   SlotState* st = p.slots + slot;
   if (st->status != SLOT_RUNNING) return;
   const SolveDims& d = p.d;
-  const int kDepth = p.depth;
-  const int NS = kDepth + R + 1;   // the stage of plane c is read R steps after its arrival
-  const int TY = d.tile_y;
-  const int EY = TY + 2 * R;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int NS = p.depth + R + 1;   // the stage of plane c is read R steps after its arrival
+  const int TX = d.tile_x, TY = d.tile_y;
+  const int BW = TX + 2 * kUBoxOff, EY = TY + 2 * R;
+  const int tid = threadIdx.x;
   const int tz = cta % d.nzchunks;
   const int txy = cta / d.nzchunks;
   const int tx = txy % d.tiles_x, ty = txy / d.tiles_x;
   const int z0 = tz * d.zchunk;
   const int z1 = min(z0 + d.zchunk, d.nz);
-  const int x0 = tx * kTileX, y0 = ty * TY;
-  const int gx = x0 + lane, gy = y0 + warp;
-  const bool own = gx < d.nx && gy < d.ny;
-  const long long plane_elems = (long long)d.nxp * d.ny;
+  // double-float: x-tiles of 32 columns, the last one with the remainder; else tiles of TX columns
+  const int x0 = tx * (LOG ? 32 : TX), y0 = ty * d.rows_cta;
+  const int xend = (LOG && tx + 1 < d.tiles_x) ? x0 + 32 : d.nx;   // columns and rows this CTA owns end here
+  const int yend = min(d.ny, y0 + d.rows_cta);
+  const int nsteps = (z1 - z0) + 2 * R;
 
   // shared memory: per stage the box of r_n (plane q) and the tile of V (plane q - R)
-  const size_t PBb = (size_t)BW * EY * sizeof(C);
-  const int PE = (int)(((PBb + 127) & ~(size_t)127) / sizeof(C));
-  const size_t PVb = (size_t)kTileX * TY * sizeof(VT);
-  const int PV = (int)(((PVb + 127) & ~(size_t)127) / sizeof(VT));
-  C* ring = (C*)(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
-  VT* vring = (VT*)(ring + (size_t)NS * PE);
-
-  struct Coefs {
-    typename O::Real zre, zim, mh1, mh2;
-    int n;
-  };
-  __shared__ Coefs sc;
-  if (tid == 0) {
-    const double2 Zs0 = st->Zs;
-    // BFP: the diagonal of s A is s (Z_s - hd) - s V
-    const double sd = BFP ? p.uscale : 1.0;
-    sc.zre = O::real(sd * (Zs0.x - p.hd));
-    sc.zim = O::real(sd * Zs0.y);
-    sc.mh1 = O::real(-p.hk1);
-    sc.mh2 = O::real(-p.hk2);
-    sc.n = st->n;
-  }
-  __syncthreads();
-  const int n = sc.n;
-  const int io = n % 3, iuo = 3 + n % 2;
-  const long long vec = (long long)d.nz * plane_elems;
-  C* uout = reinterpret_cast<C*>(p.rbuf) + ((size_t)slot * 5 + iuo) * vec;
-  const typename O::Real zre = sc.zre, zim = sc.zim, mh1 = sc.mh1, mh2 = sc.mh2;
-  float mxu = 0.f;
-
-  constexpr int mR = (MODE == RSFD_DF64) ? 4 : 2;
-  constexpr int mV = (MODE == RSFD_DF64) ? 2 : 1;
-  const int xr = mR * (x0 - kUBoxOff), yb = y0 - R, xv = mV * x0;
-  const int nsteps = (z1 - z0) + 2 * R;
-  const int wr = slot * 5 + io;
-  auto issue = [&](int bnd) {
-    const int k = bnd % NS;
-    const uint32_t bar = smem_u32(&bars[k]);
-    mbar_expect_tx(bar, (uint32_t)(PBb + PVb));
-    tma_load_4d(smem_u32(ring + (size_t)k * PE), &tmR, xr, yb, z0 - R + bnd, wr, bar);
-    tma_load_3d(smem_u32(vring + (size_t)k * PV), &tmV, xv, y0, z0 - 2 * R + bnd, bar);
-  };
-  const int nwarps = blockDim.x >> 5;
+  const uint32_t PBb = (uint32_t)(BW * EY * sizeof(C)), PVb = (uint32_t)(TX * TY * sizeof(VT));
+  const uint32_t PEb = (PBb + 127) & ~127u, PVs = (PVb + 127) & ~127u;   // stage strides in bytes
+  unsigned char* ring = (unsigned char*)(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
+  unsigned char* vring = ring + (size_t)NS * PEb;
+  const int nthr = blockDim.x;
+  float4* accA = (float4*)(vring + (size_t)NS * PVs);   // LOG: per row and thread the pair sum of (r, A r), at the end
+  const int n = st->n;
   if (tid == 0) {
     for (int k = 0; k < NS; ++k) {
       mbar_init(smem_u32(&bars[k]), 1);
-      mbar_init(smem_u32(&ebars[k]), (uint32_t)nwarps);
+      mbar_init(smem_u32(&ebars[k]), blockDim.x >> 5);
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     s_abort = 0;
   }
-  __syncthreads();
-  int issued = 0;
-  if (tid == 0) {
-    for (int bnd = 0; bnd < kDepth && bnd < nsteps; ++bnd) issue(bnd);
-    issued = min(kDepth, nsteps);
-  }
-  typename AccOf<MODE>::type acc;
-  // step s: plane q = z0 - R + s and the potential of plane c = q - R arrive in stage s % NS; from
-  // step 2R on, A r_n on plane c, whose r_n box is in stage (s - R) % NS.  A stage is released after
-  // its plane served as plane c (R steps after it arrived).
-  int ist = 0, par = 0, ic = NS - R, s = 0;
-  const int oc = (warp + R) * BW + lane + kUBoxOff;   // this thread's point in a stage
-  const int ov = warp * kTileX + lane;                // and in the potential's tile
+  struct Coefs {
+    typename O::Real zre, zim, mh1, mh2;
+  };
+  __shared__ Coefs sc;
+  const int cap = (int)first_wait_cap(d);
+  // bounded wait; also gives up when another thread has
+  auto wait = [&](uint32_t bar, uint32_t parity) -> bool {
+    for (int i = 0; i < cap; ++i) {
+      if (mbar_wait(bar, parity, 1)) return true;
+      if (s_abort) return false;
+    }
+    return false;
+  };
   auto fail_now = [&]() {
     s_abort = 1;
     atomicExch(p.error_flag, 1);
   };
-  auto begin_step = [&]() -> bool {
-    if (tid == 0 && s + kDepth < nsteps && !s_abort) {
-      const int b = s + kDepth;
-      // the stage's previous bundle (b - NS) must have been released by every warp
-      if (b >= NS && !mbar_wait(smem_u32(&ebars[b % NS]), (uint32_t)(((b / NS) - 1) & 1), first_wait_cap(d))) {
-        fail_now();
-      } else {
-        issue(b);
-        issued = b + 1;
+  typename AccSplit<MODE>::type acc[LOG ? 2 : 1];   // LOG: one per row
+  float mxu = 0.f;
+  int issued = 0;   // thread 0: bundles issued
+  {
+    constexpr int mR = (MODE == RSFD_DF64) ? 4 : 2;   // tensor-map elements per grid point along x
+    constexpr int mV = (MODE == RSFD_DF64) ? 2 : 1;
+    const int xr = mR * (x0 - kUBoxOff), yb = y0 - R, xv = mV * x0, wr = slot * 5 + n % 3;
+    int ik = 0, ipar = 1;   // stage of the next bundle, parity of its last release
+    auto issue = [&]() {
+      const uint32_t bar = smem_u32(&bars[ik]);
+      mbar_expect_tx(bar, PBb + PVb);
+      tma_load_4d(smem_u32(ring) + ik * PEb, &tmR, xr, yb, z0 - R + issued, wr, bar);
+      tma_load_3d(smem_u32(vring) + ik * PVs, &tmV, xv, y0, z0 - 2 * R + issued, bar);
+      if (++ik == NS) { ik = 0; ipar ^= 1; }
+      ++issued;
+    };
+    if (tid == 0) {
+      while (issued < p.depth && issued < nsteps) issue();
+      // the coefficients are converted while the first planes are on their way
+      const double2 Zs0 = st->Zs;
+      const double sd = BFP ? p.uscale : 1.0;   // BFP: the diagonal of s A is s (Z_s - hd) - s V
+      sc.zre = O::real(sd * (Zs0.x - p.hd));
+      sc.zim = O::real(sd * Zs0.y);
+      sc.mh1 = O::real(-p.hk1);
+      sc.mh2 = O::real(-p.hk2);
+    }
+    __syncthreads();
+    const int half = TY >> 1;
+    const bool act = tid < TX * half;
+    const int xl = act ? tid % TX : 0, yl = act ? 2 * (tid / TX) : 0;   // the points (xl, yl) and (xl, yl + 1)
+    const int gx = x0 + xl, gy = y0 + yl;
+    const bool own0 = act && gx < xend && gy < yend, own1 = act && gx < xend && gy + 1 < yend;
+    const long long plane_elems = (long long)d.nxp * d.ny;
+    // the points' place in a stage and in u_n
+    const uint32_t oc = (uint32_t)((yl + R) * BW + xl + kUBoxOff) * (uint32_t)sizeof(C);
+    const uint32_t ov = (uint32_t)(yl * TX + xl) * (uint32_t)sizeof(VT);
+    const uint32_t row = (uint32_t)BW * (uint32_t)sizeof(C), vrow = (uint32_t)TX * (uint32_t)sizeof(VT);
+    C* uout = reinterpret_cast<C*>(p.rbuf) + ((size_t)slot * 5 + 3 + n % 2) * (size_t)d.nz * plane_elems +
+              (size_t)z0 * plane_elems + (size_t)gy * d.nxp + gx;
+    const typename O::Real zre = sc.zre, zim = sc.zim, mh1 = sc.mh1, mh2 = sc.mh2;
+    // step s: plane q = z0 - R + s and the potential of plane c = q - R arrive in stage ist; from step 2R on, A r_n
+    // on plane c, whose box is in stage ic.  A stage is released after its plane served as plane c.
+    int ist = 0, ic = NS - R, s = 0;
+    uint32_t par = 0;
+    C zq[2][Q];
+    auto at = [&](const unsigned char* b, uint32_t o) -> C { return *reinterpret_cast<const C*>(b + o); };
+    auto end_step = [&]() {
+      __syncwarp();
+      if (s >= R && (tid & 31) == 0) mbar_arrive(smem_u32(&ebars[ic]));
+      if (++ist == NS) { ist = 0; par ^= 1; }
+      if (++ic == NS) ic = 0;
+      ++s;
+    };
+    auto arrive_plane = [&](auto ph_c) -> bool {   // waits for plane q and takes the thread's points of it
+      constexpr int PH = decltype(ph_c)::value;
+      bool ok = true;
+      if (tid == 0 && issued < nsteps) {   // refill: the stage's previous bundle must have been released
+        ok = issued < NS || wait(smem_u32(&ebars[ik]), (uint32_t)ipar);
+        if (ok) issue();
       }
-    }
-    if (s_abort) return false;
-    if (!mbar_wait(smem_u32(&bars[ist]), (uint32_t)par, first_wait_cap(d))) {
-      fail_now();
-      return false;
-    }
-    return true;
-  };
-  auto end_step = [&]() -> bool {
-    __syncwarp();
-    if (s >= R && lane == 0) mbar_arrive(smem_u32(&ebars[ic]));   // stage of bundle s - R
-    if (s_abort) return false;
-    if (++ist == NS) { ist = 0; par ^= 1; }
-    if (++ic == NS) ic = 0;
-    ++s;
-    return true;
-  };
-  bool ok = true;
-  C zq[Q];
-#pragma unroll
-  for (int t = 0; t < Q; ++t) zq[t] = O::zero();
-#pragma unroll
-  for (int t = 0; t < 2 * R; ++t) {
-    if (ok && s < nsteps) {
-      ok = begin_step();
-      if (!ok) break;
-      const C own_v = ring[(size_t)ist * PE + oc];
-      if (t == 0) zq[0] = own_v;
-      if (t == 1) zq[1 % Q] = own_v;
-      if (t == 2) zq[2 % Q] = own_v;
-      if (t == 3) zq[3 % Q] = own_v;
-      ok = end_step();
-    }
-  }
-  auto steady = [&](auto j_c) {
-    constexpr int PH = (2 * R + decltype(j_c)::value) % Q;   // ring slot of plane q
-    constexpr int CC = (PH + Q - R) % Q;                     // ring slot of plane c = q - R
-    if (!begin_step()) {
-      ok = false;
-      return;
-    }
-    zq[PH] = ring[(size_t)ist * PE + oc];
-    const int c = z0 - 2 * R + s;
-    const C* P0 = ring + (size_t)ic * PE;
-    C n1[6], n2[6];
-    n1[0] = zq[(CC + Q - 1) % Q];
-    n1[1] = zq[(CC + 1) % Q];
-    n1[2] = P0[oc - 1];
-    n1[3] = P0[oc + 1];
-    n1[4] = P0[oc - BW];
-    n1[5] = P0[oc + BW];
-    if (R == 2) {
-      n2[0] = zq[(CC + Q - 2) % Q];
-      n2[1] = zq[(CC + 2) % Q];
-      n2[2] = P0[oc - 2];
-      n2[3] = P0[oc + 2];
-      n2[4] = P0[oc - 2 * BW];
-      n2[5] = P0[oc + 2 * BW];
-    } else {
-#pragma unroll
-      for (int m = 0; m < 6; ++m) n2[m] = O::zero();
-    }
-    if (own) {
-      const C rc = zq[CC];
-      const VT v = vring[(size_t)ist * PV + ov];
+      ok = ok && wait(smem_u32(&bars[ist]), par);
+      if (!__all_sync(0xffffffffu, ok)) {   // the warp stops as a whole
+        if (!s_abort) fail_now();
+        return false;
+      }
+      const unsigned char* b = ring + ist * PEb;
+      zq[0][PH] = at(b, oc);
+      zq[1][PH] = at(b, oc + row);
+      return true;
+    };
+    // A r_n at point k of the thread, given its neighbours
+    auto point = [&](int k, const C& rc, const C (&n1)[6], const C (&n2)[6], VT v, bool own, C* dst) {
       if constexpr (BFP) {
         const float2 zh = make_float2(-zim.h, zim.h), zl = make_float2(-zim.l, zim.l);
         const dfc u = StencilBFP<R>::applyA(rc, n1, n2, v, zre, zh, zl);
         dfc rn;   // normalised r_n for the exact products of the dot
         fast_two_sum2(rc.h, rc.l, rn.h, rn.l);
-        acc.add_ra(rn, u);
-        mxu = fmaxf(mxu, fmaxf(fabsf(u.h.x), fabsf(u.h.y)));
-        uout[(long long)c * plane_elems + (long long)gy * d.nxp + gx] = u;
+        if (own) {
+          acc[k].add_ra(rn, u);
+          mxu = fmaxf(mxu, fmaxf(fabsf(u.h.x), fabsf(u.h.y)));
+          *dst = u;
+        }
       } else {
-        const C u = Stencil<MODE, R>::applyA(rc, n1, n2, v, zre, zim, mh1, mh2);
-        acc.add_ra(rc, u);
-        uout[(long long)c * plane_elems + (long long)gy * d.nxp + gx] = u;
+        if (own) {
+          const C u = Stencil<MODE, R>::applyA(rc, n1, n2, v, zre, zim, mh1, mh2);
+          acc[LOG ? k : 0].add_ra(rc, u);
+          *dst = u;
+        }
+      }
+    };
+    auto steady = [&](auto j_c) -> bool {
+      constexpr int PH = (2 * R + decltype(j_c)::value) % Q;   // register of plane q
+      constexpr int CC = (PH + Q - R) % Q;                     // register of plane c = q - R
+      if (!arrive_plane(std::integral_constant<int, PH>())) return false;
+      const unsigned char* b = ring + ic * PEb;
+      const unsigned char* vb = vring + ist * PVs;
+      C n1[6], n2[6];
+      const C um1 = at(b, oc - row), dp1 = at(b, oc + 2 * row);
+      C um2 = O::zero(), dp2 = O::zero();
+      if (R == 2) { um2 = at(b, oc - 2 * row); dp2 = at(b, oc + 3 * row); }
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const uint32_t o = oc + k * row;
+        n1[0] = zq[k][(CC + Q - 1) % Q];
+        n1[1] = zq[k][(CC + 1) % Q];
+        n1[2] = at(b, o - (uint32_t)sizeof(C));
+        n1[3] = at(b, o + (uint32_t)sizeof(C));
+        n1[4] = k == 0 ? um1 : zq[0][CC];
+        n1[5] = k == 0 ? zq[1][CC] : dp1;
+        if (R == 2) {
+          n2[0] = zq[k][(CC + Q - 2) % Q];
+          n2[1] = zq[k][(CC + 2) % Q];
+          n2[2] = at(b, o - 2 * (uint32_t)sizeof(C));
+          n2[3] = at(b, o + 2 * (uint32_t)sizeof(C));
+          n2[4] = k == 0 ? um2 : um1;
+          n2[5] = k == 0 ? dp1 : dp2;
+        } else {
+#pragma unroll
+          for (int m = 0; m < 6; ++m) n2[m] = O::zero();
+        }
+        const VT v = *reinterpret_cast<const VT*>(vb + ov + k * vrow);
+        point(k, zq[k][CC], n1, n2, v, k == 0 ? own0 : own1, uout + (k == 0 ? 0 : d.nxp));
+      }
+      uout += plane_elems;
+      end_step();
+      return true;
+    };
+    bool ok = true;
+#pragma unroll
+    for (int t = 0; t < 2 * R; ++t) {
+      if (ok) {
+        if (t == 0) ok = arrive_plane(std::integral_constant<int, 0>());
+        if (t == 1) ok = arrive_plane(std::integral_constant<int, 1>());
+        if (t == 2) ok = arrive_plane(std::integral_constant<int, 2 % Q>());
+        if (t == 3) ok = arrive_plane(std::integral_constant<int, 3 % Q>());
+        if (ok) end_step();
       }
     }
-    ok = end_step();
-  };
-  while (ok && s < nsteps) {
-    steady(std::integral_constant<int, 0>());
-    if (ok && s < nsteps) steady(std::integral_constant<int, 1>());
-    if (ok && s < nsteps) steady(std::integral_constant<int, 2>());
-    if (R == 2) {
-      if (ok && s < nsteps) steady(std::integral_constant<int, 3>());
-      if (ok && s < nsteps) steady(std::integral_constant<int, 4>());
+    while (ok && s < nsteps) {
+      ok = steady(std::integral_constant<int, 0>());
+      if (ok && s < nsteps) ok = steady(std::integral_constant<int, 1>());
+      if (ok && s < nsteps) ok = steady(std::integral_constant<int, 2>());
+      if (R == 2) {
+        if (ok && s < nsteps) ok = steady(std::integral_constant<int, 3>());
+        if (ok && s < nsteps) ok = steady(std::integral_constant<int, 4>());
+      }
     }
   }
-  (void)ok;
   __syncthreads();   // every thread, finished or stopped by an expired wait
   if (s_abort) {
-    // drain the transfers still in flight: per stage, the last bundle thread 0 issued into it (the
+    // per stage, the last transfer issued into it lands before the CTA's shared memory is released (the
     // earlier ones on that stage completed before it was refilled)
-    if (tid == 0) {
-      for (int bnd = max(0, issued - NS); bnd < issued; ++bnd)
-        mbar_wait(smem_u32(&bars[bnd % NS]), (uint32_t)((bnd / NS) & 1));
-    }
+    for (int bnd = max(0, issued - NS); bnd < issued; ++bnd)
+      mbar_wait(smem_u32(&bars[bnd % NS]), (uint32_t)((bnd / NS) & 1));
     return;
   }
-  double v5[5];
-  acc.get(v5);
-  if (pass_finish(p, slot, cta, v5, S, s_last, mxu)) {
+  if constexpr (LOG) {
+    // rows of 32 columns, one warp each: the 32 columns' sums in a fixed tree, then the rows of a block in order
+    __shared__ double s_rows[kMaxRowSums * 2];
+    for (int k = 0; k < 2; ++k) accA[k * nthr + tid] = make_float4(acc[k].ra_s.x, acc[k].ra_s.y, acc[k].ra_l.x, acc[k].ra_l.y);
+    __syncthreads();
+    const int lty = d.lty, nlx = (xend - x0 + 31) / 32, nly = (d.rows_cta + lty - 1) / lty, nseg = nlx * TY;
+    const int lane = tid & 31;
+    for (int g = tid >> 5; g < nseg; g += nthr >> 5) {
+      const int row = g / nlx, x = (g - row * nlx) * 32 + lane;
+      AccDF a;
+      if (x < TX && x < xend - x0) {
+        const int t = (row >> 1) * TX + x, k = row & 1;
+        const float4 v = accA[k * nthr + t];
+        a.ra_s = make_float2(v.x, v.y);
+        a.ra_l = make_float2(v.z, v.w);
+      }
+      double o[5];
+      a.get(o);
+      if (lane == 0) {
+        s_rows[g * 2] = o[2];
+        s_rows[g * 2 + 1] = o[3];
+      }
+    }
+    if (BFP) mxu = block_max0(mxu, reinterpret_cast<float*>(S.red));
+    __syncthreads();
+    // block (lx, ly) of the CTA is block (tx + lx, ty nly + ly) of the slot
+    const int ltx = (d.nx + 31) / 32, lty_n = (d.ny + lty - 1) / lty;
+    for (int e = tid; e < nlx * nly * 2; e += nthr) {
+      const int k = e % 2, lx = (e / 2) % nlx, ly = e / (2 * nlx);
+      const int by = ty * nly + ly;
+      if (by < lty_n) {
+        double t = 0.0;
+        for (int r = ly * lty; r < min(TY, (ly + 1) * lty); ++r) t += s_rows[(r * nlx + lx) * 2 + k];
+        double* dst = p.partials + ((size_t)slot * d.npart + ((size_t)by * ltx + tx + lx) * d.nzchunks + tz) * 8;
+        dst[2 + k] = t;
+        if (!d.rr_blocks) dst[k] = 0.0;   // (r, r) and ||r||^2 are in the combine's own entries
+        if (k == 0) {
+          if (!d.rr_blocks) dst[4] = 0.0;
+          dst[5] = 0.0;
+          dst[6] = 0.0;
+        }
+      }
+    }
+    __syncthreads();
+    if (BFP && tid == 0)
+      p.partials[((size_t)slot * d.npart + ((size_t)(ty * nly) * ltx + tx) * d.nzchunks + tz) * 8 + 6] = (double)mxu;
+    __threadfence();   // the partials, before the ticket
+    __syncthreads();
+  }
+  bool last;
+  if constexpr (LOG) {
+    last = pass_tail(p, slot, S, s_last);
+  } else {
+    double v5[5];
+    acc[0].get(v5);
+    last = pass_finish(p, slot, cta, v5, S, s_last);
+  }
+  if (last) {
     if (p.has_proj) {
       if (tid == 0) {
         double* o = p.pdots + (size_t)slot * 8;
@@ -1993,12 +2245,6 @@ __device__ __forceinline__ void stencil_body(const PassParams& p, const CUtensor
       scalar_step(p, slot, S);
     }
   }
-}
-
-template <int MODE, int R, int NT, int MINB, bool BFP = false>
-__global__ void __launch_bounds__(NT, MINB) stencil_kernel(PassParams p, const __grid_constant__ CUtensorMap tmR,
-                                                             const __grid_constant__ CUtensorMap tmV) {
-  stencil_body<MODE, R, BFP>(p, tmR, tmV, blockIdx.y, blockIdx.x);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -2477,6 +2723,12 @@ PassParams pass_params(const SolveDims& d, const SolverBuffers& b, const Stencil
   return p;
 }
 
+// threads of combine_blocks_kernel: a warp per 32, 16 or 8 columns' rows
+int block_threads(int nx, int lty) {
+  const int hw = nx <= 8 ? 4 : (nx <= 16 ? 2 : 1);
+  return (lty + hw - 1) / hw * 32;
+}
+
 template <int MODE, int R>
 cudaError_t launch_pass_t(const SolveDims& d, const SolverBuffers& b, const StencilCoef& c, double tol, int maxit,
                           int hist_len, cudaStream_t st, cudaEvent_t mid, bool mid_external) {
@@ -2484,11 +2736,13 @@ cudaError_t launch_pass_t(const SolveDims& d, const SolverBuffers& b, const Sten
   const bool bfp = p.bfp != 0;
   dim3 grid(d.ctas_per_slot, d.W);
   if (d.kind == RSFD_PASS_SPLIT || d.kind == RSFD_PASS_SPLIT_BFP) {
+    const dim3 gc(d.ctas_c, d.W);
     if constexpr (MODE == RSFD_DF64) {
-      if (bfp) combine_kernel<MODE, true><<<dim3(d.ctas_c, d.W), kCombThreads, 0, st>>>(p);
-      else combine_kernel<MODE, false><<<dim3(d.ctas_c, d.W), kCombThreads, 0, st>>>(p);
+      if (bfp) combine_planes_kernel<true><<<gc, kCombThreads, 0, st>>>(p);
+      else if (d.rr_blocks) combine_blocks_kernel<<<gc, block_threads(d.nx, d.lty), 0, st>>>(p);
+      else combine_planes_kernel<false><<<gc, kCombThreads, 0, st>>>(p);
     } else {
-      combine_kernel<MODE, false><<<dim3(d.ctas_c, d.W), kCombThreads, 0, st>>>(p);
+      combine_kernel<MODE><<<gc, kCombThreads, 0, st>>>(p);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -2496,23 +2750,15 @@ cudaError_t launch_pass_t(const SolveDims& d, const SolverBuffers& b, const Sten
       e = mid_external ? cudaEventRecordWithFlags(mid, st, cudaEventRecordExternal) : cudaEventRecord(mid, st);
       if (e != cudaSuccess) return e;
     }
-    const size_t smem = split_smem(MODE, R, d.tile_y, d.depth);
-    const int thr = split_threads(d.tile_y);
+    const size_t smem = split_smem(MODE, R, d.tile_x, d.tile_y, d.depth);
+    const int thr = split_threads(d.tile_x, d.tile_y);
     if constexpr (MODE == RSFD_DF64) {
       if (bfp) {
-        // register budget 1: at most 64 registers, two 512-thread (four 256-thread) CTAs per SM
-        if (d.regs == 1) {
-          if (thr <= 256) stencil_kernel<MODE, R, 256, 4, true><<<grid, thr, smem, st>>>(p, *b.tmR, *b.tmVs);
-          else stencil_kernel<MODE, R, 512, 2, true><<<grid, thr, smem, st>>>(p, *b.tmR, *b.tmVs);
-        } else {
-          if (thr <= 256) stencil_kernel<MODE, R, 256, 3, true><<<grid, thr, smem, st>>>(p, *b.tmR, *b.tmVs);
-          else stencil_kernel<MODE, R, 512, 1, true><<<grid, thr, smem, st>>>(p, *b.tmR, *b.tmVs);
-        }
+        stencil_kernel<MODE, R, true><<<grid, thr, smem, st>>>(p, *b.tmR, *b.tmVs);
         return cudaGetLastError();
       }
     }
-    if (thr <= 256) stencil_kernel<MODE, R, 256, 3><<<grid, thr, smem, st>>>(p, *b.tmR, *b.tmV);
-    else stencil_kernel<MODE, R, 512, 1><<<grid, thr, smem, st>>>(p, *b.tmR, *b.tmV);
+    stencil_kernel<MODE, R, false><<<grid, thr, smem, st>>>(p, *b.tmR, *b.tmV);
     return cudaGetLastError();
   }
   if (d.kind == RSFD_PASS_STORED) {
@@ -2546,17 +2792,28 @@ size_t pass_smem(int prec, int R, int tile_y, int depth) {
   return (size_t)(R + 1 + depth + stages + R + 2) * pc + stages * pv + 128;
 }
 int pass_max_depth() { return kMaxDepth; }
-int split_threads(int tile_y) { return 32 * tile_y; }
-size_t split_smem(int prec, int R, int tile_y, int depth) {
+int split_threads(int tile_x, int tile_y) { return (tile_x * (tile_y / 2) + 31) / 32 * 32; }
+int split_max_points() { return 2 * kStencilThreads; }
+size_t split_smem(int prec, int R, int tile_x, int tile_y, int depth) {
   const size_t es = prec == RSFD_MIXED ? 8 : 16;
-  const size_t pb = ((size_t)(kTileX + 2 * kUBoxOff) * (tile_y + 2 * R) * es + 127) & ~(size_t)127;
+  const size_t pb = ((size_t)(tile_x + 2 * kUBoxOff) * (tile_y + 2 * R) * es + 127) & ~(size_t)127;
   // per TMA stage the box of r_n and the tile of the potential
   const size_t vs = prec == RSFD_MIXED ? 4 : 8;
-  const size_t pv = ((size_t)kTileX * tile_y * vs + 127) & ~(size_t)127;
-  return (size_t)(depth + R + 1) * (pb + pv) + 128;
+  const size_t pv = ((size_t)tile_x * tile_y * vs + 127) & ~(size_t)127;
+  // double-float: two rows' accumulators per thread
+  const size_t ac = prec == RSFD_DF64 ? (size_t)split_threads(tile_x, tile_y) * 2 * 16 : 0;
+  return (size_t)(depth + R + 1) * (pb + pv) + ac + 128;
 }
-int split_combine_ctas(int nz, int W, int sms) {
-  // about eight 256-thread CTAs per SM over all slots, at least one plane each
+// Combine CTAs per slot.  Plain ranges: by the vector's length alone, so that a column's sums do not depend on how
+// many columns run beside it: 2048 16-byte units per CTA (four steps of its 256 threads), at most 64 CTAs (longer
+// ranges from there on).
+int split_combine_ctas(int prec, long long vec) {
+  const long long c = vec * (prec == RSFD_MIXED ? 8 : 16) / (2048 * 16);
+  return (int)(c < 1 ? 1 : (c > 64 ? 64 : c));
+}
+// Ranges of planes (double-float, with its sums): about eight 256-thread CTAs per SM over all slots, at least one
+// plane each
+int split_plane_ctas(int nz, int W, int sms) {
   int c = (8 * sms + W - 1) / W;
   if (c > nz) c = nz;
   if (c > 256) c = 256;
@@ -2599,24 +2856,18 @@ cudaError_t kernels_init() {
   RSFD_ATTR(RSFD_DF64, 1)
   RSFD_ATTR(RSFD_DF64, 2)
 #undef RSFD_ATTR
-#define RSFD_ATTR_S(M, R)                                                                                \
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(stencil_kernel<M, R, 256, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim); \
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(stencil_kernel<M, R, 512, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  RSFD_ATTR_S(RSFD_FP64, 1)
-  RSFD_ATTR_S(RSFD_FP64, 2)
-  RSFD_ATTR_S(RSFD_MIXED, 1)
-  RSFD_ATTR_S(RSFD_MIXED, 2)
-  RSFD_ATTR_S(RSFD_DF64, 1)
-  RSFD_ATTR_S(RSFD_DF64, 2)
+#define RSFD_ATTR_S(M, R, F)                                                                             \
+  if (e == cudaSuccess)                                                                                 \
+    e = cudaFuncSetAttribute(stencil_kernel<M, R, F>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+  RSFD_ATTR_S(RSFD_FP64, 1, false)
+  RSFD_ATTR_S(RSFD_FP64, 2, false)
+  RSFD_ATTR_S(RSFD_MIXED, 1, false)
+  RSFD_ATTR_S(RSFD_MIXED, 2, false)
+  RSFD_ATTR_S(RSFD_DF64, 1, false)
+  RSFD_ATTR_S(RSFD_DF64, 2, false)
+  RSFD_ATTR_S(RSFD_DF64, 1, true)
+  RSFD_ATTR_S(RSFD_DF64, 2, true)
 #undef RSFD_ATTR_S
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(stencil_kernel<RSFD_DF64, 1, 256, 3, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(stencil_kernel<RSFD_DF64, 1, 512, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(stencil_kernel<RSFD_DF64, 2, 256, 3, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(stencil_kernel<RSFD_DF64, 2, 512, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(stencil_kernel<RSFD_DF64, 1, 256, 4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(stencil_kernel<RSFD_DF64, 1, 512, 2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(stencil_kernel<RSFD_DF64, 2, 256, 4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(stencil_kernel<RSFD_DF64, 2, 512, 2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(chunk_apply_kernel<RSFD_FP64>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(chunk_apply_kernel<RSFD_MIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(chunk_apply_kernel<RSFD_DF64>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);

@@ -207,8 +207,8 @@ static PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
 // TMA descriptors of the Krylov vectors [nvec W][Nz][Ny][Nxp] and of the potential [Nz][Ny][Nxp].
 // Rows are padded to Nxp (a multiple of 4) so every stride is a multiple of 16 bytes; the x extent
 // is the true Nx, so reads past the last column (and outside the grid) come back as zeros.
-// Boxes: fused pass 40 x (tile_y + 4R) for both; stored-product pass 36 x (tile_y + 2R) for the
-// vectors and the 32 x tile_y tile for the potential.
+// Boxes: fused pass 40 x (tile_y + 4R) for both; stored-product and split passes (tile_x + 4) x (tile_y + 2R)
+// for the vectors and the tile_x x tile_y tile for the potential.
 static rsfd_status make_maps(Handle* h, int W, int tile_y, int kind, int tile_x) {
   PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
   if (!enc) return fail(h, RSFD_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
@@ -250,14 +250,65 @@ static rsfd_status make_maps(Handle* h, int W, int tile_y, int kind, int tile_x)
 }
 
 // the block-floating-point split pass serves double-float handles; the others run the plain split pass
-static int resolve_kind(int prec, int opt) {
+static int resolve_kind(int prec, const rsfd_solve_opts& o) {
+  const int opt = o.pass_kind;
   if (opt == RSFD_PASS_SPLIT_BFP) return prec == RSFD_DF64 ? opt : RSFD_PASS_SPLIT;
   if (opt == RSFD_PASS_RECOMPUTE || opt == RSFD_PASS_STORED || opt == RSFD_PASS_SPLIT) return opt;
-  return RSFD_PASS_STORED;
+  // automatic: the split pass, which evaluates every point once on tiles cut to the grid; a launch shape that
+  // was given in terms of the stored pass keeps the stored pass
+  const bool shaped = o.tile_y > 0 || o.tile_x == 16 || o.rows_per_thread > 1 || o.reg_budget > 0 || o.prefetch > 0;
+  return shaped ? RSFD_PASS_STORED : RSFD_PASS_SPLIT;
+}
+
+// Width of the split pass's tiles for rows of nx points in tiles of at most `most`: equal tiles, rounded up to the
+// 16-byte granularity of the TMA boxes (4 points of a float potential, 2 of the others).
+static int split_tile_x(int prec, int nx, int most) {
+  const int g = prec == RSFD_MIXED ? 4 : 2, n = (nx + most - 1) / most;
+  return ((nx + n - 1) / n + g - 1) / g * g;
+}
+
+// Tile of the split pass when it is not given: equal tiles with at most 512 points, by the fewest thread slots per
+// grid point (ragged edges, partly filled warps), a tenth of the halo's share and a quarter warp per CTA.
+static void split_tile(int prec, int R, int nx, int ny, int& tx, int& ty) {
+  double best = 1e30;
+  for (int nt = 1; nt <= nx; ++nt) {
+    const int X = split_tile_x(prec, nx, (nx + nt - 1) / nt);
+    if (X > 60) continue;
+    if (X < 8 && nt > 1) break;
+    for (int mt = 1; mt <= ny; ++mt) {
+      const int Y = ((ny + mt - 1) / mt + 1) / 2 * 2;
+      if (X * Y > split_max_points()) continue;
+      const int warps = (X * Y / 2 + 31) / 32;
+      const double slots = (double)((nx + X - 1) / X) * ((ny + Y - 1) / Y) * (warps * 64.0) / ((double)nx * ny);
+      const double halo = (double)(X + 4) * (Y + 2 * R) / ((double)X * Y) - 1.0;
+      const double cost = slots * (1.0 + 0.1 * halo + 0.25 / warps);
+      if (cost < best) {
+        best = cost;
+        tx = X;
+        ty = Y;
+      }
+      if (Y <= 2) break;
+    }
+  }
+}
+
+// Tile of the double-float split pass, made of summation blocks of 32 x lty columns: the x-remainder joins the last
+// tile when that stays within 60 columns (TMA box), and blocks are stacked in y while the tile keeps at most
+// 256 threads (two points each) and half the rows are used.
+static void split_tile_blocks(int nx, int ny, int lty, int& tx, int& ty) {
+  const int rem = nx % 32;
+  ty = (lty + 1) / 2 * 2;
+  tx = std::min(32, (nx + 1) / 2 * 2);
+  if (nx > 32 && rem > 0 && rem <= 28) {
+    const int wide = 32 + (rem + 1) / 2 * 2;
+    if (wide * ty <= split_max_points()) tx = wide;
+  }
+  if (lty % 2 == 0)
+    while (2 * tx * ty <= split_max_points() && ty < ny && 2 * ty <= 64) ty *= 2;
 }
 
 static size_t kind_smem(int prec, int R, int tile_y, int depth, int kind, int tile_x = 32) {
-  if (is_split(kind)) return split_smem(prec, R, tile_y, depth);
+  if (is_split(kind)) return split_smem(prec, R, tile_x, (tile_y + 1) / 2 * 2, depth);
   return kind == RSFD_PASS_STORED ? passu_smem(prec, R, tile_y, depth, tile_x) : pass_smem(prec, R, tile_y, depth);
 }
 
@@ -271,7 +322,7 @@ static bool tile_ok(int prec, int R, int tile_y, int kind, int rows, int budget 
   if (is_split(kind)) {
     // one row per thread, 32-wide tiles, at most 16 rows (512 threads)
     if (tile_x != 32 || rows != 1 || tile_y > 16) return false;
-    return split_smem(prec, R, tile_y, 1) <= (size_t)(216 * 1024);
+    return split_smem(prec, R, 32, (tile_y + 1) / 2 * 2, 1) <= (size_t)(216 * 1024);
   }
   if (tile_x != 32) {
     // the 16-wide tile: one-row double-float stored pass with the default register budget only
@@ -599,7 +650,7 @@ static rsfd_status rsfd_set_solve_options_impl(rsfd_handle h, const rsfd_solve_o
   const int rows = resolve_rows(o->rows_per_thread);
   if (o->prefetch > pass_max_depth())
     return fail(h, RSFD_ERR_ARG, "rsfd_set_solve_options: prefetch must be <= " + std::to_string(pass_max_depth()));
-  const int kind = resolve_kind(h->prec, o->pass_kind);
+  const int kind = resolve_kind(h->prec, *o);
   if (o->reg_budget < 0 || o->reg_budget > 1)
     return fail(h, RSFD_ERR_ARG, "rsfd_set_solve_options: reg_budget must be 0 or 1");
   if (o->tile_x != 0 && o->tile_x != 16 && o->tile_x != 32)
@@ -688,7 +739,7 @@ static rsfd_status rsfd_shifted_cocg_impl(rsfd_handle h, const int64_t* cols, in
   d.K = K;
   d.kreq = Kout;
   d.ncols = ncols;
-  d.kind = resolve_kind(prec, h->opts.pass_kind);
+  d.kind = resolve_kind(prec, h->opts);
   // the projector term follows a pass that stores A r (stored-product or split)
   if (h->n_atoms > 0 && d.kind == RSFD_PASS_RECOMPUTE) d.kind = RSFD_PASS_STORED;
   d.nvec = d.kind == RSFD_PASS_RECOMPUTE ? 3 : 5;
@@ -698,30 +749,50 @@ static rsfd_status rsfd_shifted_cocg_impl(rsfd_handle h, const int64_t* cols, in
                ? h->opts.reg_budget
                : 0;
   d.tile_x = (h->opts.tile_x == 16 && d.kind == RSFD_PASS_STORED) ? 16 : 32;
-  d.wait_cap = h->opts.wait_cap;
-  d.brk_tol = h->opts.breakdown_tol > 0.0 ? h->opts.breakdown_tol : 1e-28;
   if (!tile_ok(prec, h->R, d.tile_y, d.kind, d.rows, d.regs, d.tile_x))
     return fail(h, RSFD_ERR_ARG, "rsfd_shifted_cocg: invalid tile_y / tile_x");
+  // Double-float: the split pass that replaces the stored one (automatic pass) forms every sum in the stored pass's
+  // blocks (32 x tile_y columns, z_chunk planes), and a given split pass forms (r, A r) in blocks of its own
+  // tile, so that these results do not depend on the launch shape in their last digits; the tiles are made of such
+  // blocks.
+  const bool logical = is_split(d.kind) && prec == RSFD_DF64;
+  d.rr_blocks = logical && h->opts.pass_kind == RSFD_PASS_AUTO;
+  d.lty = d.rr_blocks ? default_tile_y(prec, h->R, h->ny, RSFD_PASS_STORED, 1) : d.tile_y;
+  if (logical) {
+    split_tile_blocks(h->nx, h->ny, d.lty, d.tile_x, d.tile_y);
+  } else if (is_split(d.kind)) {
+    if (h->opts.tile_y > 0) {
+      d.tile_x = split_tile_x(prec, h->nx, 32);
+      d.tile_y = (d.tile_y + 1) / 2 * 2;
+    } else {
+      split_tile(prec, h->R, h->nx, h->ny, d.tile_x, d.tile_y);
+    }
+  }
+  d.wait_cap = h->opts.wait_cap;
+  d.brk_tol = h->opts.breakdown_tol > 0.0 ? h->opts.breakdown_tol : 1e-28;
   // TMA prefetch depth: the option, else the deepest that fits in shared memory (fused pass: a CTA
-  // alone on its SM) or 3 (stored-product pass: bundles are three times larger)
+  // alone on its SM), 3 (stored-product pass: bundles are three times larger), or 4 with two CTAs per SM (split
+  // pass: a third stage less costs nothing measurable, one CTA per SM 17 % on 38 columns of 64 x 64 x 128)
   if (h->opts.prefetch > 0) {
     d.depth = h->opts.prefetch;
   } else {
     d.depth = 1;
     const int dmax = d.kind == RSFD_PASS_STORED ? 3 : (is_split(d.kind) ? 4 : pass_max_depth());
     for (int dp = dmax; dp >= 1; --dp)
-      if (kind_smem(prec, h->R, d.tile_y, dp, d.kind, d.tile_x) <= (size_t)(216 * 1024)) {
+      if (kind_smem(prec, h->R, d.tile_y, dp, d.kind, d.tile_x) <= (size_t)((is_split(d.kind) ? 106 : 216) * 1024)) {
         d.depth = dp;
         break;
       }
   }
   if (kind_smem(prec, h->R, d.tile_y, d.depth, d.kind, d.tile_x) > (size_t)(216 * 1024))
     return fail(h, RSFD_ERR_ARG, "rsfd_shifted_cocg: prefetch depth does not fit in shared memory");
-  {
-    const int tw = d.kind == RSFD_PASS_RECOMPUTE ? pass_tile_x(h->R) : d.tile_x;
-    d.tiles_x = (h->nx + tw - 1) / tw;
-  }
-  d.tiles_y = (h->ny + d.tile_y - 1) / d.tile_y;
+  // tiles of the sums (the launch's own, except for double-float split passes)
+  const int ltiles_x = logical ? (h->nx + 31) / 32
+                               : (h->nx + d.tile_x - 1) / (d.kind == RSFD_PASS_RECOMPUTE ? pass_tile_x(h->R) : d.tile_x);
+  const int ltiles_y = logical ? (h->ny + d.lty - 1) / d.lty : (h->ny + d.tile_y - 1) / d.tile_y;
+  d.tiles_x = !logical ? ltiles_x : (d.tile_x > 32 ? std::max(1, h->nx / 32) : ltiles_x);
+  d.rows_cta = logical && d.lty % 2 != 0 ? d.lty : d.tile_y;
+  d.tiles_y = (h->ny + d.rows_cta - 1) / d.rows_cta;
   int W0 = h->opts.slots > 0 ? h->opts.slots : 256;
   W0 = std::min(W0, ncols);
   if (h->opts.z_chunk > 0) {
@@ -731,11 +802,12 @@ static rsfd_status rsfd_shifted_cocg_impl(rsfd_handle h, const int64_t* cols, in
     int sms = 152;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
     d.zchunk = h->nz;
-    while (d.zchunk > 16 && (long long)d.tiles_x * d.tiles_y * ((h->nz + d.zchunk - 1) / d.zchunk) * W0 < 4LL * sms)
+    while (d.zchunk > 16 && (long long)ltiles_x * ltiles_y * ((h->nz + d.zchunk - 1) / d.zchunk) * W0 < 4LL * sms)
       d.zchunk = (d.zchunk + 1) / 2;
   }
   d.nzchunks = (h->nz + d.zchunk - 1) / d.zchunk;
   d.ctas_per_slot = d.tiles_x * d.tiles_y * d.nzchunks;
+  d.nlog = ltiles_x * ltiles_y * d.nzchunks;   // the pass's CTAs, or the double-float split pass's blocks
   d.ctas_c = 0;
   const int C = h->opts.iters_per_sync > 0 ? h->opts.iters_per_sync : 32;
   if (C > kMaxHist) return fail(h, RSFD_ERR_ARG, "rsfd_shifted_cocg: iters_per_sync too large");
@@ -746,7 +818,7 @@ static rsfd_status rsfd_shifted_cocg_impl(rsfd_handle h, const int64_t* cols, in
     RSFD_CK(h, cudaMemGetInfo(&freeb, &totb));
     const size_t per_slot = (size_t)d.nvec * vec * vsz + 2 * (size_t)K * h->nr * vsz + (size_t)C * h->nr * hsz +
                             (size_t)K * C * sizeof(ShiftCoef) + (size_t)K * sizeof(ShiftState) +
-                            (size_t)(d.ctas_per_slot + 64) * 64 + 256;
+                            (size_t)(d.nlog + 64) * 64 + 256;
     const size_t have = h->rbuf.bytes + h->xbuf.bytes + h->pbuf.bytes + h->rhist.bytes + h->coef.bytes;
     const size_t budget = (size_t)(0.6 * (double)(freeb + have));
     if (h->opts.slots <= 0) {
@@ -754,12 +826,14 @@ static rsfd_status rsfd_shifted_cocg_impl(rsfd_handle h, const int64_t* cols, in
     }
   }
   d.W = W;
-  if (is_split(d.kind)) {
+  if (logical && !d.rr_blocks) {
     int sms = 152;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
-    d.ctas_c = split_combine_ctas(h->nz, W, sms);
+    d.ctas_c = split_plane_ctas(h->nz, W, sms);
+  } else if (is_split(d.kind)) {
+    d.ctas_c = d.rr_blocks ? d.nlog : split_combine_ctas(prec, vec);
   }
-  d.npart = d.ctas_per_slot + d.ctas_c;
+  d.npart = d.nlog + (d.rr_blocks ? 0 : d.ctas_c);
   const bool use_graphs = h->opts.use_graphs >= 0;
 
   // ---- workspace
@@ -1181,24 +1255,23 @@ static rsfd_status rsfd_autotune_impl(rsfd_handle h, const double* energies, int
   const int kinds[4] = {RSFD_PASS_STORED, RSFD_PASS_RECOMPUTE, RSFD_PASS_SPLIT, RSFD_PASS_SPLIT_BFP};
   const int zcs[3] = {0, h->nz, (h->nz + 1) / 2};
   for (int kind : kinds) {
-    if (kind == RSFD_PASS_SPLIT_BFP && resolve_kind(h->prec, kind) != kind) continue;
+    if (kind == RSFD_PASS_SPLIT_BFP && h->prec != RSFD_DF64) continue;
     if (is_split(kind)) {
       // the split pass: tile height and z-chunk
-      const int tys[3] = {8, 4, 16};
+      const int tys[3] = {16, 8, 4};
       const int pfs[2] = {0, 3};
       for (int ty : tys) {
         if (ty > h->ny && ty != 4) continue;
         if (!tile_ok(h->prec, h->R, ty, kind, 1)) continue;
         for (int zc : zcs)
-        for (int pf : pfs)
-        for (int rb = 0; rb < (kind == RSFD_PASS_SPLIT_BFP ? 2 : 1); ++rb) {
+        for (int pf : pfs) {
           if (zc > 0 && zc < 8) continue;
           rsfd_solve_opts o = keep;
           o.pass_kind = kind;
           o.rows_per_thread = 0;
           o.tile_y = ty;
           o.z_chunk = zc;
-          o.reg_budget = rb;
+          o.reg_budget = 0;
           o.tile_x = 0;
           o.slots = ncols;
           o.iters_per_sync = C;
@@ -1256,7 +1329,9 @@ static rsfd_status rsfd_autotune_impl(rsfd_handle h, const double* energies, int
     const double its = (double)h->stats.slot_iterations;
     if (its <= 0) continue;
     const double us = (h->stats.ms_pass + h->stats.ms_shift) * 1e3 / its;
-    if (best_us < 0 || us < best_us) {
+    // a clear gain only: in double-float the blocks of the sums follow tile_y and z_chunk, so candidates that are
+    // equally fast would otherwise give results that differ in their last digits from run to run
+    if (best_us < 0 || us < 0.985 * best_us) {
       best_us = us;
       best_o = o;
     }

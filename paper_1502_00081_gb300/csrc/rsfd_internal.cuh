@@ -121,7 +121,11 @@ struct SolveDims {
   int depth;          // TMA prefetch depth of the pass kernel
   int tiles_x, tiles_y, zchunk, nzchunks, ctas_per_slot;
   int ctas_c;         // split pass: CTAs per slot of the combine kernel (0 for the other forms)
-  int npart;          // partial-sum entries per slot: ctas_per_slot + ctas_c
+  int npart;          // partial-sum entries per slot: nlog, then the combine's where it forms sums
+  int nlog;           // partial-sum entries of the pass (or stencil) kernel: its CTAs, or its 32 x lty x zchunk blocks
+  int rows_cta;       // split pass: rows a CTA owns (tile_y, or an odd lty in a tile one row taller)
+  int lty;            // double-float split pass: rows of a summation block
+  int rr_blocks;      // double-float split pass: the combine runs, and sums, in the same blocks as the stencil
   int ncols;
   int ntrack;         // interior planes recorded after the boundary planes
   int track[16];      // their z indices (rows 2 nface Nx Ny + e Nx Ny ...)
@@ -129,7 +133,7 @@ struct SolveDims {
   int nvec;           // Krylov vectors per slot in rbuf: 3 (r ring) or 5 (r ring + A r pair)
   int rows;           // stored-product pass: tile rows per thread (1, 2 or 4)
   int regs;           // register budget of the one-row double-float pass (0, 1)
-  int tile_x;         // stored-product pass tile width in x: 32, or 16 (one-row double-float pass)
+  int tile_x;         // tile width in x: 32, 16 (one-row double-float stored pass) or, split passes, by the grid's width
   int wait_cap;       // attempts of the passes' first TMA waits: 0 = default, < 0 = none (test)
   double brk_tol;     // quasi-null threshold of (r, r) relative to ||r||^2
 };
@@ -217,9 +221,11 @@ int passu_max_threads(int rows, int budget);
 int passu_box_x(int tile_x);
 int passu_box_off();
 int pass_max_depth();
-int split_threads(int tile_y);
-size_t split_smem(int prec, int R, int tile_y, int depth);
-int split_combine_ctas(int nz, int W, int sms);
+int split_threads(int tile_x, int tile_y);   // tile_y even
+int split_max_points();                      // tile_x * tile_y at most
+size_t split_smem(int prec, int R, int tile_x, int tile_y, int depth);
+int split_combine_ctas(int prec, long long vec);
+int split_plane_ctas(int nz, int W, int sms);
 int pass_box_x();
 int pass_box_off();
 int pass_max_threads(int prec);
