@@ -17,7 +17,7 @@
 // They are added to 64-bit integers, so the k-sum has no further rounding; the result is rounded to
 // FP64 once.  Elements below 2^-9 of their row's (column's) largest lose bits below 2^-63 of it.
 //
-// Kernel.  One CTA makes a 128 x 32 tile of complex C: eight accumulators of 128 x 32 for Re and eight for
+// Kernel.  One CTA per SM works through 128 x 32 tiles of complex C: eight accumulators of 128 x 32 for Re and eight for
 // Im fill the 512 columns of tensor memory.  The digit planes are laid out in global memory exactly as
 // the tensor core wants them in shared memory (K-major core matrices, no swizzle), so a k-step of 16
 // is three contiguous bulk copies: one plane of A (8 digits x 128 rows, 32 KB), the other, and both
@@ -26,9 +26,10 @@
 // weights i-1..7.  18 warps: 16 read the accumulators, one thread of the 17th issues the copies,
 // one thread of the 18th the MMAs.
 //
-// Bound: tensor rate (144 real bf16 MACs per complex FP64 MAC; 36 B per clock and SM of operands from L2).
-// Measured: 16 products of 1024^3 in 4.6 ms, 3.8e12 complex multiply-adds/s, 1.08 PFLOP/s of bf16 MMAs = 0.56 of
-// the measured cuBLAS bf16 burst; the CUDA-core kernel takes 132 ms for the same (FP64 pipe, 1.3e11/s).
+// Bound: tensor rate (144 real bf16 MACs per complex FP64 MAC, 40 per FP32 one; 36 B per clock and SM of operands from L2).
+// Measured: 16 products of 1024^3 in 4.0 ms, 4.3e12 complex multiply-adds/s, 1.24 PFLOP/s of bf16 MMAs = 0.64 of the
+// measured cuBLAS bf16 burst (132 ms on the FP64 pipe, 1.3e11/s).  One tile per CTA instead of a persistent CTA, so
+// that a tile's set-up and write-back are not hidden: 4.6 ms, and 157 instead of 96 us for the FP32 LU's k = 128 updates.
 
 #include <cuda_runtime.h>
 #include <math_constants.h>
@@ -269,6 +270,7 @@ template <typename T> struct OzGemm {
   const unsigned char *A, *B;
   const unsigned int *exA, *exB;
   int m, n, m_pad, n_pad, ksteps;
+  int tiles;          // 128 x BN tiles of all matrices
   int sign;           // alpha (+1 or -1)
   int add;            // 1: add C
   T* C;
@@ -330,7 +332,14 @@ template <typename T> __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_k
   unsigned char* sA = smem;
   unsigned char* sB = smem + NA * ABLK;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int mt = blockIdx.x, nt = blockIdx.y, b = blockIdx.z;
+  const int mtiles = q.m_pad / OZ_BM, ntiles = q.n_pad / BN;
+  // tile t: row tile fastest, then column tile, then matrix
+  auto decode = [&](int t, int& mt, int& nt, int& b) {
+    mt = t % mtiles;
+    const int r = t / mtiles;
+    nt = r % ntiles;
+    b = r / ntiles;
+  };
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(oz_saddr(&tmem_s)), "r"(512)
                  : "memory");
@@ -362,27 +371,33 @@ template <typename T> __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_k
   const int nchunks = (ksteps + OZ_CHUNK - 1) / OZ_CHUNK;
 
   if (warp == OZ_EPI / 32) {
-    // copies: per k-step B (both planes), then the two planes of A
+    // copies: per k-step B (both planes), then the two planes of A; ring positions run on over the tiles
     if (lane == 0) {
-      const unsigned char* gA = q.A + ((size_t)b * (q.m_pad / OZ_BM) + mt) * ksteps * (2 * ABLK);
-      const unsigned char* gB = q.B + ((size_t)b * (q.n_pad / BN) + nt) * ksteps * OZ_BBLK;
       bool ok = true;
       int issuedA = 0, issuedB = 0;
-      for (int t = 0; t < ksteps && ok; ++t) {
-        const int sb = t % OZ_NB;
-        if (t >= OZ_NB) ok = oz_wait(oz_saddr(&emptyB[sb]), (uint32_t)((t / OZ_NB - 1) & 1));
-        if (!ok || s_abort) break;
-        oz_bulk(oz_saddr(sB + sb * OZ_BBLK), gB + (size_t)t * OZ_BBLK, OZ_BBLK, oz_saddr(&fullB[sb]));
-        issuedB = t + 1;
-        for (int h = 0; h < 2 && ok; ++h) {
-          const int a = 2 * t + h, sa = a % NA;
-          if (a >= NA) ok = oz_wait(oz_saddr(&emptyA[sa]), (uint32_t)((a / NA - 1) & 1));
-          if (!ok || s_abort) break;
-          oz_bulk(oz_saddr(sA + sa * ABLK), gA + (size_t)a * ABLK, ABLK, oz_saddr(&fullA[sa]));
-          issuedA = a + 1;
+      for (int tile = blockIdx.x; tile < q.tiles && ok; tile += gridDim.x) {
+        int mt, nt, b;
+        decode(tile, mt, nt, b);
+        const unsigned char* gA = q.A + ((size_t)b * mtiles + mt) * ksteps * (2 * ABLK);
+        const unsigned char* gB = q.B + ((size_t)b * ntiles + nt) * ksteps * OZ_BBLK;
+        for (int t = 0; t < ksteps && ok; ++t) {
+          const int sb = issuedB % OZ_NB;
+          if (issuedB >= OZ_NB) ok = oz_wait(oz_saddr(&emptyB[sb]), (uint32_t)((issuedB / OZ_NB - 1) & 1));
+          ok = ok && !s_abort;
+          if (!ok) break;
+          oz_bulk(oz_saddr(sB + sb * OZ_BBLK), gB + (size_t)t * OZ_BBLK, OZ_BBLK, oz_saddr(&fullB[sb]));
+          ++issuedB;
+          for (int h = 0; h < 2; ++h) {
+            const int sa = issuedA % NA;
+            if (issuedA >= NA) ok = oz_wait(oz_saddr(&emptyA[sa]), (uint32_t)((issuedA / NA - 1) & 1));
+            ok = ok && !s_abort;
+            if (!ok) break;
+            oz_bulk(oz_saddr(sA + sa * ABLK), gA + (size_t)(2 * t + h) * ABLK, ABLK, oz_saddr(&fullA[sa]));
+            ++issuedA;
+          }
         }
       }
-      if (!ok || s_abort) {
+      if (!ok) {
         // let the copies in flight land before the CTA's shared memory is released: per ring entry
         // the last one issued (earlier ones completed before the entry was refilled)
         s_abort = 1;
@@ -396,39 +411,46 @@ template <typename T> __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_k
   } else if (warp == OZ_EPI / 32 + 1) {
     if (lane == 0) {
       bool ok = true;
-      for (int t = 0; t < ksteps && ok; ++t) {
-        const int c = t / OZ_CHUNK;
-        const bool first = t % OZ_CHUNK == 0;
-        if (first && c > 0) {
-          ok = oz_wait(oz_saddr(&accEmpty), (uint32_t)((c - 1) & 1));
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        }
-        const int sb = t % OZ_NB;
-        ok = ok && oz_wait(oz_saddr(&fullB[sb]), (uint32_t)((t / OZ_NB) & 1));
-        const uint32_t b0 = oz_saddr(sB + sb * OZ_BBLK);
-        const uint64_t bre = oz_desc(b0, OZ_LBO_B), bim = oz_desc(b0 + OZ_BPLANE, OZ_LBO_B);
-        for (int h = 0; h < 2 && ok; ++h) {
-          const int a = 2 * t + h, sa = a % NA;
-          ok = oz_wait(oz_saddr(&fullA[sa]), (uint32_t)((a / NA) & 1));
-          if (!ok || s_abort) {
-            ok = false;
-            break;
+      int ia = 0, ib = 0, cc = 0;   // planes of A, blocks of B and chunks so far
+      for (int tile = blockIdx.x; tile < q.tiles && ok; tile += gridDim.x) {
+        for (int t = 0; t < ksteps && ok; ++t) {
+          const bool first = t % OZ_CHUNK == 0;
+          if (first && cc > 0) {   // the accumulators have been read
+            ok = oz_wait(oz_saddr(&accEmpty), (uint32_t)((cc - 1) & 1));
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           }
-          const uint32_t a0 = oz_saddr(sA + sa * ABLK);
-          // h = 0: Re += Ar Br, Im += Ar Bi;  h = 1: Re -= Ai Bi, Im += Ai Br
+          const int sb = ib % OZ_NB;
+          ok = ok && oz_wait(oz_saddr(&fullB[sb]), (uint32_t)((ib / OZ_NB) & 1));
+          const uint32_t b0 = oz_saddr(sB + sb * OZ_BBLK);
+          const uint64_t bre = oz_desc(b0, OZ_LBO_B), bim = oz_desc(b0 + OZ_BPLANE, OZ_LBO_B);
+          for (int h = 0; h < 2 && ok; ++h) {
+            const int sa = ia % NA;
+            ok = oz_wait(oz_saddr(&fullA[sa]), (uint32_t)((ia / NA) & 1));
+            if (!ok || s_abort) {
+              ok = false;
+              break;
+            }
+            const uint32_t a0 = oz_saddr(sA + sa * ABLK);
+            // h = 0: Re += Ar Br, Im += Ar Bi;  h = 1: Re -= Ai Bi, Im += Ai Br
 #pragma unroll
-          for (int i = 0; i < S; ++i) {
-            const uint64_t ad = oz_desc(a0 + i * (OZ_BM * OZ_KS * 2), OZ_LBO_A);
-            const uint32_t acc = (first && h == 0 && i == 0) ? 0u : 1u;
-            const int N = BN * (S - i);
-            oz_mma(tmem + i * BN, ad, h ? bim : bre, h ? oz_idesc(N, 1) : oz_idesc(N, 0), acc);
-            oz_mma(tmem + 256 + i * BN, ad, h ? bre : bim, oz_idesc(N, 0), acc);
+            for (int i = 0; i < S; ++i) {
+              const uint64_t ad = oz_desc(a0 + i * (OZ_BM * OZ_KS * 2), OZ_LBO_A);
+              const uint32_t acc = (first && h == 0 && i == 0) ? 0u : 1u;
+              const int N = BN * (S - i);
+              oz_mma(tmem + i * BN, ad, h ? bim : bre, h ? oz_idesc(N, 1) : oz_idesc(N, 0), acc);
+              oz_mma(tmem + 256 + i * BN, ad, h ? bre : bim, oz_idesc(N, 0), acc);
+            }
+            oz_commit(oz_saddr(&emptyA[sa]));
+            ++ia;
           }
-          oz_commit(oz_saddr(&emptyA[sa]));
+          if (!ok) break;
+          oz_commit(oz_saddr(&emptyB[sb]));
+          ++ib;
+          if (t % OZ_CHUNK == OZ_CHUNK - 1 || t == ksteps - 1) {
+            oz_commit(oz_saddr(&accFull));
+            ++cc;
+          }
         }
-        if (!ok) break;
-        oz_commit(oz_saddr(&emptyB[sb]));
-        if (t % OZ_CHUNK == OZ_CHUNK - 1 || t == ksteps - 1) oz_commit(oz_saddr(&accFull));
       }
       if (!ok) {
         // the MMAs issued so far end before the tensor memory is given back
@@ -442,6 +464,10 @@ template <typename T> __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_k
     // epilogue threads: row 32 (warp % 4) + lane, columns EC (warp / 4) ... of Re and of Im
     const int ch = (warp >> 2) * EC;
     const uint32_t tl = tmem + ((uint32_t)((warp & 3) * 32) << 16) + ch;
+    bool ok = true;
+    int cc = 0;   // chunks so far
+    // the sums of a tile are written while the next tile's MMAs run: they only wait for the accumulators to be read
+    for (int tile = blockIdx.x; tile < q.tiles && ok; tile += gridDim.x) {
     long long sum[2][SW][EC];
 #pragma unroll
     for (int p = 0; p < 2; ++p)
@@ -449,9 +475,8 @@ template <typename T> __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_k
       for (int w = 0; w < SW; ++w)
 #pragma unroll
         for (int j = 0; j < EC; ++j) sum[p][w][j] = 0;
-    bool ok = true;
-    for (int c = 0; c < nchunks; ++c) {
-      ok = oz_wait(oz_saddr(&accFull), (uint32_t)(c & 1));
+    for (int c = 0; c < nchunks; ++c, ++cc) {
+      ok = oz_wait(oz_saddr(&accFull), (uint32_t)(cc & 1));
       if (!ok || s_abort) {
         ok = false;
         break;
@@ -486,10 +511,8 @@ template <typename T> __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_k
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(oz_saddr(&accEmpty)) : "memory");
     }
-    if (!ok) {
-      s_abort = 1;
-      atomicExch(q.err, 1);
-    }
+    int mt, nt, b;
+    decode(tile, mt, nt, b);
     const int row = mt * OZ_BM + (warp & 3) * 32 + lane;
     if (ok && row < q.m) {
       const unsigned int wa = q.exA[(size_t)b * q.m_pad + row];
@@ -523,6 +546,11 @@ template <typename T> __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_k
         }
       }
     }
+    }
+    if (!ok) {
+      s_abort = 1;
+      atomicExch(q.err, 1);
+    }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   }
   __syncthreads();
@@ -546,6 +574,8 @@ cudaError_t oz_gemm_t(cudaStream_t st, int batch, int m, int n, int k, int sign,
   int nb = (int)(work_bytes / per < (size_t)batch ? work_bytes / per : (size_t)batch);
   if (nb < 1) return cudaErrorInvalidValue;
   if (nb > 32767) nb = 32767;   // gridDim.z carries (matrix, operand)
+  int dev = 0, sms = 152;
+  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int mp = (int)up(m, OZ_BM), np = (int)up(n, BN), ks = (k + OZ_KS - 1) / OZ_KS;
   cudaError_t e = cudaFuncSetAttribute(oz_gemm_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, oz_smem<T>());
   if (e != cudaSuccess) return e;
@@ -566,8 +596,10 @@ cudaError_t oz_gemm_t(cudaStream_t st, int batch, int m, int n, int k, int sign,
     const int rows = m > n ? m : n, rpad = mp > np ? mp : np;
     oz_rowmax<T><<<dim3((rows + 31) / 32, (k + 63) / 64, 2 * bn), 256, 0, st>>>(q);
     oz_digits<T><<<dim3((rpad + 31) / 32, (2 * ks + 7) / 8, 2 * bn), 256, 0, st>>>(q);
-    OzGemm<T> g{dA, dB, xA, xB, m, n, mp, np, ks, sign, add, C + b0 * sC, ldc, sC, err};
-    oz_gemm_kernel<T><<<dim3(mp / OZ_BM, np / BN, bn), OZ_THREADS, oz_smem<T>(), st>>>(g);
+    const long long tiles = (long long)(mp / OZ_BM) * (np / BN) * bn;
+    if (tiles > 0x7fffffffll) return cudaErrorInvalidValue;
+    OzGemm<T> g{dA, dB, xA, xB, m, n, mp, np, ks, (int)tiles, sign, add, C + b0 * sC, ldc, sC, err};
+    oz_gemm_kernel<T><<<(int)(tiles < sms ? tiles : sms), OZ_THREADS, oz_smem<T>(), st>>>(g);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
