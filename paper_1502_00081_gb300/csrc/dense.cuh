@@ -21,6 +21,10 @@ struct Gemm {
 // C[b] = sign * op(A[b]) B[b] + (add ? C[b] : 0); op = N or conjugate transpose (opA = 1)
 void gemm(Gemm& g, int batch, int m, int n, int k, double sign, const double2* A, int lda, long long sA, int opA,
           const double2* B, int ldb, long long sB, bool add, double2* C, int ldc, long long sC);
+// the same on the tensor cores, C may be B; false (nothing done) where gemm() would not slice
+bool gemm_sliced(Gemm& g, int batch, int m, int n, int k, double sign, const double2* A, int lda, long long sA, int opA,
+                 const double2* B, int ldb, long long sB, bool add, double2* C, int ldc, long long sC);
+constexpr double kSliceMin = 8e6;   // complex multiply-adds of an FP64 product from which it is sliced
 void gemm(Gemm& g, int batch, int m, int n, int k, double sign, const float2* A, int lda, long long sA, int opA,
           const float2* B, int ldb, long long sB, bool add, float2* C, int ldc, long long sC);
 
@@ -31,8 +35,11 @@ int lu_swap_ints(int nb);       // scratch per matrix of lu_factor, ints
 // info [K] (zeroed by the caller): first column without a usable pivot, 1-based; swp [K][lu_swap_ints(nb)] scratch.
 void lu_factor(Gemm& g, double2* M, int nb, int K, int* perm, int* info, int* swp);
 void lu_factor(Gemm& g, float2* M, int nb, int K, int* perm, int* info, int* swp);
+// inverses of the factors' diagonal blocks for lu_solve with nrhs columns (handle workspace 10, valid until the next
+// call), or null where substitution is as fast
+const double2* lu_inverses(Gemm& g, const double2* LU, int nb, int K, int nrhs);
 // X[b] = U^{-1} L^{-1} X[b] for nrhs columns of nb rows (batch stride nb nrhs), rows already permuted
-void lu_solve(Gemm& g, const double2* LU, int nb, int K, double2* X, int nrhs);
+void lu_solve(Gemm& g, const double2* LU, int nb, int K, double2* X, int nrhs, const double2* dinv);
 void lu_solve(Gemm& g, const float2* LU, int nb, int K, float2* X, int nrhs);
 // X[b][:, c][i] = B[b][:, c][perm[b][i]], with conversion where the types differ; X may be B (same type)
 void lu_permute(Gemm& g, const double2* B, int nb, int K, const int* perm, double2* X, int nrhs);

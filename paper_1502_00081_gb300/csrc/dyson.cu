@@ -118,15 +118,19 @@ template <typename T> void* oz_work(Gemm& g, int batch, int m, int n, int k, siz
 // (1.3e11 complex multiply-adds/s) earns back from there.  Two products of ns x ns x ns and the rest of
 // rsfd_transmission, CUDA cores / sliced, us: ns = 64, 16 energies (4.2e6) 143 / 154; 192, 1 (7.1e6) 251 / 266;
 // 128, 4 (8.4e6) 242 / 208; 96, 16 (1.4e7) 291 / 190; 256, 16 (2.7e8) 3869 / 600.
-void gemm(Gemm& g, int batch, int m, int n, int k, double sign, const double2* A, int lda, long long sA, int opA,
-          const double2* B, int ldb, long long sB, bool add, double2* C, int ldc, long long sC) {
+bool gemm_sliced(Gemm& g, int batch, int m, int n, int k, double sign, const double2* A, int lda, long long sA, int opA,
+                 const double2* B, int ldb, long long sB, bool add, double2* C, int ldc, long long sC) {
   size_t wb = 0;
-  void* w = g.h && k >= 32 && m >= 32 && n >= 16 && (double)m * n * k * batch >= 8e6
+  void* w = g.h && k >= 32 && m >= 32 && n >= 16 && (double)m * n * k * batch >= kSliceMin
                 ? oz_work<double2>(g, batch, m, n, k, wb)
                 : nullptr;
-  if (w)
-    g.note(oz_gemm(g.st, batch, m, n, k, sign < 0 ? -1 : 1, A, lda, sA, opA, B, ldb, sB, add ? 1 : 0, C, ldc, sC, w, wb, g.err));
-  else
+  if (!w) return false;
+  g.note(oz_gemm(g.st, batch, m, n, k, sign < 0 ? -1 : 1, A, lda, sA, opA, B, ldb, sB, add ? 1 : 0, C, ldc, sC, w, wb, g.err));
+  return true;
+}
+void gemm(Gemm& g, int batch, int m, int n, int k, double sign, const double2* A, int lda, long long sA, int opA,
+          const double2* B, int ldb, long long sB, bool add, double2* C, int ldc, long long sC) {
+  if (!gemm_sliced(g, batch, m, n, k, sign, A, lda, sA, opA, B, ldb, sB, add, C, ldc, sC))
     zgemm(g.st, batch, m, n, k, make_double2(sign, 0.0), A, lda, sA, opA, B, ldb, sB, make_double2(add ? 1.0 : 0.0, 0.0),
           C, ldc, sC);
 }
@@ -161,7 +165,6 @@ __global__ void copy_c128(const double2* src, double2* dst, long long n) {
 }
 __device__ __forceinline__ void cvt(double2 a, double2& b) { b = a; }
 __device__ __forceinline__ void cvt(double2 a, float2& b) { b = make_float2((float)a.x, (float)a.y); }
-__device__ __forceinline__ void cvt(float2 a, double2& b) { b = make_double2((double)a.x, (double)a.y); }
 // dst[b ds + i] = src[b ss + i] for i < n, b < batch (a block of leading columns of each energy's
 // matrix, with a type conversion where the types differ)
 template <typename S, typename D>
@@ -470,6 +473,7 @@ rsfd_status dyson_run(Handle* h, const void* G0, const void* SL, const void* SR,
   copy_c128<<<grid_for(tot), 256, 0, st>>>(dM, dLU, tot);
   DY_CK(h, cudaMemsetAsync(info, 0, K * sizeof(int), st));
   lu_factor(gc, dLU, nb, K, perm, info, swp);
+  const double2* dinv = lu_inverses(gc, dLU, nb, K, nc);
   // right-hand sides: the first nc columns of every energy, compact (stride sx)
   const double2* b0 = dG0;
   if (nc < nb) {
@@ -479,13 +483,13 @@ rsfd_status dyson_run(Handle* h, const void* G0, const void* SL, const void* SR,
     b0 = (const double2*)pB;
   }
   lu_permute(gc, b0, nb, K, perm, dX, nc);
-  lu_solve(gc, dLU, nb, K, dX, nc);
+  lu_solve(gc, dLU, nb, K, dX, nc, dinv);
   // iterative refinement in FP64
   for (int it = 0; it < 2; ++it) {
     copy_c128<<<grid_for(totx), 256, 0, st>>>(b0, dR, totx);
     gemm(gc, K, nb, nc, nb, -1.0, dM, nb, n2, 0, dX, nb, sx, true, dR, nb, sx);
     lu_permute(gc, dR, nb, K, perm, dR, nc);
-    lu_solve(gc, dLU, nb, K, dR, nc);
+    lu_solve(gc, dLU, nb, K, dR, nc, dinv);
     axpy_c128<<<grid_for(totx), 256, 0, st>>>(dX, dR, totx);
   }
   if (refres) {
@@ -563,13 +567,14 @@ rsfd_status dyson_tracked_run(Handle* h, int nr, const void* G0, const void* SL,
   lu_factor(gc, dLU, nb, K, perm, info, swp);
   // Y = M^{-1} G0[b, :] with two FP64 refinement steps
   copy_rows_c128<<<grid_for(ntot), 256, 0, st>>>(dG0, nr, dRHS, nb, nb, nr, K);
+  const double2* dinv = lu_inverses(gc, dLU, nb, K, nr);
   lu_permute(gc, dRHS, nb, K, perm, dY, nr);
-  lu_solve(gc, dLU, nb, K, dY, nr);
+  lu_solve(gc, dLU, nb, K, dY, nr, dinv);
   for (int it = 0; it < 2; ++it) {
     copy_c128<<<grid_for(ntot), 256, 0, st>>>(dRHS, dR, ntot);
     gemm(gc, K, nb, nr, nb, -1.0, dM, nb, b2, 0, dY, nb, bn, true, dR, nb, bn);
     lu_permute(gc, dR, nb, K, perm, dR, nr);
-    lu_solve(gc, dLU, nb, K, dR, nr);
+    lu_solve(gc, dLU, nb, K, dR, nr, dinv);
     axpy_c128<<<grid_for(ntot), 256, 0, st>>>(dY, dR, ntot);
   }
   if (refres) {
@@ -611,32 +616,15 @@ rsfd_status dyson_tracked_run(Handle* h, int nr, const void* G0, const void* SL,
 // until max |alpha|, |beta| fall below 1e-15 max |H01| for every energy; then g_s = (Z - eps_s)^{-1} and
 // Sigma_R = H01 g_s H01^T, Sigma_L = H01^T g_s H01.
 // ------------------------------------------------------------------------------------------------
-__global__ void zi_minus(double2* A, const double2* E, const double2* Z, int n, int batch) {
+__global__ void zi_minus(double2* A, const double2* E, const double2* Z, int n, int batch, int nz) {
   const long long n2 = (long long)n * n;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n2 * batch;
        t += (long long)gridDim.x * blockDim.x) {
     const long long b = t / n2, e = t - b * n2;
     const long long c = e / n, r = e - c * n;
-    const double2 v = E[t];
-    A[t] = r == c ? make_double2(Z[b].x - v.x, Z[b].y - v.y) : make_double2(-v.x, -v.y);
+    const double2 v = E[t], z = Z[b % nz];
+    A[t] = r == c ? make_double2(z.x - v.x, z.y - v.y) : make_double2(-v.x, -v.y);
   }
-}
-// out[b] = max |re| + |im| over n2 entries of X[b] and of Y[b]
-__global__ void maxabs2_batched(const double2* X, const double2* Y, long long n2, double* out) {
-  const int b = blockIdx.x;
-  double m = 0.0;
-  for (long long i = threadIdx.x; i < n2; i += blockDim.x) {
-    const double2 x = X[(long long)b * n2 + i], y = Y[(long long)b * n2 + i];
-    m = fmax(m, fmax(fabs(x.x) + fabs(x.y), fabs(y.x) + fabs(y.y)));
-  }
-  __shared__ double red[256];
-  red[threadIdx.x] = m;
-  __syncthreads();
-  for (int k = blockDim.x / 2; k > 0; k >>= 1) {
-    if (threadIdx.x < k) red[threadIdx.x] = fmax(red[threadIdx.x], red[threadIdx.x + k]);
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) out[b] = red[0];
 }
 // dst[b] = src (one n x n matrix broadcast to the batch)
 __global__ void bcast_c128(const double2* src, double2* dst, long long n2, int batch) {
@@ -644,13 +632,44 @@ __global__ void bcast_c128(const double2* src, double2* dst, long long n2, int b
        t += (long long)gridDim.x * blockDim.x)
     dst[t] = src[t % n2];
 }
-// rhs[b] = [X[b] | Y[b]]  (n x 2n, column-major)
-__global__ void concat_cols(const double2* X, const double2* Y, double2* rhs, long long n2, int batch) {
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < 2 * n2 * batch;
-       t += (long long)gridDim.x * blockDim.x) {
-    const long long b = t / (2 * n2), e = t - b * 2 * n2;
-    rhs[t] = e < n2 ? X[b * n2 + e] : Y[b * n2 + e - n2];
+// One step of the iteration around its product P = [alpha; beta] [g alpha, g beta] (2n x 2n; FIRST: alpha and beta are
+// given in rhs and there is no product yet):
+//   eps_s += alpha g beta;  eps += alpha g beta + beta g alpha;  alpha = alpha g alpha;  beta = beta g beta,
+// the next system's A = Z - eps, its right-hand sides rhs = [alpha | beta], the stacked left factor ab = [alpha; beta], and
+// the largest |re| + |im| of the new alpha and beta per matrix in mx (bits of a non-negative double; zero before).
+template <bool FIRST>
+__global__ void __launch_bounds__(256) decimation_step(const double2* P, double2* eps_s, double2* eps, double2* ab, double2* rhs,
+                                                       double2* A, const double2* Z, int n, int nz, unsigned long long* mx) {
+  const long long n2 = (long long)n * n;
+  const int b = blockIdx.y;
+  const double2 z = Z[b % nz];
+  const double2* p = P + b * 4 * n2;
+  double m = 0.0;
+  for (long long e = blockIdx.x * 256ll + threadIdx.x; e < n2; e += gridDim.x * 256ll) {
+    const int c = (int)(e / n), r = (int)(e - (long long)c * n);
+    double2 al, be, ev = eps[b * n2 + e];
+    if (FIRST) {
+      al = rhs[b * 2 * n2 + e];
+      be = rhs[b * 2 * n2 + n2 + e];
+    } else {
+      const double2* pc = p + (long long)c * 2 * n;
+      const double2* pd = p + (long long)(c + n) * 2 * n;
+      al = pc[r];
+      be = pd[n + r];
+      const double2 agb = pd[r], bga = pc[n + r];
+      eps_s[b * n2 + e] = cadd(eps_s[b * n2 + e], agb);
+      ev = cadd(cadd(ev, agb), bga);
+      eps[b * n2 + e] = ev;
+      rhs[b * 2 * n2 + e] = al;
+      rhs[b * 2 * n2 + n2 + e] = be;
+    }
+    ab[b * 2 * n2 + (long long)c * 2 * n + r] = al;
+    ab[b * 2 * n2 + (long long)c * 2 * n + n + r] = be;
+    A[b * n2 + e] = r == c ? make_double2(z.x - ev.x, z.y - ev.y) : make_double2(-ev.x, -ev.y);
+    m = fmax(m, fmax(fabs(al.x) + fabs(al.y), fabs(be.x) + fabs(be.y)));   // NaN is passed over
   }
+  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0) atomicMax(mx + b, (unsigned long long)__double_as_longlong(m));
 }
 
 static void layer_blocks(int nx, int ny, double hh, int fd_order, const double* V, std::vector<double2>& H00,
@@ -695,103 +714,99 @@ rsfd_status lead_decimation_run(Handle* h, const double* VL, const double* VR, c
   std::vector<double2> H01T((size_t)n2);
   for (int r = 0; r < n; ++r)
     for (int c = 0; c < n; ++c) H01T[(size_t)c * n + r] = H01[(size_t)r * n + c];
-  // per energy: eps_s, eps, alpha, beta, A (LU), Y (n x 2n), rhs (n x 2n), 2 products
-  const long long per = n2 * 11 * (long long)sizeof(double2) + (n + 1 + lu_swap_ints(n)) * (long long)sizeof(int) + 64;
+  // per matrix (an energy has two, the right and the left lead's): eps_s, eps, [alpha; beta], A (LU), Y and rhs (n x 2n),
+  // P (2n x 2n)
+  const long long per = 2 * (n2 * 13 * (long long)sizeof(double2) + (n + 1 + lu_swap_ints(n)) * (long long)sizeof(int) + 64);
   size_t free_b = 0, tot_b = 0;
   DY_CK(h, cudaMemGetInfo(&free_b, &tot_b));
   long long kc = (long long)(0.5 * (double)free_b) / per;
   if (kc > K) kc = K;
+  if (kc > 32767) kc = 32767;
   if (kc < 1) kc = 1;
-  const int Kc = (int)kc;
+  const int Kc = (int)kc, Bc = 2 * Kc;
   rsfd_status s;
   void *pW, *pC, *pPiv, *pZ;
-  if ((s = handle_ensure(h, 1, (size_t)n2 * 11 * Kc * sizeof(double2), &pW)) != RSFD_OK) return s;
-  if ((s = handle_ensure(h, 2, (size_t)n2 * 3 * sizeof(double2), &pC)) != RSFD_OK) return s;
-  if ((s = handle_ensure(h, 5, (size_t)Kc * (n + 1 + lu_swap_ints(n)) * sizeof(int), &pPiv)) != RSFD_OK) return s;
-  if ((s = handle_ensure(h, 6, (size_t)Kc * (sizeof(double2) + sizeof(double)), &pZ)) != RSFD_OK) return s;
+  if ((s = handle_ensure(h, 1, (size_t)n2 * 13 * Bc * sizeof(double2), &pW)) != RSFD_OK) return s;
+  if ((s = handle_ensure(h, 2, (size_t)n2 * 4 * sizeof(double2), &pC)) != RSFD_OK) return s;
+  if ((s = handle_ensure(h, 5, (size_t)Bc * (n + 1 + lu_swap_ints(n)) * sizeof(int), &pPiv)) != RSFD_OK) return s;
+  if ((s = handle_ensure(h, 6, (size_t)Kc * sizeof(double2) + (size_t)Bc * sizeof(unsigned long long), &pZ)) != RSFD_OK) return s;
   if ((s = handle_begin(h)) != RSFD_OK) return s;
   cudaStream_t st = handle_stream(h);
   Gemm gc;
   if ((s = gemm_begin(h, gc)) != RSFD_OK) return s;
   double2* W = (double2*)pW;
-  double2 *eps_s = W, *eps = W + n2 * Kc, *al = W + 2 * n2 * Kc, *be = W + 3 * n2 * Kc, *A = W + 4 * n2 * Kc;
-  double2 *Y = W + 5 * n2 * Kc, *rhs = W + 7 * n2 * Kc, *P1 = W + 9 * n2 * Kc, *P2 = W + 10 * n2 * Kc;
-  double2 *dH00 = (double2*)pC, *dH01 = dH00 + n2, *dH01T = dH00 + 2 * n2;
+  double2 *eps_s = W, *eps = W + n2 * Bc, *ab = W + 2 * n2 * Bc, *A = W + 4 * n2 * Bc;
+  double2 *Y = W + 5 * n2 * Bc, *rhs = W + 7 * n2 * Bc, *P = W + 9 * n2 * Bc;
+  double2 *dH00R = (double2*)pC, *dH00L = dH00R + n2, *dH01 = dH00R + 2 * n2, *dH01T = dH00R + 3 * n2;
   int* perm = (int*)pPiv;
-  int* info = perm + (long long)Kc * n;
-  int* swp = info + Kc;
+  int* info = perm + (long long)Bc * n;
+  int* swp = info + Bc;
   double2* dZ = (double2*)pZ;
-  double* dmax = (double*)(dZ + Kc);
+  unsigned long long* dmax = (unsigned long long*)(dZ + Kc);
+  DY_CK(h, cudaMemcpyAsync(dH00R, H00R.data(), n2 * sizeof(double2), cudaMemcpyHostToDevice, st));
+  DY_CK(h, cudaMemcpyAsync(dH00L, H00L.data(), n2 * sizeof(double2), cudaMemcpyHostToDevice, st));
   DY_CK(h, cudaMemcpyAsync(dH01, H01.data(), n2 * sizeof(double2), cudaMemcpyHostToDevice, st));
   DY_CK(h, cudaMemcpyAsync(dH01T, H01T.data(), n2 * sizeof(double2), cudaMemcpyHostToDevice, st));
   int it_max = 0;
-  for (int lead = 0; lead < 2; ++lead) {
-    const std::vector<double2>& H00 = lead == 0 ? H00R : H00L;
-    double2* out = (double2*)(lead == 0 ? SRo : SLo);
-    const double2* a0 = lead == 0 ? dH01 : dH01T;
-    const double2* b0 = lead == 0 ? dH01T : dH01;
-    DY_CK(h, cudaMemcpyAsync(dH00, H00.data(), n2 * sizeof(double2), cudaMemcpyHostToDevice, st));
-    for (int k0 = 0; k0 < K; k0 += Kc) {
-      const int kb = K - k0 < Kc ? K - k0 : Kc;
-      const long long tot = n2 * kb;
-      std::vector<double2> Zh(kb);
-      for (int k = 0; k < kb; ++k) Zh[k] = make_double2(E[k0 + k], eta);
-      DY_CK(h, cudaMemcpyAsync(dZ, Zh.data(), kb * sizeof(double2), cudaMemcpyHostToDevice, st));
-      bcast_c128<<<grid_for(tot), 256, 0, st>>>(dH00, eps_s, n2, kb);
-      bcast_c128<<<grid_for(tot), 256, 0, st>>>(dH00, eps, n2, kb);
-      bcast_c128<<<grid_for(tot), 256, 0, st>>>(a0, al, n2, kb);
-      bcast_c128<<<grid_for(tot), 256, 0, st>>>(b0, be, n2, kb);
-      int it = 0;
-      for (; it < maxit; ++it) {
-        maxabs2_batched<<<kb, 256, 0, st>>>(al, be, n2, dmax);
-        std::vector<double> hm(kb);
-        DY_CK(h, cudaMemcpyAsync(hm.data(), dmax, kb * sizeof(double), cudaMemcpyDeviceToHost, st));
-        DY_CK(h, cudaStreamSynchronize(st));
-        bool done = true;
-        for (int k = 0; k < kb; ++k) done &= hm[k] < tol;
-        if (done) break;
-        // g [alpha | beta] by LU of Z - eps
-        zi_minus<<<grid_for(tot), 256, 0, st>>>(A, eps, dZ, n, kb);
-        DY_CK(h, cudaMemsetAsync(info, 0, kb * sizeof(int), st));
-        lu_factor(gc, A, n, kb, perm, info, swp);
-        concat_cols<<<grid_for(2 * tot), 256, 0, st>>>(al, be, rhs, n2, kb);
-        lu_permute(gc, rhs, n, kb, perm, Y, 2 * n);
-        lu_solve(gc, A, n, kb, Y, 2 * n);
-        const double2* ga = Y;        // g alpha, per energy stride 2 n2
-        const double2* gb = Y + n2;   // g beta
-        // P1 = alpha g beta, P2 = beta g alpha
-        gemm(gc, kb, n, n, n, 1.0, al, n, n2, 0, gb, n, 2 * n2, false, P1, n, n2);
-        gemm(gc, kb, n, n, n, 1.0, be, n, n2, 0, ga, n, 2 * n2, false, P2, n, n2);
-        axpy_c128<<<grid_for(tot), 256, 0, st>>>(eps_s, P1, tot);
-        axpy_c128<<<grid_for(tot), 256, 0, st>>>(eps, P1, tot);
-        axpy_c128<<<grid_for(tot), 256, 0, st>>>(eps, P2, tot);
-        // alpha <- alpha g alpha, beta <- beta g beta (through the product buffers)
-        gemm(gc, kb, n, n, n, 1.0, al, n, n2, 0, ga, n, 2 * n2, false, P1, n, n2);
-        gemm(gc, kb, n, n, n, 1.0, be, n, n2, 0, gb, n, 2 * n2, false, P2, n, n2);
-        copy_c128<<<grid_for(tot), 256, 0, st>>>(P1, al, tot);
-        copy_c128<<<grid_for(tot), 256, 0, st>>>(P2, be, tot);
-      }
-      it_max = it > it_max ? it : it_max;
-      // Sigma = b0 g_s a0 with g_s = (Z - eps_s)^{-1}:  X = g_s a0, Sigma = b0 X
-      //   right lead: b0 = H01, a0 = H01^T... the coupling into the lead and back out:
-      //   Sigma_R = H01 g_s H01^T, Sigma_L = H01^T g_s H01
-      zi_minus<<<grid_for(tot), 256, 0, st>>>(A, eps_s, dZ, n, kb);
-      DY_CK(h, cudaMemsetAsync(info, 0, kb * sizeof(int), st));
-      lu_factor(gc, A, n, kb, perm, info, swp);
-      bcast_c128<<<grid_for(tot), 256, 0, st>>>(lead == 0 ? dH01T : dH01, rhs, n2, kb);
-      lu_permute(gc, rhs, n, kb, perm, Y, n);
-      lu_solve(gc, A, n, kb, Y, n);
-      gemm(gc, kb, n, n, n, 1.0, lead == 0 ? dH01 : dH01T, n, 0, 0, Y, n, n2, false, out + n2 * k0, n, n2);
-      std::vector<int> hinfo(kb);
-      DY_CK(h, cudaMemcpyAsync(hinfo.data(), info, kb * sizeof(int), cudaMemcpyDeviceToHost, st));
-      if ((s = gemm_end(gc, "rsfd_lead_sigma_decimation")) != RSFD_OK) return s;
-      for (int k = 0; k < kb; ++k)
-        if (hinfo[k] != 0)
-          return handle_fail(h, RSFD_ERR_BREAKDOWN, "rsfd_lead_sigma_decimation: singular Z - eps at energy " +
-                                                        std::to_string(k0 + k));
-      if (it >= maxit)
-        return handle_fail(h, RSFD_ERR_NOT_CONVERGED, "rsfd_lead_sigma_decimation: no convergence in maxit steps");
+  for (int k0 = 0; k0 < K; k0 += Kc) {
+    const int kb = K - k0 < Kc ? K - k0 : Kc, nm = 2 * kb;   // matrices 0 .. kb - 1: right leads, kb .. 2 kb - 1: left leads
+    const long long tot = n2 * kb;
+    std::vector<double2> Zh(kb);
+    for (int k = 0; k < kb; ++k) Zh[k] = make_double2(E[k0 + k], eta);
+    DY_CK(h, cudaMemcpyAsync(dZ, Zh.data(), kb * sizeof(double2), cudaMemcpyHostToDevice, st));
+    for (int lead = 0; lead < 2; ++lead) {
+      const double2* h0 = lead == 0 ? dH00R : dH00L;
+      bcast_c128<<<grid_for(tot), 256, 0, st>>>(h0, eps_s + lead * tot, n2, kb);
+      bcast_c128<<<grid_for(tot), 256, 0, st>>>(h0, eps + lead * tot, n2, kb);
     }
+    // rhs = [alpha_0 | beta_0]: right [H01 | H01^T], left [H01^T | H01]
+    for (int k = 0; k < nm; ++k) {
+      const double2 *a0 = k < kb ? dH01 : dH01T, *b0 = k < kb ? dH01T : dH01;
+      DY_CK(h, cudaMemcpyAsync(rhs + k * 2 * n2, a0, n2 * sizeof(double2), cudaMemcpyDeviceToDevice, st));
+      DY_CK(h, cudaMemcpyAsync(rhs + k * 2 * n2 + n2, b0, n2 * sizeof(double2), cudaMemcpyDeviceToDevice, st));
+    }
+    const dim3 gs((unsigned)((n2 + 511) / 512 < 64 ? (n2 + 511) / 512 : 64), nm);
+    DY_CK(h, cudaMemsetAsync(dmax, 0, nm * sizeof(unsigned long long), st));
+    decimation_step<true><<<gs, 256, 0, st>>>(nullptr, eps_s, eps, ab, rhs, A, dZ, n, kb, dmax);
+    int it = 0;
+    for (; it < maxit; ++it) {
+      std::vector<double> hm(nm);
+      DY_CK(h, cudaMemcpyAsync(hm.data(), dmax, nm * sizeof(double), cudaMemcpyDeviceToHost, st));
+      DY_CK(h, cudaStreamSynchronize(st));
+      bool done = true;
+      for (int k = 0; k < nm; ++k) done &= hm[k] < tol;
+      if (done) break;
+      // Y = g [alpha | beta] by LU of Z - eps, then P = [alpha; beta] Y
+      DY_CK(h, cudaMemsetAsync(info, 0, nm * sizeof(int), st));
+      lu_factor(gc, A, n, nm, perm, info, swp);
+      const double2* dinv = lu_inverses(gc, A, n, nm, 2 * n);
+      lu_permute(gc, rhs, n, nm, perm, Y, 2 * n);
+      lu_solve(gc, A, n, nm, Y, 2 * n, dinv);
+      gemm(gc, nm, 2 * n, 2 * n, n, 1.0, ab, 2 * n, 2 * n2, 0, Y, n, 2 * n2, false, P, 2 * n, 4 * n2);
+      DY_CK(h, cudaMemsetAsync(dmax, 0, nm * sizeof(unsigned long long), st));
+      decimation_step<false><<<gs, 256, 0, st>>>(P, eps_s, eps, ab, rhs, A, dZ, n, kb, dmax);
+    }
+    it_max = it > it_max ? it : it_max;
+    // g_s = (Z - eps_s)^{-1}:  Sigma_R = H01 g_s H01^T, Sigma_L = H01^T g_s H01
+    zi_minus<<<grid_for(2 * tot), 256, 0, st>>>(A, eps_s, dZ, n, nm, kb);
+    DY_CK(h, cudaMemsetAsync(info, 0, nm * sizeof(int), st));
+    lu_factor(gc, A, n, nm, perm, info, swp);
+    bcast_c128<<<grid_for(tot), 256, 0, st>>>(dH01T, rhs, n2, kb);
+    bcast_c128<<<grid_for(tot), 256, 0, st>>>(dH01, rhs + tot, n2, kb);
+    const double2* dinv = lu_inverses(gc, A, n, nm, n);
+    lu_permute(gc, rhs, n, nm, perm, Y, n);
+    lu_solve(gc, A, n, nm, Y, n, dinv);
+    gemm(gc, kb, n, n, n, 1.0, dH01, n, 0, 0, Y, n, n2, false, (double2*)SRo + n2 * k0, n, n2);
+    gemm(gc, kb, n, n, n, 1.0, dH01T, n, 0, 0, Y + tot, n, n2, false, (double2*)SLo + n2 * k0, n, n2);
+    std::vector<int> hinfo(nm);
+    DY_CK(h, cudaMemcpyAsync(hinfo.data(), info, nm * sizeof(int), cudaMemcpyDeviceToHost, st));
+    if ((s = gemm_end(gc, "rsfd_lead_sigma_decimation")) != RSFD_OK) return s;
+    for (int k = 0; k < nm; ++k)
+      if (hinfo[k] != 0)
+        return handle_fail(h, RSFD_ERR_BREAKDOWN, "rsfd_lead_sigma_decimation: singular Z - eps at energy " +
+                                                      std::to_string(k0 + k % kb));
+    if (it >= maxit)
+      return handle_fail(h, RSFD_ERR_NOT_CONVERGED, "rsfd_lead_sigma_decimation: no convergence in maxit steps");
   }
   DY_CK(h, cudaGetLastError());
   if ((s = handle_end(h)) != RSFD_OK) return s;
@@ -944,12 +959,12 @@ rsfd_status dyson_noalloc_run(int32_t nb, int32_t K, const void* G0_bb, const vo
   copy_c128<<<grid_for(tot), 256, 0, st>>>(dM, dLU, tot);
   lu_factor(gc, dLU, nb, K, perm, info, swp);
   lu_permute(gc, G0, nb, K, perm, dX, nb);
-  lu_solve(gc, dLU, nb, K, dX, nb);
+  lu_solve(gc, dLU, nb, K, dX, nb, nullptr);
   for (int it = 0; it < 2; ++it) {
     copy_c128<<<grid_for(tot), 256, 0, st>>>(G0, dR, tot);
     gemm(gc, K, nb, nb, nb, -1.0, dM, nb, n2, 0, dX, nb, n2, true, dR, nb, n2);
     lu_permute(gc, dR, nb, K, perm, dR, nb);
-    lu_solve(gc, dLU, nb, K, dR, nb);
+    lu_solve(gc, dLU, nb, K, dR, nb, nullptr);
     axpy_c128<<<grid_for(tot), 256, 0, st>>>(dX, dR, tot);
   }
   copy_c128<<<grid_for(tot), 256, 0, st>>>(G0, dR, tot);

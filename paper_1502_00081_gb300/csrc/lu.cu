@@ -1,8 +1,8 @@
 // Batched LU with partial pivoting and triangular solves in FP32 and FP64 complex arithmetic, for the
 // boundary solve (I - G0 Sigma) G = G0 (Eq. sec3-01a) and the lead decimation.
 //
-// Right-looking, two levels.  Outer blocks of 128 columns end in one tensor-core product
-// A22 -= L21 U12 (k = 128).  Inside an outer block, panels of W columns take three launches:
+// Right-looking, two levels.  Outer blocks of 128 (FP32) or 64 (FP64) columns end in one tensor-core product
+// A22 -= L21 U12; FP64 takes the narrower block because the updates inside it run on the FP64 pipe.  Inside an outer block, panels of W columns take three launches:
 //   lu_panel   factorises rows x W: every row of the panel lives in one thread's registers, the rows are
 //              spread over up to 8 CTAs of a cluster, and a column costs one block and one cluster barrier
 //              (the pivot candidates, the pivot row and the row it replaces travel through
@@ -13,10 +13,12 @@
 // The exchanges then reach the other columns (lu_swap_rest), and U12 = L11^{-1} A12 is a triangular solve.
 // Triangular solves: blocks of 64 (FP64) or 128 (FP32) rows by substitution (lu_trsm), the rest by products.
 //
-// Measured (16 matrices of 1024 rows, FP32): panel_getrf + laswp + trsm + 3xTF32 updates 48 ms before, 14 ms now; 4 of
-// 2048: 123 -> 21 ms; 8 of 512 in FP64 with three solves of 512 columns: 213 -> 12 ms (one thread a column before).
-// What bounds it: the panels are a chain of nb column steps (barriers and reductions, ~1-2 us each); the
-// FP64 pipe for lu_update and lu_trsm in FP64; the products run at tensor rate.
+// Measured (16 matrices of 1024 rows, FP32 LU and two solves of 1024 columns): panel_getrf + laswp + trsm + 3xTF32
+// updates 48 ms before, 11 ms now; 4 of 2048: 123 -> 17 ms; 8 of 512 in FP64 with three solves of 512 columns: 213 ->
+// 8 ms (one thread a column before).  The FP64 panel step: 6.3 us a column with FP64 compares, Smith reciprocals and
+// rows fetched after the barrier, 4.2 us as it is.
+// What bounds it: the panels are a chain of nb column steps (two barriers, a reciprocal and the row update each); the
+// FP64 pipe for lu_update, lu_trsm and lu_invert in FP64; the products run at tensor rate.
 
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
@@ -28,7 +30,6 @@ namespace cg = cooperative_groups;
 namespace rsfd {
 namespace {
 
-constexpr int kOuter = 128;      // columns per outer block = k of the trailing products
 constexpr int kPanelThreads = 512;
 constexpr int kMaxCluster = 8;   // portable cluster size
 constexpr int kMaxPanels = 16;   // panels of an outer block (at least 8 columns each)
@@ -36,7 +37,7 @@ constexpr int kMaxPanels = 16;   // panels of an outer block (at least 8 columns
 template <typename T> struct Num;
 template <> struct Num<float2> {
   typedef float R;
-  static constexpr int NBLK = 128;   // rows per substitution block
+  static constexpr int NBLK = 128;   // columns per outer block = k of the products, and rows per substitution block
   // pivot measure, as in the FP32 form's reference: |re| + |im|
   static __device__ __forceinline__ float mag(float2 a) { return fabsf(a.x) + fabsf(a.y); }
   static __device__ __forceinline__ float2 mul(float2 a, float2 b) {
@@ -66,7 +67,13 @@ template <> struct Num<double2> {
   }
   static __device__ __forceinline__ double2 recip(double2 d) {
     if (d.x == 0.0 && d.y == 0.0) return make_double2(0.0, 0.0);
-    return cdiv(make_double2(1.0, 0.0), d);
+    // d* / |d|^2 with d scaled to a component near 1 (no overflow or underflow): one division instead of Smith's three
+    const int hx = __double2hiint(d.x) & 0x7ff00000, hy = __double2hiint(d.y) & 0x7ff00000;
+    const int h = hx > hy ? hx : hy;
+    if (h < 0x00200000 || h > 0x7fd00000) return cdiv(make_double2(1.0, 0.0), d);   // near the ends of the range
+    const double s = __hiloint2double(0x7fe00000 - h, 0);
+    const double x = d.x * s, y = d.y * s, q = s / fma(x, x, y * y);
+    return make_double2(x * q, -y * q);
   }
 };
 
@@ -100,23 +107,27 @@ template <int W> __device__ void swap_list(const int* piv, int j0, int jw, int* 
   out[32 + lane] = label;
 }
 
+// Pivot keys: the leading word of the pivot measure, ordered like it as an integer (-1 for NaN).  The search compares
+// FP64 measures to 20 bits, which moves the growth bound by 1e-6 and takes it off the FP64 pipe.
+__device__ __forceinline__ int pivot_key(float v) { return v == v ? __float_as_int(v) : -1; }
+__device__ __forceinline__ int pivot_key(double v) { return v == v ? __double2hiint(v) : -1; }
+
 // Factorise columns j0 .. j0 + jw - 1 (jw <= W <= 16) of matrix blockIdx.y, rows j0 .. nb - 1; grid (cluster size, K).
-// Ties in the pivot search go to the lowest row.
+// Ties in the pivot search go to the lowest row.  What a column step waits for: two warp reductions, one block
+// barrier, the reciprocal of the candidate pivots, one cluster barrier; every CTA pushes its candidate row (and the one
+// that holds row j also that row) into the shared memory of all before the barrier, so nothing is fetched after it.
 template <typename T, int W, int RPT>
 __global__ void __launch_bounds__(kPanelThreads) lu_panel(T* M, int nb, int j0, int jw, int* swp, int ss, int* info) {
   typedef Num<T> N;
-  typedef typename N::R R;
   cg::cluster_group cl = cg::this_cluster();
   const int C = gridDim.x, rank = blockIdx.x, b = blockIdx.y;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockDim.x, nw = nt >> 5;
-  // what a CTA shows to its cluster, double-buffered by column parity: a CTA that writes entry (jj + 2) has
-  // passed the barrier of column jj + 1, at which every CTA has finished reading column jj
-  __shared__ T s_cand[2][W], s_rowj[2][W], s_inv[2];
-  __shared__ R s_bv[2];
-  __shared__ int s_bi[2];
-  __shared__ R s_wv[kPanelThreads / 32];
-  __shared__ int s_wi[kPanelThreads / 32];
-  __shared__ T s_w[kPanelThreads / 32][2 * W + 1];   // per warp: pivot row, replaced row, 1 / pivot
+  // what the CTAs show each other, double-buffered by column parity: a CTA that writes for column jj + 2 has passed
+  // the barrier of column jj + 1, at which every CTA has finished reading what belongs to column jj.
+  // s_cand[.][r]: candidate row of CTA r and, last, the reciprocal of its pivot
+  __shared__ T s_cand[2][kMaxCluster][W + 1], s_rowj[2][W];
+  __shared__ int2 s_best[2][kMaxCluster];   // key and row of every CTA's candidate
+  __shared__ int2 s_wbest[kPanelThreads / 32];
   __shared__ int s_piv[W];
   T* A = M + (long long)b * nb * nb + (long long)j0 * nb;
   const int row0 = j0 + rank * nt * RPT + tid;
@@ -128,115 +139,96 @@ __global__ void __launch_bounds__(kPanelThreads) lu_panel(T* M, int nb, int j0, 
       const int i = row0 + r * nt;
       a[r][c] = (i < nb && c < jw) ? A[(long long)c * nb + i] : T();
     }
+  if (C > 1) cl.sync();   // every CTA of the cluster runs before its shared memory is written
 #pragma unroll
   for (int jj = 0; jj < W; ++jj) {
     if (jj < jw) {
       const int gj = j0 + jj, par = jj & 1;
-      R best = (R)-1;
-      int bi = 0x7fffffff;
+      int key = -1, bi = 0x7fffffff;
 #pragma unroll
       for (int r = 0; r < RPT; ++r) {
         const int i = row0 + r * nt;
-        const R v = N::mag(a[r][jj]);
-        if (i >= gj && i < nb && v > best) {
-          best = v;
+        const int v = i >= gj && i < nb ? pivot_key(N::mag(a[r][jj])) : -1;
+        if (v > key) {
+          key = v;
           bi = i;
         }
       }
-      for (int o = 16; o > 0; o >>= 1) {
-        const R ov = __shfl_xor_sync(0xffffffffu, best, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (ov > best || (ov == best && oi < bi)) {
-          best = ov;
-          bi = oi;
-        }
+      {
+        const int m = __reduce_max_sync(0xffffffffu, key);
+        bi = __reduce_min_sync(0xffffffffu, key == m && m >= 0 ? bi : 0x7fffffff);
+        if (lane == 0) s_wbest[warp] = make_int2(m, bi);
       }
-      if (lane == 0) {
-        s_wv[warp] = best;
-        s_wi[warp] = bi;
-      }
-      if (rank == 0 && tid == jj) {
+      if (rank == 0 && warp == 0) {   // row gj, in thread jj's registers, to every CTA
+        T* src = &s_rowj[par][0];
+        if (tid == jj) {
 #pragma unroll
-        for (int c = 0; c < W; ++c) s_rowj[par][c] = a[0][c];
+          for (int c = 0; c < W; ++c) src[c] = a[0][c];
+        }
+        __syncwarp();
+        for (int e = lane; e < W * (C - 1); e += 32) cl.map_shared_rank(src, 1 + e / W)[e % W] = src[e % W];
       }
       __syncthreads();
-      best = s_wv[0];
-      bi = s_wi[0];
-      for (int w = 1; w < nw; ++w) {
-        const R ov = s_wv[w];
-        const int oi = s_wi[w];
-        if (ov > best || (ov == best && oi < bi)) {
-          best = ov;
-          bi = oi;
+      {
+        const int2 w = lane < nw ? s_wbest[lane] : make_int2(-1, 0x7fffffff);
+        const int m = __reduce_max_sync(0xffffffffu, w.x);
+        key = m;
+        bi = __reduce_min_sync(0xffffffffu, w.x == m && m >= 0 ? w.y : 0x7fffffff);
+      }
+      // the candidate's warp pushes its row; warp 0 pushes key and row number
+      bool mine = false;
+#pragma unroll
+      for (int r = 0; r < RPT; ++r) mine |= row0 + r * nt == bi;
+      if (__any_sync(0xffffffffu, mine)) {
+        T* src = &s_cand[par][rank][0];
+#pragma unroll
+        for (int r = 0; r < RPT; ++r)
+          if (row0 + r * nt == bi) {
+#pragma unroll
+            for (int c = 0; c < W; ++c) src[c] = a[r][c];
+            src[W] = N::recip(a[r][jj]);
+          }
+        __syncwarp();
+        for (int e = lane; e < (W + 1) * (C - 1); e += 32) {
+          const int o = e / (W + 1), c = e % (W + 1);
+          cl.map_shared_rank(src, o + (o >= rank ? 1 : 0))[c] = src[c];
         }
       }
-#pragma unroll
-      for (int r = 0; r < RPT; ++r)
-        if (row0 + r * nt == bi) {
-#pragma unroll
-          for (int c = 0; c < W; ++c) s_cand[par][c] = a[r][c];
-          s_inv[par] = N::recip(a[r][jj]);
-        }
-      if (tid == 0) {
-        s_bv[par] = best;
-        s_bi[par] = bi;
-      }
+      if (warp == 0 && lane < C) *cl.map_shared_rank(&s_best[par][rank], lane) = make_int2(key, bi);
       if (C > 1) cl.sync();
       else __syncthreads();
-      int pr = 0;
-      if (C > 1) {
-        best = (R)-1;
-        bi = 0x7fffffff;
-        if (lane < C) {
-          best = *cl.map_shared_rank(&s_bv[par], lane);
-          bi = *cl.map_shared_rank(&s_bi[par], lane);
-        }
-        for (int o = kMaxCluster / 2; o > 0; o >>= 1) {
-          const R ov = __shfl_xor_sync(0xffffffffu, best, o);
-          const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-          if (ov > best || (ov == best && oi < bi)) {
-            best = ov;
-            bi = oi;
-          }
-        }
-        best = __shfl_sync(0xffffffffu, best, 0);
-        bi = __shfl_sync(0xffffffffu, bi, 0);
+      int pr;
+      {
+        const int2 w = lane < C ? s_best[par][lane] : make_int2(-1, 0x7fffffff);
+        key = __reduce_max_sync(0xffffffffu, w.x);
+        bi = __reduce_min_sync(0xffffffffu, w.x == key && key >= 0 ? w.y : 0x7fffffff);
       }
-      const bool none = bi == 0x7fffffff;   // no comparable entry in the column (all NaN)
+      const bool none = key < 0;   // no comparable entry in the column (all NaN)
       const int gp = none ? gj : bi;
       pr = (gp - j0) / (nt * RPT);
-      if (lane < W) {
-        const T* rj = C > 1 ? cl.map_shared_rank(&s_rowj[par][0], 0) : &s_rowj[par][0];
-        const T* pv = C > 1 ? cl.map_shared_rank(&s_cand[par][0], pr) : &s_cand[par][0];
-        const T vj = rj[lane];
-        s_w[warp][lane] = none ? vj : pv[lane];
-        s_w[warp][W + lane] = vj;
-      } else if (lane == W) {
-        const T* pi = C > 1 ? cl.map_shared_rank(&s_inv[par], pr) : &s_inv[par];
-        s_w[warp][2 * W] = none ? T() : *pi;
-      }
-      __syncwarp();
+      const T* prow = none ? &s_rowj[par][0] : &s_cand[par][pr][0];
+      const T* jrow = &s_rowj[par][0];
+      const T inv = none ? T() : s_cand[par][pr][W];
       if (rank == 0 && tid == 0) {
         s_piv[jj] = gp;
-        if (!(best > (R)0) && info[b] == 0) info[b] = gj + 1;
+        // a pivot of measure zero (key 0 also stands for FP64 measures below the range of a leading word)
+        if ((none || key == 0) && !(N::mag(prow[jj]) > 0) && info[b] == 0) info[b] = gj + 1;
       }
-      const T inv = s_w[warp][2 * W];
 #pragma unroll
       for (int r = 0; r < RPT; ++r) {
         const int i = row0 + r * nt;
         if (gp != gj && (i == gp || i == gj)) {
-          const int o = i == gp ? W : 0;
+          const T* o = i == gp ? jrow : prow;
 #pragma unroll
-          for (int c = 0; c < W; ++c) a[r][c] = s_w[warp][o + c];
+          for (int c = 0; c < W; ++c) a[r][c] = o[c];
         }
         if (i > gj && i < nb) {
           const T l = N::mul(a[r][jj], inv);
           a[r][jj] = l;
 #pragma unroll
-          for (int c = jj + 1; c < W; ++c) a[r][c] = N::nma(l, s_w[warp][c], a[r][c]);
+          for (int c = jj + 1; c < W; ++c) a[r][c] = N::nma(l, prow[c], a[r][c]);
         }
       }
-      __syncwarp();
     }
   }
 #pragma unroll
@@ -248,7 +240,6 @@ __global__ void __launch_bounds__(kPanelThreads) lu_panel(T* M, int nb, int j0, 
     }
   __syncthreads();
   if (rank == 0 && warp == 0) swap_list<W>(s_piv, j0, jw, swp + (long long)b * ss);
-  if (C > 1) cl.sync();   // a CTA's shared memory outlives the other CTAs' reads
 }
 
 // The same for panels taller than the clusters hold: one CTA per matrix, the panel stays in global memory.
@@ -320,11 +311,11 @@ __global__ void __launch_bounds__(kPanelThreads) lu_panel_global(T* M, int nb, i
 
 // Row exchanges of the panel (W, j0, jw) in the outer block's other columns o0 .. oend - 1, one thread per column;
 // those right of the panel are also solved with its unit lower triangle.  Bound: latency of 2 W scattered
-// loads per thread, all in flight together.
+// loads per thread, all in flight together, and in FP64 the pipe (so a CTA is one warp).
 template <typename T, int W>
-__global__ void __launch_bounds__(kOuter) lu_swap(T* M, int nb, int o0, int oend, int j0, int jw, const int* swp, int ss) {
+__global__ void __launch_bounds__(32) lu_swap(T* M, int nb, int o0, int oend, int j0, int jw, const int* swp, int ss) {
   typedef Num<T> N;
-  const int b = blockIdx.x;
+  const int b = blockIdx.y;
   __shared__ int s_dst[2 * W], s_src[2 * W];
   __shared__ T s_L[W][W];
   T* A = M + (long long)b * nb * nb;
@@ -338,7 +329,7 @@ __global__ void __launch_bounds__(kOuter) lu_swap(T* M, int nb, int o0, int oend
     s_L[r][c] = (r > c && r < jw) ? A[(long long)(j0 + c) * nb + j0 + r] : T();
   }
   __syncthreads();
-  const int c = o0 + threadIdx.x;
+  const int c = o0 + blockIdx.x * 32 + threadIdx.x;
   if (c >= oend || (c >= j0 && c < j0 + jw)) return;
   T* col = A + (long long)c * nb;
   const bool right = c >= j0 + jw;
@@ -350,9 +341,9 @@ __global__ void __launch_bounds__(kOuter) lu_swap(T* M, int nb, int o0, int oend
   }
   if (right) {
 #pragma unroll
-    for (int r = 1; r < W; ++r)
+    for (int q = 0; q < W - 1; ++q)   // by columns: the updates of one q are independent
 #pragma unroll
-      for (int q = 0; q < r; ++q) v[r] = N::nma(s_L[r][q], v[q], v[r]);
+      for (int r = q + 1; r < W; ++r) v[r] = N::nma(s_L[r][q], v[q], v[r]);
   }
 #pragma unroll
   for (int t = 0; t < 2 * W; ++t)
@@ -417,31 +408,38 @@ __global__ void __launch_bounds__(128) lu_update(T* M, int nb, int j0, int jw, i
 }
 
 // X[r0 .. r0 + ib, :] = T^{-1} X[r0 .. r0 + ib, :] for the diagonal block T of LU at (r0, r0): unit lower (LOWER) or
-// upper triangle.  Eight threads share a column (rows q, q + 8, ...), 32 columns per CTA; T passes through
+// upper triangle.  Eight threads share a column (rows q, q + 8, ...), 32 columns per CTA of 256 threads (4 per
+// warp; FP64 takes CTAs of one warp, so that the FP64 pipes of all SMs have their share); T passes through
 // shared memory in strips of 16 columns; the solved element travels by shuffle.  X has nb rows and batch stride sX.  Bound: FP64 (FP32) pipe.
-template <typename T, bool LOWER>
-__global__ void __launch_bounds__(256) lu_trsm(const T* LU, int nb, int r0, int ib, T* X, long long sX, int nrhs) {
+// INV: X is the identity and the result goes to D (64 x 64, one of a matrix's diagonal blocks' inverses).
+template <typename T, bool LOWER, bool INV>
+__device__ __forceinline__ void trsm_body(const T* LU, int nb, int r0, int ib, T* X, long long sX, int nrhs, int b, T* D) {
   typedef Num<T> N;
   constexpr int NB = Num<T>::NBLK, RP = NB / 8, NS = NB / 16;
   __shared__ T s_t[16][NB];
   __shared__ T s_d[NB];
-  const int b = blockIdx.y, tid = threadIdx.x, lane = tid & 31, q = tid & 7;
-  const int col = blockIdx.x * 32 + (tid >> 3);
+  const int tid = threadIdx.x, lane = tid & 31, q = tid & 7;
+  const int nt = blockDim.x, col = blockIdx.x * (nt >> 3) + (tid >> 3);
   const T* F = LU + (long long)b * nb * nb + (long long)r0 * nb + r0;
   T* x = X + b * sX + (long long)col * nb + r0;
   if (!LOWER)
-    for (int i = tid; i < ib; i += 256) s_d[i] = N::recip(F[(long long)i * nb + i]);
+    for (int i = tid; i < ib; i += nt) s_d[i] = N::recip(F[(long long)i * nb + i]);
   T v[RP];
 #pragma unroll
   for (int k = 0; k < RP; ++k) {
     const int r = k * 8 + q;
-    v[k] = (col < nrhs && r < ib) ? x[r] : T();
+    if (INV) {
+      v[k] = T();
+      if (r == col) v[k].x = 1;
+    } else {
+      v[k] = (col < nrhs && r < ib) ? x[r] : T();
+    }
   }
 #pragma unroll
   for (int s = 0; s < NS; ++s) {
     const int i0 = (LOWER ? s : NS - 1 - s) * 16;
     __syncthreads();
-    for (int e = tid; e < 16 * NB; e += 256) {
+    for (int e = tid; e < 16 * NB; e += nt) {
       const int c = e / NB, r = e % NB;
       s_t[c][r] = (i0 + c < ib && r < ib) ? F[(long long)(i0 + c) * nb + r] : T();
     }
@@ -467,8 +465,23 @@ __global__ void __launch_bounds__(256) lu_trsm(const T* LU, int nb, int r0, int 
 #pragma unroll
   for (int k = 0; k < RP; ++k) {
     const int r = k * 8 + q;
-    if (col < nrhs && r < ib) x[r] = v[k];
+    if (INV) D[(long long)col * NB + r] = v[k];
+    else if (col < nrhs && r < ib) x[r] = v[k];
   }
+}
+template <typename T, bool LOWER>
+__global__ void __launch_bounds__(256, sizeof(T) == 16 ? 2 : 3) lu_trsm(const T* LU, int nb, int r0, int ib, T* X,
+                                                                         long long sX, int nrhs) {
+  trsm_body<T, LOWER, false>(LU, nb, r0, ib, X, sX, nrhs, blockIdx.y, nullptr);
+}
+// Inverses of the diagonal blocks of 64 rows, for solves whose products run on the tensor cores: block (z >> 1) of matrix
+// blockIdx.y, its unit lower (z even) or upper (z odd) triangle; dinv [K][blocks][2][64 x 64].  One warp per 4 columns.
+__global__ void __launch_bounds__(32) lu_invert(const double2* LU, int nb, double2* dinv) {
+  constexpr int NB = Num<double2>::NBLK;
+  const int blk = blockIdx.z >> 1, r0 = blk * NB, ib = min(NB, nb - r0), nblk = (nb + NB - 1) / NB;
+  double2* D = dinv + (((long long)blockIdx.y * nblk + blk) * 2 + (blockIdx.z & 1)) * NB * NB;
+  if (blockIdx.z & 1) trsm_body<double2, false, true>(LU, nb, r0, ib, nullptr, 0, NB, blockIdx.y, D);
+  else trsm_body<double2, true, true>(LU, nb, r0, ib, nullptr, 0, NB, blockIdx.y, D);
 }
 
 __global__ void iota_rows(int* perm, int nb, int K) {
@@ -525,7 +538,7 @@ void launch_panel(Gemm& g, T* M, int nb, int K, int j0, int jw, int C, int* swp,
 
 template <typename T, int W>
 void launch_swap_update(Gemm& g, T* M, int nb, int K, int o0, int j0, int jw, int oend, const int* swp, int ss) {
-  if (oend - o0 > jw) lu_swap<T, W><<<K, kOuter, 0, g.st>>>(M, nb, o0, oend, j0, jw, swp, ss);
+  if (oend - o0 > jw) lu_swap<T, W><<<dim3((oend - o0 + 31) / 32, K), 32, 0, g.st>>>(M, nb, o0, oend, j0, jw, swp, ss);
   const int r0 = j0 + jw;
   if (r0 < oend) lu_update<T, W><<<dim3((nb - r0 + 63) / 64, (oend - r0 + 15) / 16, K), 128, 0, g.st>>>(M, nb, j0, jw, oend);
 }
@@ -565,15 +578,25 @@ int panel(Gemm& g, T* M, int nb, int K, int o0, int j0, int oend, int* info, int
 }
 
 // X = T^{-1} X for the unit lower triangle (LOWER) or the upper triangle of rows and columns r0 .. r1 - 1 of LU
+// (r0 a multiple of the block size).  dinv: the diagonal blocks' inverses (FP64), or null for substitution.
 template <typename T, bool LOWER>
-void solve_range(Gemm& g, const T* LU, int nb, int K, int r0, int r1, T* X, long long sX, int nrhs) {
+void solve_range(Gemm& g, const T* LU, int nb, int K, int r0, int r1, T* X, long long sX, int nrhs, const T* dinv) {
   constexpr int NB = Num<T>::NBLK;
   const long long n2 = (long long)nb * nb;
-  const dim3 grid((nrhs + 31) / 32, K);
+  const int thr = sizeof(T) == 16 ? 32 : 256, per = thr / 8;
+  const dim3 grid((nrhs + per - 1) / per, K);
   const int nblk = (r1 - r0 + NB - 1) / NB;
   for (int bi = 0; bi < nblk; ++bi) {
     const int s0 = r0 + (LOWER ? bi : nblk - 1 - bi) * NB, ib = r1 - s0 < NB ? r1 - s0 : NB;
-    lu_trsm<T, LOWER><<<grid, 256, 0, g.st>>>(LU, nb, s0, ib, X, sX, nrhs);
+    bool done = false;
+    if constexpr (sizeof(T) == 16) {
+      // X_b = T_bb^{-1} X_b in place: the digits of X_b are taken before the product is written
+      const int tot = (nb + NB - 1) / NB;
+      if (dinv)
+        done = gemm_sliced(g, K, ib, nrhs, ib, 1.0, dinv + ((long long)(s0 / NB) * 2 + (LOWER ? 0 : 1)) * NB * NB, NB,
+                           (long long)tot * 2 * NB * NB, 0, X + s0, nb, sX, false, X + s0, nb, sX);
+    }
+    if (!done) lu_trsm<T, LOWER><<<grid, thr, 0, g.st>>>(LU, nb, s0, ib, X, sX, nrhs);
     const int d0 = LOWER ? s0 + ib : r0, d1 = LOWER ? r1 : s0;   // rows still to be updated
     if (d1 > d0)
       gemm(g, K, d1 - d0, nrhs, ib, -1.0, LU + (long long)s0 * nb + d0, nb, n2, 0, X + s0, nb, sX, true, X + d0, nb, sX);
@@ -582,23 +605,24 @@ void solve_range(Gemm& g, const T* LU, int nb, int K, int r0, int r1, T* X, long
 
 template <typename T> void lu_factor_t(Gemm& g, T* M, int nb, int K, int* perm, int* info, int* swp) {
   const long long n2 = (long long)nb * nb;
+  constexpr int kOuter = Num<T>::NBLK;
   const int ss = lu_swap_ints(nb);
+  const bool one = nb <= kOuter;   // one outer block: one list per matrix, applied to perm after every panel
   iota_rows<<<grid1((long long)nb * K), 256, 0, g.st>>>(perm, nb, K);
   for (int o0 = 0; o0 < nb; o0 += kOuter) {
     const int oend = nb - o0 < kOuter ? nb : o0 + kOuter, out = nb - (oend - o0) + 1, rest = nb - oend;
     int np = 0;
     for (int j0 = o0; j0 < oend; ++np) {
       int* lists = swp + np * kSwapInts;
-      // nb <= kOuter: one list per matrix, applied to perm after every panel
-      if (ss == kSwapInts) lists = swp;
+      if (one) lists = swp;
       j0 += panel<T>(g, M, nb, K, o0, j0, oend, info, lists, ss);
-      if (ss == kSwapInts) lu_swap_rest<T><<<dim3(1, K), 64, 0, g.st>>>(M, nb, o0, oend, 1, swp, ss, perm);
+      if (one) lu_swap_rest<T><<<dim3(1, K), 64, 0, g.st>>>(M, nb, o0, oend, 1, swp, ss, perm);
     }
-    if (ss == kSwapInts) continue;
+    if (one) continue;
     lu_swap_rest<T><<<dim3((out + 63) / 64, K), 64, 0, g.st>>>(M, nb, o0, oend, np, swp, ss, perm);
     if (rest > 0) {
       // U12 = L11^{-1} A12, then A22 -= L21 U12
-      solve_range<T, true>(g, M, nb, K, o0, oend, M + (long long)oend * nb, n2, rest);
+      solve_range<T, true>(g, M, nb, K, o0, oend, M + (long long)oend * nb, n2, rest, nullptr);
       gemm(g, K, rest, rest, oend - o0, -1.0, M + (long long)o0 * nb + oend, nb, n2, 0, M + (long long)oend * nb + o0, nb, n2,
            true, M + (long long)oend * nb + oend, nb, n2);
     }
@@ -606,16 +630,16 @@ template <typename T> void lu_factor_t(Gemm& g, T* M, int nb, int K, int* perm, 
   g.note(cudaGetLastError());
 }
 
-template <typename T> void lu_solve_t(Gemm& g, const T* LU, int nb, int K, T* X, int nrhs) {
+template <typename T> void lu_solve_t(Gemm& g, const T* LU, int nb, int K, T* X, int nrhs, const T* dinv) {
   const long long sx = (long long)nb * nrhs;
-  solve_range<T, true>(g, LU, nb, K, 0, nb, X, sx, nrhs);
-  solve_range<T, false>(g, LU, nb, K, 0, nb, X, sx, nrhs);
+  solve_range<T, true>(g, LU, nb, K, 0, nb, X, sx, nrhs, dinv);
+  solve_range<T, false>(g, LU, nb, K, 0, nb, X, sx, nrhs, dinv);
   g.note(cudaGetLastError());
 }
 
 }  // namespace
 
-int lu_swap_ints(int nb) { return nb <= kOuter ? kSwapInts : kMaxPanels * kSwapInts; }
+int lu_swap_ints(int nb) { return nb <= 64 ? kSwapInts : kMaxPanels * kSwapInts; }
 
 void lu_factor(Gemm& g, double2* M, int nb, int K, int* perm, int* info, int* swp) {
   lu_factor_t<double2>(g, M, nb, K, perm, info, swp);
@@ -623,8 +647,26 @@ void lu_factor(Gemm& g, double2* M, int nb, int K, int* perm, int* info, int* sw
 void lu_factor(Gemm& g, float2* M, int nb, int K, int* perm, int* info, int* swp) {
   lu_factor_t<float2>(g, M, nb, K, perm, info, swp);
 }
-void lu_solve(Gemm& g, const double2* LU, int nb, int K, double2* X, int nrhs) { lu_solve_t<double2>(g, LU, nb, K, X, nrhs); }
-void lu_solve(Gemm& g, const float2* LU, int nb, int K, float2* X, int nrhs) { lu_solve_t<float2>(g, LU, nb, K, X, nrhs); }
+// Substitution costs 64 x 63 / 2 FP64 multiply-adds a column and block on the FP64 pipe (70-90 us a block for 400 to 512
+// columns of 8 matrices), a product with the inverse about 25 us; the inverses of all blocks together cost one block's
+// substitution.  Worth it from 2000 columns over the batch on (where gemm() slices the 64 x n x 64 products).
+const double2* lu_inverses(Gemm& g, const double2* LU, int nb, int K, int nrhs) {
+  constexpr int NB = Num<double2>::NBLK;
+  if (!g.h || (double)nrhs * K * NB * NB < kSliceMin || nb < NB) return nullptr;
+  const int nblk = (nb + NB - 1) / NB;
+  if (nblk > 32767) return nullptr;
+  void* w = nullptr;
+  if (handle_ensure(g.h, 10, (size_t)K * nblk * 2 * NB * NB * sizeof(double2), &w) != RSFD_OK) return nullptr;
+  lu_invert<<<dim3(NB / 4, K, 2 * nblk), 32, 0, g.st>>>(LU, nb, (double2*)w);
+  g.note(cudaGetLastError());
+  return (const double2*)w;
+}
+void lu_solve(Gemm& g, const double2* LU, int nb, int K, double2* X, int nrhs, const double2* dinv) {
+  lu_solve_t<double2>(g, LU, nb, K, X, nrhs, dinv);
+}
+void lu_solve(Gemm& g, const float2* LU, int nb, int K, float2* X, int nrhs) {
+  lu_solve_t<float2>(g, LU, nb, K, X, nrhs, nullptr);
+}
 
 void lu_permute(Gemm& g, const double2* B, int nb, int K, const int* perm, float2* X, int nrhs) {
   permute_rows<double2, float2><<<grid1((long long)nb * nrhs * K), 256, 0, g.st>>>(B, nb, nrhs, perm, X, K);

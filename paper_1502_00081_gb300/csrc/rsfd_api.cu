@@ -71,7 +71,7 @@ struct Handle {
   DevBuf cw, ce;                       // collapse weights and factors of the shift update
   CUtensorMap tmR, tmV, tmVs;
   // dyson / transmission workspace
-  DevBuf dy[10];
+  DevBuf dy[11];
 };
 
 static bool is_split(int kind) { return kind == RSFD_PASS_SPLIT || kind == RSFD_PASS_SPLIT_BFP; }

@@ -235,7 +235,7 @@ cudaError_t kernels_init();
 int pass_threads(int R, int tile_y);
 
 // Handle services used by other translation units (rsfd_api.cu).
-rsfd_status handle_ensure(Handle* h, int idx, size_t bytes, void** out);   // workspace slot idx < 10
+rsfd_status handle_ensure(Handle* h, int idx, size_t bytes, void** out);   // workspace slot idx < 11
 cudaStream_t handle_stream(Handle* h);
 int handle_prec(Handle* h);
 int handle_nb(Handle* h);
