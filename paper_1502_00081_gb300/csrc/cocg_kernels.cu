@@ -1952,6 +1952,9 @@ __global__ void __launch_bounds__(kStencilThreads, MODE == RSFD_MIXED ? 3 : 2)
 stencil_kernel(PassParams p, const __grid_constant__ CUtensorMap tmR, const __grid_constant__ CUtensorMap tmV) {
   static_assert(!BFP || MODE == RSFD_DF64, "the block-floating-point pass is double-float only");
   constexpr bool LOG = MODE == RSFD_DF64;
+  // The plain double-float stencil takes 320 instructions a point; unrolled over the 2R + 1 ring positions its loop
+  // does not fit the instruction cache (the first stall reason), so it moves the ring's registers instead.
+  constexpr bool ROT = MODE == RSFD_DF64 && !BFP && R == 2;
   typedef Ops<MODE> O;
   typedef typename O::C C;
   typedef typename O::VT VT;
@@ -2107,7 +2110,7 @@ stencil_kernel(PassParams p, const __grid_constant__ CUtensorMap tmR, const __gr
       }
     };
     auto steady = [&](auto j_c) -> bool {
-      constexpr int PH = (2 * R + decltype(j_c)::value) % Q;   // register of plane q
+      constexpr int PH = ROT ? 2 * R : (2 * R + decltype(j_c)::value) % Q;   // register of plane q
       constexpr int CC = (PH + Q - R) % Q;                     // register of plane c = q - R
       if (!arrive_plane(std::integral_constant<int, PH>())) return false;
       const unsigned char* b = ring + ic * PEb;
@@ -2154,7 +2157,18 @@ stencil_kernel(PassParams p, const __grid_constant__ CUtensorMap tmR, const __gr
         if (ok) end_step();
       }
     }
-    while (ok && s < nsteps) {
+    if (ROT) {
+#pragma unroll 1
+      while (ok && s < nsteps) {
+        ok = steady(std::integral_constant<int, 0>());
+#pragma unroll
+        for (int t = 0; t < 2 * R; ++t) {
+          zq[0][t] = zq[0][t + 1];
+          zq[1][t] = zq[1][t + 1];
+        }
+      }
+    }
+    while (!ROT && ok && s < nsteps) {
       ok = steady(std::integral_constant<int, 0>());
       if (ok && s < nsteps) ok = steady(std::integral_constant<int, 1>());
       if (ok && s < nsteps) ok = steady(std::integral_constant<int, 2>());
@@ -2252,12 +2266,15 @@ stencil_kernel(PassParams p, const __grid_constant__ CUtensorMap tmR, const __gr
 //   V_nl r = sum_a E_a c_a p_a,   c_a = h^3 p_a^T r,
 // so with u_loc = (Z_s - H_loc) r from the pass,
 //   A r = u_loc - sum_a E_a c_a p_a,   (r, A r) = (r, u_loc) - sum_a E_a c_a^2 / h^3.
-// proj_kernel: one block per (atom, slot) forms c_a (a gather-GEMV over the atom's support, exact
-// products in double-float or FP64), stores -E_a c_a and the dot correction; the last block of a
-// slot (atomic ticket) sums the corrections in atom order and runs the FP64 scalar step.
-// pscatter_kernel: u_n -= sum_a E_a c_a p_a over the union of the supports, one thread per support
-// point gathering its atoms (point-major CSR), so no atomics and a fixed summation order.
+// proj_kernel: a block takes one atom of four slots: it forms c_a (a gather-GEMV over the atom's support, exact
+// products in double-float or FP64; positions and projector values are read once for the four), stores -E_a c_a and
+// the dot correction.  proj_scalar_kernel, one block per slot, sums the corrections in atom order and runs the FP64
+// scalar step.  pscatter_kernel: u_n -= sum_a E_a c_a p_a over the union of the supports, one thread per support point of
+// four slots gathering its atoms (point-major CSR), so no atomics and a fixed summation order.
+// Bound: latency of the gathers; four slots keep four in flight per thread.  16 slots of 72 x 72 x 256 with 460 atoms, one
+// slot per block or thread: 108 us + 44 us an iteration.
 // ------------------------------------------------------------------------------------------------
+constexpr int kProjSlots = 4;
 struct ProjParams {
   PassParams pp;
   int n_atoms, n_supp;
@@ -2272,7 +2289,6 @@ struct ProjParams {
   double h3;
   double2* pw;
   double2* pcorr;
-  unsigned int* ptickets;
   const double* pmax;        // per atom: largest |projector value|
   int overlap;               // largest number of atoms at one support point
 };
@@ -2308,30 +2324,56 @@ template <> struct ProjAcc<RSFD_DF64> {
   }
 };
 
-// one block per (atom, slot); an atom has ~10^3 support points, so a small block keeps the per-block
-// reduction and ticket cheap against the gather
+// an atom has ~10^3 support points: a small block keeps its reduction cheap against the gather
 constexpr int kProjThreads = 128;
 template <int MODE>
 __global__ void __launch_bounds__(kProjThreads) proj_kernel(ProjParams q) {
   typedef typename Ops<MODE>::C C;
   typedef typename Ops<MODE>::VT VT;
-  __shared__ ScalarShared S;
-  __shared__ int s_last;
+  constexpr int NS = kProjSlots;
+  __shared__ double s_red[(kProjThreads / 32) * 2 * NS], s_c[2 * NS];
   const PassParams& p = q.pp;
-  const int a = blockIdx.x, slot = blockIdx.y, tid = threadIdx.x;
-  SlotState* st = p.slots + slot;
-  if (st->status != SLOT_RUNNING) return;
-  const int n = st->n;   // the pass of this iteration wrote r_n to ring entry n % 3
+  const int a = blockIdx.x, s0 = blockIdx.y * NS, tid = threadIdx.x;
   const long long vec = (long long)p.d.nz * p.d.ny * p.d.nxp;
-  const C* r = reinterpret_cast<const C*>(p.rbuf) + ((size_t)slot * p.d.nvec + n % 3) * vec;
+  const C* r[NS];
+  bool run[NS], any = false;
+#pragma unroll
+  for (int k = 0; k < NS; ++k) {
+    const int slot = min(s0 + k, p.d.W - 1);
+    const SlotState* st = p.slots + slot;
+    run[k] = s0 + k < p.d.W && st->status == SLOT_RUNNING;
+    any |= run[k];
+    // the pass of this iteration wrote r_n to ring entry n % 3
+    r[k] = reinterpret_cast<const C*>(p.rbuf) + ((size_t)slot * p.d.nvec + st->n % 3) * vec;
+  }
+  if (!any) return;   // uniform
   const VT* pv = reinterpret_cast<const VT*>(q.a_val);
-  ProjAcc<MODE> acc;
-  for (int e = q.a_ptr[a] + tid; e < q.a_ptr[a + 1]; e += blockDim.x) acc.add(pv[e], r[q.a_idx[e]]);
-  const double2 t = acc.get();
-  double v2[2] = {warp_sum(t.x), warp_sum(t.y)};
-  block_sum_lane0<2>(v2, S.red);
+  ProjAcc<MODE> acc[NS];
+  for (int e = q.a_ptr[a] + tid; e < q.a_ptr[a + 1]; e += kProjThreads) {
+    const long long i = q.a_idx[e];
+    const VT v = pv[e];
+    C x[NS];
+#pragma unroll
+    for (int k = 0; k < NS; ++k) x[k] = r[k][i];   // an idle slot's vector is valid memory
+#pragma unroll
+    for (int k = 0; k < NS; ++k) acc[k].add(v, x[k]);
+  }
+  double v[2 * NS];
+#pragma unroll
+  for (int k = 0; k < NS; ++k) {
+    const double2 t = acc[k].get();
+    v[2 * k] = warp_sum(t.x);
+    v[2 * k + 1] = warp_sum(t.y);
+  }
+  block_sum_lane0<2 * NS>(v, s_red);
   if (tid == 0) {
-    const double2 c = make_double2(v2[0] * q.h3, v2[1] * q.h3);
+#pragma unroll
+    for (int k = 0; k < 2 * NS; ++k) s_c[k] = v[k];
+  }
+  __syncthreads();
+  if (tid < NS && s0 + tid < p.d.W && p.slots[s0 + tid].status == SLOT_RUNNING) {
+    const int slot = s0 + tid;
+    const double2 c = make_double2(s_c[2 * tid] * q.h3, s_c[2 * tid + 1] * q.h3);
     const double E = q.a_E[a];
     const double us = p.uscale;   // the block-floating-point pass stores s A r
     const double2 wv = make_double2(-E * us * c.x, -E * us * c.y);
@@ -2347,18 +2389,21 @@ __global__ void __launch_bounds__(kProjThreads) proj_kernel(ProjParams q) {
     }
     const double2 c2 = cmul(c, c);
     q.pcorr[(size_t)slot * q.n_atoms + a] = make_double2(E * c2.x / q.h3, E * c2.y / q.h3);
-    __threadfence();
-    const unsigned int tk = atomicAdd(q.ptickets + slot, 1u);
-    s_last = (tk == (unsigned int)(q.n_atoms - 1));
   }
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
+}
+
+// (r_n, A r_n) of slot blockIdx.x from the pass's (r_n, u_loc) and the atoms' corrections, then the scalar step
+template <int MODE>
+__global__ void __launch_bounds__(kProjThreads) proj_scalar_kernel(ProjParams q) {
+  __shared__ ScalarShared S;
+  const PassParams& p = q.pp;
+  const int slot = blockIdx.x, tid = threadIdx.x;
+  if (p.slots[slot].status != SLOT_RUNNING) return;
   if (tid < 32) {
     double cx = 0.0, cy = 0.0;
     const double2* src = q.pcorr + (size_t)slot * q.n_atoms;
     for (int k = tid; k < q.n_atoms; k += 32) {
-      const double2 v = __ldcg(src + k);
+      const double2 v = src[k];
       cx += v.x;
       cy += v.y;
     }
@@ -2370,19 +2415,18 @@ __global__ void __launch_bounds__(kProjThreads) proj_kernel(ProjParams q) {
     if (MODE == RSFD_DF64 && p.bfp) {
       const dfc* wd = reinterpret_cast<const dfc*>(q.pw + (size_t)slot * q.n_atoms);
       for (int k = tid; k < q.n_atoms; k += 32) {
-        const float2 wh = __ldcg(&wd[k].h);
+        const float2 wh = wd[k].h;
         wm = fmax(wm, ((double)fabsf(wh.x) + (double)fabsf(wh.y)) * q.pmax[k]);
       }
       for (int o = 16; o > 0; o >>= 1) wm = fmax(wm, __shfl_xor_sync(0xffffffffu, wm, o));
     }
     if (tid == 0) {
       const double* dd = p.pdots + (size_t)slot * 8;
-      S.rr = make_double2(__ldcg(dd + 0), __ldcg(dd + 1));
-      S.rAr = make_double2(__ldcg(dd + 2) - cx, __ldcg(dd + 3) - cy);
-      S.nrm2 = __ldcg(dd + 4);
-      S.maxr = __ldcg(dd + 5);
-      S.maxu = __ldcg(dd + 6) + (double)q.overlap * wm;
-      q.ptickets[slot] = 0u;
+      S.rr = make_double2(dd[0], dd[1]);
+      S.rAr = make_double2(dd[2] - cx, dd[3] - cy);
+      S.nrm2 = dd[4];
+      S.maxr = dd[5];
+      S.maxu = dd[6] + (double)q.overlap * wm;
     }
   }
   __syncthreads();
@@ -2399,45 +2443,66 @@ template <int MODE>
 __global__ void __launch_bounds__(256) pscatter_kernel(ProjParams q) {
   typedef typename Ops<MODE>::C C;
   typedef typename Ops<MODE>::VT VT;
+  constexpr int NS = kProjSlots;
   const PassParams& p = q.pp;
-  const int slot = blockIdx.y;
-  SlotState* st = p.slots + slot;
-  if (st->status != SLOT_RUNNING) return;
-  const int n = st->n - 1;   // the scalar step of this iteration advanced n
+  const int s0 = blockIdx.y * NS;
   const long long vec = (long long)p.d.nz * p.d.ny * p.d.nxp;
-  C* u = reinterpret_cast<C*>(p.rbuf) + ((size_t)slot * p.d.nvec + 3 + n % 2) * vec;
+  C* u[NS];
+  const double2* w[NS];
+  bool run[NS], any = false;
+#pragma unroll
+  for (int k = 0; k < NS; ++k) {
+    const int slot = min(s0 + k, p.d.W - 1);
+    const SlotState* st = p.slots + slot;
+    run[k] = s0 + k < p.d.W && st->status == SLOT_RUNNING;
+    any |= run[k];
+    const int n = run[k] ? st->n - 1 : 0;   // the scalar step of this iteration advanced n
+    u[k] = reinterpret_cast<C*>(p.rbuf) + ((size_t)slot * p.d.nvec + 3 + n % 2) * vec;
+    w[k] = q.pw + (size_t)slot * q.n_atoms;
+  }
+  if (!any) return;
   const VT* tv = reinterpret_cast<const VT*>(q.t_val);
-  const double2* w = q.pw + (size_t)slot * q.n_atoms;
   for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < q.n_supp; s += gridDim.x * blockDim.x) {
     const long long gi = q.t_pidx[s];
-    if (MODE == RSFD_DF64) {
-      const dfc u0 = *reinterpret_cast<const dfc*>(&u[gi]);
-      DFAcc acc = dfacc_from(u0);
-      const dfc* wd = reinterpret_cast<const dfc*>(w);   // -E_a c_a as double-float pairs (proj_kernel)
-      for (int e = q.t_ptr[s]; e < q.t_ptr[s + 1]; ++e) {
-        const dfc wc = wd[q.t_atom[e]];
-        const float2 pf = *reinterpret_cast<const float2*>(&tv[e]);
+    const int e0 = q.t_ptr[s], e1 = q.t_ptr[s + 1];
+    C x[NS];
+#pragma unroll
+    for (int k = 0; k < NS; ++k) x[k] = u[k][gi];
+    if constexpr (MODE == RSFD_DF64) {
+      DFAcc acc[NS];
+#pragma unroll
+      for (int k = 0; k < NS; ++k) acc[k] = dfacc_from(x[k]);
+      for (int e = e0; e < e1; ++e) {
+        const int a = q.t_atom[e];
+        const float2 pf = tv[e];
         dfr c;
         c.h = pf.x;
         c.l = pf.y;
-        dfacc_mul(acc, c, wc);
+#pragma unroll
+        for (int k = 0; k < NS; ++k)   // -E_a c_a as double-float pairs (proj_kernel)
+          dfacc_mul(acc[k], c, reinterpret_cast<const dfc*>(w[k])[a]);
       }
-      *reinterpret_cast<dfc*>(&u[gi]) = dfacc_get(acc);
+#pragma unroll
+      for (int k = 0; k < NS; ++k)
+        if (run[k]) u[k][gi] = dfacc_get(acc[k]);
     } else {
-      double2 uu;
-      if (MODE == RSFD_FP64) {
-        uu = *reinterpret_cast<const double2*>(&u[gi]);
-      } else {
-        const float2 uf = *reinterpret_cast<const float2*>(&u[gi]);
-        uu = make_double2((double)uf.x, (double)uf.y);
+      double2 uu[NS];
+#pragma unroll
+      for (int k = 0; k < NS; ++k) uu[k] = make_double2((double)x[k].x, (double)x[k].y);
+      for (int e = e0; e < e1; ++e) {
+        const int a = q.t_atom[e];
+        const double pd = (double)tv[e];
+#pragma unroll
+        for (int k = 0; k < NS; ++k) scat_add(uu[k], pd, w[k][a]);
       }
-      for (int e = q.t_ptr[s]; e < q.t_ptr[s + 1]; ++e) {
-        const double pd = (MODE == RSFD_FP64) ? (double)*reinterpret_cast<const double*>(&tv[e])
-                                              : (double)*reinterpret_cast<const float*>(&tv[e]);
-        scat_add(uu, pd, w[q.t_atom[e]]);
-      }
-      if (MODE == RSFD_FP64) *reinterpret_cast<double2*>(&u[gi]) = uu;
-      else *reinterpret_cast<float2*>(&u[gi]) = make_float2((float)uu.x, (float)uu.y);
+#pragma unroll
+      for (int k = 0; k < NS; ++k)
+        if (run[k]) {
+          C o;
+          o.x = uu[k].x;
+          o.y = uu[k].y;
+          u[k][gi] = o;
+        }
     }
   }
 }
@@ -2943,14 +3008,15 @@ cudaError_t launch_proj_t(const SolveDims& d, const SolverBuffers& b, const Sten
   q.h3 = b.h3;
   q.pw = b.pw;
   q.pcorr = b.pcorr;
-  q.ptickets = b.ptickets;
   q.pmax = b.a_pmax;
   q.overlap = b.proj_overlap;
-  proj_kernel<MODE><<<dim3(b.n_atoms, d.W), kProjThreads, 0, st>>>(q);
+  const int groups = (d.W + kProjSlots - 1) / kProjSlots;
+  proj_kernel<MODE><<<dim3(b.n_atoms, groups), kProjThreads, 0, st>>>(q);
+  proj_scalar_kernel<MODE><<<d.W, kProjThreads, 0, st>>>(q);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const int gx = (b.n_supp + 255) / 256;
-  pscatter_kernel<MODE><<<dim3(gx < 1 ? 1 : gx, d.W), 256, 0, st>>>(q);
+  pscatter_kernel<MODE><<<dim3(gx < 1 ? 1 : gx, groups), 256, 0, st>>>(q);
   return cudaGetLastError();
 }
 

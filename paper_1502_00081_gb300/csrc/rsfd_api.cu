@@ -33,6 +33,25 @@ struct DevBuf {
   size_t bytes = 0;
 };
 
+// page-locked host staging, grown on demand
+struct PinBuf {
+  void* p = nullptr;
+  size_t bytes = 0;
+  cudaError_t ensure(size_t n) {
+    if (bytes >= n) return cudaSuccess;
+    release();
+    const cudaError_t e = cudaMallocHost(&p, n);
+    if (e == cudaSuccess) bytes = n;
+    else p = nullptr;
+    return e;
+  }
+  void release() {
+    if (p) cudaFreeHost(p);
+    p = nullptr;
+    bytes = 0;
+  }
+};
+
 struct Handle {
   int nx = 0, ny = 0, nz = 0;
   int nxp = 0;          // padded row length of the internal vectors
@@ -67,11 +86,12 @@ struct Handle {
   std::string err = "no error";
   // solver workspace
   DevBuf rbuf, xbuf, pbuf, rhist, coef, eflag, slots, shifts, partials, tickets, Z, init_list, init_grid, counters;
-  DevBuf pw, pcorr, pdots, ptickets;   // projector term of the solve
+  DevBuf pw, pcorr, pdots;   // projector term of the solve
   DevBuf cw, ce;                       // collapse weights and factors of the shift update
   CUtensorMap tmR, tmV, tmVs;
   // dyson / transmission workspace
   DevBuf dy[11];
+  PinBuf pin[3];                       // slot states, column lists, residuals of a solve
 };
 
 static bool is_split(int kind) { return kind == RSFD_PASS_SPLIT || kind == RSFD_PASS_SPLIT_BFP; }
@@ -148,7 +168,7 @@ static void free_all(Handle* h) {
   DevBuf* bufs[] = {&h->rbuf,  &h->xbuf,      &h->pbuf,      &h->rhist,    &h->coef,
                     &h->eflag, &h->slots,     &h->shifts,    &h->partials, &h->tickets,
                     &h->Z,     &h->init_list, &h->init_grid, &h->counters, &h->pw,
-                    &h->pcorr, &h->pdots,     &h->ptickets,  &h->sweep, &h->cw, &h->ce};
+                    &h->pcorr, &h->pdots,     &h->sweep, &h->cw, &h->ce};
   for (DevBuf* b : bufs) {
     if (b->p) cudaFree(b->p);
     b->p = nullptr;
@@ -159,6 +179,7 @@ static void free_all(Handle* h) {
     b.p = nullptr;
     b.bytes = 0;
   }
+  for (auto& b : h->pin) b.release();
   if (h->dV) cudaFree(h->dV);
   if (h->dVs) cudaFree(h->dVs);
   if (h->dbrow) cudaFree(h->dbrow);
@@ -802,7 +823,15 @@ static rsfd_status rsfd_shifted_cocg_impl(rsfd_handle h, const int64_t* cols, in
     int sms = 152;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
     d.zchunk = h->nz;
-    while (d.zchunk > 16 && (long long)ltiles_x * ltiles_y * ((h->nz + d.zchunk - 1) / d.zchunk) * W0 < 4LL * sms)
+    // (FP64 and complex64 split passes, whose sums are not tied to the chunk: fewer than 8 warps per SM, down to 4
+    // planes; 128 columns of 8 x 8 x 12 in FP64 take 34 us a stencil with one chunk, one warp per SM)
+    if (is_split(d.kind) && !logical) {
+      const long long warps = split_threads(d.tile_x, d.tile_y) / 32;
+      while (d.zchunk > 4 &&
+             (long long)ltiles_x * ltiles_y * ((h->nz + d.zchunk - 1) / d.zchunk) * W0 * warps < 8LL * sms)
+        d.zchunk = (d.zchunk + 1) / 2;
+    }
+    while (!(is_split(d.kind) && !logical) && d.zchunk > 16 && (long long)ltiles_x * ltiles_y * ((h->nz + d.zchunk - 1) / d.zchunk) * W0 < 4LL * sms)
       d.zchunk = (d.zchunk + 1) / 2;
   }
   d.nzchunks = (h->nz + d.zchunk - 1) / d.zchunk;
@@ -885,7 +914,6 @@ static rsfd_status rsfd_shifted_cocg_impl(rsfd_handle h, const int64_t* cols, in
     if ((s = ensure(h, h->pw, (size_t)W * h->n_atoms * sizeof(double2))) != RSFD_OK) return s;
     if ((s = ensure(h, h->pcorr, (size_t)W * h->n_atoms * sizeof(double2))) != RSFD_OK) return s;
     if ((s = ensure(h, h->pdots, (size_t)W * 8 * sizeof(double))) != RSFD_OK) return s;
-    if ((s = ensure(h, h->ptickets, (size_t)W * sizeof(unsigned int))) != RSFD_OK) return s;
     b.n_atoms = h->n_atoms;
     b.n_supp = h->n_supp;
     b.a_ptr = h->d_aptr;
@@ -902,7 +930,6 @@ static rsfd_status rsfd_shifted_cocg_impl(rsfd_handle h, const int64_t* cols, in
     b.pw = (double2*)h->pw.p;
     b.pcorr = (double2*)h->pcorr.p;
     b.pdots = (double*)h->pdots.p;
-    b.ptickets = (unsigned int*)h->ptickets.p;
   }
   const StencilCoef coef = stencil_coef(h->fd_order, h->h);
 
@@ -917,7 +944,6 @@ static rsfd_status rsfd_shifted_cocg_impl(rsfd_handle h, const int64_t* cols, in
   for (int k = 0; k < K; ++k) Zh[k] = make_double2(k < Kout ? energies[k] : aux_energies[k - Kout], eta);
   RSFD_CK(h, cudaMemcpyAsync(b.Z, Zh.data(), K * sizeof(double2), cudaMemcpyHostToDevice, st));
   RSFD_CK(h, cudaMemsetAsync(b.tickets, 0, W * sizeof(unsigned int), st));
-  if (b.n_atoms > 0) RSFD_CK(h, cudaMemsetAsync(b.ptickets, 0, W * sizeof(unsigned int), st));
   RSFD_CK(h, cudaMemsetAsync(b.counters, 0, 4 * sizeof(unsigned long long), st));
   RSFD_CK(h, cudaMemsetAsync(b.error_flag, 0, sizeof(int), st));
   std::vector<SlotState> hs(W);
@@ -934,14 +960,11 @@ static rsfd_status rsfd_shifted_cocg_impl(rsfd_handle h, const int64_t* cols, in
   h->stats.iters_per_sync = C;
   // Pinned host staging, double-buffered by chunk parity: the slot states copied after a chunk,
   // the error flag, the lists of finished and new columns, and the finished columns' residuals.
-  struct Pinned {
-    void* p = nullptr;
-    ~Pinned() { if (p) cudaFreeHost(p); }
-  };
-  Pinned pin_states, pin_lists, pin_res;
-  RSFD_CK(h, cudaMallocHost(&pin_states.p, 2 * (W * sizeof(SlotState) + 64)));
-  RSFD_CK(h, cudaMallocHost(&pin_lists.p, 2 * (4 * W * sizeof(int) + W * sizeof(long long) + 64)));
-  if (final_res) RSFD_CK(h, cudaMallocHost(&pin_res.p, (size_t)ncols * K * sizeof(double) + 64));
+  // (kept by the handle between calls; page-locking costs about as much as a short solve's set-up)
+  PinBuf &pin_states = h->pin[0], &pin_lists = h->pin[1], &pin_res = h->pin[2];
+  RSFD_CK(h, pin_states.ensure(2 * (W * sizeof(SlotState) + 64)));
+  RSFD_CK(h, pin_lists.ensure(2 * (4 * W * sizeof(int) + W * sizeof(long long) + 64)));
+  if (final_res) RSFD_CK(h, pin_res.ensure((size_t)ncols * K * sizeof(double) + 64));
   auto states_of = [&](int par) -> SlotState* {
     return (SlotState*)((char*)pin_states.p + par * (W * sizeof(SlotState) + 64));
   };
@@ -1009,14 +1032,14 @@ static rsfd_status rsfd_shifted_cocg_impl(rsfd_handle h, const int64_t* cols, in
       for (auto& e : gr.ev[i]) RSFD_CK(h, cudaEventCreate(&e));
     }
   }
-  auto rec = [&](cudaEvent_t e) -> cudaError_t {
-    return use_graphs ? cudaEventRecordWithFlags(e, st, cudaEventRecordExternal) : cudaEventRecord(e, st);
-  };
-  auto issue_chunk = [&](int par) -> rsfd_status {
+  auto issue_chunk = [&](int par, bool captured) -> rsfd_status {
+    auto rec = [&](cudaEvent_t e) -> cudaError_t {
+      return captured ? cudaEventRecordWithFlags(e, st, cudaEventRecordExternal) : cudaEventRecord(e, st);
+    };
     std::vector<cudaEvent_t>& pev = gr.ev[par];
     for (int t = 0; t < C; ++t) {
       if (h->opts.profile) RSFD_CK(h, rec(pev[t]));
-      RSFD_CK(h, launch_pass(prec, d, b, coef, tol, maxit, C, st, split_ev ? pev[C + 2 + t] : nullptr, use_graphs));
+      RSFD_CK(h, launch_pass(prec, d, b, coef, tol, maxit, C, st, split_ev ? pev[C + 2 + t] : nullptr, captured));
       if (b.n_atoms > 0) RSFD_CK(h, launch_proj(prec, d, b, coef, tol, maxit, C, st));
     }
     if (h->opts.profile) RSFD_CK(h, rec(pev[C]));
@@ -1024,16 +1047,20 @@ static rsfd_status rsfd_shifted_cocg_impl(rsfd_handle h, const int64_t* cols, in
     if (h->opts.profile) RSFD_CK(h, rec(pev[C + 1]));
     return RSFD_OK;
   };
-  if (use_graphs) {
-    for (int i = 0; i < 2; ++i) {
+  // Chunk 0 is launched kernel by kernel; the host captures and instantiates the graph of the later chunks while it
+  // runs.  Without profiling events one graph serves both parities.
+  const int ngraphs = h->opts.profile ? 2 : 1;
+  auto capture_graphs = [&]() -> rsfd_status {
+    for (int i = 0; i < ngraphs; ++i) {
       RSFD_CK(h, cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-      rsfd_status cs = issue_chunk(i);
+      rsfd_status cs = issue_chunk(i, true);
       cudaError_t ce = cudaStreamEndCapture(st, &gr.g[i]);
       if (cs != RSFD_OK) return cs;
       RSFD_CK(h, ce);
       RSFD_CK(h, cudaGraphInstantiate(&gr.x[i], gr.g[i], 0));
     }
-  }
+    return RSFD_OK;
+  };
   // chunk k, followed by the copy of the slot states and the error flag into staging set k % 2
   cudaEvent_t copied[2] = {nullptr, nullptr};
   struct EvPair {
@@ -1043,15 +1070,15 @@ static rsfd_status rsfd_shifted_cocg_impl(rsfd_handle h, const int64_t* cols, in
   for (int i = 0; i < 2; ++i) RSFD_CK(h, cudaEventCreateWithFlags(&copied[i], cudaEventDisableTiming));
   auto launch_chunk_k = [&](long long k) -> rsfd_status {
     const int par = (int)(k & 1);
-    if (use_graphs) {
-      RSFD_CK(h, cudaGraphLaunch(gr.x[par], st));
+    if (use_graphs && k > 0) {
+      RSFD_CK(h, cudaGraphLaunch(gr.x[par < ngraphs ? par : 0], st));
     } else {
-      rsfd_status cs = issue_chunk(par);
+      rsfd_status cs = issue_chunk(par, false);
       if (cs != RSFD_OK) return cs;
     }
     h->stats.n_pass += (int64_t)C * (is_split(d.kind) ? 2 : 1);   // the split passes launch twice per iteration
     h->stats.n_shift += 1;
-    h->stats.n_other += 2 + (b.n_atoms > 0 ? 2 * C : 0);   // collapse coefficients, history reset, projectors
+    h->stats.n_other += 2 + (b.n_atoms > 0 ? 3 * C : 0);   // collapse coefficients, history reset, projectors
     RSFD_CK(h, cudaMemcpyAsync(states_of(par), b.slots, W * sizeof(SlotState), cudaMemcpyDeviceToHost, st));
     RSFD_CK(h, cudaMemcpyAsync(err_of(par), b.error_flag, sizeof(int), cudaMemcpyDeviceToHost, st));
     RSFD_CK(h, cudaEventRecord(copied[par], st));
@@ -1060,6 +1087,7 @@ static rsfd_status rsfd_shifted_cocg_impl(rsfd_handle h, const int64_t* cols, in
 
   int64_t iter_sum = 0;
   if ((s = launch_chunk_k(0)) != RSFD_OK) return s;
+  if (use_graphs && (s = capture_graphs()) != RSFD_OK) return s;
   for (long long k = 0;; ++k) {
     // enqueue chunk k + 1 before reading chunk k's states; a slot that finished in chunk k is idle in
     // chunk k + 1 (its kernels return at once), so its x_b is still final when it is written out

@@ -183,7 +183,6 @@ struct SolverBuffers {
   double2* pw;            // [W][n_atoms] -E_a c_a of the last pass (double-float handles: as a (hi, lo) float pair)
   double2* pcorr;         // [W][n_atoms] E_a c_a^2 / h^3
   double* pdots;          // [W][8] (r,r), (r, u_loc), ||r||^2 of the last pass
-  unsigned int* ptickets; // [W]
 };
 
 struct StencilCoef {
