@@ -137,9 +137,11 @@ typedef enum {
 /* Form of the Dyson solve (rsfd_solve_opts.dyson_kind). */
 typedef enum {
   RSFD_DYSON_AUTO = 0, /* RSFD_DYSON_TC for double-float and complex64 handles, RSFD_DYSON_FP64 for FP64 handles */
-  RSFD_DYSON_FP64 = 1, /* LU, triangular solves and refinement in FP64 on the CUDA cores */
-  RSFD_DYSON_TC = 2    /* LU and triangular solves in FP32 with their O(nb^3) updates on the tensor cores
-                          (3xTF32, rsfd_cgemm_tf32x3), FP64 residuals and corrections (iterative refinement) */
+  RSFD_DYSON_FP64 = 1, /* LU, triangular solves and refinement in FP64; the matrix products on the tensor cores as
+                          products of exact 8-bit digits, panels and substitution on the CUDA cores */
+  RSFD_DYSON_TC = 2    /* LU and triangular solves in FP32 with their O(nb^3) updates on the tensor cores (exact
+                          digits; rsfd_cgemm_tf32x3 when there is no memory for them), FP64 residuals and
+                          corrections (iterative refinement) */
 } rsfd_dyson_kind;
 
 /* Launch options of the solver; zero fields mean "choose automatically". */
@@ -205,8 +207,8 @@ typedef struct {
  *   proj      = NULL or the nonlocal projectors (host arrays, copied; entries of one atom at distinct
  *               grid points).  With projectors the solver uses a pass that stores A r (the
  *               stored-product pass or a split pass; RSFD_PASS_RECOMPUTE becomes RSFD_PASS_STORED):
- *               after each pass a projection kernel forms c_a = h^3 p_a^T r_n, corrects (r_n, A r_n)
- *               and runs the scalar step, and a scatter kernel adds -sum_a E_a c_a p_a to A r_n.
+ *               after each pass a projection kernel forms c_a = h^3 p_a^T r_n, a scalar kernel corrects
+ *               (r_n, A r_n) and runs the scalar step, and a scatter kernel adds -sum_a E_a c_a p_a to A r_n.
  *   precision = RSFD_FP64, RSFD_MIXED or RSFD_DF64.
  *   stream    = cudaStream_t for every device operation of this handle.
  * Returns RSFD_ERR_ARG on invalid sizes, RSFD_ERR_ALLOC / RSFD_ERR_CUDA on
@@ -342,9 +344,10 @@ rsfd_status rsfd_get_stats(rsfd_handle h, rsfd_stats* out);
  * for every k < K.  G0_bb must hold all boundary columns in b order
  * (ncols = nb).  The solve is an LU with partial pivoting followed by FP64
  * iterative refinement of the residual G0 - (I - G0 Sigma) G.  Form (rsfd_solve_opts.dyson_kind):
- * FP64 LU on the CUDA cores (FP64 handles by default), or FP32 LU and triangular solves whose
- * updates run on the tensor cores (3xTF32) with FP64 residuals (double-float and complex64 handles
- * by default); energies are processed in chunks that fit the free device memory.
+ * FP64 LU (FP64 handles by default), or FP32 LU and triangular solves with FP64 residuals (double-float
+ * and complex64 handles by default); in both the matrix products run on the tensor cores as products of exact
+ * digits (at FP64 or better than FP32 accuracy); the FP32 form processes energies in chunks that fit the free
+ * device memory.
  *   G0_bb    device [K][nb][nb] (handle precision).
  *   Sigma_L, Sigma_R  device [K][ns][ns] c128.
  *   G_bb     device output, same layout and type as G0_bb (may not alias G0_bb).
@@ -352,8 +355,8 @@ rsfd_status rsfd_get_stats(rsfd_handle h, rsfd_stats* out);
 rsfd_status rsfd_dyson_boundary(rsfd_handle h, const void* G0_bb, const void* Sigma_L, const void* Sigma_R,
                                 int32_t K, void* G_bb, double* refine_residual);
 
-/* Batched complex GEMM on the tensor cores: the building block of the Dyson solve's LU and triangular
- * solves (Eq. sec3-01a; see rsfd_dyson_boundary), exposed for direct use and testing.
+/* Batched complex FP32 GEMM on the tensor cores, for direct use; the Dyson solve (rsfd_dyson_boundary) falls back on
+ * it for its FP32 updates when the device has no memory for their digits.
  *   C[b] = alpha A[b] B[b] + beta C[b],  b < batch,
  * complex FP32 (interleaved re, im floats), column-major.  Every product is taken in 3xTF32 form
  * (hi*hi + hi*lo + lo*hi of the TF32 splits) with FP32 accumulation: FP32-class accuracy.

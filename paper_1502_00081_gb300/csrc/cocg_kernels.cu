@@ -1,7 +1,8 @@
 // Shifted COCG kernels for sm_103a.
 //
-// Seed iteration (Appendix, Eqs. rvec, alpha, beta).  One fused pass per iteration and right-hand
-// side ("slot") computes
+// Seed iteration (Appendix, Eqs. rvec, alpha, beta).  Four forms of the pass; the automatic one is the split
+// pass (combine_*_kernel, then stencil_kernel, further down).  The fused pass, once per iteration and
+// right-hand side ("slot"), computes
 //
 //   r_n = a1 r_{n-1} + a2 r_{n-2} + aA (A r_{n-1}),     A = Z_s - H_T,
 //   (r_n, r_n), (r_n, A r_n) (unconjugated bilinear form) and ||r_n||^2,
@@ -1953,7 +1954,8 @@ stencil_kernel(PassParams p, const __grid_constant__ CUtensorMap tmR, const __gr
   static_assert(!BFP || MODE == RSFD_DF64, "the block-floating-point pass is double-float only");
   constexpr bool LOG = MODE == RSFD_DF64;
   // The plain double-float stencil takes 320 instructions a point; unrolled over the 2R + 1 ring positions its loop
-  // does not fit the instruction cache (the first stall reason), so it moves the ring's registers instead.
+  // does not fit the instruction cache (the first stall reason), so it moves the ring's registers instead: 63
+  // iterations of 1024 slots of 16 x 16 x 48 in 39.2 instead of 44.3 ms.
   constexpr bool ROT = MODE == RSFD_DF64 && !BFP && R == 2;
   typedef Ops<MODE> O;
   typedef typename O::C C;
@@ -2271,8 +2273,9 @@ stencil_kernel(PassParams p, const __grid_constant__ CUtensorMap tmR, const __gr
 // the dot correction.  proj_scalar_kernel, one block per slot, sums the corrections in atom order and runs the FP64
 // scalar step.  pscatter_kernel: u_n -= sum_a E_a c_a p_a over the union of the supports, one thread per support point of
 // four slots gathering its atoms (point-major CSR), so no atomics and a fixed summation order.
-// Bound: latency of the gathers; four slots keep four in flight per thread.  16 slots of 72 x 72 x 256 with 460 atoms, one
-// slot per block or thread: 108 us + 44 us an iteration.
+// Bound: latency of the gathers; four slots keep four in flight per thread.  16 slots of 72 x 72 x 256 with 460 atoms:
+// 59 + 24 + 41 us an iteration (one slot per block or thread, scalar step in the gather: 108 + 44; 95 iterations of the whole
+// solve 79.1 -> 75.4 ms).
 // ------------------------------------------------------------------------------------------------
 constexpr int kProjSlots = 4;
 struct ProjParams {

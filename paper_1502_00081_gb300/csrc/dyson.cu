@@ -322,10 +322,10 @@ __global__ void set_f32_to_c128(double2* y, const float2* x, long long n) {
 }
 
 // Tensor-core form of the Dyson step, energies processed in chunks that fit the device:
-//   M = I - G0 Sigma                       FP64 (CUDA cores)
-//   F = P L U of M in FP32                 panels on the CUDA cores, trailing updates 3xTF32 (tcgen05)
-//   X = F^{-1} G0                          blocked triangular solves, updates 3xTF32 (tcgen05)
-//   nref times: R = G0 - M X (FP64), X += F^{-1} R
+//   M = I - G0 Sigma                       FP64 (sliced products)
+//   F = P L U of M in FP32                 panels on the CUDA cores, trailing updates sliced (tcgen05)
+//   X = F^{-1} G0                          blocked triangular solves, updates sliced (tcgen05)
+//   nref times: R = G0 - M X (FP64, sliced), X += F^{-1} R
 // Reported residual ||G0 - M X|| / ||G0|| is the FP64 one after the last correction.
 rsfd_status dyson_tc_run(Handle* h, const void* G0, const void* SL, const void* SR, int K, void* G, double* refres) {
   const int nb = handle_nb(h);
