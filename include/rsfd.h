@@ -109,8 +109,9 @@ typedef struct {
 
 /* Form of the seed iteration's pass (rsfd_solve_opts.pass_kind). */
 typedef enum {
-  RSFD_PASS_AUTO = 0,      /* RSFD_PASS_SPLIT on tiles cut to the grid when the options are not tuned (double-float: with
-                              the sums in RSFD_PASS_STORED's blocks, so the two agree bit for bit), RSFD_PASS_STORED
+  RSFD_PASS_AUTO = 0,      /* RSFD_PASS_SPLIT on tiles cut to the grid when the options are not tuned (double-float and
+                              complex64: with the sums in RSFD_PASS_STORED's blocks, so the two agree bit for bit; FP64:
+                              sums in other blocks, the two agree to FP64 round-off), RSFD_PASS_STORED
                               when tile_y, tile_x = 16, rows_per_thread > 1, reg_budget or prefetch is given;
                               rsfd_autotune times every form (on the 64^2 x 128 workload it picks
                               RSFD_PASS_SPLIT_BFP for double-float) */

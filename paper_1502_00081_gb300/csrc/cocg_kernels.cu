@@ -520,6 +520,16 @@ struct AccDF {
     addprod(ra_s, ra_l, make_float2(-rh.y, rh.y), make_float2(-rl.y, rl.y), make_float2(v.h.y, v.h.x),
             make_float2(v.l.y, v.l.x));
   }
+  // one thread's (r, A r) sum, to shared memory and back; and its (r, r) as a leading and a trailing part
+  __device__ __forceinline__ float4 ra_state() const { return make_float4(ra_s.x, ra_s.y, ra_l.x, ra_l.y); }
+  __device__ __forceinline__ void set_ra(float4 v) {
+    ra_s = make_float2(v.x, v.y);
+    ra_l = make_float2(v.z, v.w);
+  }
+  __device__ __forceinline__ void rr_pair(float2& s, float2& l) const {
+    s = rr_s;
+    l = rr_l;
+  }
   static __device__ __forceinline__ float2 shfl2(float2 v, int o) {
     return make_float2(__shfl_down_sync(0xffffffffu, v.x, o), __shfl_down_sync(0xffffffffu, v.y, o));
   }
@@ -568,6 +578,23 @@ struct AccK {
     kahan(ra, ra_c, tra);
     nn = __fmaf_rn(r.x, r.x, __fmaf_rn(r.y, r.y, nn));
   }
+  // the split pass's halves of add(): the same products and sums
+  __device__ __forceinline__ void add_r(float2 r) {
+    kahan(rr, rr_c, make_float2(__fmaf_rn(r.x, r.x, -r.y * r.y), 2.f * r.x * r.y));
+    nn = __fmaf_rn(r.x, r.x, __fmaf_rn(r.y, r.y, nn));
+  }
+  __device__ __forceinline__ void add_ra(float2 r, float2 v) {
+    kahan(ra, ra_c, make_float2(__fmaf_rn(r.x, v.x, -r.y * v.y), __fmaf_rn(r.x, v.y, r.y * v.x)));
+  }
+  __device__ __forceinline__ float4 ra_state() const { return make_float4(ra.x, ra.y, ra_c.x, ra_c.y); }
+  __device__ __forceinline__ void set_ra(float4 v) {
+    ra = make_float2(v.x, v.y);
+    ra_c = make_float2(v.z, v.w);
+  }
+  __device__ __forceinline__ void rr_pair(float2& s, float2& l) const {
+    s = rr;
+    l = f2neg(rr_c);
+  }
   // The Kahan pairs (s, -c) are double-float values: reduce them over the warp with TwoSum merges
   // (whole warps only) and convert once; lane 0 returns the warp's sums, the other lanes zeros.
   __device__ __forceinline__ void get(double* o) {
@@ -588,36 +615,9 @@ struct AccK {
   }
 };
 
-// complex64 vectors in the split pass: the products are formed exactly (FMA) and summed in double-float, as for
-// double-float vectors without their low parts.  The split kernels are not bound by this arithmetic, and rounded
-// products can keep a solve at small eta from ever reaching its tolerance.
-struct AccX {
-  AccDF a;
-  static __device__ __forceinline__ void addprod(float2& s, float2& l, float2 x, float2 y) {
-    const float2 p = f2mul(x, y);
-    const float2 ne = f2fma(f2neg(x), y, p);   // p - x y, exact
-    float2 t, te;
-    two_sum2(s, p, t, te);
-    s = t;
-    l = f2add(l, f2sub(te, ne));
-  }
-  __device__ __forceinline__ void add_r(float2 r) {
-    addprod(a.rr_s, a.rr_l, bc(r.x), r);
-    addprod(a.rr_s, a.rr_l, make_float2(-r.y, r.y), make_float2(r.y, r.x));
-    a.nn = __fmaf_rn(r.x, r.x, __fmaf_rn(r.y, r.y, a.nn));
-  }
-  __device__ __forceinline__ void add_ra(float2 r, float2 v) {
-    addprod(a.ra_s, a.ra_l, bc(r.x), v);
-    addprod(a.ra_s, a.ra_l, make_float2(-r.y, r.y), make_float2(v.y, v.x));
-  }
-  __device__ __forceinline__ void get(double* o) { a.get(o); }
-};
-
 template <int MODE> struct AccOf { typedef AccDF type; };
 template <> struct AccOf<RSFD_MIXED> { typedef AccK type; };
 template <> struct AccOf<RSFD_FP64> { typedef Acc<double> type; };
-template <int MODE> struct AccSplit { typedef typename AccOf<MODE>::type type; };   // the split pass's
-template <> struct AccSplit<RSFD_MIXED> { typedef AccX type; };
 
 // index of plane z among the recorded planes (boundary planes, then the tracked interior planes),
 // -1 when its rows are not recorded
@@ -1667,18 +1667,18 @@ template <> struct Requant<true, dfc> {
   static __device__ __forceinline__ float amax(const dfc& x) { return fmaxf(fabsf(x.h.x), fabsf(x.h.y)); }
 };
 
-// Combine over a contiguous range (block blockIdx.x of d.ctas_c) of one slot's padded elements (planes are not a unit,
-// so small planes fill the threads too), in 16-byte units (one element, or two of complex64); each thread handles
-// two units per step, so that six 16-byte loads are in flight.  Coordinates are only formed where they are
-// needed: x in padded rows, all of them in the planes whose rows are recorded.
-template <int MODE> __global__ void __launch_bounds__(kCombThreads, 4) combine_kernel(PassParams p) {
+// Combine of FP64 vectors over a contiguous range (block blockIdx.x of d.ctas_c) of one slot's padded elements (planes are
+// not a unit, so small planes fill the threads too); each thread handles two elements per step, so that six 16-byte loads are
+// in flight.  Coordinates are only formed where they are needed: x in padded rows, all of them in the planes whose rows
+// are recorded.
+__global__ void __launch_bounds__(kCombThreads, 4) combine_kernel(PassParams p) {
   const int slot = blockIdx.y, cblk = blockIdx.x;
-  typedef Ops<MODE> O;
-  typedef Stencil<MODE, 1> ST;   // combine() does not depend on the stencil reach
-  typedef typename O::C C;
-  typedef typename O::H H;
+  typedef Ops<RSFD_FP64> O;
+  typedef Stencil<RSFD_FP64, 1> ST;   // combine() does not depend on the stencil reach
+  typedef O::C C;
+  typedef O::H H;
   __shared__ double s_red[32 * 5];
-  __shared__ typename O::Cplx s_a[3];
+  __shared__ O::Cplx s_a[3];
   __shared__ int s_n, s_hc;
   const SlotState* st = p.slots + slot;
   if (st->status != SLOT_RUNNING) return;
@@ -1689,31 +1689,28 @@ template <int MODE> __global__ void __launch_bounds__(kCombThreads, 4) combine_k
     s_hc = st->hcnt;
   }
   __syncthreads();
-  const typename O::Cplx a1 = s_a[0], a2 = s_a[1], aA = s_a[2];
+  const O::Cplx a1 = s_a[0], a2 = s_a[1], aA = s_a[2];
   const int n = s_n;
   const int i1 = (n + 2) % 3, i2 = (n + 1) % 3, io = n % 3, iu1 = 3 + (n + 1) % 2;
   const int pe = d.nxp * d.ny;   // padded elements per plane
-  const long long vec = (long long)d.nz * pe;
+  const long long vec = (long long)d.nz * pe;   // below 2^32: five such vectors fit the device's memory
   const C* R1 = reinterpret_cast<const C*>(p.rbuf) + ((size_t)slot * 5 + i1) * vec;
   const C* R2 = reinterpret_cast<const C*>(p.rbuf) + ((size_t)slot * 5 + i2) * vec;
   const C* U1 = reinterpret_cast<const C*>(p.rbuf) + ((size_t)slot * 5 + iu1) * vec;
   C* RO = reinterpret_cast<C*>(p.rbuf) + ((size_t)slot * 5 + io) * vec;
   H* hist = reinterpret_cast<H*>(p.rhist) + ((size_t)slot * p.hist_len + s_hc) * d.nb;
-  constexpr int U = 16 / sizeof(C);   // elements per unit (vec is a multiple of 4)
-  const long long nu = vec / U;         // below 2^32: five such vectors fit the device's memory
-  const unsigned lo = (unsigned)(nu * cblk / d.ctas_c), hi = (unsigned)(nu * (cblk + 1) / d.ctas_c);
+  const unsigned lo = (unsigned)(vec * cblk / d.ctas_c), hi = (unsigned)(vec * (cblk + 1) / d.ctas_c);
   // elements from which planes are not recorded, and from which they are again
   const long long in0 = (long long)d.nface * pe, in1 = (long long)(d.nz - d.nface) * pe;
-  const bool padded = d.nxp != d.nx, small = vec < (1ll << 32);
-  typename AccSplit<MODE>::type acc;
-  struct alignas(16) Unit {
-    C c[U];
-  };
-  auto finish = [&](long long e, const C& r) {
+  const bool padded = d.nxp != d.nx;
+  Acc<double> acc;
+  auto element = [&](unsigned e, const C& r1, const C& r2, const C& u1) {
+    const C r = ST::combine(a1, r1, a2, r2, aA, u1);   // Eq. rvec
+    RO[e] = r;
     const bool rec = e < in0 || e >= in1 || d.ntrack > 0;
     if (padded || rec) {
-      const unsigned row = small ? (unsigned)e / (unsigned)d.nxp : (unsigned)(e / d.nxp);
-      const int x = (int)(e - (long long)row * d.nxp);
+      const unsigned row = e / (unsigned)d.nxp;
+      const int x = (int)(e - row * (unsigned)d.nxp);
       if (x >= d.nx) return;   // row padding
       if (rec) {
         const int z = (int)(row / (unsigned)d.ny), y = (int)(row - (unsigned)z * (unsigned)d.ny);
@@ -1723,30 +1720,14 @@ template <int MODE> __global__ void __launch_bounds__(kCombThreads, 4) combine_k
     }
     acc.add_r(r);
   };
-  auto unit = [&](unsigned u, const Unit& r1, const Unit& r2, const Unit& u1) {
-    if constexpr (U == 1) {
-      const C r = ST::combine(a1, r1.c[0], a2, r2.c[0], aA, u1.c[0]);   // Eq. rvec
-      RO[u] = r;
-      finish(u, r);
-    } else {
-      Unit r;
-#pragma unroll
-      for (int k = 0; k < U; ++k) r.c[k] = ST::combine(a1, r1.c[k], a2, r2.c[k], aA, u1.c[k]);
-      reinterpret_cast<Unit*>(RO)[u] = r;
-#pragma unroll
-      for (int k = 0; k < U; ++k) finish((long long)u * U + k, r.c[k]);
-    }
-  };
-  const Unit *P1 = reinterpret_cast<const Unit*>(R1), *P2 = reinterpret_cast<const Unit*>(R2),
-             *PU = reinterpret_cast<const Unit*>(U1);
-  for (unsigned u = lo + threadIdx.x; u < hi; u += 2 * kCombThreads) {
-    const unsigned u2 = u + kCombThreads;   // may lie past the range
-    const bool has2 = u2 < hi;
-    const Unit r1a = P1[u], r2a = P2[u], ua = PU[u];
-    Unit r1b = r1a, r2b = r2a, ub = ua;
-    if (has2) { r1b = P1[u2]; r2b = P2[u2]; ub = PU[u2]; }
-    unit(u, r1a, r2a, ua);
-    if (has2) unit(u2, r1b, r2b, ub);
+  for (unsigned e = lo + threadIdx.x; e < hi; e += 2 * kCombThreads) {
+    const unsigned e2 = e + kCombThreads;   // may lie past the range
+    const bool has2 = e2 < hi;
+    const C r1a = R1[e], r2a = R2[e], ua = U1[e];
+    C r1b = r1a, r2b = r2a, ub = ua;
+    if (has2) { r1b = R1[e2]; r2b = R2[e2]; ub = U1[e2]; }
+    element(e, r1a, r2a, ua);
+    if (has2) element(e2, r1b, r2b, ub);
   }
   double v5[5];
   acc.get(v5);
@@ -1758,19 +1739,19 @@ template <int MODE> __global__ void __launch_bounds__(kCombThreads, 4) combine_k
   }
 }
 
-// Combine with its sums, double-float: CTA = 256 threads over a range of z-planes (block blockIdx.x of d.ctas_c); each
+// Combine with its sums, double-float and complex64: CTA = 256 threads over a range of z-planes (block blockIdx.x of d.ctas_c); each
 // thread walks the plane's padded elements with stride 256 (x, y tracked by a running counter), two elements per
 // step so that six 16-byte loads are in flight.  The ranges and this order fix the rounding of (r_n, r_n).
 // At most 64 registers: four CTAs (32 warps) per SM keep enough loads in flight for HBM.
-template <bool BFP> __global__ void __launch_bounds__(kCombThreads, 4) combine_planes_kernel(PassParams p) {
-  typedef Ops<RSFD_DF64> O;
-  typedef Stencil<RSFD_DF64, 1> ST;   // combine() does not depend on the stencil reach
+template <int MODE, bool BFP> __global__ void __launch_bounds__(kCombThreads, 4) combine_planes_kernel(PassParams p) {
+  typedef Ops<MODE> O;
+  typedef Stencil<MODE, 1> ST;   // combine() does not depend on the stencil reach
   const int slot = blockIdx.y, cblk = blockIdx.x;
-  typedef O::C C;
-  typedef O::H H;
+  typedef typename O::C C;
+  typedef typename O::H H;
   typedef Requant<BFP, C> RQ;
   __shared__ double s_red[32 * 5];
-  __shared__ O::Cplx s_a[3];
+  __shared__ typename O::Cplx s_a[3];
   __shared__ int s_n, s_hc;
   __shared__ float s_cq;
   const SlotState* st = p.slots + slot;
@@ -1785,7 +1766,7 @@ template <bool BFP> __global__ void __launch_bounds__(kCombThreads, 4) combine_p
     s_cq = BFP ? (float)(1.5 * 8388608.0 * st->q) : 0.f;
   }
   __syncthreads();
-  const O::Cplx a1 = s_a[0], a2 = s_a[1], aA = s_a[2];
+  const typename O::Cplx a1 = s_a[0], a2 = s_a[1], aA = s_a[2];
   const float2 cq = make_float2(s_cq, s_cq);
   float mxr = 0.f;
   const int n = s_n;
@@ -1803,7 +1784,7 @@ template <bool BFP> __global__ void __launch_bounds__(kCombThreads, 4) combine_p
   const int tid = threadIdx.x;
   const int nthr = blockDim.x;
   const int dx = nthr % d.nxp, dy = nthr / d.nxp;
-  AccDF acc;
+  typename AccOf<MODE>::type acc;
   for (int z = za; z < zb; ++z) {
     const long long zo = (long long)z * pe;
     const int pl = recorded_plane(d, z);
@@ -1855,23 +1836,26 @@ template <bool BFP> __global__ void __launch_bounds__(kCombThreads, 4) combine_p
   }
 }
 
-// Combine with its sums in the stored pass's blocks, double-float: CTA = one block of 32 x lty columns and a z-chunk, a
-// thread a column, two planes per step (six 16-byte loads in flight; a warp reads rows of 512 bytes).  Grids of at most
-// 16 (8) columns put two (four) rows into a warp: the missing columns of a row add zeros, which change no sum.
-__global__ void __launch_bounds__(kCombThreads, 4) combine_blocks_kernel(PassParams p) {
-  typedef Ops<RSFD_DF64> O;
-  typedef Stencil<RSFD_DF64, 1> ST;
+// Combine with its sums in the stored pass's blocks, double-float and complex64: CTA = one block of 32 x lty columns and a
+// z-chunk, a thread a column, two (complex64: four) planes per step, so that six 16-byte (twelve 8-byte) loads are in flight; a
+// warp reads rows of 512 (256) bytes.  Grids of at most 16 (8) columns put two (four) rows into a warp: the missing columns
+// of a row add zeros, which change no sum.
+template <int MODE> __global__ void __launch_bounds__(kCombThreads, 4) combine_blocks_kernel(PassParams p) {
+  typedef Ops<MODE> O;
+  typedef Stencil<MODE, 1> ST;
+  typedef typename O::C C;
+  constexpr int NP = MODE == RSFD_MIXED ? 4 : 2;   // planes per step
   const int slot = blockIdx.y, cta = blockIdx.x;
   const SlotState* st = p.slots + slot;
   if (st->status != SLOT_RUNNING) return;
-  __shared__ O::Cplx s_a[3];
+  __shared__ typename O::Cplx s_a[3];
   __shared__ double s_rows[8 * 3];
   const SolveDims& d = p.d;
   const int tid = threadIdx.x, lane = tid & 31;
   if (tid < 3) s_a[tid] = O::cplx(tid == 0 ? st->a1 : (tid == 1 ? st->a2 : st->aA));
   const int n = st->n, hc = st->hcnt;
   __syncthreads();
-  const O::Cplx a1 = s_a[0], a2 = s_a[1], aA = s_a[2];
+  const typename O::Cplx a1 = s_a[0], a2 = s_a[1], aA = s_a[2];
   const int hw = d.nx <= 8 ? 4 : (d.nx <= 16 ? 2 : 1), wd = 32 / hw;   // rows and columns per warp
   const int ltx = (d.nx + 31) / 32;
   const int tz = cta % d.nzchunks, txy = cta / d.nzchunks;
@@ -1880,45 +1864,48 @@ __global__ void __launch_bounds__(kCombThreads, 4) combine_blocks_kernel(PassPar
   const int z0 = tz * d.zchunk, z1 = min(z0 + d.zchunk, d.nz);
   const bool own = x < d.nx && y < d.ny && row < d.lty;
   const long long pe = (long long)d.nxp * d.ny, vec = d.nz * pe, o = z0 * pe + (long long)y * d.nxp + x;
-  dfc* base = reinterpret_cast<dfc*>(p.rbuf) + (size_t)slot * 5 * vec + o;
-  const dfc *R1 = base + ((n + 2) % 3) * vec, *R2 = base + ((n + 1) % 3) * vec, *U1 = base + (3 + (n + 1) % 2) * vec;
-  dfc* RO = base + (n % 3) * vec;
+  C* base = reinterpret_cast<C*>(p.rbuf) + (size_t)slot * 5 * vec + o;
+  const C *R1 = base + ((n + 2) % 3) * vec, *R2 = base + ((n + 1) % 3) * vec, *U1 = base + (3 + (n + 1) % 2) * vec;
+  C* RO = base + (n % 3) * vec;
   float2* hist = reinterpret_cast<float2*>(p.rhist) + ((size_t)slot * p.hist_len + hc) * d.nb + (size_t)y * d.nx + x;
   const size_t nxy = (size_t)d.nx * d.ny;
-  AccDF acc;
+  typename AccOf<MODE>::type acc;
   if (own) {
-    for (int z = z0; z < z1; z += 2) {
-      const bool has2 = z + 1 < z1;
-      const dfc r1a = R1[0], r2a = R2[0], ua = U1[0];
-      dfc r1b = r1a, r2b = r2a, ub = ua;
-      if (has2) { r1b = R1[pe]; r2b = R2[pe]; ub = U1[pe]; }
-      const dfc ra = ST::combine(a1, r1a, a2, r2a, aA, ua);   // Eq. rvec
-      RO[0] = ra;
-      acc.add_r(ra);
-      int pl = recorded_plane(d, z);
-      if (pl >= 0) hist[pl * nxy] = ra.h;
-      if (has2) {
-        const dfc rb = ST::combine(a1, r1b, a2, r2b, aA, ub);
-        RO[pe] = rb;
-        acc.add_r(rb);
-        pl = recorded_plane(d, z + 1);
-        if (pl >= 0) hist[pl * nxy] = rb.h;
+    for (int z = z0; z < z1; z += NP) {
+      C r1[NP] = {}, r2[NP] = {}, u1[NP] = {};
+#pragma unroll
+      for (int k = 0; k < NP; ++k) {
+        r1[k] = r1[0];   // past the chunk: not used
+        r2[k] = r2[0];
+        u1[k] = u1[0];
+        if (k == 0 || z + k < z1) { r1[k] = R1[k * pe]; r2[k] = R2[k * pe]; u1[k] = U1[k * pe]; }
       }
-      R1 += 2 * pe;
-      R2 += 2 * pe;
-      U1 += 2 * pe;
-      RO += 2 * pe;
+#pragma unroll
+      for (int k = 0; k < NP; ++k)
+        if (z + k < z1) {
+          const C r = ST::combine(a1, r1[k], a2, r2[k], aA, u1[k]);   // Eq. rvec
+          RO[k * pe] = r;
+          acc.add_r(r);
+          const int pl = recorded_plane(d, z + k);
+          if (pl >= 0) hist[pl * nxy] = O::hi(r);
+        }
+      R1 += NP * pe;
+      R2 += NP * pe;
+      U1 += NP * pe;
+      RO += NP * pe;
     }
   }
   // a row's columns in the fixed tree of a whole warp (narrower groups skip its steps over zeros), then the rows
+  float2 rs, rl;
+  acc.rr_pair(rs, rl);
   for (int off = wd / 2; off > 0; off >>= 1) {
-    const float2 a = AccDF::shfl2(acc.rr_s, off), b = AccDF::shfl2(acc.rr_l, off);
-    AccDF::merge(acc.rr_s, acc.rr_l, a, b);
+    const float2 a = AccDF::shfl2(rs, off), b = AccDF::shfl2(rl, off);
+    AccDF::merge(rs, rl, a, b);
     acc.nn += __shfl_down_sync(0xffffffffu, acc.nn, off);
   }
   if (lane % wd == 0 && row < d.lty) {
-    s_rows[row * 3] = (double)acc.rr_s.x + (double)acc.rr_l.x;
-    s_rows[row * 3 + 1] = (double)acc.rr_s.y + (double)acc.rr_l.y;
+    s_rows[row * 3] = (double)rs.x + (double)rl.x;
+    s_rows[row * 3 + 1] = (double)rs.y + (double)rl.y;
     s_rows[row * 3 + 2] = (double)acc.nn;
   }
   __syncthreads();
@@ -1938,21 +1925,22 @@ __global__ void __launch_bounds__(kCombThreads, 4) combine_blocks_kernel(PassPar
 // There is no CTA-wide barrier per plane: a stage has a "full" mbarrier (the TMA bytes) and an "empty" one
 // on which each warp arrives when it is done with it; thread 0 refills (an extra warp for that would cost a
 // quarter of the register file's third warp slot per scheduler: 96 registers a thread instead of 128).
-// Double-float vectors (LOG): the rounding of the sums is that of blocks of 32 x d.lty columns and a z-chunk (a warp a
-// row, the rows in order), whatever tile the CTA has: a tile is made of such blocks, every column keeps its own
-// accumulators over the z-range, and they are added in that order at the end.
+// Double-float and complex64 vectors (LOG): the rounding of the sums is that of blocks of 32 x d.lty columns and a z-chunk (a
+// warp a row, the rows in order), whatever tile the CTA has: a tile is made of such blocks, every column keeps its own
+// accumulators over the z-range, and they are added in that order at the end.  The recurrence amplifies a changed last bit
+// of a sum to 1e-8 of G0_bb in double-float and to 1e-5 (single elements: 1e-3 of the rms) in complex64.
 // BFP (double-float handles): the r_n it reads has block-floating-point leading parts, tmV maps s V, and it
 // stores u_n = s A r_n (StencilBFP) with the largest leading-part component of u_n.
 constexpr int kMaxStagesS = kMaxDepth + 3;
 constexpr int kStencilThreads = 256;
-constexpr int kMaxRowSums = 128;   // rows of 32 columns in a double-float tile (at most 60 wide, 512 points)
+constexpr int kMaxRowSums = 128;   // rows of 32 columns in a tile made of blocks (at most 60 wide, 512 points)
 
 // Two 256-thread CTAs per SM (128 registers): three (80 registers) spill 90 bytes a point and were 1.6 times slower.
 template <int MODE, int R, bool BFP>
 __global__ void __launch_bounds__(kStencilThreads, MODE == RSFD_MIXED ? 3 : 2)
 stencil_kernel(PassParams p, const __grid_constant__ CUtensorMap tmR, const __grid_constant__ CUtensorMap tmV) {
   static_assert(!BFP || MODE == RSFD_DF64, "the block-floating-point pass is double-float only");
-  constexpr bool LOG = MODE == RSFD_DF64;
+  constexpr bool LOG = MODE != RSFD_FP64;
   // The plain double-float stencil takes 320 instructions a point; unrolled over the 2R + 1 ring positions its loop
   // does not fit the instruction cache (the first stall reason), so it moves the ring's registers instead: 63
   // iterations of 1024 slots of 16 x 16 x 48 in 39.2 instead of 44.3 ms.
@@ -2021,7 +2009,7 @@ stencil_kernel(PassParams p, const __grid_constant__ CUtensorMap tmR, const __gr
     s_abort = 1;
     atomicExch(p.error_flag, 1);
   };
-  typename AccSplit<MODE>::type acc[LOG ? 2 : 1];   // LOG: one per row
+  typename AccOf<MODE>::type acc[LOG ? 2 : 1];   // LOG: one per row
   float mxu = 0.f;
   int issued = 0;   // thread 0: bundles issued
   {
@@ -2191,19 +2179,14 @@ stencil_kernel(PassParams p, const __grid_constant__ CUtensorMap tmR, const __gr
   if constexpr (LOG) {
     // rows of 32 columns, one warp each: the 32 columns' sums in a fixed tree, then the rows of a block in order
     __shared__ double s_rows[kMaxRowSums * 2];
-    for (int k = 0; k < 2; ++k) accA[k * nthr + tid] = make_float4(acc[k].ra_s.x, acc[k].ra_s.y, acc[k].ra_l.x, acc[k].ra_l.y);
+    for (int k = 0; k < 2; ++k) accA[k * nthr + tid] = acc[k].ra_state();
     __syncthreads();
     const int lty = d.lty, nlx = (xend - x0 + 31) / 32, nly = (d.rows_cta + lty - 1) / lty, nseg = nlx * TY;
     const int lane = tid & 31;
     for (int g = tid >> 5; g < nseg; g += nthr >> 5) {
       const int row = g / nlx, x = (g - row * nlx) * 32 + lane;
-      AccDF a;
-      if (x < TX && x < xend - x0) {
-        const int t = (row >> 1) * TX + x, k = row & 1;
-        const float4 v = accA[k * nthr + t];
-        a.ra_s = make_float2(v.x, v.y);
-        a.ra_l = make_float2(v.z, v.w);
-      }
+      typename AccOf<MODE>::type a;
+      if (x < TX && x < xend - x0) a.set_ra(accA[(row & 1) * nthr + (row >> 1) * TX + x]);
       double o[5];
       a.get(o);
       if (lane == 0) {
@@ -2805,12 +2788,15 @@ cudaError_t launch_pass_t(const SolveDims& d, const SolverBuffers& b, const Sten
   dim3 grid(d.ctas_per_slot, d.W);
   if (d.kind == RSFD_PASS_SPLIT || d.kind == RSFD_PASS_SPLIT_BFP) {
     const dim3 gc(d.ctas_c, d.W);
-    if constexpr (MODE == RSFD_DF64) {
-      if (bfp) combine_planes_kernel<true><<<gc, kCombThreads, 0, st>>>(p);
-      else if (d.rr_blocks) combine_blocks_kernel<<<gc, block_threads(d.nx, d.lty), 0, st>>>(p);
-      else combine_planes_kernel<false><<<gc, kCombThreads, 0, st>>>(p);
+    if constexpr (MODE == RSFD_FP64) {
+      combine_kernel<<<gc, kCombThreads, 0, st>>>(p);
+    } else if (d.rr_blocks) {
+      combine_blocks_kernel<MODE><<<gc, block_threads(d.nx, d.lty), 0, st>>>(p);
+    } else if constexpr (MODE == RSFD_DF64) {
+      if (bfp) combine_planes_kernel<MODE, true><<<gc, kCombThreads, 0, st>>>(p);
+      else combine_planes_kernel<MODE, false><<<gc, kCombThreads, 0, st>>>(p);
     } else {
-      combine_kernel<MODE><<<gc, kCombThreads, 0, st>>>(p);
+      combine_planes_kernel<MODE, false><<<gc, kCombThreads, 0, st>>>(p);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -2868,15 +2854,15 @@ size_t split_smem(int prec, int R, int tile_x, int tile_y, int depth) {
   // per TMA stage the box of r_n and the tile of the potential
   const size_t vs = prec == RSFD_MIXED ? 4 : 8;
   const size_t pv = ((size_t)tile_x * tile_y * vs + 127) & ~(size_t)127;
-  // double-float: two rows' accumulators per thread
-  const size_t ac = prec == RSFD_DF64 ? (size_t)split_threads(tile_x, tile_y) * 2 * 16 : 0;
+  // double-float and complex64: two rows' accumulators per thread
+  const size_t ac = prec != RSFD_FP64 ? (size_t)split_threads(tile_x, tile_y) * 2 * 16 : 0;
   return (size_t)(depth + R + 1) * (pb + pv) + ac + 128;
 }
 // Combine CTAs per slot.  Plain ranges: by the vector's length alone, so that a column's sums do not depend on how
 // many columns run beside it: 2048 16-byte units per CTA (four steps of its 256 threads), at most 64 CTAs (longer
 // ranges from there on).
-int split_combine_ctas(int prec, long long vec) {
-  const long long c = vec * (prec == RSFD_MIXED ? 8 : 16) / (2048 * 16);
+int split_combine_ctas(long long vec) {
+  const long long c = vec / 2048;
   return (int)(c < 1 ? 1 : (c > 64 ? 64 : c));
 }
 // Ranges of planes (double-float, with its sums): about eight 256-thread CTAs per SM over all slots, at least one

@@ -281,19 +281,19 @@ static int resolve_kind(int prec, const rsfd_solve_opts& o) {
   return shaped ? RSFD_PASS_STORED : RSFD_PASS_SPLIT;
 }
 
-// Width of the split pass's tiles for rows of nx points in tiles of at most `most`: equal tiles, rounded up to the
-// 16-byte granularity of the TMA boxes (4 points of a float potential, 2 of the others).
-static int split_tile_x(int prec, int nx, int most) {
-  const int g = prec == RSFD_MIXED ? 4 : 2, n = (nx + most - 1) / most;
-  return ((nx + n - 1) / n + g - 1) / g * g;
+// Width of the FP64 split pass's tiles for rows of nx points in tiles of at most `most`: equal tiles, rounded up to the
+// 16-byte granularity of the TMA boxes (2 points of the potential).
+static int split_tile_x(int nx, int most) {
+  const int n = (nx + most - 1) / most;
+  return ((nx + n - 1) / n + 1) / 2 * 2;
 }
 
-// Tile of the split pass when it is not given: equal tiles with at most 512 points, by the fewest thread slots per
+// Tile of the FP64 split pass when it is not given: equal tiles with at most 512 points, by the fewest thread slots per
 // grid point (ragged edges, partly filled warps), a tenth of the halo's share and a quarter warp per CTA.
-static void split_tile(int prec, int R, int nx, int ny, int& tx, int& ty) {
+static void split_tile(int R, int nx, int ny, int& tx, int& ty) {
   double best = 1e30;
   for (int nt = 1; nt <= nx; ++nt) {
-    const int X = split_tile_x(prec, nx, (nx + nt - 1) / nt);
+    const int X = split_tile_x(nx, (nx + nt - 1) / nt);
     if (X > 60) continue;
     if (X < 8 && nt > 1) break;
     for (int mt = 1; mt <= ny; ++mt) {
@@ -313,15 +313,16 @@ static void split_tile(int prec, int R, int nx, int ny, int& tx, int& ty) {
   }
 }
 
-// Tile of the double-float split pass, made of summation blocks of 32 x lty columns: the x-remainder joins the last
-// tile when that stays within 60 columns (TMA box), and blocks are stacked in y while the tile keeps at most
-// 256 threads (two points each) and half the rows are used.
-static void split_tile_blocks(int nx, int ny, int lty, int& tx, int& ty) {
-  const int rem = nx % 32;
+// Tile of the double-float and complex64 split pass, made of summation blocks of 32 x lty columns: the x-remainder joins
+// the last tile when that stays within 60 columns (TMA box), and blocks are stacked in y while the tile keeps at most
+// 256 threads (two points each) and half the rows are used.  Widths are multiples of the TMA boxes' 16 bytes (4 points of a
+// float potential, 2 of a double-float one).
+static void split_tile_blocks(int prec, int nx, int ny, int lty, int& tx, int& ty) {
+  const int rem = nx % 32, g = prec == RSFD_MIXED ? 4 : 2;
   ty = (lty + 1) / 2 * 2;
-  tx = std::min(32, (nx + 1) / 2 * 2);
+  tx = std::min(32, (nx + g - 1) / g * g);
   if (nx > 32 && rem > 0 && rem <= 28) {
-    const int wide = 32 + (rem + 1) / 2 * 2;
+    const int wide = 32 + (rem + g - 1) / g * g;
     if (wide * ty <= split_max_points()) tx = wide;
   }
   if (lty % 2 == 0)
@@ -772,21 +773,20 @@ static rsfd_status rsfd_shifted_cocg_impl(rsfd_handle h, const int64_t* cols, in
   d.tile_x = (h->opts.tile_x == 16 && d.kind == RSFD_PASS_STORED) ? 16 : 32;
   if (!tile_ok(prec, h->R, d.tile_y, d.kind, d.rows, d.regs, d.tile_x))
     return fail(h, RSFD_ERR_ARG, "rsfd_shifted_cocg: invalid tile_y / tile_x");
-  // Double-float: the split pass that replaces the stored one (automatic pass) forms every sum in the stored pass's
-  // blocks (32 x tile_y columns, z_chunk planes), and a given split pass forms (r, A r) in blocks of its own
-  // tile, so that these results do not depend on the launch shape in their last digits; the tiles are made of such
-  // blocks.
-  const bool logical = is_split(d.kind) && prec == RSFD_DF64;
+  // Double-float and complex64: the split pass that replaces the stored one (automatic pass) forms every sum in the stored
+  // pass's blocks (32 x tile_y columns, z_chunk planes), and a given split pass forms (r, A r) in blocks of 32 x tile_y,
+  // so that these results do not depend on the launch shape in their last digits; the tiles are made of such blocks.
+  const bool logical = is_split(d.kind) && prec != RSFD_FP64;
   d.rr_blocks = logical && h->opts.pass_kind == RSFD_PASS_AUTO;
   d.lty = d.rr_blocks ? default_tile_y(prec, h->R, h->ny, RSFD_PASS_STORED, 1) : d.tile_y;
   if (logical) {
-    split_tile_blocks(h->nx, h->ny, d.lty, d.tile_x, d.tile_y);
+    split_tile_blocks(prec, h->nx, h->ny, d.lty, d.tile_x, d.tile_y);
   } else if (is_split(d.kind)) {
     if (h->opts.tile_y > 0) {
-      d.tile_x = split_tile_x(prec, h->nx, 32);
+      d.tile_x = split_tile_x(h->nx, 32);
       d.tile_y = (d.tile_y + 1) / 2 * 2;
     } else {
-      split_tile(prec, h->R, h->nx, h->ny, d.tile_x, d.tile_y);
+      split_tile(h->R, h->nx, h->ny, d.tile_x, d.tile_y);
     }
   }
   d.wait_cap = h->opts.wait_cap;
@@ -807,7 +807,7 @@ static rsfd_status rsfd_shifted_cocg_impl(rsfd_handle h, const int64_t* cols, in
   }
   if (kind_smem(prec, h->R, d.tile_y, d.depth, d.kind, d.tile_x) > (size_t)(216 * 1024))
     return fail(h, RSFD_ERR_ARG, "rsfd_shifted_cocg: prefetch depth does not fit in shared memory");
-  // tiles of the sums (the launch's own, except for double-float split passes)
+  // tiles of the sums (the launch's own, except for double-float and complex64 split passes)
   const int ltiles_x = logical ? (h->nx + 31) / 32
                                : (h->nx + d.tile_x - 1) / (d.kind == RSFD_PASS_RECOMPUTE ? pass_tile_x(h->R) : d.tile_x);
   const int ltiles_y = logical ? (h->ny + d.lty - 1) / d.lty : (h->ny + d.tile_y - 1) / d.tile_y;
@@ -823,7 +823,7 @@ static rsfd_status rsfd_shifted_cocg_impl(rsfd_handle h, const int64_t* cols, in
     int sms = 152;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
     d.zchunk = h->nz;
-    // (FP64 and complex64 split passes, whose sums are not tied to the chunk: fewer than 8 warps per SM, down to 4
+    // (the FP64 split pass, whose sums are not tied to the chunk: fewer than 8 warps per SM, down to 4
     // planes; 128 columns of 8 x 8 x 12 in FP64 take 34 us a stencil with one chunk, one warp per SM)
     if (is_split(d.kind) && !logical) {
       const long long warps = split_threads(d.tile_x, d.tile_y) / 32;
@@ -836,7 +836,7 @@ static rsfd_status rsfd_shifted_cocg_impl(rsfd_handle h, const int64_t* cols, in
   }
   d.nzchunks = (h->nz + d.zchunk - 1) / d.zchunk;
   d.ctas_per_slot = d.tiles_x * d.tiles_y * d.nzchunks;
-  d.nlog = ltiles_x * ltiles_y * d.nzchunks;   // the pass's CTAs, or the double-float split pass's blocks
+  d.nlog = ltiles_x * ltiles_y * d.nzchunks;   // the pass's CTAs, or the blocks of the sums
   d.ctas_c = 0;
   const int C = h->opts.iters_per_sync > 0 ? h->opts.iters_per_sync : 32;
   if (C > kMaxHist) return fail(h, RSFD_ERR_ARG, "rsfd_shifted_cocg: iters_per_sync too large");
@@ -860,7 +860,7 @@ static rsfd_status rsfd_shifted_cocg_impl(rsfd_handle h, const int64_t* cols, in
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
     d.ctas_c = split_plane_ctas(h->nz, W, sms);
   } else if (is_split(d.kind)) {
-    d.ctas_c = d.rr_blocks ? d.nlog : split_combine_ctas(prec, vec);
+    d.ctas_c = d.rr_blocks ? d.nlog : split_combine_ctas(vec);
   }
   d.npart = d.nlog + (d.rr_blocks ? 0 : d.ctas_c);
   const bool use_graphs = h->opts.use_graphs >= 0;

@@ -124,8 +124,8 @@ struct SolveDims {
   int npart;          // partial-sum entries per slot: nlog, then the combine's where it forms sums
   int nlog;           // partial-sum entries of the pass (or stencil) kernel: its CTAs, or its 32 x lty x zchunk blocks
   int rows_cta;       // split pass: rows a CTA owns (tile_y, or an odd lty in a tile one row taller)
-  int lty;            // double-float split pass: rows of a summation block
-  int rr_blocks;      // double-float split pass: the combine runs, and sums, in the same blocks as the stencil
+  int lty;            // double-float and complex64 split pass: rows of a summation block
+  int rr_blocks;      // double-float and complex64 split pass: the combine runs, and sums, in the same blocks as the stencil
   int ncols;
   int ntrack;         // interior planes recorded after the boundary planes
   int track[16];      // their z indices (rows 2 nface Nx Ny + e Nx Ny ...)
@@ -223,7 +223,7 @@ int pass_max_depth();
 int split_threads(int tile_x, int tile_y);   // tile_y even
 int split_max_points();                      // tile_x * tile_y at most
 size_t split_smem(int prec, int R, int tile_x, int tile_y, int depth);
-int split_combine_ctas(int prec, long long vec);
+int split_combine_ctas(long long vec);
 int split_plane_ctas(int nz, int W, int sms);
 int pass_box_x();
 int pass_box_off();
