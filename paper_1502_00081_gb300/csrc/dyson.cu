@@ -119,18 +119,22 @@ template <typename T> void* oz_work(Gemm& g, int batch, int m, int n, int k, siz
 // rsfd_transmission, CUDA cores / sliced, us: ns = 64, 16 energies (4.2e6) 143 / 154; 192, 1 (7.1e6) 251 / 266;
 // 128, 4 (8.4e6) 242 / 208; 96, 16 (1.4e7) 291 / 190; 256, 16 (2.7e8) 3869 / 600.
 bool gemm_sliced(Gemm& g, int batch, int m, int n, int k, double sign, const double2* A, int lda, long long sA, int opA,
-                 const double2* B, int ldb, long long sB, bool add, double2* C, int ldc, long long sC) {
+                 const double2* B, int ldb, long long sB, bool add, double2* C, int ldc, long long sC, int ksplit) {
   size_t wb = 0;
+  const int k1 = ksplit > 0 && ksplit < k ? ksplit : k, k2 = k - k1;
   void* w = g.h && k >= 32 && m >= 32 && n >= 16 && (double)m * n * k * batch >= kSliceMin
-                ? oz_work<double2>(g, batch, m, n, k, wb)
+                ? oz_work<double2>(g, batch, m, n, k1 > k2 ? k1 : k2, wb)
                 : nullptr;
   if (!w) return false;
-  g.note(oz_gemm(g.st, batch, m, n, k, sign < 0 ? -1 : 1, A, lda, sA, opA, B, ldb, sB, add ? 1 : 0, C, ldc, sC, w, wb, g.err));
+  const int sg = sign < 0 ? -1 : 1;
+  g.note(oz_gemm(g.st, batch, m, n, k1, sg, A, lda, sA, opA, B, ldb, sB, add ? 1 : 0, C, ldc, sC, w, wb, g.err));
+  if (k2 > 0)
+    g.note(oz_gemm(g.st, batch, m, n, k2, sg, A + (long long)k1 * lda, lda, sA, opA, B + k1, ldb, sB, 1, C, ldc, sC, w, wb, g.err));
   return true;
 }
 void gemm(Gemm& g, int batch, int m, int n, int k, double sign, const double2* A, int lda, long long sA, int opA,
-          const double2* B, int ldb, long long sB, bool add, double2* C, int ldc, long long sC) {
-  if (!gemm_sliced(g, batch, m, n, k, sign, A, lda, sA, opA, B, ldb, sB, add, C, ldc, sC))
+          const double2* B, int ldb, long long sB, bool add, double2* C, int ldc, long long sC, int ksplit) {
+  if (!gemm_sliced(g, batch, m, n, k, sign, A, lda, sA, opA, B, ldb, sB, add, C, ldc, sC, ksplit))
     zgemm(g.st, batch, m, n, k, make_double2(sign, 0.0), A, lda, sA, opA, B, ldb, sB, make_double2(add ? 1.0 : 0.0, 0.0),
           C, ldc, sC);
 }
@@ -394,18 +398,18 @@ rsfd_status dyson_tc_run(Handle* h, const void* G0, const void* SL, const void* 
     DY_CK(h, cudaMemsetAsync(info, 0, kb * sizeof(int), st));
     lu_factor(gc, dF, nb, kb, perm, info, swp);
     lu_permute(gc, b0, nb, kb, perm, dXf, nc);
-    lu_solve(gc, dF, nb, kb, dXf, nc);
+    lu_solve(gc, dF, nb, kb, dXf, nc, ns);
     set_f32_to_c128<<<grid_for(totx), 256, 0, st>>>(dX, dXf, totx);
     for (int it = 0; it < nref; ++it) {
       copy_c128<<<grid_for(totx), 256, 0, st>>>(b0, dR, totx);
-      gemm(gc, kb, nb, nc, nb, -1.0, dM, nb, n2, 0, dX, nb, sx, true, dR, nb, sx);
+      gemm(gc, kb, nb, nc, nb, -1.0, dM, nb, n2, 0, dX, nb, sx, true, dR, nb, sx, ns);
       lu_permute(gc, dR, nb, kb, perm, dXf, nc);
-      lu_solve(gc, dF, nb, kb, dXf, nc);
+      lu_solve(gc, dF, nb, kb, dXf, nc, ns);
       add_f32_to_c128<<<grid_for(totx), 256, 0, st>>>(dX, dXf, totx);
     }
     if (refres) {
       copy_c128<<<grid_for(totx), 256, 0, st>>>(b0, dR, totx);
-      gemm(gc, kb, nb, nc, nb, -1.0, dM, nb, n2, 0, dX, nb, sx, true, dR, nb, sx);
+      gemm(gc, kb, nb, nc, nb, -1.0, dM, nb, n2, 0, dX, nb, sx, true, dR, nb, sx, ns);
       frob2_batched(st, dR, sx, kb, red + 2 * K, red + k0);
       frob2_batched(st, b0, sx, kb, red + 2 * K, red + K + k0);
     }
@@ -473,7 +477,7 @@ rsfd_status dyson_run(Handle* h, const void* G0, const void* SL, const void* SR,
   copy_c128<<<grid_for(tot), 256, 0, st>>>(dM, dLU, tot);
   DY_CK(h, cudaMemsetAsync(info, 0, K * sizeof(int), st));
   lu_factor(gc, dLU, nb, K, perm, info, swp);
-  const double2* dinv = lu_inverses(gc, dLU, nb, K, nc);
+  const double2* dinv = lu_inverses(gc, dLU, nb, K, nc, ns);
   // right-hand sides: the first nc columns of every energy, compact (stride sx)
   const double2* b0 = dG0;
   if (nc < nb) {
@@ -483,18 +487,18 @@ rsfd_status dyson_run(Handle* h, const void* G0, const void* SL, const void* SR,
     b0 = (const double2*)pB;
   }
   lu_permute(gc, b0, nb, K, perm, dX, nc);
-  lu_solve(gc, dLU, nb, K, dX, nc, dinv);
+  lu_solve(gc, dLU, nb, K, dX, nc, dinv, ns);
   // iterative refinement in FP64
   for (int it = 0; it < 2; ++it) {
     copy_c128<<<grid_for(totx), 256, 0, st>>>(b0, dR, totx);
-    gemm(gc, K, nb, nc, nb, -1.0, dM, nb, n2, 0, dX, nb, sx, true, dR, nb, sx);
+    gemm(gc, K, nb, nc, nb, -1.0, dM, nb, n2, 0, dX, nb, sx, true, dR, nb, sx, ns);
     lu_permute(gc, dR, nb, K, perm, dR, nc);
-    lu_solve(gc, dLU, nb, K, dR, nc, dinv);
+    lu_solve(gc, dLU, nb, K, dR, nc, dinv, ns);
     axpy_c128<<<grid_for(totx), 256, 0, st>>>(dX, dR, totx);
   }
   if (refres) {
     copy_c128<<<grid_for(totx), 256, 0, st>>>(b0, dR, totx);
-    gemm(gc, K, nb, nc, nb, -1.0, dM, nb, n2, 0, dX, nb, sx, true, dR, nb, sx);
+    gemm(gc, K, nb, nc, nb, -1.0, dM, nb, n2, 0, dX, nb, sx, true, dR, nb, sx, ns);
     frob2_batched(st, dR, sx, K, red + 2 * K, red);
     frob2_batched(st, b0, sx, K, red + 2 * K, red + K);
   }
@@ -567,19 +571,19 @@ rsfd_status dyson_tracked_run(Handle* h, int nr, const void* G0, const void* SL,
   lu_factor(gc, dLU, nb, K, perm, info, swp);
   // Y = M^{-1} G0[b, :] with two FP64 refinement steps
   copy_rows_c128<<<grid_for(ntot), 256, 0, st>>>(dG0, nr, dRHS, nb, nb, nr, K);
-  const double2* dinv = lu_inverses(gc, dLU, nb, K, nr);
+  const double2* dinv = lu_inverses(gc, dLU, nb, K, nr, ns);
   lu_permute(gc, dRHS, nb, K, perm, dY, nr);
-  lu_solve(gc, dLU, nb, K, dY, nr, dinv);
+  lu_solve(gc, dLU, nb, K, dY, nr, dinv, ns);
   for (int it = 0; it < 2; ++it) {
     copy_c128<<<grid_for(ntot), 256, 0, st>>>(dRHS, dR, ntot);
-    gemm(gc, K, nb, nr, nb, -1.0, dM, nb, b2, 0, dY, nb, bn, true, dR, nb, bn);
+    gemm(gc, K, nb, nr, nb, -1.0, dM, nb, b2, 0, dY, nb, bn, true, dR, nb, bn, ns);
     lu_permute(gc, dR, nb, K, perm, dR, nr);
-    lu_solve(gc, dLU, nb, K, dR, nr, dinv);
+    lu_solve(gc, dLU, nb, K, dR, nr, dinv, ns);
     axpy_c128<<<grid_for(ntot), 256, 0, st>>>(dY, dR, ntot);
   }
   if (refres) {
     copy_c128<<<grid_for(ntot), 256, 0, st>>>(dRHS, dR, ntot);
-    gemm(gc, K, nb, nr, nb, -1.0, dM, nb, b2, 0, dY, nb, bn, true, dR, nb, bn);
+    gemm(gc, K, nb, nr, nb, -1.0, dM, nb, b2, 0, dY, nb, bn, true, dR, nb, bn, ns);
     frob2_batched(st, dR, bn, K, red + 2 * K, red);
     frob2_batched(st, dRHS, bn, K, red + 2 * K, red + K);
   }
@@ -587,7 +591,7 @@ rsfd_status dyson_tracked_run(Handle* h, int nr, const void* G0, const void* SL,
   gemm(gc, K, ns, nr, ns, 1.0, (const double2*)SL, ns, (long long)ns * ns, 0, dY, nb, bn, false, dW, nb, bn);
   gemm(gc, K, ns, nr, ns, 1.0, (const double2*)SR, ns, (long long)ns * ns, 0, dY + ns, nb, bn, false, dW + ns, nb, bn);
   copy_c128<<<grid_for(rtot), 256, 0, st>>>(dG0, dX, rtot);
-  gemm(gc, K, nr, nr, nb, 1.0, dG0, nr, r2, 0, dW, nb, bn, true, dX, nr, r2);
+  gemm(gc, K, nr, nr, nb, 1.0, dG0, nr, r2, 0, dW, nb, bn, true, dX, nr, r2, ns);
   if (fp64) copy_c128<<<grid_for(rtot), 256, 0, st>>>(dX, (double2*)G, rtot);
   else from_c128_f<<<grid_for(rtot), 256, 0, st>>>(dX, (float2*)G, rtot);
   DY_CK(h, cudaGetLastError());
@@ -779,9 +783,9 @@ rsfd_status lead_decimation_run(Handle* h, const double* VL, const double* VR, c
       // Y = g [alpha | beta] by LU of Z - eps, then P = [alpha; beta] Y
       DY_CK(h, cudaMemsetAsync(info, 0, nm * sizeof(int), st));
       lu_factor(gc, A, n, nm, perm, info, swp);
-      const double2* dinv = lu_inverses(gc, A, n, nm, 2 * n);
+      const double2* dinv = lu_inverses(gc, A, n, nm, 2 * n, 0);
       lu_permute(gc, rhs, n, nm, perm, Y, 2 * n);
-      lu_solve(gc, A, n, nm, Y, 2 * n, dinv);
+      lu_solve(gc, A, n, nm, Y, 2 * n, dinv, 0);
       gemm(gc, nm, 2 * n, 2 * n, n, 1.0, ab, 2 * n, 2 * n2, 0, Y, n, 2 * n2, false, P, 2 * n, 4 * n2);
       DY_CK(h, cudaMemsetAsync(dmax, 0, nm * sizeof(unsigned long long), st));
       decimation_step<false><<<gs, 256, 0, st>>>(P, eps_s, eps, ab, rhs, A, dZ, n, kb, dmax);
@@ -793,9 +797,9 @@ rsfd_status lead_decimation_run(Handle* h, const double* VL, const double* VR, c
     lu_factor(gc, A, n, nm, perm, info, swp);
     bcast_c128<<<grid_for(tot), 256, 0, st>>>(dH01T, rhs, n2, kb);
     bcast_c128<<<grid_for(tot), 256, 0, st>>>(dH01, rhs + tot, n2, kb);
-    const double2* dinv = lu_inverses(gc, A, n, nm, n);
+    const double2* dinv = lu_inverses(gc, A, n, nm, n, 0);
     lu_permute(gc, rhs, n, nm, perm, Y, n);
-    lu_solve(gc, A, n, nm, Y, n, dinv);
+    lu_solve(gc, A, n, nm, Y, n, dinv, 0);
     gemm(gc, kb, n, n, n, 1.0, dH01, n, 0, 0, Y, n, n2, false, (double2*)SRo + n2 * k0, n, n2);
     gemm(gc, kb, n, n, n, 1.0, dH01T, n, 0, 0, Y + tot, n, n2, false, (double2*)SLo + n2 * k0, n, n2);
     std::vector<int> hinfo(nm);
@@ -959,12 +963,12 @@ rsfd_status dyson_noalloc_run(int32_t nb, int32_t K, const void* G0_bb, const vo
   copy_c128<<<grid_for(tot), 256, 0, st>>>(dM, dLU, tot);
   lu_factor(gc, dLU, nb, K, perm, info, swp);
   lu_permute(gc, G0, nb, K, perm, dX, nb);
-  lu_solve(gc, dLU, nb, K, dX, nb, nullptr);
+  lu_solve(gc, dLU, nb, K, dX, nb, nullptr, 0);
   for (int it = 0; it < 2; ++it) {
     copy_c128<<<grid_for(tot), 256, 0, st>>>(G0, dR, tot);
     gemm(gc, K, nb, nb, nb, -1.0, dM, nb, n2, 0, dX, nb, n2, true, dR, nb, n2);
     lu_permute(gc, dR, nb, K, perm, dR, nb);
-    lu_solve(gc, dLU, nb, K, dR, nb, nullptr);
+    lu_solve(gc, dLU, nb, K, dR, nb, nullptr, 0);
     axpy_c128<<<grid_for(tot), 256, 0, st>>>(dX, dR, tot);
   }
   copy_c128<<<grid_for(tot), 256, 0, st>>>(G0, dR, tot);

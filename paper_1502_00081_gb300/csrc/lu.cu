@@ -488,11 +488,25 @@ __global__ void __launch_bounds__(256, sizeof(T) == 16 ? 2 : 3) lu_trsm(const T*
                                                                          long long sX, int nrhs) {
   trsm_body<T, LOWER, false>(LU, nb, r0, ib, X, sX, nrhs, blockIdx.y, nullptr);
 }
-// Inverses of the diagonal blocks of 64 rows, for solves whose products run on the tensor cores: block (z >> 1) of matrix
-// blockIdx.y, its unit lower (z even) or upper (z odd) triangle; dinv [K][blocks][2][64 x 64].  One warp per 4 columns.
-__global__ void __launch_bounds__(32) lu_invert(const double2* LU, int nb, double2* dinv) {
+// Blocks of at most NB rows of [0, n), none of them across row split (0: no such row)
+struct RowBlocks {
+  int n, NB, split, n1;   // n1 blocks end at split
+  __host__ __device__ RowBlocks(int n_, int NB_, int split_)
+      : n(n_), NB(NB_), split(split_ < n_ ? split_ : 0), n1((split + NB_ - 1) / NB_) {}
+  __host__ __device__ int count() const { return n1 + (n - split + NB - 1) / NB; }
+  __host__ __device__ int row(int b) const { return b < n1 ? b * NB : split + (b - n1) * NB; }
+  __host__ __device__ int rows(int b) const {
+    const int left = (b < n1 ? split : n) - row(b);
+    return left < NB ? left : NB;
+  }
+};
+
+// Inverses of the diagonal blocks of (at most) 64 rows, for solves whose products run on the tensor cores: block (z >> 1) of
+// matrix blockIdx.y, its unit lower (z even) or upper (z odd) triangle; dinv [K][blocks][2][64 x 64].  One warp per 4 columns.
+__global__ void __launch_bounds__(32) lu_invert(const double2* LU, int nb, int split, double2* dinv) {
   constexpr int NB = Num<double2>::NBLK;
-  const int blk = blockIdx.z >> 1, r0 = blk * NB, ib = min(NB, nb - r0), nblk = (nb + NB - 1) / NB;
+  const RowBlocks bl(nb, NB, split);
+  const int blk = blockIdx.z >> 1, r0 = bl.row(blk), ib = bl.rows(blk), nblk = bl.count();
   double2* D = dinv + (((long long)blockIdx.y * nblk + blk) * 2 + (blockIdx.z & 1)) * NB * NB;
   if (blockIdx.z & 1) trsm_body<double2, false, true>(LU, nb, r0, ib, nullptr, 0, NB, blockIdx.y, D);
   else trsm_body<double2, true, true>(LU, nb, r0, ib, nullptr, 0, NB, blockIdx.y, D);
@@ -591,24 +605,24 @@ int panel(Gemm& g, T* M, int nb, int K, int o0, int j0, int oend, int* info, int
   return jw;
 }
 
-// X = T^{-1} X for the unit lower triangle (LOWER) or the upper triangle of rows and columns r0 .. r1 - 1 of LU
-// (r0 a multiple of the block size).  dinv: the diagonal blocks' inverses (FP64), or null for substitution.
+// X = T^{-1} X for the unit lower triangle (LOWER) or the upper triangle of rows and columns r0 .. r1 - 1 of LU, in blocks
+// that do not cross row r0 + split.  dinv: the diagonal blocks' inverses (FP64, r0 = 0), or null for substitution.
 template <typename T, bool LOWER>
-void solve_range(Gemm& g, const T* LU, int nb, int K, int r0, int r1, T* X, long long sX, int nrhs, const T* dinv) {
+void solve_range(Gemm& g, const T* LU, int nb, int K, int r0, int r1, T* X, long long sX, int nrhs, const T* dinv, int split) {
   constexpr int NB = Num<T>::NBLK;
   const long long n2 = (long long)nb * nb;
   const int thr = sizeof(T) == 16 ? 32 : 256, per = thr / 8;
   const dim3 grid((nrhs + per - 1) / per, K);
-  const int nblk = (r1 - r0 + NB - 1) / NB;
+  const RowBlocks bl(r1 - r0, NB, split);
+  const int nblk = bl.count();
   for (int bi = 0; bi < nblk; ++bi) {
-    const int s0 = r0 + (LOWER ? bi : nblk - 1 - bi) * NB, ib = r1 - s0 < NB ? r1 - s0 : NB;
+    const int blk = LOWER ? bi : nblk - 1 - bi, s0 = r0 + bl.row(blk), ib = bl.rows(blk);
     bool done = false;
     if constexpr (sizeof(T) == 16) {
       // X_b = T_bb^{-1} X_b in place: the digits of X_b are taken before the product is written
-      const int tot = (nb + NB - 1) / NB;
       if (dinv)
-        done = gemm_sliced(g, K, ib, nrhs, ib, 1.0, dinv + ((long long)(s0 / NB) * 2 + (LOWER ? 0 : 1)) * NB * NB, NB,
-                           (long long)tot * 2 * NB * NB, 0, X + s0, nb, sX, false, X + s0, nb, sX);
+        done = gemm_sliced(g, K, ib, nrhs, ib, 1.0, dinv + ((long long)blk * 2 + (LOWER ? 0 : 1)) * NB * NB, NB,
+                           (long long)nblk * 2 * NB * NB, 0, X + s0, nb, sX, false, X + s0, nb, sX);
     }
     if (!done) lu_trsm<T, LOWER><<<grid, thr, 0, g.st>>>(LU, nb, s0, ib, X, sX, nrhs);
     const int d0 = LOWER ? s0 + ib : r0, d1 = LOWER ? r1 : s0;   // rows still to be updated
@@ -636,7 +650,7 @@ template <typename T> void lu_factor_t(Gemm& g, T* M, int nb, int K, int* perm, 
     lu_swap_rest<T><<<dim3((out + 63) / 64, K), 64, 0, g.st>>>(M, nb, o0, oend, np, swp, ss, perm);
     if (rest > 0) {
       // U12 = L11^{-1} A12, then A22 -= L21 U12
-      solve_range<T, true>(g, M, nb, K, o0, oend, M + (long long)oend * nb, n2, rest, nullptr);
+      solve_range<T, true>(g, M, nb, K, o0, oend, M + (long long)oend * nb, n2, rest, nullptr, 0);
       gemm(g, K, rest, rest, oend - o0, -1.0, M + (long long)o0 * nb + oend, nb, n2, 0, M + (long long)oend * nb + o0, nb, n2,
            true, M + (long long)oend * nb + oend, nb, n2);
     }
@@ -644,10 +658,14 @@ template <typename T> void lu_factor_t(Gemm& g, T* M, int nb, int K, int* perm, 
   g.note(cudaGetLastError());
 }
 
-template <typename T> void lu_solve_t(Gemm& g, const T* LU, int nb, int K, T* X, int nrhs, const T* dinv) {
+// A matrix of one block is solved by substitution alone, which needs no split
+template <typename T> int solve_split(int nb, int split) { return nb <= Num<T>::NBLK ? 0 : split; }
+
+template <typename T> void lu_solve_t(Gemm& g, const T* LU, int nb, int K, T* X, int nrhs, const T* dinv, int split) {
   const long long sx = (long long)nb * nrhs;
-  solve_range<T, true>(g, LU, nb, K, 0, nb, X, sx, nrhs, dinv);
-  solve_range<T, false>(g, LU, nb, K, 0, nb, X, sx, nrhs, dinv);
+  split = solve_split<T>(nb, split);
+  solve_range<T, true>(g, LU, nb, K, 0, nb, X, sx, nrhs, dinv, split);
+  solve_range<T, false>(g, LU, nb, K, 0, nb, X, sx, nrhs, dinv, split);
   g.note(cudaGetLastError());
 }
 
@@ -664,22 +682,22 @@ void lu_factor(Gemm& g, float2* M, int nb, int K, int* perm, int* info, int* swp
 // Substitution costs 64 x 63 / 2 FP64 multiply-adds a column and block on the FP64 pipe (70-90 us a block for 400 to 512
 // columns of 8 matrices), a product with the inverse about 25 us; the inverses of all blocks together cost one block's
 // substitution.  Worth it from 2000 columns over the batch on (where gemm() slices the 64 x n x 64 products).
-const double2* lu_inverses(Gemm& g, const double2* LU, int nb, int K, int nrhs) {
+const double2* lu_inverses(Gemm& g, const double2* LU, int nb, int K, int nrhs, int split) {
   constexpr int NB = Num<double2>::NBLK;
-  if (!g.h || (double)nrhs * K * NB * NB < kSliceMin || nb < NB) return nullptr;
-  const int nblk = (nb + NB - 1) / NB;
+  if (!g.h || (double)nrhs * K * NB * NB < kSliceMin || nb < NB || (nb == NB && split > 0)) return nullptr;
+  const int nblk = RowBlocks(nb, NB, split).count();
   if (nblk > 32767) return nullptr;
   void* w = nullptr;
   if (handle_ensure(g.h, 10, (size_t)K * nblk * 2 * NB * NB * sizeof(double2), &w) != RSFD_OK) return nullptr;
-  lu_invert<<<dim3(NB / 4, K, 2 * nblk), 32, 0, g.st>>>(LU, nb, (double2*)w);
+  lu_invert<<<dim3(NB / 4, K, 2 * nblk), 32, 0, g.st>>>(LU, nb, split, (double2*)w);
   g.note(cudaGetLastError());
   return (const double2*)w;
 }
-void lu_solve(Gemm& g, const double2* LU, int nb, int K, double2* X, int nrhs, const double2* dinv) {
-  lu_solve_t<double2>(g, LU, nb, K, X, nrhs, dinv);
+void lu_solve(Gemm& g, const double2* LU, int nb, int K, double2* X, int nrhs, const double2* dinv, int split) {
+  lu_solve_t<double2>(g, LU, nb, K, X, nrhs, dinv, split);
 }
-void lu_solve(Gemm& g, const float2* LU, int nb, int K, float2* X, int nrhs) {
-  lu_solve_t<float2>(g, LU, nb, K, X, nrhs, nullptr);
+void lu_solve(Gemm& g, const float2* LU, int nb, int K, float2* X, int nrhs, int split) {
+  lu_solve_t<float2>(g, LU, nb, K, X, nrhs, nullptr, split);
 }
 
 void lu_permute(Gemm& g, const double2* B, int nb, int K, const int* perm, float2* X, int nrhs) {
