@@ -172,7 +172,9 @@ typedef struct {
   int32_t wait_cap;       /* attempts of a pass's bounded wait for its TMA transfers before the wait is
                              declared lost (each attempt sleeps up to 1 ms): 0 = 4096; -1 = none, so every
                              CTA's first wait expires at once (a test of the RSFD_ERR_TIMEOUT path: the CTA
-                             still drains its issued transfers with the full cap before it returns) */
+                             still drains its issued transfers with the full cap before it returns).  Also of the
+                             waits inside the sliced tensor-core products of the Dyson step, the transmission and
+                             the lead decimation */
   int32_t dyson_cols;     /* columns of G_bb rsfd_dyson_boundary solves: 0 = all nb; 1 = the left slab's nb/2
                              only (solve, refinement and residual on half the right-hand sides), the
                              block rsfd_transmission reads (G_RL); the other columns are set to zero */

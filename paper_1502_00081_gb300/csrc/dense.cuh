@@ -12,6 +12,7 @@ struct Gemm {
   Handle* h = nullptr;
   cudaStream_t st = nullptr;
   int* err = nullptr;              // device flag of expired waits
+  int wait_cap = 0;                // the handle's solve option
   cudaError_t fail = cudaSuccess;  // first launch error
   void note(cudaError_t e) {
     if (e != cudaSuccess && fail == cudaSuccess) fail = e;

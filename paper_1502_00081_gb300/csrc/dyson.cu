@@ -90,6 +90,7 @@ rsfd_status gemm_begin(Handle* h, Gemm& g) {
   const rsfd_status s = handle_ensure(h, 9, 256, &p);
   if (s != RSFD_OK) return s;
   g.err = (int*)p;
+  g.wait_cap = handle_wait_cap(h);
   g.fail = cudaMemsetAsync(g.err, 0, sizeof(int), g.st);
   return RSFD_OK;
 }
@@ -127,9 +128,11 @@ bool gemm_sliced(Gemm& g, int batch, int m, int n, int k, double sign, const dou
                 : nullptr;
   if (!w) return false;
   const int sg = sign < 0 ? -1 : 1;
-  g.note(oz_gemm(g.st, batch, m, n, k1, sg, A, lda, sA, opA, B, ldb, sB, add ? 1 : 0, C, ldc, sC, w, wb, g.err));
+  g.note(oz_gemm(g.st, batch, m, n, k1, sg, A, lda, sA, opA, B, ldb, sB, add ? 1 : 0, C, ldc, sC, w, wb, g.err,
+                 g.wait_cap));
   if (k2 > 0)
-    g.note(oz_gemm(g.st, batch, m, n, k2, sg, A + (long long)k1 * lda, lda, sA, opA, B + k1, ldb, sB, 1, C, ldc, sC, w, wb, g.err));
+    g.note(oz_gemm(g.st, batch, m, n, k2, sg, A + (long long)k1 * lda, lda, sA, opA, B + k1, ldb, sB, 1, C, ldc, sC, w, wb, g.err,
+                 g.wait_cap));
   return true;
 }
 void gemm(Gemm& g, int batch, int m, int n, int k, double sign, const double2* A, int lda, long long sA, int opA,
@@ -146,7 +149,8 @@ void gemm(Gemm& g, int batch, int m, int n, int k, double sign, const float2* A,
   size_t wb = 0;
   void* w = oz_work<float2>(g, batch, m, n, k, wb);
   if (w)
-    g.note(oz_gemm(g.st, batch, m, n, k, sign < 0 ? -1 : 1, A, lda, sA, opA, B, ldb, sB, add ? 1 : 0, C, ldc, sC, w, wb, g.err));
+    g.note(oz_gemm(g.st, batch, m, n, k, sign < 0 ? -1 : 1, A, lda, sA, opA, B, ldb, sB, add ? 1 : 0, C, ldc, sC, w, wb, g.err,
+                 g.wait_cap));
   else
     g.note(cgemm_tf32x3(g.st, batch, m, n, k, make_float2((float)sign, 0.f), A, lda, sA, B, ldb, sB, add ? 1.f : 0.f, C, ldc,
                         sC, g.err));

@@ -69,19 +69,31 @@ constexpr uint32_t kOzHintNs = 1000000;
 
 __device__ __forceinline__ uint32_t oz_saddr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-__device__ __forceinline__ bool oz_wait(uint32_t bar, uint32_t parity) {
-  for (int i = 0; i < kOzWaitCap; ++i) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity), "r"(kOzHintNs)
-        : "memory");
-    if (ok) return true;
+// one attempt, up to 1 ms
+__device__ __forceinline__ bool oz_try(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity), "r"(kOzHintNs)
+      : "memory");
+  return ok != 0;
+}
+// bounded wait; also gives up when another thread has (looked at between attempts only: a role that goes on for a while
+// does no harm, it soon waits for the one that stopped)
+__device__ __forceinline__ bool oz_wait(uint32_t bar, uint32_t parity, int cap, const volatile int& abort) {
+  for (int i = 0; i < cap; ++i) {
+    if (oz_try(bar, parity)) return true;
+    if (abort) return false;
   }
   return false;
+}
+// bounded wait for what is in flight (after an abort, before the CTA's memory is given back)
+__device__ __forceinline__ void oz_drain(uint32_t bar, uint32_t parity) {
+  for (int i = 0; i < kOzWaitCap && !oz_try(bar, parity); ++i) {
+  }
 }
 __device__ __forceinline__ void oz_bulk(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
@@ -277,6 +289,7 @@ template <typename T> struct OzGemm {
   int ldc;
   long long sC;
   int* err;
+  int cap;            // attempts of a bounded wait
 };
 
 // (hi 2^32 + lo) 2^e rounded to nearest, by integer arithmetic (conversions and FP64 arithmetic run at 2 a
@@ -328,6 +341,7 @@ template <typename T> __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_k
   __shared__ __align__(8) uint64_t fullA[NA], emptyA[NA], fullB[OZ_NB], emptyB[OZ_NB], accFull, accEmpty, mmaDone;
   __shared__ uint32_t tmem_s;
   __shared__ volatile int s_abort;
+  __shared__ int s_issuedA, s_issuedB;   // copies issued (read after an abort)
   unsigned char* smem = (unsigned char*)(((uintptr_t)oz_smem_raw + 1023) & ~(uintptr_t)1023);
   unsigned char* sA = smem;
   unsigned char* sB = smem + NA * ABLK;
@@ -382,30 +396,24 @@ template <typename T> __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_k
         const unsigned char* gB = q.B + ((size_t)b * ntiles + nt) * ksteps * OZ_BBLK;
         for (int t = 0; t < ksteps && ok; ++t) {
           const int sb = issuedB % OZ_NB;
-          if (issuedB >= OZ_NB) ok = oz_wait(oz_saddr(&emptyB[sb]), (uint32_t)((issuedB / OZ_NB - 1) & 1));
-          ok = ok && !s_abort;
+          ok = issuedB < OZ_NB || oz_wait(oz_saddr(&emptyB[sb]), (uint32_t)((issuedB / OZ_NB - 1) & 1), q.cap, s_abort);
           if (!ok) break;
           oz_bulk(oz_saddr(sB + sb * OZ_BBLK), gB + (size_t)t * OZ_BBLK, OZ_BBLK, oz_saddr(&fullB[sb]));
           ++issuedB;
           for (int h = 0; h < 2; ++h) {
             const int sa = issuedA % NA;
-            if (issuedA >= NA) ok = oz_wait(oz_saddr(&emptyA[sa]), (uint32_t)((issuedA / NA - 1) & 1));
-            ok = ok && !s_abort;
+            ok = issuedA < NA || oz_wait(oz_saddr(&emptyA[sa]), (uint32_t)((issuedA / NA - 1) & 1), q.cap, s_abort);
             if (!ok) break;
             oz_bulk(oz_saddr(sA + sa * ABLK), gA + (size_t)(2 * t + h) * ABLK, ABLK, oz_saddr(&fullA[sa]));
             ++issuedA;
           }
         }
       }
+      s_issuedA = issuedA;
+      s_issuedB = issuedB;
       if (!ok) {
-        // let the copies in flight land before the CTA's shared memory is released: per ring entry
-        // the last one issued (earlier ones completed before the entry was refilled)
         s_abort = 1;
         atomicExch(q.err, 1);
-        for (int a = max(0, issuedA - NA); a < issuedA; ++a)
-          oz_wait(oz_saddr(&fullA[a % NA]), (uint32_t)((a / NA) & 1));
-        for (int c = max(0, issuedB - OZ_NB); c < issuedB; ++c)
-          oz_wait(oz_saddr(&fullB[c % OZ_NB]), (uint32_t)((c / OZ_NB) & 1));
       }
     }
   } else if (warp == OZ_EPI / 32 + 1) {
@@ -416,20 +424,17 @@ template <typename T> __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_k
         for (int t = 0; t < ksteps && ok; ++t) {
           const bool first = t % OZ_CHUNK == 0;
           if (first && cc > 0) {   // the accumulators have been read
-            ok = oz_wait(oz_saddr(&accEmpty), (uint32_t)((cc - 1) & 1));
+            ok = oz_wait(oz_saddr(&accEmpty), (uint32_t)((cc - 1) & 1), q.cap, s_abort);
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           }
           const int sb = ib % OZ_NB;
-          ok = ok && oz_wait(oz_saddr(&fullB[sb]), (uint32_t)((ib / OZ_NB) & 1));
+          ok = ok && oz_wait(oz_saddr(&fullB[sb]), (uint32_t)((ib / OZ_NB) & 1), q.cap, s_abort);
           const uint32_t b0 = oz_saddr(sB + sb * OZ_BBLK);
           const uint64_t bre = oz_desc(b0, OZ_LBO_B), bim = oz_desc(b0 + OZ_BPLANE, OZ_LBO_B);
           for (int h = 0; h < 2 && ok; ++h) {
             const int sa = ia % NA;
-            ok = oz_wait(oz_saddr(&fullA[sa]), (uint32_t)((ia / NA) & 1));
-            if (!ok || s_abort) {
-              ok = false;
-              break;
-            }
+            ok = oz_wait(oz_saddr(&fullA[sa]), (uint32_t)((ia / NA) & 1), q.cap, s_abort);
+            if (!ok) break;
             const uint32_t a0 = oz_saddr(sA + sa * ABLK);
             // h = 0: Re += Ar Br, Im += Ar Bi;  h = 1: Re -= Ai Bi, Im += Ai Br
 #pragma unroll
@@ -456,8 +461,10 @@ template <typename T> __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_k
         // the MMAs issued so far end before the tensor memory is given back
         s_abort = 1;
         atomicExch(q.err, 1);
-        oz_commit(oz_saddr(&mmaDone));
-        oz_wait(oz_saddr(&mmaDone), 0);
+        if (ia > 0) {
+          oz_commit(oz_saddr(&mmaDone));
+          oz_drain(oz_saddr(&mmaDone), 0);
+        }
       }
     }
   } else {
@@ -476,12 +483,9 @@ template <typename T> __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_k
 #pragma unroll
         for (int j = 0; j < EC; ++j) sum[p][w][j] = 0;
     for (int c = 0; c < nchunks; ++c, ++cc) {
-      ok = oz_wait(oz_saddr(&accFull), (uint32_t)(cc & 1));
-      if (!ok || s_abort) {
-        ok = false;
-        break;
-      }
-      __syncwarp();
+      // the warp goes on or stops as a whole: what follows is warp-aligned
+      ok = __all_sync(0xffffffffu, oz_wait(oz_saddr(&accFull), (uint32_t)(cc & 1), q.cap, s_abort));
+      if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
       for (int p = 0; p < 2; ++p) {
@@ -554,6 +558,16 @@ template <typename T> __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_k
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   }
   __syncthreads();
+  if (s_abort) {
+    // the copies in flight land before the CTA's shared memory is released: per ring entry the last one issued (earlier
+    // ones completed before the entry was refilled)
+    if (tid == 0) {
+      for (int a = max(0, s_issuedA - NA); a < s_issuedA; ++a) oz_drain(oz_saddr(&fullA[a % NA]), (uint32_t)((a / NA) & 1));
+      for (int c = max(0, s_issuedB - OZ_NB); c < s_issuedB; ++c)
+        oz_drain(oz_saddr(&fullB[c % OZ_NB]), (uint32_t)((c / OZ_NB) & 1));
+    }
+    __syncthreads();
+  }
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
 }
 
@@ -568,7 +582,7 @@ template <typename T> size_t oz_bytes_t(int m, int n, int k) {
 template <typename T>
 cudaError_t oz_gemm_t(cudaStream_t st, int batch, int m, int n, int k, int sign, const T* A, int lda, long long sA,
                       int opA, const T* B, int ldb, long long sB, int add, T* C, int ldc, long long sC, void* work,
-                      size_t work_bytes, int* err) {
+                      size_t work_bytes, int* err, int wait_cap) {
   constexpr int S = OzOf<T>::S, BN = OzDim<S>::BN, ABLK = OzDim<S>::ABLK;
   const size_t per = oz_bytes_t<T>(m, n, k);
   int nb = (int)(work_bytes / per < (size_t)batch ? work_bytes / per : (size_t)batch);
@@ -598,7 +612,8 @@ cudaError_t oz_gemm_t(cudaStream_t st, int batch, int m, int n, int k, int sign,
     oz_digits<T><<<dim3((rpad + 31) / 32, (2 * ks + 7) / 8, 2 * bn), 256, 0, st>>>(q);
     const long long tiles = (long long)(mp / OZ_BM) * (np / BN) * bn;
     if (tiles > 0x7fffffffll) return cudaErrorInvalidValue;
-    OzGemm<T> g{dA, dB, xA, xB, m, n, mp, np, ks, (int)tiles, sign, add, C + b0 * sC, ldc, sC, err};
+    OzGemm<T> g{dA, dB, xA, xB, m, n, mp, np, ks, (int)tiles, sign, add, C + b0 * sC, ldc, sC, err,
+                wait_cap == 0 ? kOzWaitCap : (wait_cap < 0 ? 0 : wait_cap)};
     oz_gemm_kernel<T><<<(int)(tiles < sms ? tiles : sms), OZ_THREADS, oz_smem<T>(), st>>>(g);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -614,13 +629,15 @@ size_t oz_bytes(int m, int n, int k, bool fp64) {
 
 cudaError_t oz_gemm(cudaStream_t st, int batch, int m, int n, int k, int sign, const double2* A, int lda, long long sA,
                     int opA, const double2* B, int ldb, long long sB, int add, double2* C, int ldc, long long sC,
-                    void* work, size_t work_bytes, int* err) {
-  return oz_gemm_t<double2>(st, batch, m, n, k, sign, A, lda, sA, opA, B, ldb, sB, add, C, ldc, sC, work, work_bytes, err);
+                    void* work, size_t work_bytes, int* err, int wait_cap) {
+  return oz_gemm_t<double2>(st, batch, m, n, k, sign, A, lda, sA, opA, B, ldb, sB, add, C, ldc, sC, work, work_bytes, err,
+                            wait_cap);
 }
 cudaError_t oz_gemm(cudaStream_t st, int batch, int m, int n, int k, int sign, const float2* A, int lda, long long sA,
                     int opA, const float2* B, int ldb, long long sB, int add, float2* C, int ldc, long long sC, void* work,
-                    size_t work_bytes, int* err) {
-  return oz_gemm_t<float2>(st, batch, m, n, k, sign, A, lda, sA, opA, B, ldb, sB, add, C, ldc, sC, work, work_bytes, err);
+                    size_t work_bytes, int* err, int wait_cap) {
+  return oz_gemm_t<float2>(st, batch, m, n, k, sign, A, lda, sA, opA, B, ldb, sB, add, C, ldc, sC, work, work_bytes, err,
+                           wait_cap);
 }
 
 }  // namespace rsfd

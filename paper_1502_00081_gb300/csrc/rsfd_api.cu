@@ -143,6 +143,7 @@ int handle_dyson_kind(Handle* h) {
   if (h->opts.dyson_kind != RSFD_DYSON_AUTO) return h->opts.dyson_kind;
   return h->prec == RSFD_FP64 ? RSFD_DYSON_FP64 : RSFD_DYSON_TC;
 }
+int handle_wait_cap(Handle* h) { return h->opts.wait_cap; }
 int handle_dyson_cols(Handle* h) { return h->opts.dyson_cols; }
 int handle_dyson_refine(Handle* h) {
   if (h->opts.dyson_refine > 0) return h->opts.dyson_refine;

@@ -248,6 +248,7 @@ int handle_fd_order(Handle* h);
 double handle_h(Handle* h);
 int handle_dyson_kind(Handle* h);     // resolved: RSFD_DYSON_FP64 or RSFD_DYSON_TC
 int handle_dyson_refine(Handle* h);   // FP64 refinement steps of the Dyson solve
+int handle_wait_cap(Handle* h);       // the solve option wait_cap
 int handle_dyson_cols(Handle* h);     // 0: every column of G_bb; 1: the left slab's columns only
 
 // Tensor-core building blocks of the Dyson step (tc_gemm.cu).  err: device flag set when a bounded
@@ -258,14 +259,14 @@ cudaError_t cgemm_tf32x3(cudaStream_t st, int batch, int m, int n, int k, float2
 
 // Complex GEMM on the tensor cores by digit slices (oz_gemm.cu): C = sign op(A) B + (add ? C : 0), op = N or
 // conjugate transpose, batched, FP64-accurate (double2) or FP32-accurate (float2); work holds at least
-// oz_bytes(m, n, k, fp64); err is set when a bounded wait expires.
+// oz_bytes(m, n, k, fp64); err is set when a bounded wait expires (wait_cap: the solve option of that name).
 size_t oz_bytes(int m, int n, int k, bool fp64);
 cudaError_t oz_gemm(cudaStream_t st, int batch, int m, int n, int k, int sign, const double2* A, int lda, long long sA,
                     int opA, const double2* B, int ldb, long long sB, int add, double2* C, int ldc, long long sC,
-                    void* work, size_t work_bytes, int* err);
+                    void* work, size_t work_bytes, int* err, int wait_cap);
 cudaError_t oz_gemm(cudaStream_t st, int batch, int m, int n, int k, int sign, const float2* A, int lda, long long sA,
                     int opA, const float2* B, int ldb, long long sB, int add, float2* C, int ldc, long long sC, void* work,
-                    size_t work_bytes, int* err);
+                    size_t work_bytes, int* err, int wait_cap);
 
 // Dyson / transmission launchers (dyson.cu).
 rsfd_status dyson_run(Handle* h, const void* G0, const void* SL, const void* SR, int K, void* G, double* refres);
