@@ -290,7 +290,8 @@ static int split_tile_x(int nx, int most) {
 }
 
 // Tile of the FP64 split pass when it is not given: equal tiles with at most 512 points, by the fewest thread slots per
-// grid point (ragged edges, partly filled warps), a tenth of the halo's share and a quarter warp per CTA.
+// grid point (ragged edges, partly filled warps), a tenth of the halo's share and a quarter warp per CTA.  At most 64 rows,
+// as in split_tile_blocks: a TMA box has at most 256, and the deepest prefetch of a taller box does not fit in shared memory.
 static void split_tile(int R, int nx, int ny, int& tx, int& ty) {
   double best = 1e30;
   for (int nt = 1; nt <= nx; ++nt) {
@@ -299,7 +300,7 @@ static void split_tile(int R, int nx, int ny, int& tx, int& ty) {
     if (X < 8 && nt > 1) break;
     for (int mt = 1; mt <= ny; ++mt) {
       const int Y = ((ny + mt - 1) / mt + 1) / 2 * 2;
-      if (X * Y > split_max_points()) continue;
+      if (X * Y > split_max_points() || Y > 64) continue;
       const int warps = (X * Y / 2 + 31) / 32;
       const double slots = (double)((nx + X - 1) / X) * ((ny + Y - 1) / Y) * (warps * 64.0) / ((double)nx * ny);
       const double halo = (double)(X + 4) * (Y + 2 * R) / ((double)X * Y) - 1.0;
