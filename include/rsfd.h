@@ -279,8 +279,9 @@ rsfd_status rsfd_shifted_cocg_aux(rsfd_handle h, const int64_t* cols, int32_t nc
  * `slots` boundary columns at the given energies for every candidate pass form, tile height, rows per
  * thread and z-chunk, at the RHS block width `slots` and the handle's collapse length, and keeps the
  * candidate with the least device time per (column, iteration).  The result is applied to the handle
- * (rsfd_set_solve_options) and cached for the process by (grid, order, precision, projectors, K,
- * slots); the Dyson options and the profile flag are kept.
+ * (rsfd_set_solve_options) and cached for the process by (grid, order, precision, projectors, recorded rows, K,
+ * slots, iters_per_sync).  Only the launch shape (pass_kind, tile_y, tile_x, rows_per_thread, z_chunk, reg_budget,
+ * slots and a split pass's prefetch) is set; the handle's other options are kept.
  *   energies host [K];  eta > 0;  slots >= 1 (at most the number of boundary rows is used);
  *   best (nullable) receives the options;  us_per_slot_iteration (nullable) the measured time.
  * The trial solves allocate their own output buffer.  RSFD_ERR_ARG on bad arguments,

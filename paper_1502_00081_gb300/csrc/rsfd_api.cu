@@ -14,6 +14,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <array>
 #include <exception>
 #include <new>
 #include <map>
@@ -1237,40 +1238,43 @@ void rsfd_destroy(rsfd_handle h) {
 // Launch-option autotuner: short solves (iters seed iterations, profile events on) of the handle's
 // first boundary columns at the caller's energies for every candidate (pass form, tile height, rows
 // per thread, z-chunk), keeping the least device time per slot-iteration.  Results are cached per
-// process by (grid, order, precision, projectors, K, slots).
-struct TuneKey {
-  int nx, ny, nz, fd, prec, proj, K, slots;
-  bool operator<(const TuneKey& o) const {
-    const int a[8] = {nx, ny, nz, fd, prec, proj, K, slots};
-    const int b[8] = {o.nx, o.ny, o.nz, o.fd, o.prec, o.proj, o.K, o.slots};
-    return std::lexicographical_compare(a, a + 8, b, b + 8);
-  }
-};
+// process by (grid, order, precision, projectors, recorded rows, K, slots, chunk length).  Only the launch shape is tuned and
+// cached; the caller's other options stay the caller's.
+typedef std::array<int, 10> TuneKey;
 static std::mutex g_tune_mu;
 static std::map<TuneKey, std::pair<rsfd_solve_opts, double>> g_tune_cache;
+
+static rsfd_solve_opts with_launch_shape(rsfd_solve_opts o, const rsfd_solve_opts& tuned, int iters_per_sync) {
+  o.pass_kind = tuned.pass_kind;
+  o.rows_per_thread = tuned.rows_per_thread;
+  o.tile_y = tuned.tile_y;
+  o.tile_x = tuned.tile_x;
+  o.z_chunk = tuned.z_chunk;
+  o.reg_budget = tuned.reg_budget;
+  o.slots = tuned.slots;
+  if (is_split(tuned.pass_kind)) o.prefetch = tuned.prefetch;   // the split pass tunes its depth
+  o.iters_per_sync = iters_per_sync;
+  return o;
+}
 
 static rsfd_status rsfd_autotune_impl(rsfd_handle h, const double* energies, int32_t K, double eta, int32_t slots, int32_t iters,
                           rsfd_solve_opts* best, double* us_per_slot_iteration) {
   if (!h || !energies || K < 1 || !(eta > 0) || slots < 1 || iters < 1)
     return fail(h, RSFD_ERR_ARG, "rsfd_autotune: bad argument");
   const int ncols = std::min<long long>(slots, (long long)h->brow.size());
-  const TuneKey key{h->nx, h->ny, h->nz, h->fd_order, h->prec, h->n_atoms > 0 ? 1 : 0, (int)K, ncols};
+  const rsfd_solve_opts keep = h->opts;
+  const int C = keep.iters_per_sync > 0 ? keep.iters_per_sync : 32;
+  const TuneKey key{h->nx, h->ny, h->nz, h->fd_order, h->prec, h->n_atoms > 0 ? 1 : 0, h->nr, (int)K, ncols, C};
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tune_cache.find(key);
     if (it != g_tune_cache.end()) {
-      rsfd_solve_opts o = it->second.first;
-      o.profile = h->opts.profile;
-      o.dyson_kind = h->opts.dyson_kind;
-      o.dyson_refine = h->opts.dyson_refine;
-      h->opts = o;
-      if (best) *best = o;
+      h->opts = with_launch_shape(keep, it->second.first, C);
+      if (best) *best = h->opts;
       if (us_per_slot_iteration) *us_per_slot_iteration = it->second.second;
       return RSFD_OK;
     }
   }
-  const rsfd_solve_opts keep = h->opts;
-  const int C = keep.iters_per_sync > 0 ? keep.iters_per_sync : 32;
   const int maxit = std::max<int>(iters, 2 * C);
   std::vector<int64_t> cols(h->brow.begin(), h->brow.begin() + ncols);
   void* G0 = nullptr;
@@ -1371,15 +1375,12 @@ static rsfd_status rsfd_autotune_impl(rsfd_handle h, const double* energies, int
     h->opts = keep;
     return fail(h, RSFD_ERR_CUDA, "rsfd_autotune: no candidate ran");
   }
-  best_o.profile = keep.profile;
-  best_o.use_graphs = keep.use_graphs;
-  if (!is_split(best_o.pass_kind)) best_o.prefetch = keep.prefetch;   // the split pass tunes its depth
-  h->opts = best_o;
+  h->opts = with_launch_shape(keep, best_o, C);
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     g_tune_cache[key] = std::make_pair(best_o, best_us);
   }
-  if (best) *best = best_o;
+  if (best) *best = h->opts;
   if (us_per_slot_iteration) *us_per_slot_iteration = best_us;
   return RSFD_OK;
 }
