@@ -724,14 +724,16 @@ rsfd_status lead_decimation_run(Handle* h, const double* VL, const double* VR, c
     for (int c = 0; c < n; ++c) H01T[(size_t)c * n + r] = H01[(size_t)r * n + c];
   // per matrix (an energy has two, the right and the left lead's): eps_s, eps, [alpha; beta], A (LU), Y and rhs (n x 2n),
   // P (2n x 2n)
-  const long long per = 2 * (n2 * 13 * (long long)sizeof(double2) + (n + 1 + lu_swap_ints(n)) * (long long)sizeof(int) + 64);
+  const long long per = n2 * 13 * (long long)sizeof(double2) + (n + 1 + lu_swap_ints(n)) * (long long)sizeof(int) + 64;
   size_t free_b = 0, tot_b = 0;
   DY_CK(h, cudaMemGetInfo(&free_b, &tot_b));
-  long long kc = (long long)(0.5 * (double)free_b) / per;
+  const long long fit = (long long)(0.5 * (double)free_b) / per;
+  const int nl = fit < 2 ? 1 : 2;   // both leads in one batch, or one after the other where memory is short
+  long long kc = fit / nl;
   if (kc > K) kc = K;
   if (kc > 32767) kc = 32767;
   if (kc < 1) kc = 1;
-  const int Kc = (int)kc, Bc = 2 * Kc;
+  const int Kc = (int)kc, Bc = nl * Kc;
   rsfd_status s;
   void *pW, *pC, *pPiv, *pZ;
   if ((s = handle_ensure(h, 1, (size_t)n2 * 13 * Bc * sizeof(double2), &pW)) != RSFD_OK) return s;
@@ -756,20 +758,22 @@ rsfd_status lead_decimation_run(Handle* h, const double* VL, const double* VR, c
   DY_CK(h, cudaMemcpyAsync(dH01, H01.data(), n2 * sizeof(double2), cudaMemcpyHostToDevice, st));
   DY_CK(h, cudaMemcpyAsync(dH01T, H01T.data(), n2 * sizeof(double2), cudaMemcpyHostToDevice, st));
   int it_max = 0;
+  for (int l0 = 0; l0 < 2; l0 += nl)   // lead 0: right, 1: left
   for (int k0 = 0; k0 < K; k0 += Kc) {
-    const int kb = K - k0 < Kc ? K - k0 : Kc, nm = 2 * kb;   // matrices 0 .. kb - 1: right leads, kb .. 2 kb - 1: left leads
+    const int kb = K - k0 < Kc ? K - k0 : Kc, nm = nl * kb;   // matrices q kb .. q kb + kb - 1 are lead l0 + q's
     const long long tot = n2 * kb;
     std::vector<double2> Zh(kb);
     for (int k = 0; k < kb; ++k) Zh[k] = make_double2(E[k0 + k], eta);
     DY_CK(h, cudaMemcpyAsync(dZ, Zh.data(), kb * sizeof(double2), cudaMemcpyHostToDevice, st));
-    for (int lead = 0; lead < 2; ++lead) {
-      const double2* h0 = lead == 0 ? dH00R : dH00L;
-      bcast_c128<<<grid_for(tot), 256, 0, st>>>(h0, eps_s + lead * tot, n2, kb);
-      bcast_c128<<<grid_for(tot), 256, 0, st>>>(h0, eps + lead * tot, n2, kb);
+    for (int q = 0; q < nl; ++q) {
+      const double2* h0 = l0 + q == 0 ? dH00R : dH00L;
+      bcast_c128<<<grid_for(tot), 256, 0, st>>>(h0, eps_s + q * tot, n2, kb);
+      bcast_c128<<<grid_for(tot), 256, 0, st>>>(h0, eps + q * tot, n2, kb);
     }
     // rhs = [alpha_0 | beta_0]: right [H01 | H01^T], left [H01^T | H01]
     for (int k = 0; k < nm; ++k) {
-      const double2 *a0 = k < kb ? dH01 : dH01T, *b0 = k < kb ? dH01T : dH01;
+      const bool right = l0 + k / kb == 0;
+      const double2 *a0 = right ? dH01 : dH01T, *b0 = right ? dH01T : dH01;
       DY_CK(h, cudaMemcpyAsync(rhs + k * 2 * n2, a0, n2 * sizeof(double2), cudaMemcpyDeviceToDevice, st));
       DY_CK(h, cudaMemcpyAsync(rhs + k * 2 * n2 + n2, b0, n2 * sizeof(double2), cudaMemcpyDeviceToDevice, st));
     }
@@ -796,16 +800,18 @@ rsfd_status lead_decimation_run(Handle* h, const double* VL, const double* VR, c
     }
     it_max = it > it_max ? it : it_max;
     // g_s = (Z - eps_s)^{-1}:  Sigma_R = H01 g_s H01^T, Sigma_L = H01^T g_s H01
-    zi_minus<<<grid_for(2 * tot), 256, 0, st>>>(A, eps_s, dZ, n, nm, kb);
+    zi_minus<<<grid_for(nl * tot), 256, 0, st>>>(A, eps_s, dZ, n, nm, kb);
     DY_CK(h, cudaMemsetAsync(info, 0, nm * sizeof(int), st));
     lu_factor(gc, A, n, nm, perm, info, swp);
-    bcast_c128<<<grid_for(tot), 256, 0, st>>>(dH01T, rhs, n2, kb);
-    bcast_c128<<<grid_for(tot), 256, 0, st>>>(dH01, rhs + tot, n2, kb);
+    for (int q = 0; q < nl; ++q) bcast_c128<<<grid_for(tot), 256, 0, st>>>(l0 + q == 0 ? dH01T : dH01, rhs + q * tot, n2, kb);
     const double2* dinv = lu_inverses(gc, A, n, nm, n, 0);
     lu_permute(gc, rhs, n, nm, perm, Y, n);
     lu_solve(gc, A, n, nm, Y, n, dinv, 0);
-    gemm(gc, kb, n, n, n, 1.0, dH01, n, 0, 0, Y, n, n2, false, (double2*)SRo + n2 * k0, n, n2);
-    gemm(gc, kb, n, n, n, 1.0, dH01T, n, 0, 0, Y + tot, n, n2, false, (double2*)SLo + n2 * k0, n, n2);
+    for (int q = 0; q < nl; ++q) {
+      const bool right = l0 + q == 0;
+      gemm(gc, kb, n, n, n, 1.0, right ? dH01 : dH01T, n, 0, 0, Y + q * tot, n, n2, false,
+           (double2*)(right ? SRo : SLo) + n2 * k0, n, n2);
+    }
     std::vector<int> hinfo(nm);
     DY_CK(h, cudaMemcpyAsync(hinfo.data(), info, nm * sizeof(int), cudaMemcpyDeviceToHost, st));
     if ((s = gemm_end(gc, "rsfd_lead_sigma_decimation")) != RSFD_OK) return s;
