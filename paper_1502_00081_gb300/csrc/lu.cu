@@ -107,10 +107,13 @@ template <int W> __device__ void swap_list(const int* piv, int j0, int jw, int* 
   out[32 + lane] = label;
 }
 
-// Pivot keys: the leading word of the pivot measure, ordered like it as an integer (-1 for NaN).  The search compares
-// FP64 measures to 20 bits, which moves the growth bound by 1e-6 and takes it off the FP64 pipe.
+// Pivot keys: the leading word of the pivot measure, ordered like it as an integer (-1 for NaN, 0 only for 0).  The search
+// compares FP64 measures to 20 bits, which moves the growth bound by 1e-6 and takes it off the FP64 pipe.
 __device__ __forceinline__ int pivot_key(float v) { return v == v ? __float_as_int(v) : -1; }
-__device__ __forceinline__ int pivot_key(double v) { return v == v ? __double2hiint(v) : -1; }
+__device__ __forceinline__ int pivot_key(double v) {
+  const int hi = __double2hiint(v);
+  return v == v ? (hi == 0 && __double2loint(v) != 0 ? 1 : hi) : -1;
+}
 
 // Factorise columns j0 .. j0 + jw - 1 (jw <= W <= 16) of matrix blockIdx.y, rows j0 .. nb - 1; grid (cluster size, K).
 // Ties in the pivot search go to the lowest row.  What a column step waits for: two warp reductions, one block
@@ -216,8 +219,7 @@ __global__ void __launch_bounds__(kPanelThreads) lu_panel(T* M, int nb, int j0, 
       const T inv = none ? T() : s_cand[par][pr][W];
       if (rank == 0 && tid == 0) {
         s_piv[jj] = gp;
-        // a pivot of measure zero (key 0 also stands for FP64 measures below the range of a leading word)
-        if ((none || key == 0) && !(N::mag(prow[0]) > 0) && info[b] == 0) info[b] = gj + 1;
+        if ((none || key == 0) && info[b] == 0) info[b] = gj + 1;   // no pivot, or one of measure zero
       }
 #pragma unroll
       for (int r = 0; r < RPT; ++r) {
