@@ -113,8 +113,8 @@ typedef enum {
                               complex64: with the sums in RSFD_PASS_STORED's blocks, so the two agree bit for bit; FP64:
                               sums in other blocks, the two agree to FP64 round-off), RSFD_PASS_STORED
                               when tile_y, tile_x = 16, rows_per_thread > 1, reg_budget or prefetch is given;
-                              rsfd_autotune times every form (on the 64^2 x 128 workload it picks
-                              RSFD_PASS_SPLIT_BFP for double-float) */
+                              rsfd_autotune times every form in several launch shapes (on the 64^2 x 128 workload
+                              it picks RSFD_PASS_SPLIT_BFP for double-float) */
   RSFD_PASS_RECOMPUTE = 1, /* three vectors per iteration (r_{n-1}, r_{n-2} in, r_n out); A r_{n-1} is
                               recomputed on the tile plus halo and A r_n again for the dot products */
   RSFD_PASS_STORED = 2,    /* five vectors per iteration (r_{n-1}, r_{n-2}, A r_{n-1} in; r_n, A r_n out);
@@ -281,7 +281,9 @@ rsfd_status rsfd_shifted_cocg_aux(rsfd_handle h, const int64_t* cols, int32_t nc
  * candidate with the least device time per (column, iteration).  The result is applied to the handle
  * (rsfd_set_solve_options) and cached for the process by (grid, order, precision, projectors, recorded rows, K,
  * slots, iters_per_sync).  Only the launch shape (pass_kind, tile_y, tile_x, rows_per_thread, z_chunk, reg_budget,
- * slots and a split pass's prefetch) is set; the handle's other options are kept.
+ * slots and a split pass's prefetch) is set; the handle's other options are kept.  The pass that an untuned
+ * complex64 or FP64 handle runs is among the candidates (complex64: pass_kind RSFD_PASS_AUTO; FP64: RSFD_PASS_SPLIT
+ * with tile_y = 0).
  *   energies host [K];  eta > 0;  slots >= 1 (at most the number of boundary rows is used);
  *   best (nullable) receives the options;  us_per_slot_iteration (nullable) the measured time.
  * The trial solves allocate their own output buffer.  RSFD_ERR_ARG on bad arguments,

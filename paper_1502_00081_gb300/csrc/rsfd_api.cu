@@ -345,7 +345,7 @@ static int resolve_rows(int opt) {
 static bool tile_ok(int prec, int R, int tile_y, int kind, int rows, int budget = 0, int tile_x = 32) {
   if (tile_y < 1) return false;
   if (is_split(kind)) {
-    // one row per thread, 32-wide tiles, at most 16 rows (512 threads)
+    // in terms of blocks of 32 x tile_y columns: at most 16 rows, the options of the stored pass's tile unset
     if (tile_x != 32 || rows != 1 || tile_y > 16) return false;
     return split_smem(prec, R, 32, (tile_y + 1) / 2 * 2, 1) <= (size_t)(216 * 1024);
   }
@@ -770,9 +770,7 @@ static rsfd_status rsfd_shifted_cocg_impl(rsfd_handle h, const int64_t* cols, in
   d.nvec = d.kind == RSFD_PASS_RECOMPUTE ? 3 : 5;
   d.rows = is_split(d.kind) ? 1 : resolve_rows(h->opts.rows_per_thread);
   d.tile_y = h->opts.tile_y > 0 ? h->opts.tile_y : default_tile_y(prec, h->R, h->ny, d.kind, d.rows);
-  d.regs = (prec == RSFD_DF64 && d.rows == 1 && (d.kind == RSFD_PASS_STORED || d.kind == RSFD_PASS_SPLIT_BFP))
-               ? h->opts.reg_budget
-               : 0;
+  d.regs = (prec == RSFD_DF64 && d.rows == 1 && d.kind == RSFD_PASS_STORED) ? h->opts.reg_budget : 0;
   d.tile_x = (h->opts.tile_x == 16 && d.kind == RSFD_PASS_STORED) ? 16 : 32;
   if (!tile_ok(prec, h->R, d.tile_y, d.kind, d.rows, d.regs, d.tile_x))
     return fail(h, RSFD_ERR_ARG, "rsfd_shifted_cocg: invalid tile_y / tile_x");
@@ -1252,7 +1250,8 @@ static rsfd_solve_opts with_launch_shape(rsfd_solve_opts o, const rsfd_solve_opt
   o.z_chunk = tuned.z_chunk;
   o.reg_budget = tuned.reg_budget;
   o.slots = tuned.slots;
-  if (is_split(tuned.pass_kind)) o.prefetch = tuned.prefetch;   // the split pass tunes its depth
+  // a split pass tunes its depth (and the automatic pass is one while no depth is given)
+  if (is_split(tuned.pass_kind) || tuned.pass_kind == RSFD_PASS_AUTO) o.prefetch = tuned.prefetch;
   o.iters_per_sync = iters_per_sync;
   return o;
 }
@@ -1288,6 +1287,22 @@ static rsfd_status rsfd_autotune_impl(rsfd_handle h, const double* energies, int
   std::vector<rsfd_solve_opts> cand;
   const int kinds[4] = {RSFD_PASS_STORED, RSFD_PASS_RECOMPUTE, RSFD_PASS_SPLIT, RSFD_PASS_SPLIT_BFP};
   const int zcs[3] = {0, h->nz, (h->nz + 1) / 2};
+  // First what an untuned handle runs, so that tuning never ends with a slower pass: complex64 the automatic pass; FP64 its
+  // tiles, which the split pass takes when no height is given; double-float has both halves among the candidates below (the
+  // automatic pass's stencil with the given split pass's combine, and the stored pass of the same sums)
+  if (h->prec != RSFD_DF64)
+    for (int zc : zcs) {
+      if ((zc > 0 && zc < 8) || (zc > 0 && h->prec == RSFD_MIXED)) continue;
+      rsfd_solve_opts o = keep;
+      o.pass_kind = h->prec == RSFD_MIXED ? RSFD_PASS_AUTO : RSFD_PASS_SPLIT;
+      o.rows_per_thread = o.tile_y = o.tile_x = o.reg_budget = o.prefetch = 0;
+      o.z_chunk = zc;
+      o.slots = ncols;
+      o.iters_per_sync = C;
+      o.profile = 1;
+      o.use_graphs = 0;
+      cand.push_back(o);
+    }
   for (int kind : kinds) {
     if (kind == RSFD_PASS_SPLIT_BFP && h->prec != RSFD_DF64) continue;
     if (is_split(kind)) {
