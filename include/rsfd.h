@@ -112,6 +112,7 @@ typedef enum {
   RSFD_PASS_AUTO = 0,      /* RSFD_PASS_SPLIT on tiles cut to the grid when the options are not tuned (double-float and
                               complex64: with the sums in RSFD_PASS_STORED's blocks, so the two agree bit for bit; FP64:
                               sums in other blocks, the two agree to FP64 round-off), RSFD_PASS_STORED
+                              for complex64 launches of at most one of its CTAs per SM, and
                               when tile_y, tile_x = 16, rows_per_thread > 1, reg_budget or prefetch is given;
                               rsfd_autotune times every form in several launch shapes (on the 64^2 x 128 workload
                               it picks RSFD_PASS_SPLIT_BFP for double-float) */

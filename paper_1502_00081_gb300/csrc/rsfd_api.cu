@@ -389,6 +389,24 @@ static int default_tile_y(int prec, int R, int ny, int kind, int rows) {
   return best > 0 ? best : 4;
 }
 
+// z-chunk of the stored pass, and of the sums in its blocks: whole z-columns per CTA (no pipeline refill) unless that leaves
+// fewer than ~4 CTAs per SM over W0 columns; not below 16 planes
+static int stored_zchunk(int nz, int tiles, int W0, int sms) {
+  int zc = nz;
+  while (zc > 16 && (long long)tiles * ((nz + zc - 1) / zc) * W0 < 4LL * sms) zc = (zc + 1) / 2;
+  return zc;
+}
+
+// The automatic pass of complex64 handles is the stored pass, bit for bit the same, while that has at most one CTA per SM: an
+// iteration is then one latency-bound launch instead of two.  127 iterations, stored / split: 8 columns of 8 x 8 x 12 5.06 / 5.77
+// ms, 128 of them (128 CTAs) 5.54 / 6.34, 8 columns of 30 x 30 x 20 5.00 / 5.71; 128 of 12 x 12 x 24 (512 CTAs) 8.08 / 6.45.
+static bool few_stored_ctas(const Handle* h, int W0, int sms) {
+  const int ty = default_tile_y(h->prec, h->R, h->ny, RSFD_PASS_STORED, 1);
+  const int tiles = (h->nx + 31) / 32 * ((h->ny + ty - 1) / ty);
+  const int zc = h->opts.z_chunk > 0 ? h->opts.z_chunk : stored_zchunk(h->nz, tiles, W0, sms);
+  return (long long)tiles * ((h->nz + zc - 1) / zc) * W0 <= sms;
+}
+
 }  // namespace rsfd
 
 using namespace rsfd;
@@ -765,6 +783,12 @@ static rsfd_status rsfd_shifted_cocg_impl(rsfd_handle h, const int64_t* cols, in
   d.kreq = Kout;
   d.ncols = ncols;
   d.kind = resolve_kind(prec, h->opts);
+  int W0 = h->opts.slots > 0 ? h->opts.slots : 256;
+  W0 = std::min(W0, ncols);
+  int sms = 152;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
+  if (prec == RSFD_MIXED && h->opts.pass_kind == RSFD_PASS_AUTO && d.kind == RSFD_PASS_SPLIT && few_stored_ctas(h, W0, sms))
+    d.kind = RSFD_PASS_STORED;
   // the projector term follows a pass that stores A r (stored-product or split)
   if (h->n_atoms > 0 && d.kind == RSFD_PASS_RECOMPUTE) d.kind = RSFD_PASS_STORED;
   d.nvec = d.kind == RSFD_PASS_RECOMPUTE ? 3 : 5;
@@ -815,25 +839,18 @@ static rsfd_status rsfd_shifted_cocg_impl(rsfd_handle h, const int64_t* cols, in
   d.tiles_x = !logical ? ltiles_x : (d.tile_x > 32 ? std::max(1, h->nx / 32) : ltiles_x);
   d.rows_cta = logical && d.lty % 2 != 0 ? d.lty : d.tile_y;
   d.tiles_y = (h->ny + d.rows_cta - 1) / d.rows_cta;
-  int W0 = h->opts.slots > 0 ? h->opts.slots : 256;
-  W0 = std::min(W0, ncols);
   if (h->opts.z_chunk > 0) {
     d.zchunk = h->opts.z_chunk;
-  } else {
-    // whole z-columns per CTA (no pipeline refill) unless that leaves fewer than ~4 CTAs per SM
-    int sms = 152;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
+  } else if (is_split(d.kind) && !logical) {
+    // the FP64 split pass, whose sums are not tied to the stored pass's chunk: fewer than 8 warps per SM, down to 4
+    // planes (128 columns of 8 x 8 x 12 in FP64 take 34 us a stencil with one chunk, one warp per SM)
+    const long long warps = split_threads(d.tile_x, d.tile_y) / 32;
     d.zchunk = h->nz;
-    // (the FP64 split pass, whose sums are not tied to the chunk: fewer than 8 warps per SM, down to 4
-    // planes; 128 columns of 8 x 8 x 12 in FP64 take 34 us a stencil with one chunk, one warp per SM)
-    if (is_split(d.kind) && !logical) {
-      const long long warps = split_threads(d.tile_x, d.tile_y) / 32;
-      while (d.zchunk > 4 &&
-             (long long)ltiles_x * ltiles_y * ((h->nz + d.zchunk - 1) / d.zchunk) * W0 * warps < 8LL * sms)
-        d.zchunk = (d.zchunk + 1) / 2;
-    }
-    while (!(is_split(d.kind) && !logical) && d.zchunk > 16 && (long long)ltiles_x * ltiles_y * ((h->nz + d.zchunk - 1) / d.zchunk) * W0 < 4LL * sms)
+    while (d.zchunk > 4 &&
+           (long long)ltiles_x * ltiles_y * ((h->nz + d.zchunk - 1) / d.zchunk) * W0 * warps < 8LL * sms)
       d.zchunk = (d.zchunk + 1) / 2;
+  } else {
+    d.zchunk = stored_zchunk(h->nz, ltiles_x * ltiles_y, W0, sms);
   }
   d.nzchunks = (h->nz + d.zchunk - 1) / d.zchunk;
   d.ctas_per_slot = d.tiles_x * d.tiles_y * d.nzchunks;
@@ -857,8 +874,6 @@ static rsfd_status rsfd_shifted_cocg_impl(rsfd_handle h, const int64_t* cols, in
   }
   d.W = W;
   if (logical && !d.rr_blocks) {
-    int sms = 152;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
     d.ctas_c = split_plane_ctas(h->nz, W, sms);
   } else if (is_split(d.kind)) {
     d.ctas_c = d.rr_blocks ? d.nlog : split_combine_ctas(vec);
