@@ -8,14 +8,19 @@
 //
 // Arithmetic.  Every row of A (column of B) is scaled by a power of two so that its largest component
 // is below 1 and written as a 62-bit fixed-point integer X = rint(x 2^62); X is cut into 8 balanced
-// base-256 digits in [-128, 127] (the leading one within +-65), which are exact in bf16.  A product of
-// digits is at most 2^14, so the tensor core's FP32 sums are exact while a sum has at most 2^10 terms.
-// Digit pairs (i, j) of equal weight 256^-(i+j) share an accumulator; pairs with i + j <= 9 are kept (36
-// of 64; the dropped ones are below 2^-62 of the row and column maxima per term).  The accumulators are
-// emptied every 128 complex k (256 real products): the sums of weights 0..3 then have at most 4 x 256
-// terms and are exact; those of weights 4..7 (2^-32 and less) may round once at 2^-24, below 2^-56.
-// They are added to 64-bit integers, so the k-sum has no further rounding; the result is rounded to
-// FP64 once.  Elements below 2^-9 of their row's (column's) largest lose bits below 2^-63 of it.
+// base-256 digits in [-128, 127] (the leading one within +-64), which are exact in bf16.  A product of
+// digits is at most 2^14 (2^13 with a leading one), so the tensor core's FP32 sums are exact up to 2^24.
+// Digit pairs (i, j), i, j = 0 .. 7, of equal weight 256^-(i+j) share an accumulator; pairs with i + j <= 7 are kept
+// (36 of 64).  The accumulators are emptied every 128 complex k (256 real products): the sums of weights 0 .. 4
+// are then at most 2^24 and exact; those of weights 5, 6 and 7 can reach 1.25, 1.5 and 1.75 x 2^24 (all digits near
+// -128, all products of one sign), where every MMA that adds beyond 2^24 may lose up to 2 units of the weight.  The sums
+// are added to 64-bit integers, so the k-sum has no further rounding, and the result is rounded to FP64 once.
+// Error, in units of the row's scale times the column's (each at most twice the largest component): 7 x 2^-62 per real
+// product from the dropped pairs, 2^-62 from the fixed point, and, only where a sum passes 2^24, up to 20 x 2 x 2^-52 per 128
+// complex k from weight 5 (2^-54.7 per real product).  It is a bound relative to the largest element of the row and of
+// the column, not to each element: elements below 2^-9 of their row's (column's) largest lose bits below 2^-63 of it.
+// Callers whose sums mix parts of very different size cut the k-range between them (dense.cuh).
+// FP32 operands take 30 bits and 4 digits, 10 pairs: all sums exact, 3 x 2^-30 per real product from the dropped pairs.
 //
 // Kernel.  One CTA per SM works through 128 x 32 tiles of complex C: eight accumulators of 128 x 32 for Re and eight for
 // Im fill the 512 columns of tensor memory.  The digit planes are laid out in global memory exactly as
