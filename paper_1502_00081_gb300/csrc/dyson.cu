@@ -751,11 +751,10 @@ rsfd_status lead_decimation_run(Handle* h, const double* VL, const double* VR, c
   int* perm = (int*)pPiv;
   int* info = perm + (long long)Bc * n;
   int* swp = info + Bc;
-  // Solves by the inverses of diagonal blocks only from more than two blocks of 64 rows on: nothing refines these solves, and
-  // where a block is most of the matrix its explicit inverse shows.  Error against the closed form, geometric mean at eta 0.01 to
-  // 0.05, LAPACK / substitution / inverses: 64 rows 2.3e-15 / 2.9e-15 / 3.7e-15, 81 rows 3.2e-15 / 2.9e-15 / 5.0e-15; 200 rows
-  // 4.0e-15 / 4.2e-15 (substitution / inverses), where 16 matrices take 41.0 / 38.1 ms.
-  const bool block_inverses = n > 128;
+  // Solves by substitution: nothing refines them, and explicit inverses of the diagonal blocks show.  Error, geometric means,
+  // substitution / inverses: closed form at eta 0.01 to 0.05, 64 rows 2.9e-15 / 3.7e-15, 81 rows 2.9e-15 / 5.0e-15 (LAPACK 2.3e-15,
+  // 3.2e-15); layers of 200 rows with random potentials against 80-bit arithmetic 3.4e-15 / 5.7e-15.  16 matrices of 200 rows
+  // take 41.0 ms, 38.1 with inverses.
   double2* dZ = (double2*)pZ;
   unsigned long long* dmax = (unsigned long long*)(dZ + Kc);
   DY_CK(h, cudaMemcpyAsync(dH00R, H00R.data(), n2 * sizeof(double2), cudaMemcpyHostToDevice, st));
@@ -796,9 +795,8 @@ rsfd_status lead_decimation_run(Handle* h, const double* VL, const double* VR, c
       // Y = g [alpha | beta] by LU of Z - eps, then P = [alpha; beta] Y
       DY_CK(h, cudaMemsetAsync(info, 0, nm * sizeof(int), st));
       lu_factor(gc, A, n, nm, perm, info, swp);
-      const double2* dinv = block_inverses ? lu_inverses(gc, A, n, nm, 2 * n, 0) : nullptr;
       lu_permute(gc, rhs, n, nm, perm, Y, 2 * n);
-      lu_solve(gc, A, n, nm, Y, 2 * n, dinv, 0);
+      lu_solve(gc, A, n, nm, Y, 2 * n, nullptr, 0);
       gemm(gc, nm, 2 * n, 2 * n, n, 1.0, ab, 2 * n, 2 * n2, 0, Y, n, 2 * n2, false, P, 2 * n, 4 * n2);
       DY_CK(h, cudaMemsetAsync(dmax, 0, nm * sizeof(unsigned long long), st));
       decimation_step<false><<<gs, 256, 0, st>>>(P, eps_s, eps, ab, rhs, A, dZ, n, kb, dmax);
@@ -809,9 +807,8 @@ rsfd_status lead_decimation_run(Handle* h, const double* VL, const double* VR, c
     DY_CK(h, cudaMemsetAsync(info, 0, nm * sizeof(int), st));
     lu_factor(gc, A, n, nm, perm, info, swp);
     for (int q = 0; q < nl; ++q) bcast_c128<<<grid_for(tot), 256, 0, st>>>(l0 + q == 0 ? dH01T : dH01, rhs + q * tot, n2, kb);
-    const double2* dinv = block_inverses ? lu_inverses(gc, A, n, nm, n, 0) : nullptr;
     lu_permute(gc, rhs, n, nm, perm, Y, n);
-    lu_solve(gc, A, n, nm, Y, n, dinv, 0);
+    lu_solve(gc, A, n, nm, Y, n, nullptr, 0);
     for (int q = 0; q < nl; ++q) {
       const bool right = l0 + q == 0;
       gemm(gc, kb, n, n, n, 1.0, right ? dH01 : dH01T, n, 0, 0, Y + q * tot, n, n2, false,

@@ -2,7 +2,8 @@
 // boundary solve (I - G0 Sigma) G = G0 (Eq. sec3-01a) and the lead decimation.
 //
 // Right-looking, two levels.  Outer blocks of 128 (FP32) or 64 (FP64) columns end in one tensor-core product
-// A22 -= L21 U12; FP64 takes the narrower block because the updates inside it run on the FP64 pipe.  Inside an outer block, panels of W columns take three launches:
+// A22 -= L21 U12; FP64 takes the narrower block because the updates inside it run on the FP64 pipe.  Inside an outer block,
+// panels of W columns take three launches:
 //   lu_panel   factorises rows x W: every row of the panel lives in one thread's registers, the rows are
 //              spread over up to 8 CTAs of a cluster, and a column costs one block and one cluster barrier
 //              (the pivot candidates, the pivot row and the row it replaces travel through
@@ -11,7 +12,9 @@
 //              most 2 W rows, and solves with the panel's unit lower triangle for those to its right;
 //   lu_update  the rank-W update of the rest of the outer block.
 // The exchanges then reach the other columns (lu_swap_rest), and U12 = L11^{-1} A12 is a triangular solve.
-// Triangular solves: blocks of 64 (FP64) or 128 (FP32) rows by substitution (lu_trsm), the rest by products.
+// Triangular solves: blocks of 64 (FP64) or 128 (FP32) rows by substitution (lu_trsm), the rest by products.  In the Dyson
+// step no block of a solve holds rows of both slabs (dense.cuh); the factorisation's blocks may, there the parts that a product
+// loses are squares of the coupling beside elements of order 1.
 //
 // Measured (16 matrices of 1024 rows, FP32 LU and two solves of 1024 columns): panel_getrf + laswp + trsm + 3xTF32
 // updates 48 ms before, 11 ms now; 4 of 2048: 123 -> 17 ms; 8 of 512 in FP64 with three solves of 512 columns: 213 ->
@@ -683,7 +686,9 @@ void lu_factor(Gemm& g, float2* M, int nb, int K, int* perm, int* info, int* swp
 }
 // Substitution costs 64 x 63 / 2 FP64 multiply-adds a column and block on the FP64 pipe (70-90 us a block for 400 to 512
 // columns of 8 matrices), a product with the inverse about 25 us; the inverses of all blocks together cost one block's
-// substitution.  Worth it from 2000 columns over the batch on (where gemm() slices the 64 x n x 64 products).
+// substitution.  For solves that are refined: one without refinement loses digits to the explicit inverses (lead_decimation_run).
+// The line lies where gemm() slices the 64 x n x 64 products, at 2000 columns over the batch.  Measured above it, substitution /
+// inverses: Dyson step of 8 x 512 rows (4096 columns) 11.8 / 9.9 ms, of 8 x 240 rows with two interior planes (3840) 5.6 / 4.6 ms.
 const double2* lu_inverses(Gemm& g, const double2* LU, int nb, int K, int nrhs, int split) {
   constexpr int NB = Num<double2>::NBLK;
   if (!g.h || (double)nrhs * K * NB * NB < kSliceMin || nb < NB || (nb == NB && split > 0)) return nullptr;
