@@ -111,7 +111,8 @@ typedef struct {
 typedef enum {
   RSFD_PASS_AUTO = 0,      /* RSFD_PASS_SPLIT on tiles cut to the grid when the options are not tuned (double-float and
                               complex64: with the sums in RSFD_PASS_STORED's blocks, so the two agree bit for bit; FP64:
-                              sums in other blocks, the two agree to FP64 round-off), RSFD_PASS_STORED
+                              sums in other blocks, the two agree to FP64 round-off, and the last digits follow the
+                              number of columns in flight through the z-chunk), RSFD_PASS_STORED
                               for complex64 launches of at most one of its CTAs per SM, and
                               when tile_y, tile_x = 16, rows_per_thread > 1, reg_budget or prefetch is given;
                               rsfd_autotune times every form in several launch shapes (on the 64^2 x 128 workload
@@ -140,8 +141,8 @@ typedef enum {
 typedef enum {
   RSFD_DYSON_AUTO = 0, /* RSFD_DYSON_TC for double-float and complex64 handles, RSFD_DYSON_FP64 for FP64 handles */
   RSFD_DYSON_FP64 = 1, /* LU, triangular solves and refinement in FP64; the matrix products on the tensor cores as
-                          products of exact 8-bit digits, panels and substitution on the CUDA cores */
-  RSFD_DYSON_TC = 2    /* LU and triangular solves in FP32 with their O(nb^3) updates on the tensor cores (exact
+                          products of 8-bit digits, panels and substitution on the CUDA cores */
+  RSFD_DYSON_TC = 2    /* LU and triangular solves in FP32 with their O(nb^3) updates on the tensor cores (8-bit
                           digits; rsfd_cgemm_tf32x3 when there is no memory for them), FP64 residuals and
                           corrections (iterative refinement) */
 } rsfd_dyson_kind;
@@ -352,9 +353,10 @@ rsfd_status rsfd_get_stats(rsfd_handle h, rsfd_stats* out);
  * (ncols = nb).  The solve is an LU with partial pivoting followed by FP64
  * iterative refinement of the residual G0 - (I - G0 Sigma) G.  Form (rsfd_solve_opts.dyson_kind):
  * FP64 LU (FP64 handles by default), or FP32 LU and triangular solves with FP64 residuals (double-float
- * and complex64 handles by default); in both the matrix products run on the tensor cores as products of exact
- * digits (at FP64 or better than FP32 accuracy); the FP32 form processes energies in chunks that fit the free
- * device memory.
+ * and complex64 handles by default); in both the matrix products run on the tensor cores as products of
+ * digits, accurate to 2^-62 (FP32 operands: 2^-30) of the largest element of each row and column, and summed slab by
+ * slab, so that each block of G_bb is accurate relative to its own size, however small G_RL is beside G_LL.  The FP32
+ * form processes energies in chunks that fit the free device memory.
  *   G0_bb    device [K][nb][nb] (handle precision).
  *   Sigma_L, Sigma_R  device [K][ns][ns] c128.
  *   G_bb     device output, same layout and type as G0_bb (may not alias G0_bb).

@@ -1839,7 +1839,7 @@ template <int MODE, bool BFP> __global__ void __launch_bounds__(kCombThreads, 4)
 // Combine with its sums in the stored pass's blocks, double-float and complex64: CTA = one block of 32 x lty columns and a
 // z-chunk, a thread a column, two (complex64: four) planes per step, so that six 16-byte (twelve 8-byte) loads are in flight; a
 // warp reads rows of 512 (256) bytes.  Grids of at most 16 (8) columns put two (four) rows into a warp: the missing columns
-// of a row add zeros, which change no sum.
+// of a row add zeros, which change no sum.  Bound: HBM (38 columns of 64 x 64 x 128: 6.4 TB/s in double-float, 6.2 in complex64).
 template <int MODE> __global__ void __launch_bounds__(kCombThreads, 4) combine_blocks_kernel(PassParams p) {
   typedef Ops<MODE> O;
   typedef Stencil<MODE, 1> ST;
@@ -1928,7 +1928,8 @@ template <int MODE> __global__ void __launch_bounds__(kCombThreads, 4) combine_b
 // Double-float and complex64 vectors (LOG): the rounding of the sums is that of blocks of 32 x d.lty columns and a z-chunk (a
 // warp a row, the rows in order), whatever tile the CTA has: a tile is made of such blocks, every column keeps its own
 // accumulators over the z-range, and they are added in that order at the end.  The recurrence amplifies a changed last bit
-// of a sum to 1e-8 of G0_bb in double-float and to 1e-5 (single elements: 1e-3 of the rms) in complex64.
+// of a sum to 1e-8 of G0_bb in double-float and to 1e-5 (single elements: 1e-3 of the rms) in complex64.  64 columns of 56 x 56 x 80
+// in complex64: 78 us a launch (85 with products formed exactly).
 // BFP (double-float handles): the r_n it reads has block-floating-point leading parts, tmV maps s V, and it
 // stores u_n = s A r_n (StencilBFP) with the largest leading-part component of u_n.
 constexpr int kMaxStagesS = kMaxDepth + 3;
@@ -1941,7 +1942,7 @@ __global__ void __launch_bounds__(kStencilThreads, MODE == RSFD_MIXED ? 3 : 2)
 stencil_kernel(PassParams p, const __grid_constant__ CUtensorMap tmR, const __grid_constant__ CUtensorMap tmV) {
   static_assert(!BFP || MODE == RSFD_DF64, "the block-floating-point pass is double-float only");
   constexpr bool LOG = MODE != RSFD_FP64;
-  // The plain double-float stencil takes 320 instructions a point; unrolled over the 2R + 1 ring positions its loop
+  // The plain double-float stencil takes about 300 instructions a point; unrolled over the 2R + 1 ring positions its loop
   // does not fit the instruction cache (the first stall reason), so it moves the ring's registers instead: 63
   // iterations of 1024 slots of 16 x 16 x 48 in 39.2 instead of 44.3 ms.
   constexpr bool ROT = MODE == RSFD_DF64 && !BFP && R == 2;
@@ -2858,14 +2859,14 @@ size_t split_smem(int prec, int R, int tile_x, int tile_y, int depth) {
   const size_t ac = prec != RSFD_FP64 ? (size_t)split_threads(tile_x, tile_y) * 2 * 16 : 0;
   return (size_t)(depth + R + 1) * (pb + pv) + ac + 128;
 }
-// Combine CTAs per slot.  Plain ranges: by the vector's length alone, so that a column's sums do not depend on how
-// many columns run beside it: 2048 16-byte units per CTA (four steps of its 256 threads), at most 64 CTAs (longer
-// ranges from there on).
+// Combine CTAs per slot.  Plain ranges (FP64): by the vector's length alone, 2048 elements per CTA (four steps of its 256
+// threads), at most 64 CTAs (longer ranges from there on).  So a column's (r, r) does not depend on how many columns run beside
+// it; its (r, A r) does, in the last digits, through the z-chunk.
 int split_combine_ctas(long long vec) {
   const long long c = vec / 2048;
   return (int)(c < 1 ? 1 : (c > 64 ? 64 : c));
 }
-// Ranges of planes (double-float, with its sums): about eight 256-thread CTAs per SM over all slots, at least one
+// Ranges of planes (double-float and complex64, with their sums): about eight 256-thread CTAs per SM over all slots, at least one
 // plane each
 int split_plane_ctas(int nz, int W, int sms) {
   int c = (8 * sms + W - 1) / W;

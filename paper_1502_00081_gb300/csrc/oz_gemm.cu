@@ -31,9 +31,9 @@
 // weights i-1..7.  18 warps: 16 read the accumulators, one thread of the 17th issues the copies,
 // one thread of the 18th the MMAs.
 //
-// Bound: tensor rate (144 real bf16 MACs per complex FP64 MAC, 40 per FP32 one; 36 B per clock and SM of operands from L2).
-// Measured: 16 products of 1024^3 in 4.0 ms, 4.3e12 complex multiply-adds/s, 1.24 PFLOP/s of bf16 MMAs = 0.64 of the
-// measured cuBLAS bf16 burst (132 ms on the FP64 pipe, 1.3e11/s).  One tile per CTA instead of a persistent CTA, so
+// Bound: tensor rate (144 real bf16 MACs per complex FP64 MAC, 40 per FP32 one; 36 B per clock and SM of operands from L2
+// at full rate).  Measured: 16 products of 1024^3 in 4.0 ms, 4.3e12 complex multiply-adds/s, 1.24 PFLOP/s of bf16 MMAs = 0.64
+// of the measured cuBLAS bf16 burst, tensor pipe active in 55 % of the cycles (132 ms on the FP64 pipe, 1.3e11/s).  One tile per CTA instead of a persistent CTA, so
 // that a tile's set-up and write-back are not hidden: 4.6 ms, and 157 instead of 96 us for the FP32 LU's k = 128 updates.
 
 #include <cuda_runtime.h>
