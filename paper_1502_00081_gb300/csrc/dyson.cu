@@ -754,7 +754,7 @@ rsfd_status lead_decimation_run(Handle* h, const double* VL, const double* VR, c
   // Solves by substitution: nothing refines them, and explicit inverses of the diagonal blocks show.  Error, geometric means,
   // substitution / inverses: closed form at eta 0.01 to 0.05, 64 rows 2.9e-15 / 3.7e-15, 81 rows 2.9e-15 / 5.0e-15 (LAPACK 2.3e-15,
   // 3.2e-15); layers of 200 rows with random potentials against 80-bit arithmetic 3.4e-15 / 5.7e-15.  16 matrices of 200 rows
-  // take 41.0 ms, 38.1 with inverses.
+  // take 38.9 ms, 38.1 with inverses.
   double2* dZ = (double2*)pZ;
   unsigned long long* dmax = (unsigned long long*)(dZ + Kc);
   DY_CK(h, cudaMemcpyAsync(dH00R, H00R.data(), n2 * sizeof(double2), cudaMemcpyHostToDevice, st));
